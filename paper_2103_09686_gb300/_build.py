@@ -12,7 +12,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(PKG, "libdmcr.so")
 BUILD_DIR = os.path.join(PKG, "_build")
-SOURCES = ["corr.cu", "aux.cu", "fft.cu", "gram.cu", "api.cu"]
+SOURCES = ["corr.cu", "sep.cu", "aux.cu", "fft.cu", "gram.cu", "api.cu"]
 # the benchmark's pipe-rate microbenchmark: a library of its own, not part of the C ABI
 PIPES_SRC = "pipes.cu"
 PIPES_LIB = os.path.join(PKG, "libdmcr_pipes.so")

@@ -150,6 +150,11 @@ struct Plan {
     int64_t s3Kpad = 0, s3Npad[MAX_LEVELS] = {};
     size_t o_eh[MAX_LEVELS] = {}, o_el[MAX_LEVELS] = {}, o_eth[MAX_LEVELS] = {}, o_etl[MAX_LEVELS] = {},
            o_w[MAX_LEVELS] = {}, o_gh[MAX_LEVELS] = {}, o_gl[MAX_LEVELS] = {}, o_amax[MAX_LEVELS] = {};
+    // separable path (sep.cu): all levels of the instance or none
+    bool sep = false;
+    std::shared_ptr<const SepBasis> basis;
+    size_t o_tier = 0, o_tiers = 0, o_z[MAX_LEVELS] = {}, o_q[MAX_LEVELS] = {}, o_u[MAX_LEVELS] = {},
+           o_v[MAX_LEVELS] = {}, o_sdc[MAX_LEVELS] = {}, o_spart[MAX_LEVELS] = {};
     size_t bytes = 0;
 };
 
@@ -173,14 +178,17 @@ bool fft_cheaper(const LevelGeom& g) {
 }
 
 // Upper bound of the segment-table bytes of one instance (every phase, 16-B aligned arrays).
-size_t table_bound(int levels, int phases) {
+size_t table_bound(const Plan& pl) {
+    const int levels = pl.levels, phases = pl.phases;
     const size_t pp = (size_t)phases * phases;
-    return (size_t)levels *
+    const size_t sep = !pl.sep ? 0 : pl.basis->coef.size() * sizeof(float2) +
+                                         (size_t)levels * (sizeof(SepLevel) + (size_t)SEP_KERNELS * pp * sizeof(SepItem));
+    return sep + (size_t)levels *
                (pp * (sizeof(FwdSeg) + sizeof(RedSeg) + sizeof(GSeg) + sizeof(AdjSeg)) +
                 phases * sizeof(RestrictSeg) + 2 * sizeof(TildeSeg)) +
            sizeof(PenSeg) + sizeof(LossSeg) + phases * sizeof(FinalSeg) + sizeof(InitSeg);
 }
-size_t table_slack() { return (size_t)(16 + MAX_LEVELS) * 16 + 256; }
+size_t table_slack(bool sep) { return (size_t)(16 + MAX_LEVELS + (sep ? 8 + SEP_KERNELS : 0)) * 16 + 256; }
 
 int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
@@ -288,6 +296,56 @@ void plan_level(LevelGeom& g, const int tune[4], int phases, int level) {
         }
     }
     g.nChunks = g.nZc * g.nYc * g.nXc;
+}
+
+// lengths of the window buffers of the separable path, one phase pair (float2 elements)
+int64_t sep_u_len(const LevelGeom& g) { return g.n[0] > 1 ? (int64_t)(g.P[0] + 1) * g.n[1] * g.n[2] : 0; }
+int64_t sep_v_rows(const LevelGeom& g) {
+    return g.n[0] > 1 ? (int64_t)(g.P[0] + 1) * (2 * g.P[1] + 1) : g.P[1] + 1;
+}
+
+// shape of one level for sep.cu (no pointers)
+bool sep_shape(const LevelGeom& g, int phases, int max_pairs, SepLevel& lv) {
+    lv = SepLevel{};
+    for (int a = 0; a < 3; ++a)
+        if (!sep_axis(g.n[a], lv.ax[a])) return false;
+    lv.n0 = (int)g.n[0], lv.n1 = (int)g.n[1], lv.n2 = (int)g.n[2];
+    lv.P0 = g.P[0], lv.P1 = g.P[1], lv.P2 = g.P[2];
+    lv.phases = phases;
+    lv.maxPairs = max_pairs;
+    lv.N = g.N;
+    lv.Khalf = g.Khalf;
+    lv.strideU = sep_u_len(g);
+    lv.strideV = sep_v_rows(g) * g.n[2];
+    lv.rowsF = sep_rows(lv.ax[2], SEP_SLOTS);
+    lv.rowsW = sep_rows(lv.ax[2], 1);
+    lv.colsY = sep_cols(lv.ax[1], true);
+    lv.colsL = lv.n0 > 1 ? sep_cols(lv.ax[0], true) : sep_cols(lv.ax[1], false);
+    return std::max(sep_smem_last(lv, true), sep_smem_feat(lv)) <= (size_t)SEP_MAX_SMEM;
+}
+
+// The separable path for the soft threshold's two-point descriptor: when a basis of this
+// alpha exists, every axis of every level can be transformed, its buffers stay moderate and
+// the direct kernels' pair evaluations cost more.  All levels of an instance or none.
+bool choose_sep(const dmcr_params* p, Plan& pl) {
+    if (p->path != DMCR_PATH_AUTO || p->threshold != DMCR_SOFT || pl.desc_kind == DMCR_DESC_S3) return false;
+    const double ph = pl.phases;
+    double pairs = 0.0, bytes = 0.0, points = 0.0;
+    for (int l = 0; l < pl.levels; ++l) {
+        const LevelGeom& g = pl.g[l];
+        SepLevel lv;
+        if (!sep_shape(g, pl.phases, SEP_MAX_PAIRS, lv)) return false;
+        pairs += ph * ph * (double)g.N * (double)g.Khalf;
+        bytes += 8.0 * SEP_MAX_PAIRS * (double)g.N * ph * (pl.phases > 1 ? 2 : 1);
+        double per = 0.0;
+        for (int a = 0; a < 3; ++a)
+            if (g.n[a] > 1) per += sep_axis_cost(lv.ax[a]);
+        points += ph * (double)g.N * per;
+    }
+    const double t_direct = 4.5e-5 + 5.75e-13 * pairs, t_sep = 1e-4 + points;
+    if (bytes > 8e9 || t_direct < 1.25 * t_sep) return false;
+    pl.basis = sep_basis(p->alpha);
+    return pl.basis->ntier > 0;
 }
 
 dmcr_status validate_and_plan(const dmcr_params* p, Plan& pl) {
@@ -417,6 +475,7 @@ dmcr_status validate_and_plan(const dmcr_params* p, Plan& pl) {
         const double fh = c1 / (1.0 + exp(0.25 * a)) - c1 * s0;
         pl.fh2 = fh * fh;
     }
+    pl.sep = choose_sep(p, pl);
     // App. A: f(1/2) of the threshold (1/2 for f(x) = x)
     pl.q_tilde = (float)(tc.identity ? 0.5 : 2.0 * pl.fh2);
     // the workspace, estimated in floating point first: sizes beyond any device are
@@ -439,12 +498,16 @@ dmcr_status validate_and_plan(const dmcr_params* p, Plan& pl) {
     }
     // workspace layout
     size_t o = 0;
-    pl.tab_bytes = align_up(table_bound(pl.levels, pl.phases) + table_slack());
+    pl.tab_bytes = align_up(table_bound(pl) + table_slack(pl.sep));
     pl.o_tab = o; o += pl.tab_bytes;
     pl.o_scal = o; o = align_up(o + sizeof(Scalars));
     pl.o_pen = o; o = align_up(o + 3 * NPEN_BLOCKS * sizeof(double));
     pl.o_desc = o; o = align_up(o + (size_t)pl.Ktot * sizeof(float));
     pl.o_tsum = o; o = align_up(o + (size_t)MAX_LEVELS * sizeof(float));
+    if (pl.sep) {
+        pl.o_tier = o; o = align_up(o + sizeof(int));
+        pl.o_tiers = o; o = align_up(o + SEP_RANGE_BLOCKS * sizeof(int));
+    }
     for (int l = 0; l < pl.levels; ++l) {
         const LevelGeom& g = pl.g[l];
         const size_t ph = (size_t)pl.phases;
@@ -465,6 +528,25 @@ dmcr_status validate_and_plan(const dmcr_params* p, Plan& pl) {
             pl.o_gh[l] = o; o = align_up(o + Kp * Kp * sizeof(uint16_t));
             pl.o_gl[l] = o; o = align_up(o + Kp * Kp * sizeof(uint16_t));
             pl.o_amax[l] = o; o = align_up(o + 2 * sizeof(float));
+        } else if (pl.sep) {
+            // gradient of the level and window means, then the buffers of the path that runs:
+            // spectra (separable) or partials and coefficients (direct, for fields outside the
+            // separable ranges) -- a call uses one of the two
+            const size_t pp = ph * ph;
+            pl.o_spart[l] = o; o = align_up(o + ph * g.N * sizeof(float));
+            pl.o_sdc[l] = o; o = align_up(o + pp * sizeof(double));
+            const size_t start = o;
+            pl.o_z[l] = o; o = align_up(o + ph * pl.basis->max_pairs * g.N * sizeof(float2));
+            pl.o_q[l] = pl.o_z[l];
+            if (ph > 1) { pl.o_q[l] = o; o = align_up(o + ph * pl.basis->max_pairs * g.N * sizeof(float2)); }
+            pl.o_u[l] = o; o = align_up(o + pp * sep_u_len(g) * sizeof(float2));
+            pl.o_v[l] = o; o = align_up(o + pp * sep_v_rows(g) * g.n[2] * sizeof(float2));
+            size_t d = start;
+            pl.o_fwd[l] = d; d = align_up(d + ph * ph * g.fwdTiles * g.Khalf * sizeof(float));
+            pl.o_gd[l] = d; d = align_up(d + ph * ph * gd_floats(g) * sizeof(float));
+            pl.o_adj[l] = d; d = align_up(d + ph * ph * g.nChunks * g.N * sizeof(float));
+            o = std::max(o, d);
+            continue;
         } else {
             pl.o_fwd[l] = o; o = align_up(o + ph * ph * g.fwdTiles * g.Khalf * sizeof(float));
         }
@@ -486,6 +568,7 @@ dmcr_status prepare_device() {
     set_kernel_attributes();
     set_fft_attributes();
     set_gram_attributes();
+    set_sep_attributes();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_check(e, "cudaFuncSetAttribute");
     ready.push_back(dev);
@@ -561,6 +644,13 @@ struct Prepared {
     R fwd{0, 0, 0}, red{0, 0, 0}, pen{0, 0, 0}, loss{0, 0, 0}, gco{0, 0, 0}, adj{0, 0, 0}, fin{0, 0, 0},
         fin_small{0, 0, 0}, init{0, 0, 0}, tmap{0, 0, 0}, tsum{0, 0, 0};
     size_t smem_fwd = 0, smem_adj = 0;
+    // separable path, and the direct launches of its instances (run only where their gate opens)
+    R sep[SEP_KERNELS] = {};
+    size_t sep_smem[SEP_KERNELS] = {};
+    SepTables sept{};
+    size_t o_sep_level = 0, o_sep_coef = 0;
+    R gfwd{0, 0, 0}, gred{0, 0, 0}, ggco{0, 0, 0}, gadj{0, 0, 0};
+    size_t smem_gfwd = 0, smem_gadj = 0;
     struct FftJob {
         LevelGeom g;
         const float* field;
@@ -633,6 +723,106 @@ S3Job s3_job(const Inst& x, int l, bool loss) {
     return j;
 }
 
+// Tables of the separable path: one SepLevel per (instance, level), one block range per
+// kernel and phase (pair), the basis' coefficients.
+void prepare_sep(const std::vector<Inst>& in, unsigned flags, Prepared& P) {
+    std::vector<SepLevel> levels;
+    std::vector<SepItem> items[SEP_KERNELS];
+    const SepBasis* basis = nullptr;
+    const bool vjp = !(flags & F_LOSS);
+    const int *lv_tier = nullptr, *lv_done = nullptr;
+    auto add = [&](SepKernel k, int a, int b, int64_t blocks, size_t smem) {
+        SepItem it{};
+        it.level = (int)levels.size();
+        it.a = a;
+        it.b = b;
+        it.blockStart = P.sep[k].blocks;
+        it.tier = lv_tier;
+        it.done = lv_done;
+        P.sep[k].blocks += blocks;
+        P.sep_smem[k] = std::max(P.sep_smem[k], smem);
+        items[k].push_back(it);
+    };
+    for (const Inst& x : in) {
+        const Plan& pl = *x.pl;
+        if (!pl.sep) continue;
+        basis = pl.basis.get();
+        for (int l = 0; l < pl.levels; ++l) {
+            const LevelGeom& g = pl.g[l];
+            SepLevel lv;
+            sep_shape(g, pl.phases, basis->max_pairs, lv);
+            lv.field = x.lv[l];
+            lv.Z = reinterpret_cast<float2*>(x.ws + pl.o_z[l]);
+            lv.Q = reinterpret_cast<float2*>(x.ws + pl.o_q[l]);
+            lv.U = reinterpret_cast<float2*>(x.ws + pl.o_u[l]);
+            lv.V = reinterpret_cast<float2*>(x.ws + pl.o_v[l]);
+            lv.dc = reinterpret_cast<double*>(x.ws + pl.o_sdc[l]);
+            lv.tier = reinterpret_cast<int*>(x.ws + pl.o_tier);
+            lv.tiers = reinterpret_cast<int*>(x.ws + pl.o_tiers);
+            const int64_t Nall = pl.N1 * pl.phases;
+            lv.ntiers = (int)std::min<int64_t>(SEP_RANGE_BLOCKS, ceil_div(Nall, 1024));
+            lv.first = l == 0;
+            lv.desc = x.desc + pl.off[l];
+            lv.scaleD = (double)pl.w[l] / ((double)g.N * (double)g.N);
+            if (flags & F_BACK) {
+                lv.src = vjp ? x.target + pl.off[l] : x.desc + pl.off[l];
+                lv.sub = vjp ? nullptr : x.target + pl.off[l];
+                lv.sc = vjp ? nullptr : x.sc;
+                if (pl.desc_kind == DMCR_DESC_S2_TILDE) {
+                    lv.tsum = reinterpret_cast<const float*>(x.ws + pl.o_tsum) + l;
+                    lv.q = pl.q_tilde;
+                }
+                lv.scaleG = (float)((double)pl.w[l] / (double)g.N);
+                lv.part = reinterpret_cast<float*>(x.ws + pl.o_spart[l]);
+            }
+            lv.done = lv_done = x.use_done ? &x.sc->done : nullptr;
+            lv_tier = lv.tier;
+            const bool d3 = lv.n0 > 1;
+            const int64_t rows = (int64_t)lv.n0 * lv.n1;
+            const int64_t fgroups = ceil_div(rows, lv.rowsF);
+            const int64_t xl = ceil_div(lv.n2, lv.colsL), xy = ceil_div(lv.n2, lv.colsY);
+            const int64_t last = d3 ? xl * lv.n1 : xl;
+            // planes of the middle axis side by side in one block
+            const int64_t side = lv.ax[1].fast ? SEP_BLOCK_PTS / (lv.colsY * lv.n1) : 1;
+            const size_t sf = sep_smem_feat(lv), sw = sep_smem_window(lv), sy = d3 ? sep_smem_y(lv) : 0;
+            if (lv.first) add(SEP_RANGE, lv.ntiers, 0, lv.ntiers, 0);
+            for (int a = 0; a < pl.phases; ++a) {
+                add(SEP_FEAT, a, 0, fgroups, sf);
+                if (d3) add(SEP_FFT_Y, a, 0, ceil_div(xy * lv.n0, side) * basis->max_pairs, sy);
+                if (flags & F_BACK) {
+                    add(pl.phases > 1 ? SEP_MUL_PH : SEP_MUL, a, 0, last, sep_smem_last(lv, true));
+                    if (d3) add(SEP_IFFT_Y, a, 0, ceil_div(xy * lv.n0, side) * basis->max_pairs, sy);
+                    add(SEP_GRAD, a, 0, fgroups, sf);
+                }
+                for (int b = 0; b < pl.phases; ++b) {
+                    const int64_t kept = lv.P0 + 1, wrows = sep_v_rows(g);
+                    if (flags & F_FWD) {
+                        add(pl.phases > 1 ? SEP_POWER_PH : SEP_POWER, a, b, last, sep_smem_last(lv, false));
+                        if (d3) add(SEP_INV_Y, a, b, ceil_div(xy * kept, side), sy);
+                        add(SEP_DESC, a, b, ceil_div(wrows, lv.rowsW), sw);
+                    }
+                    if (flags & F_BACK) {
+                        add(SEP_GX, a, b, ceil_div(wrows, lv.rowsW), sw);
+                        if (d3) add(SEP_GY, a, b, ceil_div(xy * kept, side), sy);
+                    }
+                }
+            }
+            levels.push_back(lv);
+        }
+    }
+    if (levels.empty()) return;
+    P.o_sep_level = push(P.tb, levels);
+    P.o_sep_coef = push(P.tb, basis->coef);
+    for (int t = 0; t < SEP_TIERS; ++t) P.sept.tier[t] = basis->tier[t];
+    P.sept.ntier = basis->ntier;
+    P.sept.level = P.at<SepLevel>(P.o_sep_level);
+    P.sept.coef = P.at<float2>(P.o_sep_coef);
+    for (int k = 0; k < SEP_KERNELS; ++k) {
+        P.sep[k].off = push(P.tb, items[k]);
+        P.sep[k].nseg = (int)items[k].size();
+    }
+}
+
 // Build every table of the requested phases; `tab`/`cap` is the device table region.
 dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap, Prepared& P) {
     P.tab = tab;
@@ -687,12 +877,18 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
             FwdSeg f;
             int64_t work, blocks;
         };
-        std::vector<Item> items;
-        std::vector<RedSeg> rv;
-        int64_t rb = 0;
+        std::vector<Item> plain, gated;
+        std::vector<RedSeg> rplain, rgated;
+        int64_t rplain_b = 0, rgated_b = 0;
         for (const Inst& x : in)
             for (int l = 0; l < x.pl->levels; ++l) {
                 const LevelGeom& g = x.pl->g[l];
+                // an instance on the separable path keeps the direct kernels for fields outside its ranges
+                const int* gate = x.pl->sep ? reinterpret_cast<const int*>(x.ws + x.pl->o_tier) : nullptr;
+                std::vector<Item>& items = gate ? gated : plain;
+                std::vector<RedSeg>& rv = gate ? rgated : rplain;
+                int64_t& rb = gate ? rgated_b : rplain_b;
+                size_t& smem = gate ? P.smem_gfwd : P.smem_fwd;
                 if (x.pl->desc_kind == DMCR_DESC_S3) {
                     P.s3f.push_back(s3_job(x, l, true));
                     continue;
@@ -712,6 +908,7 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
                         it.f.tip = x.lv[l] + pb * g.N;
                         it.f.partial = reinterpret_cast<float*>(x.ws + x.pl->o_fwd[l]) + blk * g.fwdTiles * g.Khalf;
                         it.f.done = x.use_done ? &x.sc->done : nullptr;
+                        it.f.gate = gate;
                         it.work = (int64_t)g.TY * g.PPB;
                         it.blocks = g.fwdTiles * g.fwdGroupBlocks;
                         items.push_back(it);
@@ -720,24 +917,30 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
                         r.partial = it.f.partial;
                         r.desc = x.desc + x.pl->off[l] + blk * g.Khalf;
                         r.done = it.f.done;
+                        r.gate = gate;
                         r.scale = (float)((double)x.pl->w[l] / (double)g.N);
                         r.blockStart = rb;
                         rb += ceil_div(g.Khalf, RED_K);
                         rv.push_back(r);
                     }
-                P.smem_fwd = std::max(P.smem_fwd, fwd_smem_bytes(g));
+                smem = std::max(smem, fwd_smem_bytes(g));
             }
         // heaviest blocks first: the tail of the launch is made of the light ones
-        std::stable_sort(items.begin(), items.end(), [](const Item& a, const Item& b) { return a.work > b.work; });
-        std::vector<FwdSeg> fv;
-        int64_t b = 0;
-        for (Item& it : items) {
-            it.f.blockStart = b;
-            b += it.blocks;
-            fv.push_back(it.f);
-        }
-        P.fwd = {push(P.tb, fv), (int)fv.size(), b};
-        P.red = {push(P.tb, rv), (int)rv.size(), rb};
+        auto table = [&](std::vector<Item>& items) {
+            std::stable_sort(items.begin(), items.end(), [](const Item& a, const Item& b) { return a.work > b.work; });
+            std::vector<FwdSeg> fv;
+            int64_t b = 0;
+            for (Item& it : items) {
+                it.f.blockStart = b;
+                b += it.blocks;
+                fv.push_back(it.f);
+            }
+            return Prepared::R{push(P.tb, fv), (int)fv.size(), b};
+        };
+        P.fwd = table(plain);
+        P.red = {push(P.tb, rplain), (int)rplain.size(), rplain_b};
+        P.gfwd = table(gated);
+        P.gred = {push(P.tb, rgated), (int)rgated.size(), rgated_b};
         // corrected descriptor: map every level block once the whole block is written
         std::vector<TildeSeg> tv;
         int64_t tb = 0;
@@ -786,19 +989,25 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
             AdjSeg a;
             int64_t work, blocks;
         };
-        std::vector<Item> items;
-        std::vector<GSeg> gv;
+        std::vector<Item> plain, gated;
+        std::vector<GSeg> gplain, ggated;
         std::vector<TildeSeg> tsv;
         // gradient assembly: a small field has few positions for many chunk partials and its
         // segments go to the launch with FIN_SUB threads per position; the others to the one
         // with one thread per position
         std::vector<FinalSeg> fv, fvs;
-        int64_t gb = 0, fb = 0, fbs = 0;
+        int64_t gplain_b = 0, ggated_b = 0, fb = 0, fbs = 0;
         const bool vjp = !(flags & F_LOSS);
         for (const Inst& x : in) {
             const int nph = x.pl->phases;
+            const int* gate = x.pl->sep ? reinterpret_cast<const int*>(x.ws + x.pl->o_tier) : nullptr;
+            std::vector<Item>& items = gate ? gated : plain;
+            std::vector<GSeg>& gv = gate ? ggated : gplain;
+            int64_t& gb = gate ? ggated_b : gplain_b;
+            size_t& smem = gate ? P.smem_gadj : P.smem_adj;
             FinalSeg fs{};
             FinalArgs& fa = fs.a;
+            fa.tier = gate;
             fa.ndim = x.pl->ndim;
             fa.levels = x.pl->levels;
             for (int a = 0; a < 3; ++a) fa.n1[a] = x.pl->g[0].n[a];
@@ -832,6 +1041,7 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
                         gs.scale = gcoef_scale(g, x.pl->tc, x.pl->w[l]);
                         gs.Gd = Gd;
                         gs.done = x.use_done ? &x.sc->done : nullptr;
+                        gs.gate = gate;
                         if (x.pl->desc_kind == DMCR_DESC_S2_TILDE) {
                             TildeSeg t{};
                             t.src = gs.src;
@@ -861,11 +1071,12 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
                         it.a.Gd = Gd;
                         it.a.part = pblk;
                         it.a.done = gs.done;
+                        it.a.gate = gate;
                         it.work = (int64_t)g.RZ * g.RY * g.NBc;
                         it.blocks = g.adjTiles * g.nChunks;
                         items.push_back(it);
                     }
-                if (!g.fft) P.smem_adj = std::max(P.smem_adj, adj_smem_bytes(g));
+                if (!g.fft) smem = std::max(smem, adj_smem_bytes(g));
             }
             const bool pen = !vjp && x.lp.bc_on;
             fa.field = pen ? x.field : nullptr;
@@ -888,8 +1099,11 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
             for (int pa = 0; pa < nph; ++pa) {
                 FinalSeg f = fs;
                 for (int l = 0; l < x.pl->levels; ++l)
-                    if (x.pl->desc_kind != DMCR_DESC_S3)
+                    if (x.pl->desc_kind != DMCR_DESC_S3) {
                         f.a.parts[l] = fs.a.parts[l] + (int64_t)pa * nph * x.pl->g[l].nChunks * x.pl->g[l].N;
+                        if (x.pl->sep)
+                            f.a.sparts[l] = reinterpret_cast<const float*>(x.ws + x.pl->o_spart[l]) + pa * x.pl->g[l].N;
+                    }
                 auto slice = [&](auto* ptr) { return ptr != nullptr ? ptr + pa * N1 : ptr; };
                 f.a.field = slice(fs.a.field);
                 f.a.grad_out = slice(fs.a.grad_out);
@@ -907,24 +1121,31 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
                 }
             }
         }
-        std::stable_sort(items.begin(), items.end(), [](const Item& a, const Item& b) { return a.work > b.work; });
-        std::vector<AdjSeg> av;
-        int64_t ab = 0;
-        for (Item& it : items) {
-            it.a.blockStart = ab;
-            ab += it.blocks;
-            av.push_back(it.a);
-        }
-        P.gco = {push(P.tb, gv), (int)gv.size(), gb};
+        auto table = [&](std::vector<Item>& items) {
+            std::stable_sort(items.begin(), items.end(), [](const Item& a, const Item& b) { return a.work > b.work; });
+            std::vector<AdjSeg> av;
+            int64_t ab = 0;
+            for (Item& it : items) {
+                it.a.blockStart = ab;
+                ab += it.blocks;
+                av.push_back(it.a);
+            }
+            return Prepared::R{push(P.tb, av), (int)av.size(), ab};
+        };
+        P.gco = {push(P.tb, gplain), (int)gplain.size(), gplain_b};
         P.tsum = {push(P.tb, tsv), (int)tsv.size(), (int64_t)tsv.size()};
-        P.adj = {push(P.tb, av), (int)av.size(), ab};
+        P.adj = table(plain);
+        P.ggco = {push(P.tb, ggated), (int)ggated.size(), ggated_b};
+        P.gadj = table(gated);
         P.fin = {push(P.tb, fv), (int)fv.size(), fb};
         P.fin_small = {push(P.tb, fvs), (int)fvs.size(), fbs};
     }
+    if (need_pyr) prepare_sep(in, flags, P);
     if (P.tb.h.size() > cap) return fail(DMCR_ENOMEM, "segment tables (%zu bytes) exceed their region", P.tb.h.size());
     // every fused launch indexes its blocks with a 1-D grid
     int64_t most = std::max({P.fwd.blocks, P.red.blocks, P.gco.blocks, P.adj.blocks, P.fin.blocks, P.fin_small.blocks,
                              P.tmap.blocks});
+    for (const Prepared::R& r : P.sep) most = std::max(most, r.blocks);
     for (const Prepared::R& r : P.restricts) most = std::max(most, r.blocks);
     if (most > (int64_t)INT32_MAX)
         return fail(DMCR_ENOTSUP, "a fused launch would need %lld thread blocks (more than 2^31 - 1): split the batch "
@@ -1012,6 +1233,12 @@ void upload(const Prepared& P, cudaStream_t s) {
     launch_blob(P.tb.h.data(), P.tb.h.size(), P.tab, s);
 }
 
+void run_sep(const Prepared& P, SepKernel k, const char* name, cudaStream_t s) {
+    if (P.sep[k].blocks == 0) return;
+    ProfScope ps(name, -1, s);
+    launch_sep(k, P.sept, P.at<SepItem>(P.sep[k].off), P.sep[k].nseg, P.sep[k].blocks, P.sep_smem[k], s);
+}
+
 void run(const Prepared& P, cudaStream_t s) {
     if (P.flags & F_INIT) {
         ProfScope ps("scalars_init", -1, s);
@@ -1021,12 +1248,26 @@ void run(const Prepared& P, cudaStream_t s) {
         ProfScope ps("restrict", -1, s);
         launch_restrict(P.at<RestrictSeg>(r.off), r.nseg, r.blocks, s);
     }
+    if (P.flags & (F_FWD | F_BACK)) {
+        run_sep(P, SEP_RANGE, "sep_range", s);
+        run_sep(P, SEP_FEAT, "sep_feat", s);
+        run_sep(P, SEP_FFT_Y, "sep_fft_y", s);
+    }
     if (P.flags & F_FWD) {
-        {
+        run_sep(P, SEP_POWER, "sep_power", s);
+        run_sep(P, SEP_POWER_PH, "sep_power_phases", s);
+        run_sep(P, SEP_INV_Y, "sep_inv_y", s);
+        run_sep(P, SEP_DESC, "sep_desc", s);
+        if (P.gfwd.nseg > 0) {
+            ProfScope ps("corr_fwd_gated", -1, s);
+            launch_corr_fwd_gated(P.at<FwdSeg>(P.gfwd.off), P.gfwd.nseg, P.gfwd.blocks, P.smem_gfwd, P.tc, s);
+            launch_fwd_reduce_gated(P.at<RedSeg>(P.gred.off), P.gred.nseg, P.gred.blocks, s);
+        }
+        if (P.fwd.nseg > 0) {
             ProfScope ps("corr_fwd", -1, s);
             launch_corr_fwd(P.at<FwdSeg>(P.fwd.off), P.fwd.nseg, P.fwd.blocks, P.smem_fwd, P.tc, s);
         }
-        {
+        if (P.red.nseg > 0) {
             ProfScope ps("fwd_reduce", -1, s);
             launch_fwd_reduce(P.at<RedSeg>(P.red.off), P.red.nseg, P.red.blocks, s);
         }
@@ -1056,11 +1297,22 @@ void run(const Prepared& P, cudaStream_t s) {
             ProfScope ps("tilde_sum", -1, s);
             launch_tilde_sum(P.at<TildeSeg>(P.tsum.off), P.tsum.nseg, s);
         }
-        {
+        run_sep(P, SEP_GX, "sep_gx", s);
+        run_sep(P, SEP_GY, "sep_gy", s);
+        run_sep(P, SEP_MUL, "sep_mul", s);
+        run_sep(P, SEP_MUL_PH, "sep_mul_phases", s);
+        run_sep(P, SEP_IFFT_Y, "sep_ifft_y", s);
+        run_sep(P, SEP_GRAD, "sep_grad", s);
+        if (P.gadj.nseg > 0) {
+            ProfScope ps("corr_adj_gated", -1, s);
+            launch_gcoef_gated(P.at<GSeg>(P.ggco.off), P.ggco.nseg, P.ggco.blocks, P.tc, s);
+            launch_corr_adj_gated(P.at<AdjSeg>(P.gadj.off), P.gadj.nseg, P.gadj.blocks, P.smem_gadj, P.tc, s);
+        }
+        if (P.gco.nseg > 0) {
             ProfScope ps("gcoef", -1, s);
             launch_gcoef(P.at<GSeg>(P.gco.off), P.gco.nseg, P.gco.blocks, P.tc, s);
         }
-        {
+        if (P.adj.nseg > 0) {
             ProfScope ps("corr_adj", -1, s);
             launch_corr_adj(P.at<AdjSeg>(P.adj.off), P.adj.nseg, P.adj.blocks, P.smem_adj, P.tc, s);
         }
@@ -1129,10 +1381,10 @@ dmcr_status batch_layout(int count, const dmcr_params* params, BatchLayout& B) {
     if (count < 1) return fail(DMCR_EINVAL, "count must be >= 1");
     if (params == nullptr) return fail(DMCR_EINVAL, "params is NULL");
     B.plans.resize(count);
-    size_t tb = table_slack();
+    size_t tb = table_slack(true);
     for (int i = 0; i < count; ++i) {
         DMCR_TRY(validate_and_plan(&params[i], B.plans[i]));
-        tb += table_bound(B.plans[i].levels, B.plans[i].phases) + 32;
+        tb += table_bound(B.plans[i]) + 32;
     }
     size_t o = 0;
     B.o_tab = o;
@@ -1208,8 +1460,13 @@ std::string prepared_key(const Prepared& P) {
     add(&P.tc, sizeof P.tc);
     for (const Prepared::R& r : P.restricts) add(&r, sizeof r);
     for (const Prepared::R* r : {&P.fwd, &P.red, &P.pen, &P.loss, &P.gco, &P.adj, &P.fin, &P.fin_small, &P.init,
-                                   &P.tmap, &P.tsum})
+                                   &P.tmap, &P.tsum, &P.gfwd, &P.gred, &P.ggco, &P.gadj})
         add(r, sizeof *r);
+    add(P.sep, sizeof P.sep);
+    add(P.sep_smem, sizeof P.sep_smem);
+    add(&P.sept, sizeof P.sept);
+    add(&P.smem_gfwd, sizeof P.smem_gfwd);
+    add(&P.smem_gadj, sizeof P.smem_gadj);
     add(&P.smem_fwd, sizeof P.smem_fwd);
     add(&P.smem_adj, sizeof P.smem_adj);
     for (const auto* v : {&P.fftf, &P.fftb}) {
@@ -1346,8 +1603,8 @@ dmcr_status reconstruct_insts(std::vector<Inst>& in, char* tab, size_t tab_cap, 
         else if (st == DMCR_ENONFINITE) st = fail(st, "loss became non-finite in instance %d", bad);
         if (st) break;
         // one more evaluation, of the returned fields rounded to phases 0/1 (Sec. 4.1) where
-        // asked for: a rounded field goes to its first level's adjoint partials, which no
-        // forward pass uses
+        // asked for: a rounded field goes to its first level's gradient (adjoint partials on
+        // the direct path), which no forward pass uses
         std::vector<Inst> rin;
         std::vector<int> rid;
         for (int i = 0; i < count; ++i) {
@@ -1359,7 +1616,7 @@ dmcr_status reconstruct_insts(std::vector<Inst>& in, char* tab, size_t tab_cap, 
         }
         if (rin.empty()) break;
         for (Inst& y : rin) {
-            float* rf = reinterpret_cast<float*>(y.ws + y.pl->o_adj[0]);
+            float* rf = reinterpret_cast<float*>(y.ws + (y.pl->sep ? y.pl->o_spart[0] : y.pl->o_adj[0]));
             launch_round_field(y.field, rf, y.pl->N1 * y.pl->phases, s);
             y.field = rf;
             y.M = nullptr;
@@ -1963,6 +2220,8 @@ extern "C" dmcr_status dmcr_descriptor_noalloc(const dmcr_params* p, const float
         return fail(DMCR_ENOTSUP, "dmcr_descriptor_noalloc computes the direct two-point descriptor of one field only");
     // compact layout: segment tables, pyramid levels 2.. and the forward partials of every level
     Plan cp = pl;
+    cp.sep = false;            // the spectra of the separable path do not fit
+    cp.tab_bytes = align_up(table_bound(cp) + table_slack(false));
     size_t o = 0;
     cp.o_tab = o;
     o += cp.tab_bytes;

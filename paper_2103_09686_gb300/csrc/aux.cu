@@ -299,12 +299,13 @@ __device__ __forceinline__ float chunk_sums(const FinalArgs& a, int64_t i, int q
     const int64_t x = i % a.n1[2], y = (i / a.n1[2]) % a.n1[1], z = i / (a.n1[1] * a.n1[2]);
     float g = 0.f, scale = 1.f;
     const float step = a.ndim == 2 ? 0.25f : 0.125f;
+    const bool sep = a.tier != nullptr && *a.tier < SEP_TIERS;
     for (int l = 0; l < a.levels; ++l) {
         const int64_t lz = a.ndim == 2 ? 0 : (z >> l);
         const int64_t li = (lz * a.nl[l][1] + (y >> l)) * a.nl[l][2] + (x >> l);
         const int64_t jump = SUB * a.Nl[l];
-        const float* p = a.parts[l] + li + q * a.Nl[l];
-        const int nc = a.nChunks[l];
+        const float* p = (sep ? a.sparts[l] : a.parts[l]) + li + q * a.Nl[l];
+        const int nc = sep ? 1 : a.nChunks[l];
         float s = 0.f;
         int c = q;
         for (; c + 7 * SUB < nc; c += 8 * SUB) {

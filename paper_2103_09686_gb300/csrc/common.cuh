@@ -3,6 +3,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <memory>
+#include <vector>
+
 #include "scalars.h"
 
 namespace dmcr {
@@ -112,6 +115,8 @@ struct LossParams {
 };
 
 struct FinalArgs {
+    const int* tier;             // separable levels (sep.cu): below SEP_TIERS, sparts replaces parts
+    const float* sparts[8];      // their gradient, one field per level
     int ndim;
     int levels;
     int64_t n1[3];               // finest sizes (3-D embedded)
@@ -137,6 +142,7 @@ struct FwdSeg {
     const float* field;     // tails of the pairs (x)
     const float* tip;       // tips of the pairs (x + r): the same field, or another phase's
     float* partial;
+    const int* gate;        // gated launches only: run when *gate >= SEP_TIERS
     const int* done;
     int64_t blockStart;
 };
@@ -144,6 +150,7 @@ struct RedSeg {
     LevelGeom g;
     const float* partial;
     float* desc;
+    const int* gate;        // gated launches only: run when *gate >= SEP_TIERS
     const int* done;
     float scale;             // w_l / N_l
     int64_t blockStart;
@@ -154,6 +161,7 @@ struct AdjSeg {
     const float* tip;       // partners y + r: the same field, or another phase's
     const float* Gd;
     float* part;
+    const int* gate;        // gated launches only: run when *gate >= SEP_TIERS
     const int* done;
     int64_t blockStart;
 };
@@ -166,6 +174,7 @@ struct GSeg {
     const Scalars* sc;
     float scale;
     float* Gd;
+    const int* gate;
     const int* done;
     const float* tsum;      // corrected descriptor: sum_{k >= 1} (src - sub) of the block, else null
     float q;                // corrected descriptor: 2 f(1/2)^2
@@ -262,6 +271,109 @@ struct FftPass {
     double2 om3[3], om5[5];   // exp(-2 pi i t / 3), exp(-2 pi i t / 5)
 };
 
+// ---------------------------------------------------------------- separable path (sep.cu)
+constexpr int SEP_TIERS = 3;        // value ranges with a basis of their own; tier SEP_TIERS: direct kernels
+constexpr int SEP_MAX_PAIRS = 13;   // packed pairs of features of one basis at most
+constexpr int SEP_THREADS = 512;    // threads of the transform kernels
+constexpr int SEP_BLOCK_PTS = 8 * SEP_THREADS;   // points a block holds in registers (power-of-two axes)
+constexpr int SEP_SLOTS = 8;        // feature pairs a row block holds side by side at most
+constexpr int SEP_FAST_PHASES = 3;  // phases whose spectra fit behind the line buffers of sep_mul
+constexpr int SEP_MAX_DEG = 64;     // Chebyshev coefficients per feature at most
+constexpr int SEP_MAX_N = 2048;     // longest axis
+constexpr int SEP_MAX_RAD = 12;
+constexpr int SEP_OWN = 8;          // points of a column group one thread owns (at most 4096 per block)
+constexpr int SEP_MAX_SMEM = 208 * 1024;
+constexpr int SEP_RANGE_BLOCKS = 256;
+
+struct SepAxis {
+    int n, nrad;
+    int fast;                 // log2 n for powers of two 16 .. SEP_MAX_N, else 0
+    unsigned short rad[SEP_MAX_RAD];
+};
+
+__host__ __device__ inline int sep_coef_stride(int npair) { return (npair + 1) / 2 * 2; }
+
+// line pitch (float2 elements) of a column group of L adjacent columns: padded length, and
+// pitch = 16 / L (mod 16), so that the L columns of one position lie in different banks
+__host__ __device__ inline int sep_pitch(int n, int L) {
+    const int p = n - 1 + ((n - 1) >> 4) + 1;
+    const int want = L >= 16 ? 1 : 16 / L;
+    return p + ((want - p) % 16 + 16) % 16;
+}
+
+struct SepTier {
+    float lo, hi, mid, inv_half;
+    int deg, npair, npos;     // coefficients per feature, packed pairs, the first npos of them with s = +1
+    int coef;                 // offset of this tier's coefficients
+};
+
+struct SepBasis {
+    float alpha = 0.f;
+    int ntier = 0, max_pairs = 0;
+    SepTier tier[SEP_TIERS] = {};
+    std::vector<float2> coef;
+};
+
+// one (instance, level)
+struct SepLevel {
+    int n0, n1, n2;
+    int P0, P1, P2;
+    int phases, maxPairs;
+    int64_t N, Khalf;
+    SepAxis ax[3];
+    const float* field;       // this level's field(s)
+    float2 *Z, *Q;            // spectra of the features, products: phases x maxPairs grids (one phase: Q = Z)
+    float2 *U, *V;            // window spectra (3-D: [r0][y][x]; [row][x]), one per ordered phase pair
+    int64_t strideU, strideV;
+    double* dc;               // sum_k s_k conj(Z^a_k(0)) Z^b_k(0) per phase pair
+    int* tiers;               // tiers of the range blocks
+    int ntiers;
+    int* tier;                // the instance's tier
+    int first;                // finest level: writes *tier
+    int rowsF, rowsW, colsY, colsL;
+    float* desc;
+    double scaleD;            // w / N^2
+    const float* src;         // gradient coefficients: scaleG (gscale) (src - sub)
+    const float* sub;
+    const Scalars* sc;
+    const float* tsum;        // corrected descriptor
+    float q, scaleG;
+    float* part;              // this level's gradient, one field per phase
+    const int* done;
+};
+
+struct SepItem {
+    int level, a, b, pad;
+    int64_t blockStart;
+    const int* tier;
+    const int* done;
+};
+
+struct SepTables {
+    const SepLevel* level;
+    const float2* coef;
+    SepTier tier[SEP_TIERS];
+    int ntier;
+};
+
+enum SepKernel {
+    SEP_RANGE, SEP_FEAT, SEP_FFT_Y, SEP_POWER, SEP_POWER_PH, SEP_INV_Y, SEP_DESC, SEP_GX, SEP_GY, SEP_MUL, SEP_MUL_PH, SEP_IFFT_Y,
+    SEP_GRAD, SEP_KERNELS
+};
+
+std::shared_ptr<const SepBasis> sep_basis(float alpha);
+bool sep_axis(int64_t n, SepAxis& ax);
+double sep_axis_cost(const SepAxis& ax);
+int sep_cols(const SepAxis& ax, bool wide);
+int sep_rows(const SepAxis& ax, int per);
+size_t sep_smem_feat(const SepLevel& lv);
+size_t sep_smem_window(const SepLevel& lv);
+size_t sep_smem_y(const SepLevel& lv);
+size_t sep_smem_last(const SepLevel& lv, bool mul);
+void launch_sep(SepKernel k, const SepTables& tb, const SepItem* items, int nitem, int64_t blocks, size_t smem,
+                cudaStream_t s);
+void set_sep_attributes();
+
 // ---------------------------------------------------------------- launchers
 void launch_blob(const void* host, size_t bytes, void* dst, cudaStream_t s);
 void launch_restrict(const RestrictSeg* segs, int nseg, int64_t blocks, cudaStream_t s);
@@ -271,6 +383,13 @@ void launch_prolongate(int ndim, const int64_t nc[3], const float* coarse, float
 void launch_corr_fwd(const FwdSeg* segs, int nseg, int64_t blocks, size_t smem, const ThreshConst& tc,
                      cudaStream_t s);
 void launch_fwd_reduce(const RedSeg* segs, int nseg, int64_t blocks, cudaStream_t s);
+// the same for the segments whose gate says so (fields outside every separable range)
+void launch_corr_fwd_gated(const FwdSeg* segs, int nseg, int64_t blocks, size_t smem, const ThreshConst& tc,
+                           cudaStream_t s);
+void launch_fwd_reduce_gated(const RedSeg* segs, int nseg, int64_t blocks, cudaStream_t s);
+void launch_gcoef_gated(const GSeg* segs, int nseg, int64_t blocks, const ThreshConst& tc, cudaStream_t s);
+void launch_corr_adj_gated(const AdjSeg* segs, int nseg, int64_t blocks, size_t smem, const ThreshConst& tc,
+                           cudaStream_t s);
 void launch_penalty(const PenSeg* segs, int nseg, int maxblk, cudaStream_t s);
 int stats_blocks(int64_t K, int64_t N);
 void launch_loss(const LossSeg* segs, int nseg, cudaStream_t s);

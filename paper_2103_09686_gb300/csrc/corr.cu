@@ -357,16 +357,11 @@ __device__ __forceinline__ void fwd_plane(const float* xbase, const float* ybase
 }
 
 template <bool IDENT>
-__global__ void __launch_bounds__(FWD_THREADS, 4)
-corr_fwd_kernel(const FwdSeg* __restrict__ segs, int nseg, ThreshConst tc) {
-    const int si = find_segment(segs, nseg, (int64_t)blockIdx.x);
-    const FwdSeg& sg = segs[si];
-    if (sg.done != nullptr && *sg.done) return;
+__device__ __forceinline__ void corr_fwd_block(const FwdSeg& sg, const int64_t local, const ThreshConst& tc) {
     const LevelGeom g = sg.g;
     const float* __restrict__ field = sg.field;
     const float* __restrict__ tipf = sg.tip;
     float* __restrict__ partial = sg.partial;
-    const int64_t local = (int64_t)blockIdx.x - sg.blockStart;
     extern __shared__ __align__(16) float smem[];
     const int tid = threadIdx.x;
     const int64_t ts = local % g.fwdTiles;
@@ -522,17 +517,51 @@ corr_fwd_kernel(const FwdSeg* __restrict__ segs, int nseg, ThreshConst tc) {
     }
 }
 
+template <bool IDENT>
+__global__ void __launch_bounds__(FWD_THREADS, 4)
+corr_fwd_kernel(const FwdSeg* __restrict__ segs, int nseg, ThreshConst tc) {
+    const FwdSeg& sg = segs[find_segment(segs, nseg, (int64_t)blockIdx.x)];
+    if (sg.done != nullptr && *sg.done) return;
+    corr_fwd_block<IDENT>(sg, (int64_t)blockIdx.x - sg.blockStart, tc);
+}
+
+// Gated launches: the segments belong to instances on the separable path, and run here only
+// when their field left every range that path has a basis for.  A small grid that all but
+// always finds nothing to do: one parallel look at the gates, then a block-strided walk over
+// the blocks of the segments whose gate is open.
+template <typename S>
+__device__ __forceinline__ bool gate_open(const S& sg) {
+    return !(sg.done != nullptr && *sg.done) && *sg.gate >= SEP_TIERS;
+}
+
+template <typename S, typename F>
+__device__ __forceinline__ void run_gated(const S* __restrict__ segs, int nseg, int64_t total, F block) {
+    int any = 0;
+    for (int i = threadIdx.x; i < nseg; i += blockDim.x) any |= gate_open(segs[i]);
+    if (!__syncthreads_or(any)) return;
+    for (int i = 0; i < nseg; ++i) {
+        if (!gate_open(segs[i])) continue;
+        const int64_t count = (i + 1 < nseg ? segs[i + 1].blockStart : total) - segs[i].blockStart;
+        for (int64_t local = blockIdx.x; local < count; local += gridDim.x) {
+            block(segs[i], local);
+            __syncthreads();
+        }
+    }
+}
+
+__global__ void __launch_bounds__(FWD_THREADS, 4)
+corr_fwd_gated_kernel(const FwdSeg* __restrict__ segs, int nseg, int64_t total, ThreshConst tc) {
+    run_gated(segs, nseg, total, [&](const FwdSeg& sg, int64_t local) { corr_fwd_block<false>(sg, local, tc); });
+}
+
 // Fixed-order sum over tiles, scaled by w_l / N_l.  A block owns 32 consecutive shifts (one
 // per lane, coalesced rows); warp w sums the tiles t = w (mod 8) in order (Kahan, FP32) and
 // the 8 warp sums are combined in a fixed order as double-floats.
-__global__ void __launch_bounds__(256) fwd_reduce_kernel(const RedSeg* __restrict__ segs, int nseg) {
-    const int si = find_segment(segs, nseg, (int64_t)blockIdx.x);
-    const RedSeg& sg = segs[si];
-    if (sg.done != nullptr && *sg.done) return;
+__device__ __forceinline__ void fwd_reduce_block(const RedSeg& sg, int64_t local) {
     const int64_t Khalf = sg.g.Khalf, tiles = sg.g.fwdTiles;
     __shared__ DF sh[8][RED_K];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t k = ((int64_t)blockIdx.x - sg.blockStart) * RED_K + lane;
+    const int64_t k = local * RED_K + lane;
     // compensated (Kahan) FP32 sum over this warp's tiles, then a double-float (two-sum)
     // combination of the 8 warps
     float sum = 0.f, comp = 0.f;
@@ -563,6 +592,16 @@ __global__ void __launch_bounds__(256) fwd_reduce_kernel(const RedSeg* __restric
     }
 }
 
+__global__ void __launch_bounds__(256) fwd_reduce_kernel(const RedSeg* __restrict__ segs, int nseg) {
+    const RedSeg& sg = segs[find_segment(segs, nseg, (int64_t)blockIdx.x)];
+    if (sg.done != nullptr && *sg.done) return;
+    fwd_reduce_block(sg, (int64_t)blockIdx.x - sg.blockStart);
+}
+
+__global__ void __launch_bounds__(256) fwd_reduce_gated_kernel(const RedSeg* __restrict__ segs, int nseg, int64_t total) {
+    run_gated(segs, nseg, total, [](const RedSeg& sg, int64_t local) { fwd_reduce_block(sg, local); });
+}
+
 // ------------------------------------------------------------------------- adjoint
 
 // lastValid: shifts of the chunk's last rx block inside the window (T unless the chunk ends
@@ -589,17 +628,12 @@ __device__ __forceinline__ void adj_rows(const float* ys, const float* Gs, int s
 }
 
 template <bool IDENT>
-__global__ void __launch_bounds__(ADJ_THREADS, 4)
-corr_adj_kernel(const AdjSeg* __restrict__ segs, int nseg, ThreshConst tc) {
-    const int si = find_segment(segs, nseg, (int64_t)blockIdx.x);
-    const AdjSeg& sg = segs[si];
-    if (sg.done != nullptr && *sg.done) return;
+__device__ __forceinline__ void corr_adj_block(const AdjSeg& sg, const int64_t local, const ThreshConst& tc) {
     const LevelGeom g = sg.g;
     const float* __restrict__ field = sg.field;
     const float* __restrict__ tipf = sg.tip;
     const float* __restrict__ Gd = sg.Gd;
     float* __restrict__ part = sg.part;
-    const int64_t local = (int64_t)blockIdx.x - sg.blockStart;
     extern __shared__ __align__(16) float smem[];
     const int lane = threadIdx.x & 31, strip = threadIdx.x >> 5;
     const int64_t tile = local % g.adjTiles;
@@ -735,6 +769,19 @@ corr_adj_kernel(const AdjSeg* __restrict__ segs, int nseg, ThreshConst tc) {
     }
 }
 
+template <bool IDENT>
+__global__ void __launch_bounds__(ADJ_THREADS, 4)
+corr_adj_kernel(const AdjSeg* __restrict__ segs, int nseg, ThreshConst tc) {
+    const AdjSeg& sg = segs[find_segment(segs, nseg, (int64_t)blockIdx.x)];
+    if (sg.done != nullptr && *sg.done) return;
+    corr_adj_block<IDENT>(sg, (int64_t)blockIdx.x - sg.blockStart, tc);
+}
+
+__global__ void __launch_bounds__(ADJ_THREADS, 4)
+corr_adj_gated_kernel(const AdjSeg* __restrict__ segs, int nseg, int64_t total, ThreshConst tc) {
+    run_gated(segs, nseg, total, [&](const AdjSeg& sg, int64_t local) { corr_adj_block<false>(sg, local, tc); });
+}
+
 // Dense full-window coefficient grid of one level (one phase pair (a, b)), in adjoint order:
 //   G(r) = scale * (src[k] - sub[k]) for r in the half window (k its canonical index),
 //   G(r) = scale * (src2[k] - sub2[k]) for -r in it (k the index of -r),
@@ -744,14 +791,11 @@ corr_adj_kernel(const AdjSeg* __restrict__ segs, int nseg, ThreshConst tc) {
 // zero where rx > P2 (padding of the last rx block).  Row (rz, ry) holds NB blocks of 8
 // shifts; a block of GBLOCK = 48 floats stores (A, A, B, B) for m = 0..7 and then
 // (C_m, C_m, C_m+1, C_m+1) for even m: both halves of a packed pair get the same coefficient.
-__global__ void gcoef_kernel(const GSeg* __restrict__ segs, int nseg, ThreshConst tc) {
-    const int si = find_segment(segs, nseg, (int64_t)blockIdx.x);
-    const GSeg& sg = segs[si];
-    if (sg.done != nullptr && *sg.done) return;
+__device__ __forceinline__ void gcoef_block(const GSeg& sg, int64_t local, const ThreshConst& tc) {
     const LevelGeom& g = sg.g;
     const int WB = g.NB * T;
     const int64_t total = (int64_t)(2 * g.P[0] + 1) * (2 * g.P[1] + 1) * WB;
-    const int64_t i = ((int64_t)blockIdx.x - sg.blockStart) * GCOEF_TH + threadIdx.x;
+    const int64_t i = local * GCOEF_TH + threadIdx.x;
     if (i >= total) return;
     const int col = (int)(i % WB);
     const int64_t row = i / WB;
@@ -783,6 +827,16 @@ __global__ void gcoef_kernel(const GSeg* __restrict__ segs, int nseg, ThreshCons
     float* blk = sg.Gd + (row * g.NB + b) * GBLOCK;
     *reinterpret_cast<float4*>(blk + 4 * m) = make_float4(A, A, B, B);
     *reinterpret_cast<float2*>(blk + gblock_c(m)) = make_float2(C, C);
+}
+
+__global__ void gcoef_kernel(const GSeg* __restrict__ segs, int nseg, ThreshConst tc) {
+    const GSeg& sg = segs[find_segment(segs, nseg, (int64_t)blockIdx.x)];
+    if (sg.done != nullptr && *sg.done) return;
+    gcoef_block(sg, (int64_t)blockIdx.x - sg.blockStart, tc);
+}
+
+__global__ void gcoef_gated_kernel(const GSeg* __restrict__ segs, int nseg, int64_t total, ThreshConst tc) {
+    run_gated(segs, nseg, total, [&](const GSeg& sg, int64_t local) { gcoef_block(sg, local, tc); });
 }
 
 // ------------------------------------------------------------------------- launchers
@@ -825,8 +879,35 @@ void launch_corr_adj(const AdjSeg* segs, int nseg, int64_t blocks, size_t smem, 
     else corr_adj_kernel<false><<<(unsigned)blocks, ADJ_THREADS, smem, s>>>(segs, nseg, tc);
 }
 
+// resident blocks of a gated launch: as many as run at once (4 per SM; the small kernels 2)
+constexpr int64_t GATED_BLOCKS = 4 * 152, GATED_SMALL = 2 * 152;
+
+void launch_corr_fwd_gated(const FwdSeg* segs, int nseg, int64_t blocks, size_t smem, const ThreshConst& tc,
+                           cudaStream_t s) {
+    if (blocks <= 0) return;
+    corr_fwd_gated_kernel<<<(unsigned)std::min(blocks, GATED_BLOCKS), FWD_THREADS, smem, s>>>(segs, nseg, blocks, tc);
+}
+
+void launch_fwd_reduce_gated(const RedSeg* segs, int nseg, int64_t blocks, cudaStream_t s) {
+    if (blocks <= 0) return;
+    fwd_reduce_gated_kernel<<<(unsigned)std::min(blocks, GATED_SMALL), 256, 0, s>>>(segs, nseg, blocks);
+}
+
+void launch_gcoef_gated(const GSeg* segs, int nseg, int64_t blocks, const ThreshConst& tc, cudaStream_t s) {
+    if (blocks <= 0) return;
+    gcoef_gated_kernel<<<(unsigned)std::min(blocks, GATED_SMALL), GCOEF_TH, 0, s>>>(segs, nseg, blocks, tc);
+}
+
+void launch_corr_adj_gated(const AdjSeg* segs, int nseg, int64_t blocks, size_t smem, const ThreshConst& tc,
+                           cudaStream_t s) {
+    if (blocks <= 0) return;
+    corr_adj_gated_kernel<<<(unsigned)std::min(blocks, GATED_BLOCKS), ADJ_THREADS, smem, s>>>(segs, nseg, blocks, tc);
+}
+
 void set_kernel_attributes() {
     const int bytes = MAX_DYN_SMEM;
+    cudaFuncSetAttribute(corr_fwd_gated_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    cudaFuncSetAttribute(corr_adj_gated_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     cudaFuncSetAttribute(corr_fwd_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     cudaFuncSetAttribute(corr_fwd_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     cudaFuncSetAttribute(corr_adj_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);

@@ -1,0 +1,1696 @@
+// Separable evaluation of the soft-thresholded two-point descriptor and its adjoint
+// (sm_103a).  Paper: arXiv 2103.09686, Sec. 3.2.2-3.2.4 and the gradient of Sec. 3.1/3.3.
+//
+// The pair function F(u, v) = f((u + v) / 2)^2 is smooth on the bounded range of a relaxed
+// field, so its integral operator has rapidly decaying eigenvalues:
+//     F(u, v) = sum_k s_k p_k(u) p_k(v),  s_k = +-1,  p_k polynomials,
+// with 14 terms to 4e-11 on [-1/16, 17/16] at alpha = 10 (SepBasis, built on the host in
+// FP64).  The descriptor is then a sum of autocorrelations of R feature fields p_k(M), and the
+// gradient a sum of convolutions of the same features with the window coefficients G:
+//     S(r) = (1/N) sum_k s_k sum_x p_k(M_x) p_k(M_{x+r}),
+//     g(y) = sum_k s_k p_k'(M_y) sum_r G(r) p_k(M_{y+r}).
+// Both are diagonal in Fourier space: the work per position falls from the window's K pair
+// evaluations (8321 at +-64) to R transforms (5 R log2 N operations).  Features of equal sign
+// are packed in pairs, z = p_1 + i p_2: Re IDFT(|Z|^2) = autocorr(p_1) + autocorr(p_2), and a
+// real even G acts on both parts at once, so no mirrored frequency is ever read.
+//
+//   sep_range   the tier (basis) that covers the field's values; none: the direct kernels run
+//   sep_feat    features of whole rows + transform along x             -> Z
+//   sep_fft_y   3-D: transform along y, in place
+//   sep_power   last axis: transform, sum_k s_k conj(Z^a_k) Z^b_k, inverse along the same
+//               axis, cropped to the window
+//   sep_inv_y   3-D: inverse along y, cropped to the window
+//   sep_desc    inverse along x, cropped to the window: the descriptor
+//   sep_gx/gy   the window's coefficients G embedded and transformed along x (and y)
+//   sep_mul     last axis: transform of G, then per feature pair transform, product, inverse
+//   sep_grad    inverse along x and sum_k s_k p_k'(M_y) Q_k(y): the gradient of the level
+//
+// The frequency 0 carries the means, which are orders of magnitude above the fluctuations:
+// its power is summed in FP64 and added after the inverse transform, so the FP32 transforms
+// only carry fluctuations.  Fixed grids and orders: results are bitwise reproducible.
+#include <math.h>
+
+#include <algorithm>
+#include <mutex>
+#include <type_traits>
+#include <vector>
+
+#include "common.cuh"
+
+namespace dmcr {
+
+// ------------------------------------------------------------------------- basis (host)
+
+namespace {
+
+struct PairFn {
+    double a, c1, c3;
+    explicit PairFn(double alpha) : a(alpha) {
+        const double s0 = 1.0 / (1.0 + exp(0.75 * a)), s1 = 1.0 / (1.0 + exp(-0.25 * a));
+        c1 = 1.0 / (s1 - s0);
+        c3 = -c1 * s0;
+    }
+    double f(double t) const { return c1 / (1.0 + exp(-a * (0.5 * t - 0.75))) + c3; }
+    double F(double t) const { const double v = f(t); return v * v; }          // t = u + v
+    double Fu(double t) const {
+        const double s = 1.0 / (1.0 + exp(-a * (0.5 * t - 0.75)));
+        return (c1 * s + c3) * c1 * a * s * (1.0 - s);
+    }
+};
+
+// Symmetric eigenproblem by cyclic Jacobi rotations (Golub & Van Loan, Matrix Computations,
+// Sec. 8.5): A (n x n) becomes diagonal, V holds the eigenvectors in its columns.
+void jacobi_eigen(std::vector<double>& A, std::vector<double>& V, int n) {
+    V.assign((size_t)n * n, 0.0);
+    for (int i = 0; i < n; ++i) V[(size_t)i * n + i] = 1.0;
+    for (int sweep = 0; sweep < 30; ++sweep) {
+        double off = 0.0, dia = 0.0;
+        for (int i = 0; i < n; ++i)
+            for (int j = 0; j < n; ++j) (i == j ? dia : off) += A[(size_t)i * n + j] * A[(size_t)i * n + j];
+        if (off <= 1e-30 * dia) break;
+        for (int p = 0; p < n; ++p)
+            for (int q = p + 1; q < n; ++q) {
+                const double apq = A[(size_t)p * n + q];
+                if (apq == 0.0) continue;
+                const double th = (A[(size_t)q * n + q] - A[(size_t)p * n + p]) / (2.0 * apq);
+                const double t = (th >= 0 ? 1.0 : -1.0) / (fabs(th) + sqrt(th * th + 1.0));
+                const double c = 1.0 / sqrt(t * t + 1.0), s = t * c;
+                for (int k = 0; k < n; ++k) {
+                    const double x = A[(size_t)k * n + p], y = A[(size_t)k * n + q];
+                    A[(size_t)k * n + p] = c * x - s * y;
+                    A[(size_t)k * n + q] = s * x + c * y;
+                }
+                for (int k = 0; k < n; ++k) {
+                    const double x = A[(size_t)p * n + k], y = A[(size_t)q * n + k];
+                    A[(size_t)p * n + k] = c * x - s * y;
+                    A[(size_t)q * n + k] = s * x + c * y;
+                }
+                for (int k = 0; k < n; ++k) {
+                    const double x = V[(size_t)k * n + p], y = V[(size_t)k * n + q];
+                    V[(size_t)k * n + p] = c * x - s * y;
+                    V[(size_t)k * n + q] = s * x + c * y;
+                }
+            }
+    }
+}
+
+constexpr int SEP_NODES = 64;
+// accepted error of F and of dF/du over the whole range: below the FP32 rounding of a pair
+constexpr double SEP_TOL_F = 1.5e-9, SEP_TOL_FU = 1e-7;
+
+// One tier: eigenfunctions of F on [lo, hi] at SEP_NODES Chebyshev nodes, as Chebyshev series;
+// false when SEP_MAX_PAIRS pairs of features do not reach the tolerances.
+bool build_tier(const PairFn& fn, double lo, double hi, SepTier& t, std::vector<float2>& coef) {
+    constexpr int n = SEP_NODES;
+    const double mid = 0.5 * (lo + hi), half = 0.5 * (hi - lo);
+    std::vector<double> x(n), A((size_t)n * n), V;
+    for (int i = 0; i < n; ++i) x[i] = cos((i + 0.5) * M_PI / n);
+    for (int i = 0; i < n; ++i)
+        for (int j = 0; j < n; ++j) A[(size_t)i * n + j] = fn.F(2.0 * mid + half * (x[i] + x[j])) / n;
+    jacobi_eigen(A, V, n);
+    std::vector<int> ord(n);
+    for (int i = 0; i < n; ++i) ord[i] = i;
+    std::stable_sort(ord.begin(), ord.end(),
+                     [&](int a, int b) { return fabs(A[(size_t)a * n + a]) > fabs(A[(size_t)b * n + b]); });
+    // Chebyshev coefficients of sqrt(|lambda_k| n) v_k
+    auto series = [&](int k) {
+        std::vector<double> c(n);
+        const double sc = sqrt(fabs(A[(size_t)ord[k] * n + ord[k]]) * n);
+        for (int j = 0; j < n; ++j) {
+            double s = 0.0;
+            for (int i = 0; i < n; ++i) s += V[(size_t)i * n + ord[k]] * cos(j * (i + 0.5) * M_PI / n);
+            c[j] = s * sc * (j == 0 ? 1.0 : 2.0) / n;
+        }
+        return c;
+    };
+    constexpr int GRID = 49;
+    std::vector<double> E((size_t)GRID * GRID), D((size_t)GRID * GRID);
+    auto gx = [&](int i) { return -1.0 + 2.0 * i / (GRID - 1); };
+    for (int i = 0; i < GRID; ++i)
+        for (int j = 0; j < GRID; ++j) {
+            const double tt = 2.0 * mid + half * (gx(i) + gx(j));
+            E[(size_t)i * GRID + j] = fn.F(tt);
+            D[(size_t)i * GRID + j] = fn.Fu(tt);
+        }
+    std::vector<std::vector<double>> pos, neg;
+    bool ok = false;
+    for (int k = 0; k < 2 * SEP_MAX_PAIRS; ++k) {
+        const bool plus = A[(size_t)ord[k] * n + ord[k]] > 0.0;
+        std::vector<std::vector<double>>& side = plus ? pos : neg;
+        // once accurate, further terms are taken only while they fill a half-empty pair
+        if (ok && side.size() % 2 == 0) break;
+        if (!ok && (int)((pos.size() + 1) / 2 + (neg.size() + 1) / 2) + (side.size() % 2 == 0) > SEP_MAX_PAIRS) break;
+        const std::vector<double> c = series(k);
+        side.push_back(c);
+        std::vector<double> p(GRID), dp(GRID);
+        for (int i = 0; i < GRID; ++i) {
+            const double xx = gx(i);
+            double T0 = 1.0, T1 = xx, U0 = 1.0, U1 = 2.0 * xx, s = c[0] + c[1] * xx, d = c[1];
+            for (int j = 2; j < n; ++j) {
+                const double T2 = 2.0 * xx * T1 - T0;
+                s += c[j] * T2;
+                d += c[j] * j * U1;          // T_j' = j U_{j-1}
+                T0 = T1, T1 = T2;
+                const double U2 = 2.0 * xx * U1 - U0;
+                U0 = U1, U1 = U2;
+            }
+            p[i] = s;
+            dp[i] = d / half;
+        }
+        double eF = 0.0, eD = 0.0;
+        for (int i = 0; i < GRID; ++i)
+            for (int j = 0; j < GRID; ++j) {
+                E[(size_t)i * GRID + j] -= (plus ? 1.0 : -1.0) * p[i] * p[j];
+                D[(size_t)i * GRID + j] -= (plus ? 1.0 : -1.0) * dp[i] * p[j];
+                eF = std::max(eF, fabs(E[(size_t)i * GRID + j]));
+                eD = std::max(eD, fabs(D[(size_t)i * GRID + j]));
+            }
+        if (eF < SEP_TOL_F && eD < SEP_TOL_FU) ok = true;
+    }
+    if (!ok) return false;
+    int deg = 4;
+    for (const auto* side : {&pos, &neg})
+        for (const auto& c : *side)
+            for (int j = 0; j < n; ++j)
+                if (fabs(c[j]) > 3e-10) deg = std::max(deg, j + 1);
+    t.lo = (float)lo;
+    t.hi = (float)hi;
+    t.mid = (float)mid;
+    t.inv_half = (float)(1.0 / half);
+    t.deg = deg;
+    t.npos = (int)(pos.size() + 1) / 2;
+    t.npair = t.npos + (int)(neg.size() + 1) / 2;
+    t.coef = (int)coef.size();
+    // coefficients [deg][npair rounded up to even], zero padded: (feature 2p, feature 2p + 1)
+    const int stride = sep_coef_stride(t.npair);
+    coef.resize(coef.size() + (size_t)deg * stride, make_float2(0.f, 0.f));
+    for (int j = 0; j < deg; ++j)
+        for (int p = 0; p < t.npair; ++p) {
+            const auto& side = p < t.npos ? pos : neg;
+            const size_t k = 2 * (size_t)(p < t.npos ? p : p - t.npos);
+            float2& c = coef[t.coef + (size_t)j * stride + p];
+            c.x = (float)side[k][j];
+            c.y = k + 1 < side.size() ? (float)side[k + 1][j] : 0.f;
+        }
+    return true;
+}
+
+}  // namespace
+
+// The basis of one alpha.  Three ranges: a field between the phases with the overshoot of an
+// optimiser step, and two with wider excursions (a wider range needs more features).
+std::shared_ptr<const SepBasis> sep_basis(float alpha) {
+    static std::mutex mu;
+    static std::vector<std::shared_ptr<const SepBasis>>* cache = new std::vector<std::shared_ptr<const SepBasis>>();
+    constexpr size_t KEEP = 8;
+    std::lock_guard<std::mutex> lk(mu);
+    for (size_t i = 0; i < cache->size(); ++i)
+        if ((*cache)[i]->alpha == alpha) {
+            std::rotate(cache->begin(), cache->begin() + i, cache->begin() + i + 1);   // most recent first
+            return cache->front();
+        }
+    auto b = std::make_shared<SepBasis>();
+    b->alpha = alpha;
+    const PairFn fn((double)alpha);
+    const double ranges[SEP_TIERS][2] = {{-0.0625, 1.0625}, {-0.25, 1.25}, {-0.5, 1.5}};
+    for (int t = 0; t < SEP_TIERS; ++t) {
+        if (!build_tier(fn, ranges[t][0], ranges[t][1], b->tier[t], b->coef)) break;
+        b->ntier = t + 1;
+        b->max_pairs = std::max(b->max_pairs, b->tier[t].npair);
+    }
+    cache->insert(cache->begin(), b);
+    if (cache->size() > KEEP) cache->pop_back();
+    return b;
+}
+
+// ------------------------------------------------------------------------- plan (host)
+
+// Transform lengths: any n <= SEP_MAX_N; radices 8, 4, 2, 3, 5, 7, then the remaining primes
+// (a direct sum over the prime, O(p) per point).
+bool sep_axis(int64_t n, SepAxis& ax) {
+    if (n < 1 || n > SEP_MAX_N) return false;
+    ax.n = (int)n;
+    ax.nrad = 0;
+    ax.fast = 0;
+    for (int k = 4; (1 << k) <= SEP_MAX_N; ++k)
+        if (n == (1 << k)) ax.fast = k;
+    int m = (int)n;
+    auto put = [&](int r) {
+        if (ax.nrad >= SEP_MAX_RAD) return false;
+        ax.rad[ax.nrad++] = (unsigned short)r;
+        m /= r;
+        return true;
+    };
+    while (m % 8 == 0)
+        if (!put(8)) return false;
+    for (int r : {4, 2, 3, 5, 7})
+        while (m % r == 0)
+            if (!put(r)) return false;
+    for (int r = 11; m > 1; r += 2)
+        while (m % r == 0)
+            if (!put(r)) return false;
+    return true;
+}
+
+// Estimated seconds per point and axis of a loss and gradient: powers of two, and the general
+// stages (primes by their length).
+double sep_axis_cost(const SepAxis& ax) {
+    if (ax.fast) return 2e-10;
+    double c = 1.5e-10;
+    for (int i = 0; i < ax.nrad; ++i) c += 0.75e-10 * (ax.rad[i] <= 8 ? 1.0 : 0.5 * ax.rad[i]);
+    return c;
+}
+
+namespace {
+int pow2_floor(int v) {
+    int p = 1;
+    while (2 * p <= v) p *= 2;
+    return p;
+}
+}  // namespace
+
+// Adjacent columns of a strided axis per block.  A block holds SEP_BLOCK_PTS points of a power
+// of two: its remaining factor goes to feature pairs (or planes).  2-D grids stay in L2, where
+// 32-byte segments (4 columns) cost nothing and the narrow groups give more blocks; 3-D grids
+// stream from DRAM in 128-byte lines.
+int sep_cols(const SepAxis& ax, bool wide) {
+    const int n = ax.n;
+    if (ax.fast) {
+        const int lines = SEP_BLOCK_PTS / n;
+        const int narrow = std::max(4, lines / 8);       // at most 8 pairs side by side
+        return std::min(std::min(lines, 16), wide ? 16 : narrow);
+    }
+    if (n > 1024) return 2;
+    return std::max(4, std::min(16, pow2_floor(2048 / n)));
+}
+
+// Whole rows per block: of `per` feature pairs each (feature and gradient kernels), or of the window.
+int sep_rows(const SepAxis& ax, int per) {
+    const int pts = ax.fast ? SEP_BLOCK_PTS : 2048;
+    return std::max(1, std::min(ax.fast ? 64 : 16, pow2_floor(std::max(1, pts / (ax.n * per)))));
+}
+
+// ------------------------------------------------------------------------- transforms (device)
+
+namespace {
+
+__device__ __forceinline__ float2 cmulf(float2 a, float2 b) {
+    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+}
+__device__ __forceinline__ float2 caddf(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 csubf(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ float2 swapf(float2 a) { return make_float2(a.y, a.x); }
+// times -i
+__device__ __forceinline__ float2 rot(float2 a) { return make_float2(a.y, -a.x); }
+
+// Only forward transforms are written: an inverse exchanges real and imaginary parts of its
+// input and output.
+
+// Lines live in shared memory with one pad element (8 bytes) after every 16: the radix-8
+// stages' strided writes then spread over the banks.
+__device__ __forceinline__ int spad(int i) { return i + (i >> 4); }
+
+// tw[t] = exp(-2 pi i t / n), from sincospi of an argument reduced to an eighth of a turn
+__device__ __forceinline__ void fill_twiddles(float2* tw, int n) {
+    for (int t = threadIdx.x; t < n; t += blockDim.x) {
+        // angle = 2 pi t / n = (pi / 4)(o + r / n); odd octants are reflected about pi / 4
+        const int o = 8 * t / n;
+        int r = 8 * t - o * n;
+        const bool flip = o & 1;
+        if (flip) r = n - r;
+        float s, c;
+        sincospif((float)r / (float)(4 * n), &s, &c);
+        if (flip) { const float x = s; s = c; c = x; }
+        const int quad = o >> 1;
+        const float cs = quad == 0 ? c : (quad == 1 ? -s : (quad == 2 ? -c : s));
+        const float sn = quad == 0 ? s : (quad == 1 ? c : (quad == 2 ? -s : -c));
+        tw[t] = make_float2(cs, -sn);
+    }
+}
+
+__device__ __forceinline__ void bfly4(float2& a, float2& b, float2& c, float2& d) {
+    const float2 s0 = caddf(a, c), d0 = csubf(a, c), s1 = caddf(b, d), d1 = rot(csubf(b, d));
+    a = caddf(s0, s1);
+    b = caddf(d0, d1);
+    c = csubf(s0, s1);
+    d = csubf(d0, d1);
+}
+
+// V[q] = sum_r v[r] exp(-2 pi i r q / R) in place
+template <int R>
+__device__ __forceinline__ void butterfly(float2 (&v)[R]) {
+    if constexpr (R == 2) {
+        const float2 t = csubf(v[0], v[1]);
+        v[0] = caddf(v[0], v[1]);
+        v[1] = t;
+    } else if constexpr (R == 4) {
+        bfly4(v[0], v[1], v[2], v[3]);
+    } else if constexpr (R == 8) {
+        // even and odd halves, then the eighth roots
+        bfly4(v[0], v[2], v[4], v[6]);
+        bfly4(v[1], v[3], v[5], v[7]);
+        constexpr float h = 0.70710678118654752440f;
+        const float2 w1 = make_float2(h * (v[3].x + v[3].y), h * (v[3].y - v[3].x));
+        const float2 w2 = rot(v[5]);
+        const float2 w3 = make_float2(h * (v[7].y - v[7].x), -h * (v[7].x + v[7].y));
+        const float2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6], o0 = v[1];
+        v[0] = caddf(e0, o0);
+        v[4] = csubf(e0, o0);
+        v[1] = caddf(e1, w1);
+        v[5] = csubf(e1, w1);
+        v[2] = caddf(e2, w2);
+        v[6] = csubf(e2, w2);
+        v[3] = caddf(e3, w3);
+        v[7] = csubf(e3, w3);
+    } else {
+        // odd radices: pair r with R - r; the cosines and sines of 2 pi j / R are constants
+        constexpr int H = (R - 1) / 2;
+        constexpr float C3[1] = {-0.5f}, S3[1] = {0.86602540378443864676f};
+        constexpr float C5[2] = {0.30901699437494742410f, -0.80901699437494742410f},
+                        S5[2] = {0.95105651629515357212f, 0.58778525229247312917f};
+        constexpr float C7[3] = {0.62348980185873353053f, -0.22252093395631440429f, -0.90096886790241912624f},
+                        S7[3] = {0.78183148246802980871f, 0.97492791218182360702f, 0.43388373911755812048f};
+        float2 p[H], m[H];
+#pragma unroll
+        for (int r = 0; r < H; ++r) {
+            p[r] = caddf(v[r + 1], v[R - 1 - r]);
+            m[r] = rot(csubf(v[r + 1], v[R - 1 - r]));
+        }
+        const float2 v0 = v[0];
+#pragma unroll
+        for (int r = 0; r < H; ++r) v[0] = caddf(v[0], p[r]);
+#pragma unroll
+        for (int q = 1; q <= H; ++q) {
+            float2 a = v0, b = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int r = 1; r <= H; ++r) {
+                const int j = (r * q) % R, jj = j <= H ? j : R - j;      // angle index, folded
+                const float c = R == 3 ? C3[jj - 1] : (R == 5 ? C5[jj - 1 < 2 ? jj - 1 : 0] : C7[jj - 1]);
+                const float s0 = R == 3 ? S3[jj - 1] : (R == 5 ? S5[jj - 1 < 2 ? jj - 1 : 0] : S7[jj - 1]);
+                const float s = j <= H ? s0 : -s0;
+                a = make_float2(fmaf(c, p[r - 1].x, a.x), fmaf(c, p[r - 1].y, a.y));
+                b = make_float2(fmaf(s, m[r - 1].x, b.x), fmaf(s, m[r - 1].y, b.y));
+            }
+            v[q] = caddf(a, b);
+            v[R - q] = csubf(a, b);
+        }
+    }
+}
+
+// ---- powers of two: 8 points per thread in registers
+//
+// T = N / 8 threads hold a line; thread t holds the points t + e T (e = 0 .. 7) before the
+// first stage and after the last, so that a product between two transforms needs no exchange.
+// Stockham stages of radix 8 (the last one 2 or 4), exchanged through shared memory in two
+// alternating buffers: one barrier per exchange.
+template <int N>
+struct Line {
+    float2* buf[2];           // this line in the two buffers
+    const float2* tw;
+    int t;
+};
+
+// WARP: the line's threads are consecutive lanes of one warp
+template <bool WARP>
+__device__ __forceinline__ void line_sync() {
+    if (WARP) __syncwarp();
+    else __syncthreads();
+}
+
+template <int N, int Ns, bool WARP, int PAR>
+__device__ __forceinline__ void p2_stages(float2 (&v)[8], const Line<N>& ln) {
+    constexpr int T = N / 8, REM = N / Ns, R = REM >= 8 ? 8 : REM, M = 8 / R;
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+        const int k = (ln.t + m * T) & (Ns - 1);
+        float2 u[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) u[r] = v[m + r * M];
+        if (Ns > 1) {
+#pragma unroll
+            for (int r = 1; r < R; ++r) u[r] = cmulf(u[r], ln.tw[k * r * (REM / R)]);
+        }
+        butterfly<R>(u);
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[m + r * M] = u[r];
+    }
+    if constexpr (Ns * R < N) {
+        static_assert(R == 8, "only the last stage has another radix");
+        float2* b = ln.buf[PAR];
+        // point (t - k) 8 + k + q Ns of the next stage's input; the pads are constants of q
+        const int k = ln.t & (Ns - 1), o = (ln.t - k) * 8 + k;
+        float2* out = b + spad(o);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) out[q * Ns + (Ns == 1 ? 0 : (Ns == 8 ? q / 2 : q * Ns / 16))] = v[q];
+        line_sync<WARP>();
+        const float2* in = b + spad(ln.t);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = in[e * T + (T >= 16 ? e * T / 16 : (e * T) / 16)];
+        p2_stages<N, Ns * R, WARP, PAR ^ 1>(v, ln);
+    }
+}
+
+// exchanges of one transform (the buffer parity the next one starts with)
+__host__ __device__ constexpr int p2_exchanges(int N) { return N <= 8 ? 0 : (N <= 64 ? 1 : (N <= 512 ? 2 : 3)); }
+
+template <int N, bool WARP, int PAR>
+__device__ __forceinline__ void p2_fft(float2 (&v)[8], const Line<N>& ln) {
+    p2_stages<N, 1, WARP, PAR>(v, ln);
+}
+
+__device__ __forceinline__ void swap8(float2 (&v)[8]) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = swapf(v[e]);
+}
+
+// line pitch (float2 elements) of rows: consecutive lines start 2 T banks apart
+template <int N>
+__host__ __device__ constexpr int row_pitch() {
+    int p = N - 1 + (N - 1) / 16 + 1;
+    const int want = N >= 128 ? 0 : N / 8;
+    while (p % 16 != want) ++p;
+    return p;
+}
+
+// ---- any other length: stages over lines in shared memory
+
+// t / d for 0 <= t < 2^20 through a float reciprocal: (t + 1/2) / d is at least 1/(2 d) away
+// from an integer, and the rounding of the product is below t 2^-22 / d
+__device__ __forceinline__ int fdiv(int t, float inv) { return (int)(((float)t + 0.5f) * inv); }
+
+// One Stockham stage of radix R over `lines` lines (pitch elements apart) src -> dst.
+template <int R>
+__device__ __forceinline__ void sep_stage(const float2* __restrict__ src, float2* __restrict__ dst,
+                                          const float2* __restrict__ tw, int n, int lines, int pitch, int Ns) {
+    const int nR = n / R;
+    const int tstep = nR / Ns;
+    const float inv_nR = 1.0f / (float)nR, inv_Ns = 1.0f / (float)Ns;
+    for (int t = threadIdx.x; t < lines * nR; t += blockDim.x) {
+        const int l = fdiv(t, inv_nR), j = t - l * nR;
+        const int blk = fdiv(j, inv_Ns), k = j - blk * Ns;
+        const float2* in = src + l * pitch;
+        float2 v[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = in[spad(j + r * nR)];
+        if (Ns > 1) {
+#pragma unroll
+            for (int r = 1; r < R; ++r) v[r] = cmulf(v[r], tw[k * r * tstep]);
+        }
+        butterfly<R>(v);
+        float2* out = dst + l * pitch;
+        const int o = blk * Ns * R + k;
+#pragma unroll
+        for (int q = 0; q < R; ++q) out[spad(o + q * Ns)] = v[q];
+    }
+}
+
+// A prime radix p > 7: one thread per output, a direct sum over the p inputs.
+__device__ __forceinline__ void sep_stage_prime(const float2* __restrict__ src, float2* __restrict__ dst,
+                                                const float2* __restrict__ tw, int n, int lines, int pitch, int Ns,
+                                                int p) {
+    const int np = n / p, tstep = np / Ns;
+    const float inv_n = 1.0f / (float)n, inv_np = 1.0f / (float)np, inv_Ns = 1.0f / (float)Ns;
+    for (int t = threadIdx.x; t < lines * n; t += blockDim.x) {
+        const int l = fdiv(t, inv_n), e = t - l * n;
+        const int q = fdiv(e, inv_np), j = e - q * np;
+        const int blk = fdiv(j, inv_Ns), k = j - blk * Ns;
+        const float2* in = src + l * pitch;
+        const int step = k * tstep + q * np;      // < n: the angle of one input to the next
+        float2 a = in[spad(j)];
+        int w = 0, at = j;
+        for (int r = 1; r < p; ++r) {
+            w += step;
+            if (w >= n) w -= n;
+            at += np;
+            const float2 c = tw[w], x = in[spad(at)];
+            a.x = fmaf(x.x, c.x, fmaf(-x.y, c.y, a.x));
+            a.y = fmaf(x.x, c.y, fmaf(x.y, c.x, a.y));
+        }
+        dst[l * pitch + spad(blk * Ns * p + k + q * Ns)] = a;
+    }
+}
+
+// Forward transform of `lines` lines in shared memory: from `a`, through `b` and back; returns
+// the buffer that holds the result.  Begins and ends with a barrier.  One copy of the code
+// serves every call.
+__device__ __noinline__ float2* transform(const SepAxis& ax, float2* a, float2* b, const float2* tw, int lines,
+                                          int pitch) {
+    int Ns = 1;
+    __syncthreads();
+    for (int s = 0; s < ax.nrad; ++s) {
+        const int R = ax.rad[s];
+        switch (R) {
+            case 8: sep_stage<8>(a, b, tw, ax.n, lines, pitch, Ns); break;
+            case 4: sep_stage<4>(a, b, tw, ax.n, lines, pitch, Ns); break;
+            case 2: sep_stage<2>(a, b, tw, ax.n, lines, pitch, Ns); break;
+            case 3: sep_stage<3>(a, b, tw, ax.n, lines, pitch, Ns); break;
+            case 5: sep_stage<5>(a, b, tw, ax.n, lines, pitch, Ns); break;
+            case 7: sep_stage<7>(a, b, tw, ax.n, lines, pitch, Ns); break;
+            default: sep_stage_prime(a, b, tw, ax.n, lines, pitch, Ns, R); break;
+        }
+        Ns *= R;
+        float2* x = a;
+        a = b;
+        b = x;
+        __syncthreads();
+    }
+    return a;
+}
+
+// ---- what a block works on
+
+extern __shared__ __align__(16) float2 sep_smem[];
+
+// Dynamic shared memory: twiddles of the axis, then two buffers of whole lines.
+struct SepShared {
+    float2 *tw, *a, *b;
+};
+__device__ __forceinline__ SepShared sep_shared(int n, int lines, int pitch) {
+    SepShared s;
+    s.tw = sep_smem;
+    s.a = sep_smem + ((n + 1) & ~1);
+    s.b = s.a + lines * pitch;
+    return s;
+}
+
+struct SepBlock {
+    SepLevel lv;
+    int a, b, block, tier;
+};
+
+// Finds the block's item (every thread looks at one item), copies its level to shared memory
+// and reads the instance's tier.  Returns false when there is nothing to do: the instance has
+// stopped, or (TIERED) its field needs the direct kernels.
+template <bool TIERED>
+__device__ __forceinline__ bool enter(const SepTables& tb, const SepItem* __restrict__ items, int nitem,
+                                      SepBlock& bk) {
+    int count = 0;
+    for (int base = 0; base < nitem; base += blockDim.x) {
+        const int i = base + threadIdx.x;
+        count += __syncthreads_count(i < nitem && items[i].blockStart <= (int64_t)blockIdx.x);
+    }
+    const SepItem& it = items[count - 1];
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(tb.level + it.level);
+    uint32_t* dst = reinterpret_cast<uint32_t*>(&bk.lv);
+    for (int i = threadIdx.x; i < (int)(sizeof(SepLevel) / 4); i += blockDim.x) dst[i] = src[i];
+    const bool stopped = it.done != nullptr && *it.done;
+    const int tier = TIERED ? *it.tier : 0;
+    if (threadIdx.x == 0) {
+        bk.a = it.a;
+        bk.b = it.b;
+        bk.block = (int)((int64_t)blockIdx.x - it.blockStart);
+        bk.tier = tier;
+    }
+    __syncthreads();
+    return !stopped && tier < SEP_TIERS;
+}
+
+// runs body(std::integral_constant<int, N>) for the power of two N = 2^k, 16 <= N <= 2048
+template <typename F>
+__device__ __forceinline__ void for_pow2(int k, F&& body) {
+    switch (k) {
+        case 4: body(std::integral_constant<int, 16>()); break;
+        case 5: body(std::integral_constant<int, 32>()); break;
+        case 6: body(std::integral_constant<int, 64>()); break;
+        case 7: body(std::integral_constant<int, 128>()); break;
+        case 8: body(std::integral_constant<int, 256>()); break;
+        case 9: body(std::integral_constant<int, 512>()); break;
+        case 10: body(std::integral_constant<int, 1024>()); break;
+        default: body(std::integral_constant<int, 2048>()); break;
+    }
+}
+
+}  // namespace
+
+// ------------------------------------------------------------------------- range
+
+// Tier of a share of the finest field (all phases); sep_feat combines the blocks' results.
+// NaN and values beyond every tier give SEP_TIERS: direct kernels.
+__global__ void __launch_bounds__(256) sep_range_kernel(const __grid_constant__ SepTables tb,
+                                                        const SepItem* __restrict__ items, int nitem) {
+    const int it = find_segment(items, nitem, (int64_t)blockIdx.x);
+    const SepLevel& lv = tb.level[items[it].level];
+    if (lv.done != nullptr && *lv.done) return;
+    const int blk = (int)((int64_t)blockIdx.x - items[it].blockStart), nblk = items[it].a;
+    const int64_t count = lv.N * lv.phases, stride = (int64_t)nblk * blockDim.x;
+    const float* __restrict__ field = lv.field;
+    float lo = 0.f, hi = 0.f;
+    int bad = 0;
+    for (int64_t i = (int64_t)blk * blockDim.x + threadIdx.x; i < count; i += 4 * stride) {
+        float v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = i + u * stride < count ? field[i + u * stride] : 0.f;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            bad |= !(v[u] == v[u]);
+            lo = fminf(lo, v[u]);
+            hi = fmaxf(hi, v[u]);
+        }
+    }
+    int t = 0;
+    while (t < tb.ntier && !(lo >= tb.tier[t].lo && hi <= tb.tier[t].hi)) ++t;
+    if (bad || t >= tb.ntier) t = SEP_TIERS;
+    t = __reduce_max_sync(0xffffffffu, t);
+    __shared__ int sh[8];
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = t;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) t = max(t, sh[w]);
+        lv.tiers[blk] = t;
+    }
+}
+
+// ------------------------------------------------------------------------- features
+
+namespace {
+
+// Coefficients of a tier in shared memory: cf[j * SEP_STRIDE + p], DERIV: times j, for the
+// series T_j' = j U_{j-1}.
+constexpr int SEP_STRIDE = 16;
+static_assert(SEP_MAX_PAIRS <= SEP_STRIDE, "one row of coefficients holds every pair");
+
+template <bool DERIV>
+__device__ __forceinline__ void load_coef(const SepTables& tb, const SepTier& t, float2* cf) {
+    const int stride = sep_coef_stride(t.npair);
+    for (int i = threadIdx.x; i < t.deg * SEP_STRIDE; i += blockDim.x) {
+        const int j = i / SEP_STRIDE, p = i % SEP_STRIDE;
+        float2 c = p < t.npair ? tb.coef[t.coef + j * stride + p] : make_float2(0.f, 0.f);
+        if (DERIV) c = make_float2((float)j * c.x, (float)j * c.y);
+        cf[i] = c;
+    }
+}
+
+// One packed pair of features (DERIV: of their derivatives) at C normalised values:
+// sum_j c_j W_j(x), W = T_j (DERIV: U_{j-1}), both W_{j+1} = 2 x W_j - W_{j-1}.  The terms from
+// j = 4 on are summed first and the four large ones last, so that the small terms are not
+// lost against them.  Bound by the FP32 pipe: per term one FFMA2 and one FFMA.
+template <bool DERIV, int C>
+__device__ __forceinline__ void eval_features(const float2* __restrict__ cf, int deg, const float (&x)[C],
+                                              float2 (&out)[C]) {
+    float x2[C], w0[C], w1[C];
+#pragma unroll
+    for (int e = 0; e < C; ++e) {
+        x2[e] = 2.f * x[e];
+        out[e] = make_float2(0.f, 0.f);
+        // W_3 and W_4
+        if (DERIV) {
+            w0[e] = fmaf(x2[e], x2[e], -1.f);               // U_2
+            w1[e] = fmaf(x2[e], w0[e], -x2[e]);             // U_3
+        } else {
+            const float t2 = fmaf(x2[e], x[e], -1.f);
+            w0[e] = fmaf(x2[e], t2, -x[e]);                 // T_3
+            w1[e] = fmaf(x2[e], w0[e], -t2);                // T_4
+        }
+    }
+    const float2* c = cf + 4 * SEP_STRIDE;
+    int j = 4;
+    for (; j + 1 < deg; j += 2, c += 2 * SEP_STRIDE) {
+        const float2 ca = c[0], cb = c[SEP_STRIDE];
+#pragma unroll
+        for (int e = 0; e < C; ++e) {
+            out[e] = __ffma2_rn(ca, make_float2(w1[e], w1[e]), out[e]);
+            w0[e] = fmaf(x2[e], w1[e], -w0[e]);
+            out[e] = __ffma2_rn(cb, make_float2(w0[e], w0[e]), out[e]);
+            w1[e] = fmaf(x2[e], w0[e], -w1[e]);
+        }
+    }
+    if (j < deg) {
+        const float2 ca = c[0];
+#pragma unroll
+        for (int e = 0; e < C; ++e) out[e] = __ffma2_rn(ca, make_float2(w1[e], w1[e]), out[e]);
+    }
+    const float2 c0 = cf[0], c1 = cf[SEP_STRIDE], c2 = cf[2 * SEP_STRIDE], c3 = cf[3 * SEP_STRIDE];
+#pragma unroll
+    for (int e = 0; e < C; ++e) {
+        float a1, a2, a3;
+        if (DERIV) {
+            a1 = 1.f;
+            a2 = x2[e];
+            a3 = fmaf(x2[e], x2[e], -1.f);
+        } else {
+            a1 = x[e];
+            a2 = fmaf(x2[e], x[e], -1.f);
+            a3 = fmaf(x2[e], a2, -x[e]);
+        }
+        out[e] = __ffma2_rn(c3, make_float2(a3, a3), out[e]);
+        out[e] = __ffma2_rn(c2, make_float2(a2, a2), out[e]);
+        out[e] = __ffma2_rn(c1, make_float2(a1, a1), out[e]);
+        if (!DERIV) out[e] = __fadd2_rn(c0, out[e]);
+    }
+}
+
+// rows of a block of the feature and gradient kernels: SLOTS feature pairs side by side
+template <int N>
+struct RowShape {
+    static constexpr int T = N / 8, LINES = SEP_THREADS / T;
+    static constexpr int SLOTS = LINES < SEP_SLOTS ? LINES : SEP_SLOTS;
+    static constexpr int ROWS = LINES / SLOTS;
+    static constexpr bool WARP = T <= 32;
+};
+
+template <int N>
+__device__ __forceinline__ Line<N> row_line(int line, int t, int lines) {
+    constexpr int P = row_pitch<N>();
+    Line<N> ln;
+    ln.tw = sep_smem;
+    ln.buf[0] = sep_smem + N + line * P;
+    ln.buf[1] = ln.buf[0] + lines * P;
+    ln.t = t;
+    return ln;
+}
+
+}  // namespace
+
+// item: (level, phase a); blocks: groups of rows.  Features of whole rows and their transform
+// along x.  Every block first combines the range blocks' tiers; the first block of the finest
+// level leaves the result for the later kernels.
+__global__ void __launch_bounds__(SEP_THREADS, 2) sep_feat_kernel(const __grid_constant__ SepTables tb,
+                                                                  const SepItem* __restrict__ items, int nitem) {
+    __shared__ SepBlock bk;
+    __shared__ int tsh[SEP_THREADS / 32];
+    __shared__ __align__(16) float2 cf[SEP_MAX_DEG * SEP_STRIDE];
+    if (!enter<false>(tb, items, nitem, bk)) return;
+    const SepLevel& lv = bk.lv;
+    {
+        int t = 0;
+        for (int i = threadIdx.x; i < lv.ntiers; i += blockDim.x) t = max(t, lv.tiers[i]);
+        t = __reduce_max_sync(0xffffffffu, t);
+        if ((threadIdx.x & 31) == 0) tsh[threadIdx.x >> 5] = t;
+    }
+    __syncthreads();
+    int tier = tsh[0];
+    for (int i = 1; i < SEP_THREADS / 32; ++i) tier = max(tier, tsh[i]);
+    if (lv.first && bk.a == 0 && bk.block == 0 && threadIdx.x == 0) *lv.tier = tier;
+    if (tier >= SEP_TIERS) return;
+    const SepTier& t = tb.tier[tier];
+    load_coef<false>(tb, t, cf);
+    const int rowsN = lv.n0 * lv.n1, n = lv.n2;
+    const int row0 = bk.block * lv.rowsF, rows = min(lv.rowsF, rowsN - row0);
+    const float* __restrict__ field = lv.field + (int64_t)bk.a * lv.N + (int64_t)row0 * n;
+    float2* __restrict__ Z = lv.Z + (int64_t)bk.a * lv.maxPairs * lv.N + (int64_t)row0 * n;
+    fill_twiddles(sep_smem, n);
+    __syncthreads();
+    if (lv.ax[2].fast) {
+        for_pow2(lv.ax[2].fast, [&](auto c) {
+            constexpr int N = decltype(c)::value;
+            using S = RowShape<N>;
+            const int line = threadIdx.x / S::T, p = line % S::SLOTS, row = line / S::SLOTS;
+            const Line<N> ln = row_line<N>(line, threadIdx.x % S::T, S::LINES);
+            const bool in = row < rows;
+            float x[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                x[e] = in ? (field[row * N + ln.t + e * S::T] - t.mid) * t.inv_half : 0.f;
+            for (int p0 = 0; p0 < t.npair; p0 += S::SLOTS) {
+                const bool live = in && p0 + p < t.npair;
+                float2 v[8];
+                if (live) eval_features<false, 8>(cf + p0 + p, t.deg, x, v);
+                p2_fft<N, S::WARP, 0>(v, ln);
+                if (live) {
+                    float2* out = Z + (int64_t)(p0 + p) * lv.N + row * N + ln.t;
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) out[e * S::T] = v[e];
+                }
+                line_sync<S::WARP>();       // the next round starts in the buffer this one started in
+            }
+        });
+        return;
+    }
+    const int pitch = spad(n - 1) + 2;
+    const float inv_n = 1.0f / (float)n;
+    const SepShared s = sep_shared(n, lv.rowsF * SEP_SLOTS, pitch);
+    for (int p0 = 0; p0 < t.npair; p0 += SEP_SLOTS) {
+        const int nc = min(SEP_SLOTS, t.npair - p0);
+        __syncthreads();
+        for (int e = threadIdx.x; e < rows * nc * n; e += blockDim.x) {
+            const int q = fdiv(e, inv_n), i = e - q * n;        // q = l nc + c
+            const int l = q / nc, c = q - l * nc;
+            const float x[1] = {(field[l * n + i] - t.mid) * t.inv_half};
+            float2 f[1];
+            eval_features<false, 1>(cf + p0 + c, t.deg, x, f);
+            s.a[q * pitch + spad(i)] = f[0];
+        }
+        const float2* r = transform(lv.ax[2], s.a, s.b, s.tw, rows * nc, pitch);
+        for (int e = threadIdx.x; e < rows * nc * n; e += blockDim.x) {
+            const int q = fdiv(e, inv_n), i = e - q * n;
+            const int l = q / nc, c = q - l * nc;
+            Z[(int64_t)(p0 + c) * lv.N + l * n + i] = r[q * pitch + spad(i)];
+        }
+    }
+}
+
+// ------------------------------------------------------------------------- columns
+
+namespace {
+
+// Threads of a block over L adjacent columns (fastest, for coalesced rows), T per line and the
+// SLOTS = SEP_THREADS / (L T) groups side by side (feature pairs, or planes).
+template <int N>
+struct Cols {
+    static constexpr int T = N / 8;
+    int L, l, slot, slots;
+    Line<N> ln;
+    __device__ __forceinline__ explicit Cols(int L_) : L(L_) {
+        const int sh = 31 - __clz(L);
+        l = threadIdx.x & (L - 1);
+        const int r = threadIdx.x >> sh;
+        ln.t = r % T;
+        slot = r / T;
+        slots = SEP_THREADS / T >> sh;
+        const int pitch = sep_pitch(N, L);
+        ln.tw = sep_smem;
+        ln.buf[0] = sep_smem + N + (slot * L + l) * pitch;
+        ln.buf[1] = ln.buf[0] + slots * L * pitch;
+    }
+};
+
+// the columns of one block along a strided axis
+struct ColGroup {
+    int n, L, cols;
+    int64_t base, stride;      // first element of the group within one grid; step along the axis
+};
+
+// last axis: z in 3-D, y in 2-D
+__device__ __forceinline__ ColGroup last_axis(const SepLevel& lv, int block, int& x0, int& y) {
+    ColGroup g;
+    g.L = lv.colsL;
+    const int xg = (lv.n2 + g.L - 1) / g.L;
+    x0 = (block % xg) * g.L;
+    y = lv.n0 > 1 ? block / xg : 0;
+    g.n = lv.n0 > 1 ? lv.n0 : lv.n1;
+    g.cols = min(g.L, lv.n2 - x0);
+    g.stride = lv.n0 > 1 ? (int64_t)lv.n1 * lv.n2 : lv.n2;
+    g.base = (int64_t)y * lv.n2 + x0;
+    return g;
+}
+
+__device__ __forceinline__ const SepAxis& last_ax(const SepLevel& lv) { return lv.n0 > 1 ? lv.ax[0] : lv.ax[1]; }
+
+template <int N>
+__device__ __forceinline__ void load8(const float2* __restrict__ src, const ColGroup& g, const Cols<N>& c, bool on,
+                                      float2 (&v)[8]) {
+    const float2* p = src + g.base + c.ln.t * g.stride + c.l;
+    const int64_t step = (N / 8) * g.stride;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = on && c.l < g.cols ? p[e * step] : make_float2(0.f, 0.f);
+}
+
+template <int N>
+__device__ __forceinline__ void store8(float2* __restrict__ dst, const ColGroup& g, const Cols<N>& c, bool on,
+                                       const float2 (&v)[8]) {
+    float2* p = dst + g.base + c.ln.t * g.stride + c.l;
+    const int64_t step = (N / 8) * g.stride;
+    if (on && c.l < g.cols) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) p[e * step] = v[e];
+    }
+}
+
+// columns into shared lines (any length)
+__device__ __forceinline__ void load_cols(const float2* __restrict__ src, const ColGroup& g, int pitch, float2* dst) {
+    const int sh = 31 - __clz(g.L);
+    for (int e = threadIdx.x; e < g.L * g.n; e += blockDim.x) {
+        const int l = e & (g.L - 1), i = e >> sh;
+        dst[l * pitch + spad(i)] = l < g.cols ? src[g.base + i * g.stride + l] : make_float2(0.f, 0.f);
+    }
+}
+
+}  // namespace
+
+// Middle axis of 3-D, in place on Z (forward) or on the product spectra (INVERSE).  item:
+// (level, phase a); blocks: groups of planes' columns (x fastest, then z), then pairs.
+template <bool INVERSE>
+__global__ void __launch_bounds__(SEP_THREADS, 2) sep_fft_y_kernel(const __grid_constant__ SepTables tb,
+                                                                   const SepItem* __restrict__ items, int nitem) {
+    __shared__ SepBlock bk;
+    if (!enter<true>(tb, items, nitem, bk)) return;
+    const SepLevel& lv = bk.lv;
+    const int L = lv.colsY, n = lv.n1;
+    const int xg = (lv.n2 + L - 1) / L, groups = xg * lv.n0;
+    const int slots = lv.ax[1].fast ? SEP_BLOCK_PTS / (L * n) : 1;
+    const int per = (groups + slots - 1) / slots;      // blocks of one pair
+    const int p = bk.block / per, g0 = (bk.block % per) * slots;
+    if (p >= tb.tier[bk.tier].npair) return;
+    float2* grid = (INVERSE ? lv.Q : lv.Z) + ((int64_t)bk.a * lv.maxPairs + p) * lv.N;
+    fill_twiddles(sep_smem, n);
+    auto group = [&](int gi) {
+        ColGroup g;
+        g.n = n;
+        g.L = L;
+        const int x0 = (gi % xg) * L, z = gi / xg;
+        g.cols = min(L, lv.n2 - x0);
+        g.stride = lv.n2;
+        g.base = (int64_t)z * lv.n1 * lv.n2 + x0;
+        return g;
+    };
+    if (lv.ax[1].fast) {
+        __syncthreads();
+        for_pow2(lv.ax[1].fast, [&](auto cc) {
+            constexpr int N = decltype(cc)::value;
+            const Cols<N> c(L);
+            const bool on = g0 + c.slot < groups;
+            const ColGroup g = group(on ? g0 + c.slot : 0);
+            float2 v[8];
+            load8<N>(grid, g, c, on, v);
+            if (INVERSE) swap8(v);
+            p2_fft<N, false, 0>(v, c.ln);
+            if (INVERSE) swap8(v);
+            store8<N>(grid, g, c, on, v);
+        });
+        return;
+    }
+    const ColGroup g = group(g0);
+    const int pitch = sep_pitch(n, L), sh = 31 - __clz(L);
+    const SepShared s = sep_shared(n, L, pitch);
+    for (int e = threadIdx.x; e < L * n; e += blockDim.x) {
+        const int l = e & (L - 1), i = e >> sh;
+        const float2 v = l < g.cols ? grid[g.base + i * g.stride + l] : make_float2(0.f, 0.f);
+        s.a[l * pitch + spad(i)] = INVERSE ? swapf(v) : v;
+    }
+    const float2* r = transform(lv.ax[1], s.a, s.b, s.tw, L, pitch);
+    for (int e = threadIdx.x; e < L * n; e += blockDim.x) {
+        const int l = e & (L - 1), i = e >> sh;
+        const float2 v = r[l * pitch + spad(i)];
+        if (l < g.cols) grid[g.base + i * g.stride + l] = INVERSE ? swapf(v) : v;
+    }
+}
+
+// ------------------------------------------------------------------------- last axis: power
+
+// item: (level, phases a, b).  Sums s_k conj(Z^a_k) Z^b_k over the feature pairs and writes the
+// inverse along the last axis, cropped to r = 0 .. P (-r belongs to the pair (b, a)).  CROSS:
+// a and b may differ.  The next round's columns are loaded while the current one is transformed.
+template <bool CROSS>
+__global__ void __launch_bounds__(SEP_THREADS, CROSS ? 1 : 2)
+sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__ items, int nitem) {
+    __shared__ SepBlock bk;
+    __shared__ double dcs[SEP_THREADS / 2];
+    if (!enter<true>(tb, items, nitem, bk)) return;
+    const SepLevel& lv = bk.lv;
+    const SepTier& t = tb.tier[bk.tier];
+    int x0, y;
+    const ColGroup g = last_axis(lv, bk.block, x0, y);
+    const SepAxis& ax = last_ax(lv);
+    const bool dc_block = x0 == 0 && y == 0;
+    const float2* Za = lv.Z + (int64_t)bk.a * lv.maxPairs * lv.N;
+    const float2* Zb = lv.Z + (int64_t)bk.b * lv.maxPairs * lv.N;
+    const int pair = bk.a * lv.phases + bk.b;
+    const int P = lv.n0 > 1 ? lv.P0 : lv.P1;
+    // 3-D: U[r][y][x]; 2-D: V[r][x]
+    float2* out = (lv.n0 > 1 ? lv.U : lv.V) + (int64_t)pair * (lv.n0 > 1 ? lv.strideU : lv.strideV) + g.base;
+    fill_twiddles(sep_smem, g.n);
+    const bool cross = CROSS && bk.a != bk.b;
+    if (ax.fast) {
+        __syncthreads();
+        for_pow2(ax.fast, [&](auto cc) {
+            constexpr int N = decltype(cc)::value, T = N / 8;
+            constexpr int PAR1 = p2_exchanges(N) & 1;
+            const Cols<N> c(g.L);
+            float2 acc[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] = make_float2(0.f, 0.f);
+            double dc = 0.0;
+            const bool has_dc = dc_block && c.l == 0 && c.ln.t == 0;
+            float2 nx[8];
+            load8<N>(Za + (int64_t)c.slot * lv.N, g, c, c.slot < t.npair, nx);
+            for (int p0 = 0; p0 < t.npair; p0 += c.slots) {
+                const int p = p0 + c.slot;
+                const float sg = p < t.npos ? 1.f : -1.f;
+                float2 v[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] = nx[e];
+                if (!cross) {
+                    const int q = p + c.slots;
+                    if (p0 + c.slots < t.npair) load8<N>(Za + (int64_t)q * lv.N, g, c, q < t.npair, nx);
+                    p2_fft<N, false, 0>(v, c.ln);
+                    if (PAR1 != 0) __syncthreads();   // the next round starts in buffer 0 again
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) acc[e].x = fmaf(sg, fmaf(v[e].x, v[e].x, v[e].y * v[e].y), acc[e].x);
+                    if (has_dc) dc += (double)sg * ((double)v[0].x * v[0].x + (double)v[0].y * v[0].y);
+                } else {
+                    float2 u[8];
+                    load8<N>(Zb + (int64_t)p * lv.N, g, c, p < t.npair, u);
+                    p2_fft<N, false, 0>(v, c.ln);
+                    if (PAR1 != 0) __syncthreads();
+                    p2_fft<N, false, 0>(u, c.ln);
+                    if (PAR1 != 0) __syncthreads();
+                    // conj(v) u; the imaginary part as a difference of rounded products, so that
+                    // exchanging a and b gives exactly the conjugate
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        acc[e].x = fmaf(sg, __fadd_rn(__fmul_rn(v[e].x, u[e].x), __fmul_rn(v[e].y, u[e].y)), acc[e].x);
+                        acc[e].y = fmaf(sg, __fsub_rn(__fmul_rn(v[e].x, u[e].y), __fmul_rn(v[e].y, u[e].x)), acc[e].y);
+                    }
+                    if (has_dc) dc += (double)sg * ((double)v[0].x * u[0].x + (double)v[0].y * u[0].y);
+                    const int q = p + c.slots;
+                    if (p0 + c.slots < t.npair) load8<N>(Za + (int64_t)q * lv.N, g, c, q < t.npair, nx);
+                }
+            }
+            // sum over the slots in a fixed order; the mean's power goes on in FP64
+            if (has_dc) dcs[c.slot] = dc;
+            __syncthreads();
+            if (c.slots > 1) {
+                float2* red = sep_smem + N;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) red[e * SEP_THREADS + threadIdx.x] = acc[e];
+                __syncthreads();
+                const int group = SEP_THREADS / c.slots, at = threadIdx.x % group;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    float2 s = red[e * SEP_THREADS + at];
+                    for (int k = 1; k < c.slots; ++k) s = caddf(s, red[e * SEP_THREADS + at + k * group]);
+                    acc[e] = s;
+                }
+                __syncthreads();
+            }
+            if (has_dc && c.slot == 0) {
+                double s = dcs[0];
+                for (int k = 1; k < c.slots; ++k) s += dcs[k];
+                lv.dc[pair] = s;
+            }
+            if (has_dc) acc[0] = make_float2(0.f, 0.f);
+            swap8(acc);
+            p2_fft<N, false, 0>(acc, c.ln);
+            if (c.slot == 0 && c.l < g.cols) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const int i = c.ln.t + e * T;
+                    if (i <= P) out[i * g.stride + c.l] = swapf(acc[e]);
+                }
+            }
+        });
+        return;
+    }
+    const int pitch = sep_pitch(g.n, g.L), sh = 31 - __clz(g.L), total = g.L * g.n;
+    const SepShared s = sep_shared(g.n, g.L, pitch);
+    float2 acc[SEP_OWN], za[SEP_OWN];
+#pragma unroll
+    for (int q = 0; q < SEP_OWN; ++q) acc[q] = make_float2(0.f, 0.f);
+    double dc = 0.0;
+    const bool has_dc = dc_block && threadIdx.x == 0;   // element 0 is frequency 0
+    auto own = [&](auto f) {
+#pragma unroll
+        for (int q = 0; q < SEP_OWN; ++q) {
+            const int e = threadIdx.x + q * SEP_THREADS;
+            if (e < total) f(q, (e & (g.L - 1)) * pitch + spad(e >> sh));
+        }
+    };
+    for (int p = 0; p < t.npair; ++p) {
+        const float sg = p < t.npos ? 1.f : -1.f;
+        __syncthreads();
+        load_cols(Za + (int64_t)p * lv.N, g, pitch, s.a);
+        const float2* r = transform(ax, s.a, s.b, s.tw, g.L, pitch);
+        if (cross) {
+            own([&](int q, int at) { za[q] = r[at]; });
+            __syncthreads();
+            load_cols(Zb + (int64_t)p * lv.N, g, pitch, s.a);
+            r = transform(ax, s.a, s.b, s.tw, g.L, pitch);
+        }
+        own([&](int q, int at) {
+            const float2 v = r[at], u = cross ? za[q] : v;
+            acc[q].x = fmaf(sg, __fadd_rn(__fmul_rn(u.x, v.x), __fmul_rn(u.y, v.y)), acc[q].x);
+            acc[q].y = fmaf(sg, __fsub_rn(__fmul_rn(u.x, v.y), __fmul_rn(u.y, v.x)), acc[q].y);
+            if (q == 0 && has_dc) dc += (double)sg * ((double)u.x * v.x + (double)u.y * v.y);
+        });
+    }
+    if (has_dc) {
+        lv.dc[pair] = dc;
+        acc[0] = make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+    own([&](int q, int at) { s.a[at] = swapf(acc[q]); });
+    const float2* r = transform(ax, s.a, s.b, s.tw, g.L, pitch);
+    for (int e = threadIdx.x; e < g.L * (P + 1); e += blockDim.x) {
+        const int l = e & (g.L - 1), i = e >> sh;
+        if (l < g.cols) out[i * g.stride + l] = swapf(r[l * pitch + spad(i)]);
+    }
+}
+
+// ------------------------------------------------------------------------- 3-D middle axis of the window
+
+// item: (level, phases a, b); blocks: groups of columns (x fastest, then kept rz).  DESC: U -> V,
+// inverse along y cropped to -P1 .. P1.  Otherwise V -> U: G's rows embedded along y and
+// transformed.
+template <bool DESC>
+__global__ void __launch_bounds__(SEP_THREADS, 2) sep_win_y_kernel(const __grid_constant__ SepTables tb,
+                                                                   const SepItem* __restrict__ items, int nitem) {
+    __shared__ SepBlock bk;
+    if (!enter<true>(tb, items, nitem, bk)) return;
+    const SepLevel& lv = bk.lv;
+    const int L = lv.colsY, n = lv.n1, P1 = lv.P1, wy = 2 * P1 + 1;
+    const int xg = (lv.n2 + L - 1) / L, groups = xg * (lv.P0 + 1);
+    const int slots = lv.ax[1].fast ? SEP_BLOCK_PTS / (L * n) : 1;
+    const int pair = bk.a * lv.phases + bk.b;
+    float2* U = lv.U + (int64_t)pair * lv.strideU;
+    float2* V = lv.V + (int64_t)pair * lv.strideV;
+    fill_twiddles(sep_smem, n);
+    auto window = [&](const float2* src, int i, int64_t stride) {
+        // ry = i and ry = i - n (both at the aliased ry = +-n/2)
+        float2 v = make_float2(0.f, 0.f);
+        if (i <= P1) v = src[(int64_t)(i + P1) * stride];
+        if (i > 0 && n - i <= P1) v = caddf(v, src[(int64_t)(i - n + P1) * stride]);
+        return v;
+    };
+    if (lv.ax[1].fast) {
+        __syncthreads();
+        for_pow2(lv.ax[1].fast, [&](auto cc) {
+            constexpr int N = decltype(cc)::value, T = N / 8;
+            const Cols<N> c(L);
+            const int gi = bk.block * slots + c.slot, k = gi / xg, x = (gi % xg) * L + c.l;
+            const bool on = gi < groups && x < lv.n2;
+            float2* u = U + (int64_t)k * lv.n1 * lv.n2 + x;
+            float2* w = V + (int64_t)k * wy * lv.n2 + x;
+            float2 v[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int i = c.ln.t + e * T;
+                v[e] = !on ? make_float2(0.f, 0.f) : (DESC ? swapf(u[(int64_t)i * lv.n2]) : window(w, i, lv.n2));
+            }
+            p2_fft<N, false, 0>(v, c.ln);
+            if (!on) return;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int i = c.ln.t + e * T;
+                if (!DESC) {
+                    u[(int64_t)i * lv.n2] = v[e];
+                } else {
+                    if (i <= P1) w[(int64_t)(i + P1) * lv.n2] = swapf(v[e]);
+                    if (i > 0 && N - i <= P1) w[(int64_t)(i - N + P1) * lv.n2] = swapf(v[e]);
+                }
+            }
+        });
+        return;
+    }
+    const int gi = bk.block, k = gi / xg, x0 = (gi % xg) * L, cols = min(L, lv.n2 - x0);
+    const int pitch = sep_pitch(n, L), sh = 31 - __clz(L);
+    const SepShared s = sep_shared(n, L, pitch);
+    U += (int64_t)k * lv.n1 * lv.n2 + x0;
+    V += (int64_t)k * wy * lv.n2 + x0;
+    for (int e = threadIdx.x; e < L * n; e += blockDim.x) {
+        const int l = e & (L - 1), i = e >> sh;
+        float2 v = make_float2(0.f, 0.f);
+        if (l < cols) v = DESC ? swapf(U[(int64_t)i * lv.n2 + l]) : window(V + l, i, lv.n2);
+        s.a[l * pitch + spad(i)] = v;
+    }
+    const float2* r = transform(lv.ax[1], s.a, s.b, s.tw, L, pitch);
+    for (int e = threadIdx.x; e < L * (DESC ? wy : n); e += blockDim.x) {
+        const int l = e & (L - 1), i = e >> sh;
+        if (l >= cols) continue;
+        if (DESC) {
+            const int ry = i - P1;
+            V[(int64_t)i * lv.n2 + l] = swapf(r[l * pitch + spad(ry < 0 ? ry + n : ry)]);
+        } else {
+            U[(int64_t)i * lv.n2 + l] = r[l * pitch + spad(i)];
+        }
+    }
+}
+
+// ------------------------------------------------------------------------- window rows
+
+namespace {
+
+// row `row` of the kept half of the window -> (rz, ry): 3-D rz = 0 .. P0 and every ry, 2-D
+// ry = 0 .. P1
+__device__ __forceinline__ void window_row(const SepLevel& lv, int row, int& rz, int& ry) {
+    if (lv.n0 > 1) {
+        const int wy = 2 * lv.P1 + 1;
+        rz = row / wy;
+        ry = row - rz * wy - lv.P1;
+    } else {
+        rz = 0;
+        ry = row;
+    }
+}
+
+__device__ __forceinline__ int window_rows(const SepLevel& lv) {
+    return lv.n0 > 1 ? (lv.P0 + 1) * (2 * lv.P1 + 1) : lv.P1 + 1;
+}
+
+// Canonical half-window index of (rz, ry, rx), -1 if it is not in the half window.
+__device__ __forceinline__ int half_index(const SepLevel& lv, int rz, int ry, int rx) {
+    const int Px = lv.P2, Py = lv.P1;
+    if (rz == 0 && ry == 0) return rx >= 0 ? rx : -1;
+    if (rz == 0) return ry > 0 ? (Px + 1) + (ry - 1) * (2 * Px + 1) + (rx + Px) : -1;
+    if (rz < 0) return -1;
+    return (Px + 1) + Py * (2 * Px + 1) + ((rz - 1) * (2 * Py + 1) + (ry + Py)) * (2 * Px + 1) + (rx + Px);
+}
+
+}  // namespace
+
+// item: (level, phases a, b); blocks: groups of rowsW window rows.  Inverse along x: the
+// entries of block (a, b).
+__global__ void __launch_bounds__(SEP_THREADS, 2) sep_desc_kernel(const __grid_constant__ SepTables tb,
+                                                                  const SepItem* __restrict__ items, int nitem) {
+    __shared__ SepBlock bk;
+    if (!enter<true>(tb, items, nitem, bk)) return;
+    const SepLevel& lv = bk.lv;
+    const int n = lv.n2, P2 = lv.P2;
+    const int R = window_rows(lv);
+    const int row0 = bk.block * lv.rowsW, rows = min(lv.rowsW, R - row0);
+    const int pair = bk.a * lv.phases + bk.b;
+    const float2* V = lv.V + (int64_t)pair * lv.strideV + (int64_t)row0 * n;
+    const double dc = lv.dc[pair];
+    float* desc = lv.desc + (int64_t)pair * lv.Khalf;
+    auto entry = [&](int l, int rx, float c) {
+        int rz, ry;
+        window_row(lv, row0 + l, rz, ry);
+        const int k = half_index(lv, rz, ry, rx);
+        if (k >= 0) desc[k] = (float)(((double)c + dc) * lv.scaleD);
+    };
+    fill_twiddles(sep_smem, n);
+    if (lv.ax[2].fast) {
+        __syncthreads();
+        for_pow2(lv.ax[2].fast, [&](auto cc) {
+            constexpr int N = decltype(cc)::value, T = N / 8;
+            constexpr bool WARP = T <= 32;
+            const int line = threadIdx.x / T;
+            const Line<N> ln = row_line<N>(line, threadIdx.x % T, SEP_THREADS / T);
+            const bool in = line < rows;
+            float2 v[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = in ? swapf(V[line * N + ln.t + e * T]) : make_float2(0.f, 0.f);
+            p2_fft<N, WARP, 0>(v, ln);
+            if (!in) return;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int i = ln.t + e * T;
+                if (i <= P2) entry(line, i, v[e].y);
+                if (i > 0 && N - i <= P2) entry(line, i - N, v[e].y);
+            }
+        });
+        return;
+    }
+    const int pitch = spad(n - 1) + 2, wx = 2 * P2 + 1;
+    const SepShared s = sep_shared(n, lv.rowsW, pitch);
+    const float inv_n = 1.0f / (float)n;
+    for (int e = threadIdx.x; e < rows * n; e += blockDim.x) {
+        const int l = fdiv(e, inv_n), i = e - l * n;
+        s.a[l * pitch + spad(i)] = swapf(V[e]);
+    }
+    const float2* r = transform(lv.ax[2], s.a, s.b, s.tw, rows, pitch);
+    for (int e = threadIdx.x; e < rows * wx; e += blockDim.x) {
+        const int l = e / wx, rx = e - l * wx - P2;
+        entry(l, rx, r[l * pitch + spad(rx < 0 ? rx + n : rx)].y);
+    }
+}
+
+// item: (level, phases a, b); blocks: groups of rowsW window rows.  G(r) of the row (the
+// coefficient rule of the direct path's grid), embedded along x and transformed.
+__global__ void __launch_bounds__(SEP_THREADS, 2) sep_gx_kernel(const __grid_constant__ SepTables tb,
+                                                                const SepItem* __restrict__ items, int nitem) {
+    __shared__ SepBlock bk;
+    if (!enter<true>(tb, items, nitem, bk)) return;
+    const SepLevel& lv = bk.lv;
+    const int n = lv.n2, P2 = lv.P2;
+    const int R = window_rows(lv);
+    const int row0 = bk.block * lv.rowsW, rows = min(lv.rowsW, R - row0);
+    const int pair = bk.a * lv.phases + bk.b;
+    fill_twiddles(sep_smem, n);
+    const int64_t oab = (int64_t)pair * lv.Khalf, oba = ((int64_t)bk.b * lv.phases + bk.a) * lv.Khalf;
+    const float scale = lv.scaleG * (lv.sc != nullptr ? lv.sc->gscale : 1.f);
+    auto delta = [&](int64_t off, int k) {
+        float d = lv.src[off + k] - (lv.sub != nullptr ? lv.sub[off + k] : 0.f);
+        if (lv.tsum != nullptr) d = k == 0 ? d - lv.q / (1.f - lv.q) * *lv.tsum : d / (1.f - lv.q);
+        return d;
+    };
+    auto G = [&](int rz, int ry, int rx) {
+        const int k = half_index(lv, rz, ry, rx);
+        if (k == 0) return scale * (delta(oab, 0) + delta(oba, 0));
+        if (k > 0) return scale * delta(oab, k);
+        return scale * delta(oba, half_index(lv, -rz, -ry, -rx));
+    };
+    auto embedded = [&](int l, int i) {
+        int rz, ry;
+        window_row(lv, row0 + l, rz, ry);
+        float v = 0.f;
+        if (i <= P2) v = G(rz, ry, i);
+        if (i > 0 && n - i <= P2) v += G(rz, ry, i - n);
+        return v;
+    };
+    float2* V = lv.V + (int64_t)pair * lv.strideV + (int64_t)row0 * n;
+    if (lv.ax[2].fast) {
+        __syncthreads();
+        for_pow2(lv.ax[2].fast, [&](auto cc) {
+            constexpr int N = decltype(cc)::value, T = N / 8;
+            constexpr bool WARP = T <= 32;
+            const int line = threadIdx.x / T;
+            const Line<N> ln = row_line<N>(line, threadIdx.x % T, SEP_THREADS / T);
+            const bool in = line < rows;
+            float2 v[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = make_float2(in ? embedded(line, ln.t + e * T) : 0.f, 0.f);
+            p2_fft<N, WARP, 0>(v, ln);
+            if (!in) return;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) V[line * N + ln.t + e * T] = v[e];
+        });
+        return;
+    }
+    const int pitch = spad(n - 1) + 2;
+    const SepShared s = sep_shared(n, lv.rowsW, pitch);
+    const float inv_n = 1.0f / (float)n;
+    for (int e = threadIdx.x; e < rows * n; e += blockDim.x) {
+        const int l = fdiv(e, inv_n), i = e - l * n;
+        s.a[l * pitch + spad(i)] = make_float2(embedded(l, i), 0.f);
+    }
+    const float2* r = transform(lv.ax[2], s.a, s.b, s.tw, rows, pitch);
+    for (int e = threadIdx.x; e < rows * n; e += blockDim.x) {
+        const int l = fdiv(e, inv_n), i = e - l * n;
+        V[e] = r[l * pitch + spad(i)];
+    }
+}
+
+// ------------------------------------------------------------------------- last axis: products
+
+namespace {
+
+// Point i of G's column l of the phase pair (a, b), embedded along the last axis: rows
+// r = 0 .. P of the pair, and at -r the conjugates of the pair (b, a) (G^ab(-r) = G^ba(r); both
+// at r = +-n/2).
+struct GCols {
+    const float2 *ab, *ba;
+    int P, n;
+    int64_t stride;
+    __device__ __forceinline__ GCols(const SepLevel& lv, int a, int b, const ColGroup& g) {
+        P = lv.n0 > 1 ? lv.P0 : lv.P1;
+        const float2* base = (lv.n0 > 1 ? lv.U : lv.V) + g.base;
+        const int64_t size = lv.n0 > 1 ? lv.strideU : lv.strideV;
+        ab = base + (a * lv.phases + b) * size;
+        ba = base + (b * lv.phases + a) * size;
+        n = g.n;
+        stride = g.stride;
+    }
+    __device__ __forceinline__ float2 at(int i, int l) const {
+        float2 v = make_float2(0.f, 0.f);
+        if (i <= P) v = ab[i * stride + l];
+        if (i > 0 && n - i <= P) {
+            const float2 u = ba[(n - i) * stride + l];
+            v = make_float2(v.x + u.x, v.y - u.y);
+        }
+        return v;
+    }
+};
+
+}  // namespace
+
+// item: (level, phase a).  Spectrum of G along the last axis, then for every feature pair the
+// forward transform of the columns, the product sum_b conj(G^ab) Z^b and the inverse: Q^a, in
+// place of Z for a single phase (G is even then: a real spectrum).
+template <bool MULTI>
+__global__ void __launch_bounds__(SEP_THREADS, MULTI ? 1 : 2)
+sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__ items, int nitem) {
+    __shared__ SepBlock bk;
+    if (!enter<true>(tb, items, nitem, bk)) return;
+    const SepLevel& lv = bk.lv;
+    const SepTier& t = tb.tier[bk.tier];
+    int x0, y;
+    const ColGroup g = last_axis(lv, bk.block, x0, y);
+    const SepAxis& ax = last_ax(lv);
+    const float norm = 1.0f / (float)lv.N;       // of the unnormalised inverse
+    fill_twiddles(sep_smem, g.n);
+    if (ax.fast && (!MULTI || lv.phases <= SEP_FAST_PHASES)) {
+        __syncthreads();
+        for_pow2(ax.fast, [&](auto cc) {
+            constexpr int N = decltype(cc)::value, T = N / 8;
+            constexpr int EX = p2_exchanges(N), PAR1 = EX & 1;
+            const Cols<N> c(g.L);
+            // MULTI: every phase's spectrum, this thread's points, behind the line buffers
+            float2* gs = sep_smem + N + 2 * c.slots * c.L * sep_pitch(N, c.L) + threadIdx.x;
+            float gr[8];
+            float2 nx[8];
+            if (!MULTI) load8<N>(lv.Z + (int64_t)c.slot * lv.N, g, c, c.slot < t.npair, nx);
+            for (int b = 0; b < lv.phases; ++b) {
+                const GCols gc(lv, bk.a, b, g);
+                float2 v[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    v[e] = c.l < g.cols ? gc.at(c.ln.t + e * T, c.l) : make_float2(0.f, 0.f);
+                p2_fft<N, false, 0>(v, c.ln);
+                if (PAR1) __syncthreads();
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    if (MULTI) gs[(b * 8 + e) * SEP_THREADS] = make_float2(norm * v[e].x, -norm * v[e].y);
+                    else gr[e] = norm * v[e].x;
+                }
+            }
+            for (int p0 = 0; p0 < t.npair; p0 += c.slots) {
+                const int p = p0 + c.slot;
+                const bool on = p < t.npair;
+                float2 v[8];
+                if (!MULTI) {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) v[e] = nx[e];
+                    const int q = p + c.slots;
+                    if (p0 + c.slots < t.npair) load8<N>(lv.Z + (int64_t)q * lv.N, g, c, q < t.npair, nx);
+                    p2_fft<N, false, 0>(v, c.ln);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) v[e] = make_float2(gr[e] * v[e].y, gr[e] * v[e].x);
+                    p2_fft<N, false, PAR1>(v, c.ln);
+                } else {
+                    float2 acc[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) acc[e] = make_float2(0.f, 0.f);
+                    for (int b = 0; b < lv.phases; ++b) {
+                        load8<N>(lv.Z + ((int64_t)b * lv.maxPairs + p) * lv.N, g, c, on, v);
+                        p2_fft<N, false, 0>(v, c.ln);
+                        if (PAR1) __syncthreads();
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) {
+                            const float2 w = gs[(b * 8 + e) * SEP_THREADS];
+                            acc[e].x = fmaf(w.x, v[e].x, fmaf(-w.y, v[e].y, acc[e].x));
+                            acc[e].y = fmaf(w.x, v[e].y, fmaf(w.y, v[e].x, acc[e].y));
+                        }
+                    }
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) v[e] = swapf(acc[e]);
+                    p2_fft<N, false, 0>(v, c.ln);
+                    if (PAR1) __syncthreads();
+                }
+                swap8(v);
+                store8<N>(lv.Q + ((int64_t)bk.a * lv.maxPairs + p) * lv.N, g, c, on, v);
+            }
+        });
+        return;
+    }
+    const int pitch = sep_pitch(g.n, g.L), sh = 31 - __clz(g.L), total = g.L * g.n;
+    const SepShared s = sep_shared(g.n, g.L, pitch);
+    float2* gs = s.b + g.L * pitch;              // the spectra of every b, own points
+    auto own = [&](auto f) {
+#pragma unroll
+        for (int q = 0; q < SEP_OWN; ++q) {
+            const int e = threadIdx.x + q * SEP_THREADS;
+            if (e < total) f(q, e, (e & (g.L - 1)) * pitch + spad(e >> sh));
+        }
+    };
+    for (int b = 0; b < lv.phases; ++b) {
+        const GCols gc(lv, bk.a, b, g);
+        __syncthreads();
+        for (int e = threadIdx.x; e < total; e += blockDim.x) {
+            const int l = e & (g.L - 1), i = e >> sh;
+            s.a[l * pitch + spad(i)] = l < g.cols ? gc.at(i, l) : make_float2(0.f, 0.f);
+        }
+        const float2* r = transform(ax, s.a, s.b, s.tw, g.L, pitch);
+        own([&](int, int e, int at) { gs[b * total + e] = make_float2(norm * r[at].x, MULTI ? -norm * r[at].y : 0.f); });
+    }
+    for (int p = 0; p < t.npair; ++p) {
+        float2 acc[SEP_OWN];
+#pragma unroll
+        for (int q = 0; q < SEP_OWN; ++q) acc[q] = make_float2(0.f, 0.f);
+        for (int b = 0; b < lv.phases; ++b) {
+            __syncthreads();
+            load_cols(lv.Z + ((int64_t)b * lv.maxPairs + p) * lv.N, g, pitch, s.a);
+            const float2* r = transform(ax, s.a, s.b, s.tw, g.L, pitch);
+            own([&](int q, int e, int at) {
+                const float2 v = r[at], c = gs[b * total + e];
+                acc[q].x = fmaf(c.x, v.x, fmaf(-c.y, v.y, acc[q].x));
+                acc[q].y = fmaf(c.x, v.y, fmaf(c.y, v.x, acc[q].y));
+            });
+        }
+        __syncthreads();
+        own([&](int q, int, int at) { s.a[at] = swapf(acc[q]); });
+        const float2* o = transform(ax, s.a, s.b, s.tw, g.L, pitch);
+        float2* Q = lv.Q + ((int64_t)bk.a * lv.maxPairs + p) * lv.N;
+        for (int e = threadIdx.x; e < total; e += blockDim.x) {
+            const int l = e & (g.L - 1), i = e >> sh;
+            if (l < g.cols) Q[g.base + i * g.stride + l] = swapf(o[l * pitch + spad(i)]);
+        }
+    }
+}
+
+// ------------------------------------------------------------------------- gradient
+
+// item: (level, phase a); blocks: groups of rows.  Inverse along x of every feature pair and
+// g(y) = sum_k s_k p_k'(M_y) Q_k(y), the slots' shares added in a fixed order.
+__global__ void __launch_bounds__(SEP_THREADS, 1) sep_grad_kernel(const __grid_constant__ SepTables tb,
+                                                                  const SepItem* __restrict__ items, int nitem) {
+    __shared__ SepBlock bk;
+    __shared__ __align__(16) float2 cf[SEP_MAX_DEG * SEP_STRIDE];
+    if (!enter<true>(tb, items, nitem, bk)) return;
+    const SepLevel& lv = bk.lv;
+    const SepTier& t = tb.tier[bk.tier];
+    load_coef<true>(tb, t, cf);
+    const int rowsN = lv.n0 * lv.n1, n = lv.n2;
+    const int row0 = bk.block * lv.rowsF, rows = min(lv.rowsF, rowsN - row0);
+    const float* __restrict__ field = lv.field + (int64_t)bk.a * lv.N + (int64_t)row0 * n;
+    const float2* __restrict__ Q = lv.Q + (int64_t)bk.a * lv.maxPairs * lv.N + (int64_t)row0 * n;
+    float* __restrict__ part = lv.part + (int64_t)bk.a * lv.N + (int64_t)row0 * n;
+    fill_twiddles(sep_smem, n);
+    __syncthreads();
+    if (lv.ax[2].fast) {
+        for_pow2(lv.ax[2].fast, [&](auto cc) {
+            constexpr int N = decltype(cc)::value;
+            using S = RowShape<N>;
+            const int line = threadIdx.x / S::T, p = line % S::SLOTS, row = line / S::SLOTS;
+            const Line<N> ln = row_line<N>(line, threadIdx.x % S::T, S::LINES);
+            const bool in = row < rows;
+            float g[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) g[e] = 0.f;
+            for (int p0 = 0; p0 < t.npair; p0 += S::SLOTS) {
+                const bool live = in && p0 + p < t.npair;
+                float2 v[8];
+                const float2* src = Q + (int64_t)(p0 + p) * lv.N + row * N + ln.t;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] = live ? swapf(src[e * S::T]) : make_float2(0.f, 0.f);
+                p2_fft<N, S::WARP, 0>(v, ln);
+                if (live) {
+                    const float sg = p0 + p < t.npos ? t.inv_half : -t.inv_half;
+                    // four positions at a time: the series' state of eight does not fit the registers
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        float x[4];
+                        float2 f[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            x[e] = (field[row * N + ln.t + (4 * h + e) * S::T] - t.mid) * t.inv_half;
+                        eval_features<true, 4>(cf + p0 + p, t.deg, x, f);
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            g[4 * h + e] = fmaf(sg, fmaf(f[e].x, v[4 * h + e].y, f[e].y * v[4 * h + e].x), g[4 * h + e]);
+                    }
+                }
+                line_sync<S::WARP>();
+            }
+            // sum over the slots: red[slot][row][i]
+            __syncthreads();
+            float* red = reinterpret_cast<float*>(sep_smem + N);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) red[(p * S::ROWS + row) * N + ln.t + e * S::T] = g[e];
+            __syncthreads();
+            for (int o = threadIdx.x; o < rows * N; o += SEP_THREADS) {
+                float s = red[o];
+#pragma unroll
+                for (int k = 1; k < S::SLOTS; ++k) s += red[k * S::ROWS * N + o];
+                part[o] = s;
+            }
+        });
+        return;
+    }
+    const int pitch = spad(n - 1) + 2;
+    const SepShared s = sep_shared(n, lv.rowsF * SEP_SLOTS, pitch);
+    const float inv_n = 1.0f / (float)n;
+    float g[SEP_OWN];
+#pragma unroll
+    for (int q = 0; q < SEP_OWN; ++q) g[q] = 0.f;
+    for (int p0 = 0; p0 < t.npair; p0 += SEP_SLOTS) {
+        const int nc = min(SEP_SLOTS, t.npair - p0);
+        __syncthreads();
+        for (int e = threadIdx.x; e < rows * nc * n; e += blockDim.x) {
+            const int q = fdiv(e, inv_n), i = e - q * n;
+            const int l = q / nc, c = q - l * nc;
+            s.a[q * pitch + spad(i)] = swapf(Q[(int64_t)(p0 + c) * lv.N + l * n + i]);
+        }
+        const float2* r = transform(lv.ax[2], s.a, s.b, s.tw, rows * nc, pitch);
+#pragma unroll
+        for (int q = 0; q < SEP_OWN; ++q) {
+            const int e = threadIdx.x + q * SEP_THREADS;
+            if (e < rows * n) {
+                const int l = fdiv(e, inv_n), i = e - l * n;
+                const float x[1] = {(field[e] - t.mid) * t.inv_half};
+                for (int c = 0; c < nc; ++c) {
+                    float2 f[1];
+                    eval_features<true, 1>(cf + p0 + c, t.deg, x, f);
+                    const float2 v = r[(l * nc + c) * pitch + spad(i)];
+                    g[q] = fmaf(p0 + c < t.npos ? t.inv_half : -t.inv_half, fmaf(f[0].x, v.y, f[0].y * v.x), g[q]);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < SEP_OWN; ++q) {
+        const int e = threadIdx.x + q * SEP_THREADS;
+        if (e < rows * n) part[e] = g[q];
+    }
+}
+
+// ------------------------------------------------------------------------- launchers
+
+namespace {
+size_t bytes_of(int n, int lines, int pitch) { return (size_t)(((n + 1) & ~1) + 2 * lines * pitch) * sizeof(float2); }
+// power-of-two rows: the block's whole line capacity (row_pitch)
+size_t fast_row_bytes(int n) {
+    int p = n - 1 + (n - 1) / 16 + 1;
+    const int want = n >= 128 ? 0 : n / 8;
+    while (p % 16 != want) ++p;
+    return bytes_of(n, SEP_BLOCK_PTS / n, p);
+}
+}  // namespace
+
+size_t sep_smem_feat(const SepLevel& lv) {
+    const int n = lv.n2;
+    return lv.ax[2].fast ? fast_row_bytes(n) : bytes_of(n, lv.rowsF * SEP_SLOTS, n - 1 + ((n - 1) >> 4) + 2);
+}
+size_t sep_smem_window(const SepLevel& lv) {
+    const int n = lv.n2;
+    return lv.ax[2].fast ? fast_row_bytes(n) : bytes_of(n, lv.rowsW, n - 1 + ((n - 1) >> 4) + 2);
+}
+size_t sep_smem_y(const SepLevel& lv) {
+    const int lines = lv.ax[1].fast ? SEP_BLOCK_PTS / lv.n1 : lv.colsY;
+    return bytes_of(lv.n1, lines, sep_pitch(lv.n1, lv.colsY));
+}
+size_t sep_smem_last(const SepLevel& lv, bool mul) {
+    const SepAxis& ax = lv.n0 > 1 ? lv.ax[0] : lv.ax[1];
+    const int lines = ax.fast ? SEP_BLOCK_PTS / ax.n : lv.colsL;
+    size_t b = bytes_of(ax.n, lines, sep_pitch(ax.n, lv.colsL));
+    if (mul) {
+        if (!ax.fast || lv.phases > SEP_FAST_PHASES) b = bytes_of(ax.n, lv.colsL, sep_pitch(ax.n, lv.colsL)) +
+                                                         (size_t)lv.phases * lv.colsL * ax.n * sizeof(float2);
+        else if (lv.phases > 1) b += (size_t)lv.phases * SEP_BLOCK_PTS * sizeof(float2);
+    }
+    return b;
+}
+
+void launch_sep(SepKernel k, const SepTables& tb, const SepItem* items, int nitem, int64_t blocks, size_t smem,
+                cudaStream_t s) {
+    if (blocks <= 0) return;
+    const unsigned b = (unsigned)blocks;
+    constexpr int T = SEP_THREADS;
+    switch (k) {
+        case SEP_RANGE: sep_range_kernel<<<b, 256, 0, s>>>(tb, items, nitem); break;
+        case SEP_FEAT: sep_feat_kernel<<<b, T, smem, s>>>(tb, items, nitem); break;
+        case SEP_FFT_Y: sep_fft_y_kernel<false><<<b, T, smem, s>>>(tb, items, nitem); break;
+        case SEP_POWER: sep_power_kernel<false><<<b, T, smem, s>>>(tb, items, nitem); break;
+        case SEP_POWER_PH: sep_power_kernel<true><<<b, T, smem, s>>>(tb, items, nitem); break;
+        case SEP_INV_Y: sep_win_y_kernel<true><<<b, T, smem, s>>>(tb, items, nitem); break;
+        case SEP_DESC: sep_desc_kernel<<<b, T, smem, s>>>(tb, items, nitem); break;
+        case SEP_GX: sep_gx_kernel<<<b, T, smem, s>>>(tb, items, nitem); break;
+        case SEP_GY: sep_win_y_kernel<false><<<b, T, smem, s>>>(tb, items, nitem); break;
+        case SEP_MUL: sep_mul_kernel<false><<<b, T, smem, s>>>(tb, items, nitem); break;
+        case SEP_MUL_PH: sep_mul_kernel<true><<<b, T, smem, s>>>(tb, items, nitem); break;
+        case SEP_IFFT_Y: sep_fft_y_kernel<true><<<b, T, smem, s>>>(tb, items, nitem); break;
+        case SEP_GRAD: sep_grad_kernel<<<b, T, smem, s>>>(tb, items, nitem); break;
+        default: break;
+    }
+}
+
+void set_sep_attributes() {
+    const void* ks[] = {(const void*)sep_feat_kernel,         (const void*)sep_fft_y_kernel<false>,
+                        (const void*)sep_fft_y_kernel<true>,  (const void*)sep_power_kernel<false>,
+                        (const void*)sep_power_kernel<true>,  (const void*)sep_win_y_kernel<true>,
+                        (const void*)sep_win_y_kernel<false>, (const void*)sep_desc_kernel,
+                        (const void*)sep_gx_kernel,           (const void*)sep_mul_kernel<false>,
+                        (const void*)sep_mul_kernel<true>,    (const void*)sep_grad_kernel};
+    for (const void* k : ks) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SEP_MAX_SMEM);
+}
+
+}  // namespace dmcr
