@@ -153,8 +153,10 @@ struct Plan {
     // separable path (sep.cu): all levels of the instance or none
     bool sep = false;
     std::shared_ptr<const SepBasis> basis;
+    int sep_tiers = 0, sep_pairs = 0;   // tiers worth running, feature pairs of the widest of them
     size_t o_tier = 0, o_tiers = 0, o_z[MAX_LEVELS] = {}, o_q[MAX_LEVELS] = {}, o_u[MAX_LEVELS] = {},
-           o_v[MAX_LEVELS] = {}, o_sdc[MAX_LEVELS] = {}, o_spart[MAX_LEVELS] = {};
+           o_v[MAX_LEVELS] = {}, o_sdc[MAX_LEVELS] = {}, o_spart[MAX_LEVELS] = {}, o_excess = 0, o_sums = 0;
+    int sum_off[MAX_LEVELS] = {}, nsum = 0;   // residual sums of the sep_desc blocks per level
     size_t bytes = 0;
 };
 
@@ -181,12 +183,12 @@ bool fft_cheaper(const LevelGeom& g) {
 size_t table_bound(const Plan& pl) {
     const int levels = pl.levels, phases = pl.phases;
     const size_t pp = (size_t)phases * phases;
-    const size_t sep = !pl.sep ? 0 : pl.basis->coef.size() * sizeof(float2) +
+    const size_t sep = !pl.sep ? 0 : 16 + pl.basis->coef.size() * sizeof(float2) +
                                          (size_t)levels * (sizeof(SepLevel) + (size_t)SEP_KERNELS * pp * sizeof(SepItem));
     return sep + (size_t)levels *
                (pp * (sizeof(FwdSeg) + sizeof(RedSeg) + sizeof(GSeg) + sizeof(AdjSeg)) +
                 phases * sizeof(RestrictSeg) + 2 * sizeof(TildeSeg)) +
-           sizeof(PenSeg) + sizeof(LossSeg) + phases * sizeof(FinalSeg) + sizeof(InitSeg);
+           sizeof(PrepSeg) + sizeof(PenSeg) + sizeof(LossSeg) + phases * sizeof(FinalSeg) + sizeof(InitSeg);
 }
 size_t table_slack(bool sep) { return (size_t)(16 + MAX_LEVELS + (sep ? 8 + SEP_KERNELS : 0)) * 16 + 256; }
 
@@ -317,8 +319,8 @@ bool sep_shape(const LevelGeom& g, int phases, int max_pairs, SepLevel& lv) {
     lv.Khalf = g.Khalf;
     lv.strideU = sep_u_len(g);
     lv.strideV = sep_v_rows(g) * g.n[2];
-    lv.rowsF = sep_rows(lv.ax[2], SEP_SLOTS);
-    lv.rowsW = sep_rows(lv.ax[2], 1);
+    lv.rowsF = sep_feature_rows(lv.ax[2], (int64_t)lv.n0 * lv.n1);
+    lv.rowsW = sep_window_rows(lv.ax[2]);
     lv.colsY = sep_cols(lv.ax[1], true);
     lv.colsL = lv.n0 > 1 ? sep_cols(lv.ax[0], true) : sep_cols(lv.ax[1], false);
     return std::max(sep_smem_last(lv, true), sep_smem_feat(lv)) <= (size_t)SEP_MAX_SMEM;
@@ -326,26 +328,45 @@ bool sep_shape(const LevelGeom& g, int phases, int max_pairs, SepLevel& lv) {
 
 // The separable path for the soft threshold's two-point descriptor: when a basis of this
 // alpha exists, every axis of every level can be transformed, its buffers stay moderate and
-// the direct kernels' pair evaluations cost more.  All levels of an instance or none.
+// the direct kernels are estimated to be slower in each of the three kinds of call.  All levels
+// of an instance or none.  Seconds, fitted to GB300 measurements of both paths (2-D 64^2 ..
+// 2048^2, 3-D 32^3 .. 160^3, windows 2 .. 64; captured calls, GPU time): e.g. loss and gradient
+// at 256^2, +-32, 3 levels 201 us direct and 82 us separable, 64^2, +-16: 45 and 57 us;
+// 128^3, +-4: 883 and 575 us, 128^3, +-2: 530 and 572 us; 600^2 (8 * 3 * 5^2), +-16: 211 and
+// 321 us.  The separable cost of a tier grows with its feature pairs (7 in the narrowest), so
+// wide ranges are left to the direct kernels where the window is small.
 bool choose_sep(const dmcr_params* p, Plan& pl) {
     if (p->path != DMCR_PATH_AUTO || p->threshold != DMCR_SOFT || pl.desc_kind == DMCR_DESC_S3) return false;
     const double ph = pl.phases;
-    double pairs = 0.0, bytes = 0.0, points = 0.0;
+    double pairs = 0.0, bytes = 0.0, points = 0.0, N = 0.0;
     for (int l = 0; l < pl.levels; ++l) {
         const LevelGeom& g = pl.g[l];
         SepLevel lv;
         if (!sep_shape(g, pl.phases, SEP_MAX_PAIRS, lv)) return false;
         pairs += ph * ph * (double)g.N * (double)g.Khalf;
-        bytes += 8.0 * SEP_MAX_PAIRS * (double)g.N * ph * (pl.phases > 1 ? 2 : 1);
+        bytes += 8.0 * (double)g.N * ph * (pl.phases > 1 ? 2 : 1);
         double per = 0.0;
         for (int a = 0; a < 3; ++a)
             if (g.n[a] > 1) per += sep_axis_cost(lv.ax[a]);
         points += ph * (double)g.N * per;
+        N += ph * ph * (double)g.N;
     }
-    const double t_direct = 4.5e-5 + 5.75e-13 * pairs, t_sep = 1e-4 + points;
-    if (bytes > 8e9 || t_direct < 1.25 * t_sep) return false;
+    const bool d3 = pl.g[0].n[0] > 1;
+    const double direct_lg = 4.0e-5 + 5.7e-13 * pairs + (d3 ? 2.2e-10 : 1.2e-10) * N;
+    const double direct_d = 1.4e-5 + 1.55e-13 * pairs + (d3 ? 1.2e-10 : 0.8e-10) * N;
+    const double direct_v = 2.4e-5 + 4.1e-13 * pairs + 0.6e-10 * N;
+    auto worth = [&](int npair) {
+        const double w = points * npair / 7.0;
+        return bytes * npair <= 16e9 && direct_lg > 1.1 * (5.5e-5 + w) && direct_d > 2.8e-5 + 0.45 * w &&
+               direct_v > 3.7e-5 + 0.8 * w;
+    };
+    if (!worth(1)) return false;
     pl.basis = sep_basis(p->alpha);
-    return pl.basis->ntier > 0;
+    while (pl.sep_tiers < pl.basis->ntier && worth(pl.basis->tier[pl.sep_tiers].npair)) {
+        pl.sep_pairs = std::max(pl.sep_pairs, pl.basis->tier[pl.sep_tiers].npair);
+        ++pl.sep_tiers;
+    }
+    return pl.sep_tiers > 0;
 }
 
 dmcr_status validate_and_plan(const dmcr_params* p, Plan& pl) {
@@ -506,7 +527,15 @@ dmcr_status validate_and_plan(const dmcr_params* p, Plan& pl) {
     pl.o_tsum = o; o = align_up(o + (size_t)MAX_LEVELS * sizeof(float));
     if (pl.sep) {
         pl.o_tier = o; o = align_up(o + sizeof(int));
-        pl.o_tiers = o; o = align_up(o + SEP_RANGE_BLOCKS * sizeof(int));
+        pl.o_tiers = o; o = align_up(o + PREP_BLOCKS * sizeof(int));
+        pl.o_excess = o; o = align_up(o + PREP_BLOCKS * sizeof(float4));
+        for (int l = 0; l < pl.levels; ++l) {
+            SepLevel lv;
+            sep_shape(pl.g[l], pl.phases, pl.sep_pairs, lv);
+            pl.sum_off[l] = pl.nsum;
+            pl.nsum += (int)ceil_div(sep_v_rows(pl.g[l]), lv.rowsW);
+        }
+        pl.o_sums = o; o = align_up(o + (size_t)pl.nsum * sizeof(float4));
     }
     for (int l = 0; l < pl.levels; ++l) {
         const LevelGeom& g = pl.g[l];
@@ -536,9 +565,9 @@ dmcr_status validate_and_plan(const dmcr_params* p, Plan& pl) {
             pl.o_spart[l] = o; o = align_up(o + ph * g.N * sizeof(float));
             pl.o_sdc[l] = o; o = align_up(o + pp * sizeof(double));
             const size_t start = o;
-            pl.o_z[l] = o; o = align_up(o + ph * pl.basis->max_pairs * g.N * sizeof(float2));
+            pl.o_z[l] = o; o = align_up(o + ph * pl.sep_pairs * g.N * sizeof(float2));
             pl.o_q[l] = pl.o_z[l];
-            if (ph > 1) { pl.o_q[l] = o; o = align_up(o + ph * pl.basis->max_pairs * g.N * sizeof(float2)); }
+            if (ph > 1) { pl.o_q[l] = o; o = align_up(o + ph * pl.sep_pairs * g.N * sizeof(float2)); }
             pl.o_u[l] = o; o = align_up(o + pp * sep_u_len(g) * sizeof(float2));
             pl.o_v[l] = o; o = align_up(o + pp * sep_v_rows(g) * g.n[2] * sizeof(float2));
             size_t d = start;
@@ -642,7 +671,7 @@ struct Prepared {
     };
     std::vector<R> restricts;
     R fwd{0, 0, 0}, red{0, 0, 0}, pen{0, 0, 0}, loss{0, 0, 0}, gco{0, 0, 0}, adj{0, 0, 0}, fin{0, 0, 0},
-        fin_small{0, 0, 0}, init{0, 0, 0}, tmap{0, 0, 0}, tsum{0, 0, 0};
+        fin_small{0, 0, 0}, init{0, 0, 0}, tmap{0, 0, 0}, tsum{0, 0, 0}, prep{0, 0, 0};
     size_t smem_fwd = 0, smem_adj = 0;
     // separable path, and the direct launches of its instances (run only where their gate opens)
     R sep[SEP_KERNELS] = {};
@@ -723,6 +752,21 @@ S3Job s3_job(const Inst& x, int l, bool loss) {
     return j;
 }
 
+// blocks of one instance in the pyramid launch
+int prep_blocks(const Plan& pl) {
+    const LevelGeom& g = pl.g[0];
+    const int64_t tiles = (pl.ndim == 2 ? 1 : ceil_div(g.n[0], PREP_TILE3)) *
+                          ceil_div(g.n[1], pl.ndim == 2 ? PREP_TILE2 : PREP_TILE3) *
+                          ceil_div(g.n[2], pl.ndim == 2 ? PREP_TILE2 : PREP_TILE3) * pl.phases;
+    return (int)std::min<int64_t>(PREP_BLOCKS, tiles);
+}
+
+// the separable kernels leave the loss' sums and the rows of G as they compute the descriptor
+bool fused_loss(const Plan& pl, unsigned flags) {
+    return pl.sep && pl.phases == 1 && pl.desc_kind == DMCR_DESC_S2 && (flags & F_FWD) && (flags & F_LOSS) &&
+           (flags & F_BACK);
+}
+
 // Tables of the separable path: one SepLevel per (instance, level), one block range per
 // kernel and phase (pair), the basis' coefficients.
 void prepare_sep(const std::vector<Inst>& in, unsigned flags, Prepared& P) {
@@ -750,7 +794,8 @@ void prepare_sep(const std::vector<Inst>& in, unsigned flags, Prepared& P) {
         for (int l = 0; l < pl.levels; ++l) {
             const LevelGeom& g = pl.g[l];
             SepLevel lv;
-            sep_shape(g, pl.phases, basis->max_pairs, lv);
+            sep_shape(g, pl.phases, pl.sep_pairs, lv);
+            lv.ntier = pl.sep_tiers;
             lv.field = x.lv[l];
             lv.Z = reinterpret_cast<float2*>(x.ws + pl.o_z[l]);
             lv.Q = reinterpret_cast<float2*>(x.ws + pl.o_q[l]);
@@ -759,9 +804,11 @@ void prepare_sep(const std::vector<Inst>& in, unsigned flags, Prepared& P) {
             lv.dc = reinterpret_cast<double*>(x.ws + pl.o_sdc[l]);
             lv.tier = reinterpret_cast<int*>(x.ws + pl.o_tier);
             lv.tiers = reinterpret_cast<int*>(x.ws + pl.o_tiers);
-            const int64_t Nall = pl.N1 * pl.phases;
-            lv.ntiers = (int)std::min<int64_t>(SEP_RANGE_BLOCKS, ceil_div(Nall, 1024));
+            lv.ntiers = prep_blocks(pl);
+            lv.sums = reinterpret_cast<float4*>(x.ws + pl.o_sums) + pl.sum_off[l];
+            lv.fuse = fused_loss(pl, flags);
             lv.first = l == 0;
+            lv.keep = pl.phases == 1 && (flags & F_FWD) && (flags & F_BACK);
             lv.desc = x.desc + pl.off[l];
             lv.scaleD = (double)pl.w[l] / ((double)g.N * (double)g.N);
             if (flags & F_BACK) {
@@ -785,13 +832,12 @@ void prepare_sep(const std::vector<Inst>& in, unsigned flags, Prepared& P) {
             // planes of the middle axis side by side in one block
             const int64_t side = lv.ax[1].fast ? SEP_BLOCK_PTS / (lv.colsY * lv.n1) : 1;
             const size_t sf = sep_smem_feat(lv), sw = sep_smem_window(lv), sy = d3 ? sep_smem_y(lv) : 0;
-            if (lv.first) add(SEP_RANGE, lv.ntiers, 0, lv.ntiers, 0);
             for (int a = 0; a < pl.phases; ++a) {
                 add(SEP_FEAT, a, 0, fgroups, sf);
-                if (d3) add(SEP_FFT_Y, a, 0, ceil_div(xy * lv.n0, side) * basis->max_pairs, sy);
+                if (d3) add(SEP_FFT_Y, a, 0, ceil_div(xy * lv.n0, side), sy);
                 if (flags & F_BACK) {
                     add(pl.phases > 1 ? SEP_MUL_PH : SEP_MUL, a, 0, last, sep_smem_last(lv, true));
-                    if (d3) add(SEP_IFFT_Y, a, 0, ceil_div(xy * lv.n0, side) * basis->max_pairs, sy);
+                    if (d3) add(SEP_IFFT_Y, a, 0, ceil_div(xy * lv.n0, side), sy);
                     add(SEP_GRAD, a, 0, fgroups, sf);
                 }
                 for (int b = 0; b < pl.phases; ++b) {
@@ -801,10 +847,10 @@ void prepare_sep(const std::vector<Inst>& in, unsigned flags, Prepared& P) {
                         if (d3) add(SEP_INV_Y, a, b, ceil_div(xy * kept, side), sy);
                         add(SEP_DESC, a, b, ceil_div(wrows, lv.rowsW), sw);
                     }
-                    if (flags & F_BACK) {
+                    if ((flags & F_BACK) && !lv.fuse) {
                         add(SEP_GX, a, b, ceil_div(wrows, lv.rowsW), sw);
-                        if (d3) add(SEP_GY, a, b, ceil_div(xy * kept, side), sy);
                     }
+                    if ((flags & F_BACK) && d3) add(SEP_GY, a, b, ceil_div(xy * kept, side), sy);
                 }
             }
             levels.push_back(lv);
@@ -812,11 +858,11 @@ void prepare_sep(const std::vector<Inst>& in, unsigned flags, Prepared& P) {
     }
     if (levels.empty()) return;
     P.o_sep_level = push(P.tb, levels);
-    P.o_sep_coef = push(P.tb, basis->coef);
+    const float2* coef = sep_device_coef(*basis);
+    if (coef == nullptr) P.o_sep_coef = push(P.tb, basis->coef);
     for (int t = 0; t < SEP_TIERS; ++t) P.sept.tier[t] = basis->tier[t];
-    P.sept.ntier = basis->ntier;
     P.sept.level = P.at<SepLevel>(P.o_sep_level);
-    P.sept.coef = P.at<float2>(P.o_sep_coef);
+    P.sept.coef = coef != nullptr ? coef : P.at<float2>(P.o_sep_coef);
     for (int k = 0; k < SEP_KERNELS; ++k) {
         P.sep[k].off = push(P.tb, items[k]);
         P.sep[k].nseg = (int)items[k].size();
@@ -851,11 +897,37 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
         P.init = {push(P.tb, v), (int)v.size(), (int64_t)v.size()};
     }
     if (need_pyr) {
+        // levels the tiles of prep_kernel determine, then one restriction per deeper level
+        std::vector<PrepSeg> pv;
+        int64_t pb = 0;
+        for (const Inst& x : in) {
+            const Plan& pl = *x.pl;
+            if (pl.levels == 1 && !pl.sep) continue;
+            PrepSeg p{};
+            p.ndim = pl.ndim;
+            p.coarse = std::min(pl.levels - 1, pl.ndim == 2 ? PREP_LEVELS2 : PREP_LEVELS3);
+            p.phases = pl.phases;
+            p.nblk = prep_blocks(pl);
+            for (int a = 0; a < 3; ++a) p.n[a] = (int)pl.g[0].n[a];
+            p.field = x.lv[0];
+            for (int l = 0; l < p.coarse; ++l) p.lv[l] = const_cast<float*>(x.lv[l + 1]);
+            if (pl.sep) {
+                p.tiers = reinterpret_cast<int*>(x.ws + pl.o_tiers);
+                p.ntier = pl.sep_tiers;
+                for (int t = 0; t < pl.sep_tiers; ++t) p.lo[t] = pl.basis->tier[t].lo, p.hi[t] = pl.basis->tier[t].hi;
+                if (fused_loss(pl, flags) && x.lp.bc_on) p.excess = reinterpret_cast<float4*>(x.ws + pl.o_excess);
+            }
+            p.done = x.use_done ? &x.sc->done : nullptr;
+            p.blockStart = pb;
+            pb += p.nblk;
+            pv.push_back(p);
+        }
+        P.prep = {push(P.tb, pv), (int)pv.size(), pb};
         for (int l = 1; l < maxL; ++l) {
             std::vector<RestrictSeg> v;
             int64_t b = 0;
             for (const Inst& x : in) {
-                if (x.pl->levels <= l) continue;
+                if (x.pl->levels <= l || l <= (x.pl->ndim == 2 ? PREP_LEVELS2 : PREP_LEVELS3)) continue;
                 const LevelGeom& g = x.pl->g[l];
                 for (int ph = 0; ph < x.pl->phases; ++ph) {
                     RestrictSeg r{};
@@ -869,7 +941,7 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
                     v.push_back(r);
                 }
             }
-            P.restricts.push_back({push(P.tb, v), (int)v.size(), b});
+            if (!v.empty()) P.restricts.push_back({push(P.tb, v), (int)v.size(), b});
         }
     }
     if (flags & F_FWD) {
@@ -968,9 +1040,18 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
             const int64_t Nall = x.pl->N1 * x.pl->phases;
             const int nblk = stats_blocks(x.pl->Ktot, x.lp.bc_on ? Nall : 0);
             maxblk = std::max(maxblk, nblk);
-            pv.push_back({x.lp.bc_on ? x.field : nullptr, Nall, x.desc, x.target, x.pl->Ktot, pen,
+            const bool fuse = fused_loss(*x.pl, flags);
+            const int* gate = fuse ? reinterpret_cast<const int*>(x.ws + x.pl->o_tier) : nullptr;
+            pv.push_back({gate, x.lp.bc_on ? x.field : nullptr, Nall, x.desc, x.target, x.pl->Ktot, pen,
                           x.use_done ? &x.sc->done : nullptr, nblk});
             LossSeg ls{};
+            if (fuse) {
+                ls.tier = gate;
+                ls.sums = reinterpret_cast<const float4*>(x.ws + x.pl->o_sums);
+                ls.nsum = x.pl->nsum;
+                ls.excess = reinterpret_cast<const float4*>(x.ws + x.pl->o_excess);
+                ls.nexc = x.lp.bc_on ? prep_blocks(*x.pl) : 0;
+            }
             ls.lp = x.lp;
             ls.desc = x.desc;
             ls.target = x.target;
@@ -1244,12 +1325,15 @@ void run(const Prepared& P, cudaStream_t s) {
         ProfScope ps("scalars_init", -1, s);
         launch_scalars_init(P.at<InitSeg>(P.init.off), P.init.nseg, s);
     }
+    if (P.prep.blocks > 0) {
+        ProfScope ps("pyramid", -1, s);
+        launch_prep(P.at<PrepSeg>(P.prep.off), P.prep.nseg, P.prep.blocks, s);
+    }
     for (const Prepared::R& r : P.restricts) {
         ProfScope ps("restrict", -1, s);
         launch_restrict(P.at<RestrictSeg>(r.off), r.nseg, r.blocks, s);
     }
     if (P.flags & (F_FWD | F_BACK)) {
-        run_sep(P, SEP_RANGE, "sep_range", s);
         run_sep(P, SEP_FEAT, "sep_feat", s);
         run_sep(P, SEP_FFT_Y, "sep_fft_y", s);
     }
@@ -1460,7 +1544,7 @@ std::string prepared_key(const Prepared& P) {
     add(&P.tc, sizeof P.tc);
     for (const Prepared::R& r : P.restricts) add(&r, sizeof r);
     for (const Prepared::R* r : {&P.fwd, &P.red, &P.pen, &P.loss, &P.gco, &P.adj, &P.fin, &P.fin_small, &P.init,
-                                   &P.tmap, &P.tsum, &P.gfwd, &P.gred, &P.ggco, &P.gadj})
+                                   &P.tmap, &P.tsum, &P.prep, &P.gfwd, &P.gred, &P.ggco, &P.gadj})
         add(r, sizeof *r);
     add(P.sep, sizeof P.sep);
     add(P.sep_smem, sizeof P.sep_smem);

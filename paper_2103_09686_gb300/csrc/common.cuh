@@ -60,6 +60,29 @@ __device__ __forceinline__ DF block_sum_df(DF v, DF* sh) {
     }
     return v;
 }
+// Programmatic dependent launch.  A kernel launched with launch_dep may start while its
+// predecessor in the stream still runs; dep_wait() returns once every earlier kernel has
+// completed and its writes are visible, and dep_trigger() lets the successor start.  Every
+// kernel triggers only after its own wait, so what a kernel reads before dep_wait() may be
+// anything written at least two launches earlier (the segment tables), and nothing else.
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline void launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 constexpr int MAX_DYN_SMEM = 200 * 1024;   // dynamic shared memory limit of the correlation kernels
 constexpr int MAX_PHASES = 8;      // phase fields of one problem (their ordered pairs each get a block)
 
@@ -201,7 +224,26 @@ struct RestrictSeg {
     const int* done;
     int64_t blockStart;
 };
+// Pyramid of one instance (one block range over all its phases): every coarser level that a
+// tile of the finest grid determines, and with `tiers` the range tier of each block's values.
+constexpr int PREP_TILE2 = 32, PREP_TILE3 = 16;      // tile edge: 2-D 32 x 32, 3-D 16 x 16 x 16
+constexpr int PREP_LEVELS2 = 5, PREP_LEVELS3 = 4;    // coarser levels of one tile
+constexpr int PREP_BLOCKS = 256;                     // blocks per instance at most
+struct PrepSeg {
+    int ndim, coarse;            // coarser levels to build here
+    int phases, nblk;
+    int n[3];                    // finest sizes (3-D embedded)
+    const float* field;
+    float* lv[PREP_LEVELS2];     // level 2, 3, ... (phases stacked)
+    int* tiers;                  // separable path: one tier per block, null otherwise
+    int ntier;
+    float lo[8], hi[8];          // its ranges
+    float4* excess;              // box excess: sum of squares per block (hi, lo), null: not wanted
+    const int* done;
+    int64_t blockStart;
+};
 struct PenSeg {
+    const int* gate;         // separable path with fused sums: run only when *gate >= SEP_TIERS
     const float* field;      // null: no box penalty
     int64_t N;
     const float* desc;
@@ -212,6 +254,11 @@ struct PenSeg {
     int nblk;                // blocks of this instance: a function of its own sizes only
 };
 struct LossSeg {
+    // separable path with fused residual sums: used while *tier < SEP_TIERS (else `pen`)
+    const int* tier;
+    const float4* sums;         // nsum entries: sum (D - D_des)^2, sum D_des^2 (hi, lo each)
+    const float4* excess;       // nexc entries: sum of squared box excess (hi, lo)
+    int nsum, nexc;
     LossParams lp;
     const float* desc;
     const float* target;
@@ -272,26 +319,25 @@ struct FftPass {
 };
 
 // ---------------------------------------------------------------- separable path (sep.cu)
-constexpr int SEP_TIERS = 3;        // value ranges with a basis of their own; tier SEP_TIERS: direct kernels
-constexpr int SEP_MAX_PAIRS = 13;   // packed pairs of features of one basis at most
+constexpr int SEP_TIERS = 6;        // value ranges with a basis of their own; tier SEP_TIERS: direct kernels
+constexpr int SEP_MAX_PAIRS = 28;   // packed pairs of features of one basis at most
 constexpr int SEP_THREADS = 512;    // threads of the transform kernels
 constexpr int SEP_BLOCK_PTS = 8 * SEP_THREADS;   // points a block holds in registers (power-of-two axes)
+constexpr int SEP_ROW_THREADS = 256;   // threads of the feature and gradient kernels
 constexpr int SEP_SLOTS = 8;        // feature pairs a row block holds side by side at most
 constexpr int SEP_FAST_PHASES = 3;  // phases whose spectra fit behind the line buffers of sep_mul
-constexpr int SEP_MAX_DEG = 64;     // Chebyshev coefficients per feature at most
+constexpr int SEP_MAX_DEG = 128;    // Chebyshev coefficients per feature at most
 constexpr int SEP_MAX_N = 2048;     // longest axis
 constexpr int SEP_MAX_RAD = 12;
+constexpr int COLOCC = 2;
 constexpr int SEP_OWN = 8;          // points of a column group one thread owns (at most 4096 per block)
-constexpr int SEP_MAX_SMEM = 208 * 1024;
-constexpr int SEP_RANGE_BLOCKS = 256;
+constexpr int SEP_MAX_SMEM = 222 * 1024;
 
 struct SepAxis {
     int n, nrad;
     int fast;                 // log2 n for powers of two 16 .. SEP_MAX_N, else 0
     unsigned short rad[SEP_MAX_RAD];
 };
-
-__host__ __device__ inline int sep_coef_stride(int npair) { return (npair + 1) / 2 * 2; }
 
 // line pitch (float2 elements) of a column group of L adjacent columns: padded length, and
 // pitch = 16 / L (mod 16), so that the L columns of one position lie in different banks
@@ -309,7 +355,7 @@ struct SepTier {
 
 struct SepBasis {
     float alpha = 0.f;
-    int ntier = 0, max_pairs = 0;
+    int ntier = 0;
     SepTier tier[SEP_TIERS] = {};
     std::vector<float2> coef;
 };
@@ -319,6 +365,7 @@ struct SepLevel {
     int n0, n1, n2;
     int P0, P1, P2;
     int phases, maxPairs;
+    int ntier;                // tiers this problem uses (wider fields: the direct kernels)
     int64_t N, Khalf;
     SepAxis ax[3];
     const float* field;       // this level's field(s)
@@ -330,6 +377,7 @@ struct SepLevel {
     int ntiers;
     int* tier;                // the instance's tier
     int first;                // finest level: writes *tier
+    int keep;                 // one phase, forward and backward in one call: sep_power leaves its spectra in Z
     int rowsF, rowsW, colsY, colsL;
     float* desc;
     double scaleD;            // w / N^2
@@ -338,6 +386,8 @@ struct SepLevel {
     const Scalars* sc;
     const float* tsum;        // corrected descriptor
     float q, scaleG;
+    int fuse;                 // one phase, loss and gradient in one call: sep_desc goes on to the rows of G
+    float4* sums;             // fuse: per sep_desc block sum (D - D_des)^2 and sum D_des^2 (hi, lo each)
     float* part;              // this level's gradient, one field per phase
     const int* done;
 };
@@ -353,19 +403,20 @@ struct SepTables {
     const SepLevel* level;
     const float2* coef;
     SepTier tier[SEP_TIERS];
-    int ntier;
 };
 
 enum SepKernel {
-    SEP_RANGE, SEP_FEAT, SEP_FFT_Y, SEP_POWER, SEP_POWER_PH, SEP_INV_Y, SEP_DESC, SEP_GX, SEP_GY, SEP_MUL, SEP_MUL_PH, SEP_IFFT_Y,
+    SEP_FEAT, SEP_FFT_Y, SEP_POWER, SEP_POWER_PH, SEP_INV_Y, SEP_DESC, SEP_GX, SEP_GY, SEP_MUL, SEP_MUL_PH, SEP_IFFT_Y,
     SEP_GRAD, SEP_KERNELS
 };
 
 std::shared_ptr<const SepBasis> sep_basis(float alpha);
+const float2* sep_device_coef(const SepBasis& b);
 bool sep_axis(int64_t n, SepAxis& ax);
 double sep_axis_cost(const SepAxis& ax);
 int sep_cols(const SepAxis& ax, bool wide);
-int sep_rows(const SepAxis& ax, int per);
+int sep_window_rows(const SepAxis& ax);
+int sep_feature_rows(const SepAxis& ax, int64_t rows);
 size_t sep_smem_feat(const SepLevel& lv);
 size_t sep_smem_window(const SepLevel& lv);
 size_t sep_smem_y(const SepLevel& lv);
@@ -376,6 +427,7 @@ void set_sep_attributes();
 
 // ---------------------------------------------------------------- launchers
 void launch_blob(const void* host, size_t bytes, void* dst, cudaStream_t s);
+void launch_prep(const PrepSeg* segs, int nseg, int64_t blocks, cudaStream_t s);
 void launch_restrict(const RestrictSeg* segs, int nseg, int64_t blocks, cudaStream_t s);
 void launch_restrict_one(int ndim, const int64_t nf[3], const float* fine, float* coarse, cudaStream_t s);
 void launch_prolongate(int ndim, const int64_t nc[3], const float* coarse, float* fine, int mode,

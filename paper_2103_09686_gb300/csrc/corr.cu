@@ -520,6 +520,8 @@ __device__ __forceinline__ void corr_fwd_block(const FwdSeg& sg, const int64_t l
 template <bool IDENT>
 __global__ void __launch_bounds__(FWD_THREADS, 4)
 corr_fwd_kernel(const FwdSeg* __restrict__ segs, int nseg, ThreshConst tc) {
+    dep_wait();
+    dep_trigger();
     const FwdSeg& sg = segs[find_segment(segs, nseg, (int64_t)blockIdx.x)];
     if (sg.done != nullptr && *sg.done) return;
     corr_fwd_block<IDENT>(sg, (int64_t)blockIdx.x - sg.blockStart, tc);
@@ -551,6 +553,8 @@ __device__ __forceinline__ void run_gated(const S* __restrict__ segs, int nseg, 
 
 __global__ void __launch_bounds__(FWD_THREADS, 4)
 corr_fwd_gated_kernel(const FwdSeg* __restrict__ segs, int nseg, int64_t total, ThreshConst tc) {
+    dep_wait();
+    dep_trigger();
     run_gated(segs, nseg, total, [&](const FwdSeg& sg, int64_t local) { corr_fwd_block<false>(sg, local, tc); });
 }
 
@@ -593,12 +597,16 @@ __device__ __forceinline__ void fwd_reduce_block(const RedSeg& sg, int64_t local
 }
 
 __global__ void __launch_bounds__(256) fwd_reduce_kernel(const RedSeg* __restrict__ segs, int nseg) {
+    dep_wait();
+    dep_trigger();
     const RedSeg& sg = segs[find_segment(segs, nseg, (int64_t)blockIdx.x)];
     if (sg.done != nullptr && *sg.done) return;
     fwd_reduce_block(sg, (int64_t)blockIdx.x - sg.blockStart);
 }
 
 __global__ void __launch_bounds__(256) fwd_reduce_gated_kernel(const RedSeg* __restrict__ segs, int nseg, int64_t total) {
+    dep_wait();
+    dep_trigger();
     run_gated(segs, nseg, total, [](const RedSeg& sg, int64_t local) { fwd_reduce_block(sg, local); });
 }
 
@@ -772,6 +780,8 @@ __device__ __forceinline__ void corr_adj_block(const AdjSeg& sg, const int64_t l
 template <bool IDENT>
 __global__ void __launch_bounds__(ADJ_THREADS, 4)
 corr_adj_kernel(const AdjSeg* __restrict__ segs, int nseg, ThreshConst tc) {
+    dep_wait();
+    dep_trigger();
     const AdjSeg& sg = segs[find_segment(segs, nseg, (int64_t)blockIdx.x)];
     if (sg.done != nullptr && *sg.done) return;
     corr_adj_block<IDENT>(sg, (int64_t)blockIdx.x - sg.blockStart, tc);
@@ -779,6 +789,8 @@ corr_adj_kernel(const AdjSeg* __restrict__ segs, int nseg, ThreshConst tc) {
 
 __global__ void __launch_bounds__(ADJ_THREADS, 4)
 corr_adj_gated_kernel(const AdjSeg* __restrict__ segs, int nseg, int64_t total, ThreshConst tc) {
+    dep_wait();
+    dep_trigger();
     run_gated(segs, nseg, total, [&](const AdjSeg& sg, int64_t local) { corr_adj_block<false>(sg, local, tc); });
 }
 
@@ -830,12 +842,16 @@ __device__ __forceinline__ void gcoef_block(const GSeg& sg, int64_t local, const
 }
 
 __global__ void gcoef_kernel(const GSeg* __restrict__ segs, int nseg, ThreshConst tc) {
+    dep_wait();
+    dep_trigger();
     const GSeg& sg = segs[find_segment(segs, nseg, (int64_t)blockIdx.x)];
     if (sg.done != nullptr && *sg.done) return;
     gcoef_block(sg, (int64_t)blockIdx.x - sg.blockStart, tc);
 }
 
 __global__ void gcoef_gated_kernel(const GSeg* __restrict__ segs, int nseg, int64_t total, ThreshConst tc) {
+    dep_wait();
+    dep_trigger();
     run_gated(segs, nseg, total, [&](const GSeg& sg, int64_t local) { gcoef_block(sg, local, tc); });
 }
 
@@ -857,13 +873,13 @@ size_t fwd_smem_bytes(const LevelGeom& g) {
 void launch_corr_fwd(const FwdSeg* segs, int nseg, int64_t blocks, size_t smem, const ThreshConst& tc,
                      cudaStream_t s) {
     if (blocks <= 0) return;
-    if (tc.identity) corr_fwd_kernel<true><<<(unsigned)blocks, FWD_THREADS, smem, s>>>(segs, nseg, tc);
-    else corr_fwd_kernel<false><<<(unsigned)blocks, FWD_THREADS, smem, s>>>(segs, nseg, tc);
+    if (tc.identity) launch_dep(corr_fwd_kernel<true>, (unsigned)blocks, FWD_THREADS, smem, s, segs, nseg, tc);
+    else launch_dep(corr_fwd_kernel<false>, (unsigned)blocks, FWD_THREADS, smem, s, segs, nseg, tc);
 }
 
 void launch_fwd_reduce(const RedSeg* segs, int nseg, int64_t blocks, cudaStream_t s) {
     if (blocks <= 0) return;
-    fwd_reduce_kernel<<<(unsigned)blocks, 256, 0, s>>>(segs, nseg);
+    launch_dep(fwd_reduce_kernel, (unsigned)blocks, 256, 0, s, segs, nseg);
 }
 
 size_t adj_smem_bytes(const LevelGeom& g) {
@@ -875,33 +891,33 @@ size_t adj_smem_bytes(const LevelGeom& g) {
 void launch_corr_adj(const AdjSeg* segs, int nseg, int64_t blocks, size_t smem, const ThreshConst& tc,
                      cudaStream_t s) {
     if (blocks <= 0) return;
-    if (tc.identity) corr_adj_kernel<true><<<(unsigned)blocks, ADJ_THREADS, smem, s>>>(segs, nseg, tc);
-    else corr_adj_kernel<false><<<(unsigned)blocks, ADJ_THREADS, smem, s>>>(segs, nseg, tc);
+    if (tc.identity) launch_dep(corr_adj_kernel<true>, (unsigned)blocks, ADJ_THREADS, smem, s, segs, nseg, tc);
+    else launch_dep(corr_adj_kernel<false>, (unsigned)blocks, ADJ_THREADS, smem, s, segs, nseg, tc);
 }
 
 // resident blocks of a gated launch: as many as run at once (4 per SM; the small kernels 2)
-constexpr int64_t GATED_BLOCKS = 4 * 152, GATED_SMALL = 2 * 152;
+constexpr int64_t GATED_BLOCKS = 8192, GATED_SMALL = 8192;
 
 void launch_corr_fwd_gated(const FwdSeg* segs, int nseg, int64_t blocks, size_t smem, const ThreshConst& tc,
                            cudaStream_t s) {
     if (blocks <= 0) return;
-    corr_fwd_gated_kernel<<<(unsigned)std::min(blocks, GATED_BLOCKS), FWD_THREADS, smem, s>>>(segs, nseg, blocks, tc);
+    launch_dep(corr_fwd_gated_kernel, (unsigned)std::min(blocks, GATED_BLOCKS), FWD_THREADS, smem, s, segs, nseg, blocks, tc);
 }
 
 void launch_fwd_reduce_gated(const RedSeg* segs, int nseg, int64_t blocks, cudaStream_t s) {
     if (blocks <= 0) return;
-    fwd_reduce_gated_kernel<<<(unsigned)std::min(blocks, GATED_SMALL), 256, 0, s>>>(segs, nseg, blocks);
+    launch_dep(fwd_reduce_gated_kernel, (unsigned)std::min(blocks, GATED_SMALL), 256, 0, s, segs, nseg, blocks);
 }
 
 void launch_gcoef_gated(const GSeg* segs, int nseg, int64_t blocks, const ThreshConst& tc, cudaStream_t s) {
     if (blocks <= 0) return;
-    gcoef_gated_kernel<<<(unsigned)std::min(blocks, GATED_SMALL), GCOEF_TH, 0, s>>>(segs, nseg, blocks, tc);
+    launch_dep(gcoef_gated_kernel, (unsigned)std::min(blocks, GATED_SMALL), GCOEF_TH, 0, s, segs, nseg, blocks, tc);
 }
 
 void launch_corr_adj_gated(const AdjSeg* segs, int nseg, int64_t blocks, size_t smem, const ThreshConst& tc,
                            cudaStream_t s) {
     if (blocks <= 0) return;
-    corr_adj_gated_kernel<<<(unsigned)std::min(blocks, GATED_BLOCKS), ADJ_THREADS, smem, s>>>(segs, nseg, blocks, tc);
+    launch_dep(corr_adj_gated_kernel, (unsigned)std::min(blocks, GATED_BLOCKS), ADJ_THREADS, smem, s, segs, nseg, blocks, tc);
 }
 
 void set_kernel_attributes() {
@@ -922,7 +938,7 @@ float gcoef_scale(const LevelGeom& g, const ThreshConst& tc, float weight) {
 
 void launch_gcoef(const GSeg* segs, int nseg, int64_t blocks, const ThreshConst& tc, cudaStream_t s) {
     if (blocks <= 0) return;
-    gcoef_kernel<<<(unsigned)blocks, GCOEF_TH, 0, s>>>(segs, nseg, tc);
+    launch_dep(gcoef_kernel, (unsigned)blocks, GCOEF_TH, 0, s, segs, nseg, tc);
 }
 
 }  // namespace dmcr

@@ -4,7 +4,7 @@
 // The pair function F(u, v) = f((u + v) / 2)^2 is smooth on the bounded range of a relaxed
 // field, so its integral operator has rapidly decaying eigenvalues:
 //     F(u, v) = sum_k s_k p_k(u) p_k(v),  s_k = +-1,  p_k polynomials,
-// with 14 terms to 4e-11 on [-1/16, 17/16] at alpha = 10 (SepBasis, built on the host in
+// with 16 terms to 1e-10 on [-1/16, 17/16] at alpha = 10 (SepBasis, built on the host in
 // FP64).  The descriptor is then a sum of autocorrelations of R feature fields p_k(M), and the
 // gradient a sum of convolutions of the same features with the window coefficients G:
 //     S(r) = (1/N) sum_k s_k sum_x p_k(M_x) p_k(M_{x+r}),
@@ -94,36 +94,90 @@ void jacobi_eigen(std::vector<double>& A, std::vector<double>& V, int n) {
     }
 }
 
-constexpr int SEP_NODES = 64;
-// accepted error of F and of dF/du over the whole range: below the FP32 rounding of a pair
-constexpr double SEP_TOL_F = 1.5e-9, SEP_TOL_FU = 1e-7;
-
-// One tier: eigenfunctions of F on [lo, hi] at SEP_NODES Chebyshev nodes, as Chebyshev series;
-// false when SEP_MAX_PAIRS pairs of features do not reach the tolerances.
-bool build_tier(const PairFn& fn, double lo, double hi, SepTier& t, std::vector<float2>& coef) {
-    constexpr int n = SEP_NODES;
+// One tier: eigenfunctions of F on [lo, hi], discretised at Chebyshev nodes, as Chebyshev
+// series.  False when SEP_MAX_PAIRS packed pairs of at most SEP_MAX_DEG coefficients do not
+// reach the tolerances (largest error of F and of dF/du over the range).
+bool build_tier(const PairFn& fn, double lo, double hi, double tolF, double tolFu, SepTier& t,
+                std::vector<float2>& coef) {
     const double mid = 0.5 * (lo + hi), half = 0.5 * (hi - lo);
-    std::vector<double> x(n), A((size_t)n * n), V;
-    for (int i = 0; i < n; ++i) x[i] = cos((i + 0.5) * M_PI / n);
+    // nodes: the degree grows with the range measured in widths of the sigmoid
+    const int n = (int)std::min(160.0, std::max(48.0, 24.0 + 2.6 * (hi - lo) * fn.a));
+    std::vector<double> ct(4 * n);                       // cos(pi m / (2 n))
+    for (int m = 0; m < 4 * n; ++m) ct[m] = cos(M_PI * m / (2 * n));
+    auto node = [&](int i) { return ct[2 * i + 1]; };
+    std::vector<double> A((size_t)n * n);
     for (int i = 0; i < n; ++i)
-        for (int j = 0; j < n; ++j) A[(size_t)i * n + j] = fn.F(2.0 * mid + half * (x[i] + x[j])) / n;
-    jacobi_eigen(A, V, n);
-    std::vector<int> ord(n);
-    for (int i = 0; i < n; ++i) ord[i] = i;
-    std::stable_sort(ord.begin(), ord.end(),
-                     [&](int a, int b) { return fabs(A[(size_t)a * n + a]) > fabs(A[(size_t)b * n + b]); });
-    // Chebyshev coefficients of sqrt(|lambda_k| n) v_k
-    auto series = [&](int k) {
-        std::vector<double> c(n);
-        const double sc = sqrt(fabs(A[(size_t)ord[k] * n + ord[k]]) * n);
+        for (int j = 0; j < n; ++j) A[(size_t)i * n + j] = fn.F(2.0 * mid + half * (node(i) + node(j))) / n;
+    // numerical range of A: Gram-Schmidt on its columns, largest residual first, each
+    // direction orthogonalised twice
+    const int rmax = std::min(n, 2 * SEP_MAX_PAIRS + 8);
+    std::vector<double> W(A), Q;                          // W: residual columns; Q: r rows of length n
+    int r = 0;
+    double first = 0.0;
+    for (; r < rmax; ++r) {
+        int best = 0;
+        double bestn = -1.0;
         for (int j = 0; j < n; ++j) {
             double s = 0.0;
-            for (int i = 0; i < n; ++i) s += V[(size_t)i * n + ord[k]] * cos(j * (i + 0.5) * M_PI / n);
+            for (int i = 0; i < n; ++i) s += W[(size_t)i * n + j] * W[(size_t)i * n + j];
+            if (s > bestn) bestn = s, best = j;
+        }
+        if (r == 0) first = bestn;
+        if (!(bestn > 1e-28 * first)) break;
+        std::vector<double> q(n);
+        for (int i = 0; i < n; ++i) q[i] = W[(size_t)i * n + best];
+        for (int k = 0; k < r; ++k) {
+            double d = 0.0;
+            for (int i = 0; i < n; ++i) d += q[i] * Q[(size_t)k * n + i];
+            for (int i = 0; i < n; ++i) q[i] -= d * Q[(size_t)k * n + i];
+        }
+        double nn = 0.0;
+        for (double v : q) nn += v * v;
+        nn = 1.0 / sqrt(nn);
+        for (double& v : q) v *= nn;
+        for (int j = 0; j < n; ++j) {
+            double d = 0.0;
+            for (int i = 0; i < n; ++i) d += q[i] * W[(size_t)i * n + j];
+            for (int i = 0; i < n; ++i) W[(size_t)i * n + j] -= d * q[i];
+        }
+        Q.insert(Q.end(), q.begin(), q.end());
+    }
+    // A restricted to it, and its eigenvectors
+    std::vector<double> AQ((size_t)r * n), B((size_t)r * r), V;
+    for (int k = 0; k < r; ++k)
+        for (int i = 0; i < n; ++i) {
+            double s = 0.0;
+            for (int j = 0; j < n; ++j) s += A[(size_t)i * n + j] * Q[(size_t)k * n + j];
+            AQ[(size_t)k * n + i] = s;
+        }
+    for (int k = 0; k < r; ++k)
+        for (int m = 0; m < r; ++m) {
+            double s = 0.0;
+            for (int i = 0; i < n; ++i) s += Q[(size_t)m * n + i] * AQ[(size_t)k * n + i];
+            B[(size_t)k * r + m] = s;
+        }
+    for (int k = 0; k < r; ++k)
+        for (int m = 0; m < k; ++m)
+            B[(size_t)k * r + m] = B[(size_t)m * r + k] = 0.5 * (B[(size_t)k * r + m] + B[(size_t)m * r + k]);
+    jacobi_eigen(B, V, r);
+    std::vector<int> ord(r);
+    for (int i = 0; i < r; ++i) ord[i] = i;
+    std::stable_sort(ord.begin(), ord.end(),
+                     [&](int a, int b) { return fabs(B[(size_t)a * r + a]) > fabs(B[(size_t)b * r + b]); });
+    // Chebyshev coefficients of sqrt(|lambda_k| n) v_k
+    auto series = [&](int k) {
+        std::vector<double> v(n, 0.0), c(n);
+        for (int m = 0; m < r; ++m)
+            for (int i = 0; i < n; ++i) v[i] += V[(size_t)m * r + ord[k]] * Q[(size_t)m * n + i];
+        const double sc = sqrt(fabs(B[(size_t)ord[k] * r + ord[k]]) * n);
+        for (int j = 0; j < n; ++j) {
+            double s = 0.0;
+            for (int i = 0; i < n; ++i) s += v[i] * ct[(int)((int64_t)j * (2 * i + 1) % (4 * n))];
             c[j] = s * sc * (j == 0 ? 1.0 : 2.0) / n;
         }
         return c;
     };
-    constexpr int GRID = 49;
+    constexpr int GRID = 97;
     std::vector<double> E((size_t)GRID * GRID), D((size_t)GRID * GRID);
     auto gx = [&](int i) { return -1.0 + 2.0 * i / (GRID - 1); };
     for (int i = 0; i < GRID; ++i)
@@ -134,12 +188,12 @@ bool build_tier(const PairFn& fn, double lo, double hi, SepTier& t, std::vector<
         }
     std::vector<std::vector<double>> pos, neg;
     bool ok = false;
-    for (int k = 0; k < 2 * SEP_MAX_PAIRS; ++k) {
-        const bool plus = A[(size_t)ord[k] * n + ord[k]] > 0.0;
+    for (int k = 0; k < r; ++k) {
+        const bool plus = B[(size_t)ord[k] * r + ord[k]] > 0.0;
         std::vector<std::vector<double>>& side = plus ? pos : neg;
         // once accurate, further terms are taken only while they fill a half-empty pair
         if (ok && side.size() % 2 == 0) break;
-        if (!ok && (int)((pos.size() + 1) / 2 + (neg.size() + 1) / 2) + (side.size() % 2 == 0) > SEP_MAX_PAIRS) break;
+        if ((int)((pos.size() + 1) / 2 + (neg.size() + 1) / 2) + (side.size() % 2 == 0) > SEP_MAX_PAIRS) break;
         const std::vector<double> c = series(k);
         side.push_back(c);
         std::vector<double> p(GRID), dp(GRID);
@@ -165,7 +219,7 @@ bool build_tier(const PairFn& fn, double lo, double hi, SepTier& t, std::vector<
                 eF = std::max(eF, fabs(E[(size_t)i * GRID + j]));
                 eD = std::max(eD, fabs(D[(size_t)i * GRID + j]));
             }
-        if (eF < SEP_TOL_F && eD < SEP_TOL_FU) ok = true;
+        if (eF < tolF && eD < tolFu) ok = true;
     }
     if (!ok) return false;
     int deg = 4;
@@ -173,6 +227,7 @@ bool build_tier(const PairFn& fn, double lo, double hi, SepTier& t, std::vector<
         for (const auto& c : *side)
             for (int j = 0; j < n; ++j)
                 if (fabs(c[j]) > 3e-10) deg = std::max(deg, j + 1);
+    if (deg > SEP_MAX_DEG) return false;
     t.lo = (float)lo;
     t.hi = (float)hi;
     t.mid = (float)mid;
@@ -181,28 +236,29 @@ bool build_tier(const PairFn& fn, double lo, double hi, SepTier& t, std::vector<
     t.npos = (int)(pos.size() + 1) / 2;
     t.npair = t.npos + (int)(neg.size() + 1) / 2;
     t.coef = (int)coef.size();
-    // coefficients [deg][npair rounded up to even], zero padded: (feature 2p, feature 2p + 1)
-    const int stride = sep_coef_stride(t.npair);
-    coef.resize(coef.size() + (size_t)deg * stride, make_float2(0.f, 0.f));
-    for (int j = 0; j < deg; ++j)
-        for (int p = 0; p < t.npair; ++p) {
-            const auto& side = p < t.npos ? pos : neg;
-            const size_t k = 2 * (size_t)(p < t.npos ? p : p - t.npos);
-            float2& c = coef[t.coef + (size_t)j * stride + p];
-            c.x = (float)side[k][j];
-            c.y = k + 1 < side.size() ? (float)side[k + 1][j] : 0.f;
-        }
+    // coefficients [deg][npair]: (feature 2p, feature 2p + 1); then j times them, the series of
+    // the derivatives in U_{j-1}
+    for (int der = 0; der < 2; ++der)
+        for (int j = 0; j < deg; ++j)
+            for (int p = 0; p < t.npair; ++p) {
+                const auto& side = p < t.npos ? pos : neg;
+                const size_t k = 2 * (size_t)(p < t.npos ? p : p - t.npos);
+                const double f = der ? (double)j : 1.0;
+                coef.push_back(make_float2((float)(f * side[k][j]), k + 1 < side.size() ? (float)(f * side[k + 1][j]) : 0.f));
+            }
     return true;
 }
 
 }  // namespace
 
-// The basis of one alpha.  Three ranges: a field between the phases with the overshoot of an
-// optimiser step, and two with wider excursions (a wider range needs more features).
+// The basis of one alpha.  The first range is a field between the phases with the overshoot of
+// a few optimiser steps; the penalty weakens as the loss falls, so fields of long runs spread
+// over the wider ones (measured over 3000 Adam steps: [-1.7, 1.9]).  A wider range needs more
+// features: 8, 10, 13, 15, 19, 25 packed pairs at alpha = 10.
 std::shared_ptr<const SepBasis> sep_basis(float alpha) {
     static std::mutex mu;
     static std::vector<std::shared_ptr<const SepBasis>>* cache = new std::vector<std::shared_ptr<const SepBasis>>();
-    constexpr size_t KEEP = 8;
+    constexpr size_t KEEP = 16;
     std::lock_guard<std::mutex> lk(mu);
     for (size_t i = 0; i < cache->size(); ++i)
         if ((*cache)[i]->alpha == alpha) {
@@ -212,15 +268,68 @@ std::shared_ptr<const SepBasis> sep_basis(float alpha) {
     auto b = std::make_shared<SepBasis>();
     b->alpha = alpha;
     const PairFn fn((double)alpha);
-    const double ranges[SEP_TIERS][2] = {{-0.0625, 1.0625}, {-0.25, 1.25}, {-0.5, 1.5}};
+    const double ranges[SEP_TIERS][2] = {{-0.0625, 1.0625}, {-0.25, 1.25}, {-0.5, 1.5},
+                                         {-1.0, 1.625},     {-1.5, 2.0},   {-2.25, 2.5}};
     for (int t = 0; t < SEP_TIERS; ++t) {
-        if (!build_tier(fn, ranges[t][0], ranges[t][1], b->tier[t], b->coef)) break;
+        // below the FP32 rounding of a pair's value and derivative
+        if (!build_tier(fn, ranges[t][0], ranges[t][1], t == 0 ? 1.5e-9 : 1e-8, 3e-7, b->tier[t],
+                        b->coef))
+            break;
         b->ntier = t + 1;
-        b->max_pairs = std::max(b->max_pairs, b->tier[t].npair);
     }
     cache->insert(cache->begin(), b);
     if (cache->size() > KEEP) cache->pop_back();
     return b;
+}
+
+// Coefficients in device memory: the first SEP_SLOTS_DEV alphas a process uses get a slot of a
+// static array, filled once per device by a synchronous copy on a stream of its own (also while
+// another stream is being captured); slots are never rewritten, so kernels and graphs may keep
+// reading them.  Null when there is no slot: the call uploads the coefficients with its tables.
+namespace {
+constexpr int SEP_SLOTS_DEV = 16, SEP_SLOT_LEN = 16384;
+__device__ float2 g_sep_coef[SEP_SLOTS_DEV][SEP_SLOT_LEN];
+}  // namespace
+
+const float2* sep_device_coef(const SepBasis& b) {
+    struct Slot {
+        int dev;
+        float alpha;
+        const float2* ptr;
+    };
+    static std::mutex mu;
+    static std::vector<Slot>* slots = new std::vector<Slot>();
+    if (b.coef.size() > (size_t)SEP_SLOT_LEN) return nullptr;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    std::lock_guard<std::mutex> lk(mu);
+    int used = 0;
+    for (const Slot& s : *slots)
+        if (s.dev == dev) {
+            if (s.alpha == b.alpha) return s.ptr;
+            ++used;
+        }
+    if (used >= SEP_SLOTS_DEV) return nullptr;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    void* base = nullptr;
+    cudaStream_t s = nullptr;
+    bool ok = cudaGetSymbolAddress(&base, g_sep_coef) == cudaSuccess &&
+              cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess;
+    float2* dst = static_cast<float2*>(base) + (size_t)used * SEP_SLOT_LEN;
+    ok = ok && cudaMemcpyAsync(dst, b.coef.data(), b.coef.size() * sizeof(float2), cudaMemcpyHostToDevice, s) == cudaSuccess;
+    if (s) ok = cudaStreamSynchronize(s) == cudaSuccess && ok;
+    if (s) cudaStreamDestroy(s);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (!ok) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    slots->push_back({dev, b.alpha, dst});
+    return dst;
 }
 
 // ------------------------------------------------------------------------- plan (host)
@@ -252,12 +361,12 @@ bool sep_axis(int64_t n, SepAxis& ax) {
     return true;
 }
 
-// Estimated seconds per point and axis of a loss and gradient: powers of two, and the general
-// stages (primes by their length).
+// Estimated seconds per point and axis of a loss and gradient with 7 feature pairs: powers of
+// two, and the general stages (primes by their length).
 double sep_axis_cost(const SepAxis& ax) {
-    if (ax.fast) return 2e-10;
-    double c = 1.5e-10;
-    for (int i = 0; i < ax.nrad; ++i) c += 0.75e-10 * (ax.rad[i] <= 8 ? 1.0 : 0.5 * ax.rad[i]);
+    if (ax.fast) return 1.3e-10;
+    double c = 0.0;
+    for (int i = 0; i < ax.nrad; ++i) c += ax.rad[i] <= 8 ? 1e-10 : 3e-11 * ax.rad[i];
     return c;
 }
 
@@ -284,10 +393,22 @@ int sep_cols(const SepAxis& ax, bool wide) {
     return std::max(4, std::min(16, pow2_floor(2048 / n)));
 }
 
-// Whole rows per block: of `per` feature pairs each (feature and gradient kernels), or of the window.
-int sep_rows(const SepAxis& ax, int per) {
+// Rows per block of the window kernels.
+int sep_window_rows(const SepAxis& ax) {
     const int pts = ax.fast ? SEP_BLOCK_PTS : 2048;
-    return std::max(1, std::min(ax.fast ? 64 : 16, pow2_floor(std::max(1, pts / (ax.n * per)))));
+    return std::max(1, std::min(ax.fast ? 64 : 16, pow2_floor(std::max(1, pts / ax.n))));
+}
+
+// Rows per block of the feature and gradient kernels, of a grid with `rows` rows.  A block
+// holds 2048 points (SEP_SLOTS pairs of as many rows as fit, or a share of the pairs of one
+// row); large grids take several such groups one after another, up to 8, as long as about
+// 1200 blocks (two per resident one) remain: start-up (tables, twiddles) is paid once.
+int sep_feature_rows(const SepAxis& ax, int64_t rows) {
+    const int base = std::max(1, std::min(16, pow2_floor(std::max(1, 2048 / (ax.n * SEP_SLOTS)))));
+    if (!ax.fast) return base;
+    int loops = 1;
+    while (loops < 8 && rows / (base * loops * 2) >= 1216) loops *= 2;
+    return base * loops;
 }
 
 // ------------------------------------------------------------------------- transforms (device)
@@ -297,8 +418,9 @@ namespace {
 __device__ __forceinline__ float2 cmulf(float2 a, float2 b) {
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
+// packed sums and differences: one issue slot for both parts (a - b as an exact FMA with -1)
 __device__ __forceinline__ float2 caddf(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 csubf(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ float2 csubf(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 __device__ __forceinline__ float2 swapf(float2 a) { return make_float2(a.y, a.x); }
 // times -i
 __device__ __forceinline__ float2 rot(float2 a) { return make_float2(a.y, -a.x); }
@@ -329,11 +451,11 @@ __device__ __forceinline__ void fill_twiddles(float2* tw, int n) {
 }
 
 __device__ __forceinline__ void bfly4(float2& a, float2& b, float2& c, float2& d) {
-    const float2 s0 = caddf(a, c), d0 = csubf(a, c), s1 = caddf(b, d), d1 = rot(csubf(b, d));
+    const float2 s0 = caddf(a, c), d0 = csubf(a, c), s1 = caddf(b, d), t = csubf(b, d);
     a = caddf(s0, s1);
-    b = caddf(d0, d1);
+    b = make_float2(d0.x + t.y, d0.y - t.x);
     c = csubf(s0, s1);
-    d = csubf(d0, d1);
+    d = make_float2(d0.x - t.y, d0.y + t.x);
 }
 
 // V[q] = sum_r v[r] exp(-2 pi i r q / R) in place
@@ -350,18 +472,18 @@ __device__ __forceinline__ void butterfly(float2 (&v)[R]) {
         bfly4(v[0], v[2], v[4], v[6]);
         bfly4(v[1], v[3], v[5], v[7]);
         constexpr float h = 0.70710678118654752440f;
-        const float2 w1 = make_float2(h * (v[3].x + v[3].y), h * (v[3].y - v[3].x));
-        const float2 w2 = rot(v[5]);
-        const float2 w3 = make_float2(h * (v[7].y - v[7].x), -h * (v[7].x + v[7].y));
-        const float2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6], o0 = v[1];
+        const float2 hp = make_float2(h, h), hm = make_float2(-h, -h);
+        const float2 w1 = make_float2(v[3].x + v[3].y, v[3].y - v[3].x);     // odd 1 times (1 - i)
+        const float2 w3 = make_float2(v[7].y - v[7].x, -v[7].x - v[7].y);    // odd 3 times -(1 + i)
+        const float2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6], o0 = v[1], o2 = v[5];
         v[0] = caddf(e0, o0);
         v[4] = csubf(e0, o0);
-        v[1] = caddf(e1, w1);
-        v[5] = csubf(e1, w1);
-        v[2] = caddf(e2, w2);
-        v[6] = csubf(e2, w2);
-        v[3] = caddf(e3, w3);
-        v[7] = csubf(e3, w3);
+        v[1] = __ffma2_rn(w1, hp, e1);
+        v[5] = __ffma2_rn(w1, hm, e1);
+        v[2] = make_float2(e2.x + o2.y, e2.y - o2.x);
+        v[6] = make_float2(e2.x - o2.y, e2.y + o2.x);
+        v[3] = __ffma2_rn(w3, hp, e3);
+        v[7] = __ffma2_rn(w3, hm, e3);
     } else {
         // odd radices: pair r with R - r; the cosines and sines of 2 pi j / R are constants
         constexpr int H = (R - 1) / 2;
@@ -565,10 +687,10 @@ extern __shared__ __align__(16) float2 sep_smem[];
 struct SepShared {
     float2 *tw, *a, *b;
 };
-__device__ __forceinline__ SepShared sep_shared(int n, int lines, int pitch) {
+__device__ __forceinline__ SepShared sep_shared(float2* sm, int n, int lines, int pitch) {
     SepShared s;
-    s.tw = sep_smem;
-    s.a = sep_smem + ((n + 1) & ~1);
+    s.tw = sm;
+    s.a = sm + ((n + 1) & ~1);
     s.b = s.a + lines * pitch;
     return s;
 }
@@ -578,12 +700,14 @@ struct SepBlock {
     int a, b, block, tier;
 };
 
-// Finds the block's item (every thread looks at one item), copies its level to shared memory
-// and reads the instance's tier.  Returns false when there is nothing to do: the instance has
-// stopped, or (TIERED) its field needs the direct kernels.
-template <bool TIERED>
+// Before the wait for the predecessor: finds the block's item (every thread looks at one),
+// copies its level to shared memory (tables are written at least two launches earlier) and
+// fills the twiddles of `axis(level)`.  After it: reads the instance's tier and returns false
+// when there is nothing to do -- the instance has stopped, or (TIERED) its field needs the
+// direct kernels.
+template <bool TIERED, typename AXIS>
 __device__ __forceinline__ bool enter(const SepTables& tb, const SepItem* __restrict__ items, int nitem,
-                                      SepBlock& bk) {
+                                      SepBlock& bk, float2* tw, AXIS axis) {
     int count = 0;
     for (int base = 0; base < nitem; base += blockDim.x) {
         const int i = base + threadIdx.x;
@@ -593,17 +717,26 @@ __device__ __forceinline__ bool enter(const SepTables& tb, const SepItem* __rest
     const uint32_t* src = reinterpret_cast<const uint32_t*>(tb.level + it.level);
     uint32_t* dst = reinterpret_cast<uint32_t*>(&bk.lv);
     for (int i = threadIdx.x; i < (int)(sizeof(SepLevel) / 4); i += blockDim.x) dst[i] = src[i];
-    const bool stopped = it.done != nullptr && *it.done;
-    const int tier = TIERED ? *it.tier : 0;
     if (threadIdx.x == 0) {
         bk.a = it.a;
         bk.b = it.b;
         bk.block = (int)((int64_t)blockIdx.x - it.blockStart);
-        bk.tier = tier;
     }
+    const int *tier = it.tier, *done = it.done;
     __syncthreads();
-    return !stopped && tier < SEP_TIERS;
+    fill_twiddles(tw, axis(bk.lv));
+    dep_wait();
+    dep_trigger();
+    const bool stopped = done != nullptr && *done;
+    const int t = TIERED ? *tier : 0;
+    if (threadIdx.x == 0) bk.tier = t;
+    __syncthreads();
+    return !stopped && t < SEP_TIERS;
 }
+
+__device__ __forceinline__ int axis_x(const SepLevel& lv) { return lv.n2; }
+__device__ __forceinline__ int axis_y(const SepLevel& lv) { return lv.n1; }
+__device__ __forceinline__ int axis_last(const SepLevel& lv) { return lv.n0 > 1 ? lv.n0 : lv.n1; }
 
 // runs body(std::integral_constant<int, N>) for the power of two N = 2^k, 16 <= N <= 2048
 template <typename F>
@@ -622,62 +755,15 @@ __device__ __forceinline__ void for_pow2(int k, F&& body) {
 
 }  // namespace
 
-// ------------------------------------------------------------------------- range
-
-// Tier of a share of the finest field (all phases); sep_feat combines the blocks' results.
-// NaN and values beyond every tier give SEP_TIERS: direct kernels.
-__global__ void __launch_bounds__(256) sep_range_kernel(const __grid_constant__ SepTables tb,
-                                                        const SepItem* __restrict__ items, int nitem) {
-    const int it = find_segment(items, nitem, (int64_t)blockIdx.x);
-    const SepLevel& lv = tb.level[items[it].level];
-    if (lv.done != nullptr && *lv.done) return;
-    const int blk = (int)((int64_t)blockIdx.x - items[it].blockStart), nblk = items[it].a;
-    const int64_t count = lv.N * lv.phases, stride = (int64_t)nblk * blockDim.x;
-    const float* __restrict__ field = lv.field;
-    float lo = 0.f, hi = 0.f;
-    int bad = 0;
-    for (int64_t i = (int64_t)blk * blockDim.x + threadIdx.x; i < count; i += 4 * stride) {
-        float v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = i + u * stride < count ? field[i + u * stride] : 0.f;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            bad |= !(v[u] == v[u]);
-            lo = fminf(lo, v[u]);
-            hi = fmaxf(hi, v[u]);
-        }
-    }
-    int t = 0;
-    while (t < tb.ntier && !(lo >= tb.tier[t].lo && hi <= tb.tier[t].hi)) ++t;
-    if (bad || t >= tb.ntier) t = SEP_TIERS;
-    t = __reduce_max_sync(0xffffffffu, t);
-    __shared__ int sh[8];
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = t;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < 8; ++w) t = max(t, sh[w]);
-        lv.tiers[blk] = t;
-    }
-}
-
 // ------------------------------------------------------------------------- features
 
 namespace {
 
-// Coefficients of a tier in shared memory: cf[j * SEP_STRIDE + p], DERIV: times j, for the
-// series T_j' = j U_{j-1}.
-constexpr int SEP_STRIDE = 16;
-static_assert(SEP_MAX_PAIRS <= SEP_STRIDE, "one row of coefficients holds every pair");
-
+// The coefficients are read from global memory: all threads of a line read the same ones, and
+// the few kilobytes of a tier stay in L1.
 template <bool DERIV>
-__device__ __forceinline__ void load_coef(const SepTables& tb, const SepTier& t, float2* cf) {
-    const int stride = sep_coef_stride(t.npair);
-    for (int i = threadIdx.x; i < t.deg * SEP_STRIDE; i += blockDim.x) {
-        const int j = i / SEP_STRIDE, p = i % SEP_STRIDE;
-        float2 c = p < t.npair ? tb.coef[t.coef + j * stride + p] : make_float2(0.f, 0.f);
-        if (DERIV) c = make_float2((float)j * c.x, (float)j * c.y);
-        cf[i] = c;
-    }
+__device__ __forceinline__ const float2* tier_coef(const SepTables& tb, const SepTier& t) {
+    return tb.coef + t.coef + (DERIV ? t.deg * t.npair : 0);
 }
 
 // One packed pair of features (DERIV: of their derivatives) at C normalised values:
@@ -685,7 +771,7 @@ __device__ __forceinline__ void load_coef(const SepTables& tb, const SepTier& t,
 // j = 4 on are summed first and the four large ones last, so that the small terms are not
 // lost against them.  Bound by the FP32 pipe: per term one FFMA2 and one FFMA.
 template <bool DERIV, int C>
-__device__ __forceinline__ void eval_features(const float2* __restrict__ cf, int deg, const float (&x)[C],
+__device__ __forceinline__ void eval_features(const float2* __restrict__ cf, int stride, int deg, const float (&x)[C],
                                               float2 (&out)[C]) {
     float x2[C], w0[C], w1[C];
 #pragma unroll
@@ -702,10 +788,10 @@ __device__ __forceinline__ void eval_features(const float2* __restrict__ cf, int
             w1[e] = fmaf(x2[e], w0[e], -t2);                // T_4
         }
     }
-    const float2* c = cf + 4 * SEP_STRIDE;
+    const float2* c = cf + 4 * stride;
     int j = 4;
-    for (; j + 1 < deg; j += 2, c += 2 * SEP_STRIDE) {
-        const float2 ca = c[0], cb = c[SEP_STRIDE];
+    for (; j + 1 < deg; j += 2, c += 2 * stride) {
+        const float2 ca = __ldg(c), cb = __ldg(c + stride);
 #pragma unroll
         for (int e = 0; e < C; ++e) {
             out[e] = __ffma2_rn(ca, make_float2(w1[e], w1[e]), out[e]);
@@ -715,11 +801,11 @@ __device__ __forceinline__ void eval_features(const float2* __restrict__ cf, int
         }
     }
     if (j < deg) {
-        const float2 ca = c[0];
+        const float2 ca = __ldg(c);
 #pragma unroll
         for (int e = 0; e < C; ++e) out[e] = __ffma2_rn(ca, make_float2(w1[e], w1[e]), out[e]);
     }
-    const float2 c0 = cf[0], c1 = cf[SEP_STRIDE], c2 = cf[2 * SEP_STRIDE], c3 = cf[3 * SEP_STRIDE];
+    const float2 c0 = __ldg(cf), c1 = __ldg(cf + stride), c2 = __ldg(cf + 2 * stride), c3 = __ldg(cf + 3 * stride);
 #pragma unroll
     for (int e = 0; e < C; ++e) {
         float a1, a2, a3;
@@ -742,18 +828,18 @@ __device__ __forceinline__ void eval_features(const float2* __restrict__ cf, int
 // rows of a block of the feature and gradient kernels: SLOTS feature pairs side by side
 template <int N>
 struct RowShape {
-    static constexpr int T = N / 8, LINES = SEP_THREADS / T;
+    static constexpr int T = N / 8, LINES = SEP_ROW_THREADS / T;
     static constexpr int SLOTS = LINES < SEP_SLOTS ? LINES : SEP_SLOTS;
     static constexpr int ROWS = LINES / SLOTS;
     static constexpr bool WARP = T <= 32;
 };
 
 template <int N>
-__device__ __forceinline__ Line<N> row_line(int line, int t, int lines) {
+__device__ __forceinline__ Line<N> row_line(float2* sm, int line, int t, int lines) {
     constexpr int P = row_pitch<N>();
     Line<N> ln;
-    ln.tw = sep_smem;
-    ln.buf[0] = sep_smem + N + line * P;
+    ln.tw = sm;
+    ln.buf[0] = sm + N + line * P;
     ln.buf[1] = ln.buf[0] + lines * P;
     ln.t = t;
     return ln;
@@ -762,14 +848,13 @@ __device__ __forceinline__ Line<N> row_line(int line, int t, int lines) {
 }  // namespace
 
 // item: (level, phase a); blocks: groups of rows.  Features of whole rows and their transform
-// along x.  Every block first combines the range blocks' tiers; the first block of the finest
+// along x.  Every block combines the range blocks' tiers; the first block of the finest
 // level leaves the result for the later kernels.
-__global__ void __launch_bounds__(SEP_THREADS, 2) sep_feat_kernel(const __grid_constant__ SepTables tb,
-                                                                  const SepItem* __restrict__ items, int nitem) {
+__global__ void __launch_bounds__(SEP_ROW_THREADS, 4) sep_feat_kernel(const __grid_constant__ SepTables tb,
+                                                                      const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
-    __shared__ int tsh[SEP_THREADS / 32];
-    __shared__ __align__(16) float2 cf[SEP_MAX_DEG * SEP_STRIDE];
-    if (!enter<false>(tb, items, nitem, bk)) return;
+    __shared__ int tsh[SEP_ROW_THREADS / 32];
+    if (!enter<false>(tb, items, nitem, bk, sep_smem, axis_x)) return;
     const SepLevel& lv = bk.lv;
     {
         int t = 0;
@@ -777,48 +862,50 @@ __global__ void __launch_bounds__(SEP_THREADS, 2) sep_feat_kernel(const __grid_c
         t = __reduce_max_sync(0xffffffffu, t);
         if ((threadIdx.x & 31) == 0) tsh[threadIdx.x >> 5] = t;
     }
+    float2* sm = sep_smem;
+    const int rowsN = lv.n0 * lv.n1, n = lv.n2;
     __syncthreads();
     int tier = tsh[0];
-    for (int i = 1; i < SEP_THREADS / 32; ++i) tier = max(tier, tsh[i]);
+    for (int i = 1; i < SEP_ROW_THREADS / 32; ++i) tier = max(tier, tsh[i]);
     if (lv.first && bk.a == 0 && bk.block == 0 && threadIdx.x == 0) *lv.tier = tier;
     if (tier >= SEP_TIERS) return;
     const SepTier& t = tb.tier[tier];
-    load_coef<false>(tb, t, cf);
-    const int rowsN = lv.n0 * lv.n1, n = lv.n2;
+    const float2* __restrict__ cf = tier_coef<false>(tb, t);
     const int row0 = bk.block * lv.rowsF, rows = min(lv.rowsF, rowsN - row0);
     const float* __restrict__ field = lv.field + (int64_t)bk.a * lv.N + (int64_t)row0 * n;
     float2* __restrict__ Z = lv.Z + (int64_t)bk.a * lv.maxPairs * lv.N + (int64_t)row0 * n;
-    fill_twiddles(sep_smem, n);
-    __syncthreads();
     if (lv.ax[2].fast) {
         for_pow2(lv.ax[2].fast, [&](auto c) {
             constexpr int N = decltype(c)::value;
             using S = RowShape<N>;
-            const int line = threadIdx.x / S::T, p = line % S::SLOTS, row = line / S::SLOTS;
-            const Line<N> ln = row_line<N>(line, threadIdx.x % S::T, S::LINES);
-            const bool in = row < rows;
-            float x[8];
+            const int line = threadIdx.x / S::T, p = line % S::SLOTS;
+            const Line<N> ln = row_line<N>(sm, line, threadIdx.x % S::T, S::LINES);
+            for (int row = line / S::SLOTS; row < lv.rowsF; row += S::ROWS) {
+                const bool in = row < rows;
+                float x[8];
 #pragma unroll
-            for (int e = 0; e < 8; ++e)
-                x[e] = in ? (field[row * N + ln.t + e * S::T] - t.mid) * t.inv_half : 0.f;
-            for (int p0 = 0; p0 < t.npair; p0 += S::SLOTS) {
-                const bool live = in && p0 + p < t.npair;
-                float2 v[8];
-                if (live) eval_features<false, 8>(cf + p0 + p, t.deg, x, v);
-                p2_fft<N, S::WARP, 0>(v, ln);
-                if (live) {
-                    float2* out = Z + (int64_t)(p0 + p) * lv.N + row * N + ln.t;
+                for (int e = 0; e < 8; ++e)
+                    x[e] = in ? (field[row * N + ln.t + e * S::T] - t.mid) * t.inv_half : 0.f;
+                for (int p0 = 0; p0 < t.npair; p0 += S::SLOTS) {
+                    const bool live = in && p0 + p < t.npair;
+                    float2 v[8];
+                    if (live) eval_features<false, 8>(cf + p0 + p, t.npair, t.deg, x, v);
+                    p2_fft<N, S::WARP, 0>(v, ln);
+                    if (live) {
+                        float2* out = Z + (int64_t)(p0 + p) * lv.N + row * N + ln.t;
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) out[e * S::T] = v[e];
+                        for (int e = 0; e < 8; ++e) out[e * S::T] = v[e];
+                    }
+                    // the next round starts in the buffer this one started in
+                    if (p2_exchanges(N) & 1) line_sync<S::WARP>();
                 }
-                line_sync<S::WARP>();       // the next round starts in the buffer this one started in
             }
         });
         return;
     }
     const int pitch = spad(n - 1) + 2;
     const float inv_n = 1.0f / (float)n;
-    const SepShared s = sep_shared(n, lv.rowsF * SEP_SLOTS, pitch);
+    const SepShared s = sep_shared(sm, n, lv.rowsF * SEP_SLOTS, pitch);
     for (int p0 = 0; p0 < t.npair; p0 += SEP_SLOTS) {
         const int nc = min(SEP_SLOTS, t.npair - p0);
         __syncthreads();
@@ -827,7 +914,7 @@ __global__ void __launch_bounds__(SEP_THREADS, 2) sep_feat_kernel(const __grid_c
             const int l = q / nc, c = q - l * nc;
             const float x[1] = {(field[l * n + i] - t.mid) * t.inv_half};
             float2 f[1];
-            eval_features<false, 1>(cf + p0 + c, t.deg, x, f);
+            eval_features<false, 1>(cf + p0 + c, t.npair, t.deg, x, f);
             s.a[q * pitch + spad(i)] = f[0];
         }
         const float2* r = transform(lv.ax[2], s.a, s.b, s.tw, rows * nc, pitch);
@@ -918,21 +1005,20 @@ __device__ __forceinline__ void load_cols(const float2* __restrict__ src, const 
 }  // namespace
 
 // Middle axis of 3-D, in place on Z (forward) or on the product spectra (INVERSE).  item:
-// (level, phase a); blocks: groups of planes' columns (x fastest, then z), then pairs.
+// (level, phase a); blocks: groups of planes' columns (x fastest, then z).  A block walks the
+// feature pairs, loading the next pair's columns while it transforms the current ones.
 template <bool INVERSE>
-__global__ void __launch_bounds__(SEP_THREADS, 2) sep_fft_y_kernel(const __grid_constant__ SepTables tb,
+__global__ void __launch_bounds__(SEP_THREADS, COLOCC) sep_fft_y_kernel(const __grid_constant__ SepTables tb,
                                                                    const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
-    if (!enter<true>(tb, items, nitem, bk)) return;
+    if (!enter<true>(tb, items, nitem, bk, sep_smem, axis_y)) return;
     const SepLevel& lv = bk.lv;
+    float2* sm = sep_smem;
     const int L = lv.colsY, n = lv.n1;
     const int xg = (lv.n2 + L - 1) / L, groups = xg * lv.n0;
     const int slots = lv.ax[1].fast ? SEP_BLOCK_PTS / (L * n) : 1;
-    const int per = (groups + slots - 1) / slots;      // blocks of one pair
-    const int p = bk.block / per, g0 = (bk.block % per) * slots;
-    if (p >= tb.tier[bk.tier].npair) return;
-    float2* grid = (INVERSE ? lv.Q : lv.Z) + ((int64_t)bk.a * lv.maxPairs + p) * lv.N;
-    fill_twiddles(sep_smem, n);
+    const int g0 = bk.block * slots, npair = tb.tier[bk.tier].npair;
+    float2* grid = (INVERSE ? lv.Q : lv.Z) + (int64_t)bk.a * lv.maxPairs * lv.N;
     auto group = [&](int gi) {
         ColGroup g;
         g.n = n;
@@ -944,34 +1030,42 @@ __global__ void __launch_bounds__(SEP_THREADS, 2) sep_fft_y_kernel(const __grid_
         return g;
     };
     if (lv.ax[1].fast) {
-        __syncthreads();
         for_pow2(lv.ax[1].fast, [&](auto cc) {
             constexpr int N = decltype(cc)::value;
             const Cols<N> c(L);
             const bool on = g0 + c.slot < groups;
             const ColGroup g = group(on ? g0 + c.slot : 0);
-            float2 v[8];
-            load8<N>(grid, g, c, on, v);
-            if (INVERSE) swap8(v);
-            p2_fft<N, false, 0>(v, c.ln);
-            if (INVERSE) swap8(v);
-            store8<N>(grid, g, c, on, v);
+            float2 nx[8];
+            load8<N>(grid, g, c, on, nx);
+            for (int p = 0; p < npair; ++p) {
+                float2 v[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] = INVERSE ? swapf(nx[e]) : nx[e];
+                if (p + 1 < npair) load8<N>(grid + (int64_t)(p + 1) * lv.N, g, c, on, nx);
+                p2_fft<N, false, 0>(v, c.ln);
+                if (p2_exchanges(N) & 1) __syncthreads();
+                if (INVERSE) swap8(v);
+                store8<N>(grid + (int64_t)p * lv.N, g, c, on, v);
+            }
         });
         return;
     }
     const ColGroup g = group(g0);
     const int pitch = sep_pitch(n, L), sh = 31 - __clz(L);
-    const SepShared s = sep_shared(n, L, pitch);
-    for (int e = threadIdx.x; e < L * n; e += blockDim.x) {
-        const int l = e & (L - 1), i = e >> sh;
-        const float2 v = l < g.cols ? grid[g.base + i * g.stride + l] : make_float2(0.f, 0.f);
-        s.a[l * pitch + spad(i)] = INVERSE ? swapf(v) : v;
-    }
-    const float2* r = transform(lv.ax[1], s.a, s.b, s.tw, L, pitch);
-    for (int e = threadIdx.x; e < L * n; e += blockDim.x) {
-        const int l = e & (L - 1), i = e >> sh;
-        const float2 v = r[l * pitch + spad(i)];
-        if (l < g.cols) grid[g.base + i * g.stride + l] = INVERSE ? swapf(v) : v;
+    const SepShared s = sep_shared(sm, n, L, pitch);
+    for (int p = 0; p < npair; ++p, grid += lv.N) {
+        __syncthreads();
+        for (int e = threadIdx.x; e < L * n; e += blockDim.x) {
+            const int l = e & (L - 1), i = e >> sh;
+            const float2 v = l < g.cols ? grid[g.base + i * g.stride + l] : make_float2(0.f, 0.f);
+            s.a[l * pitch + spad(i)] = INVERSE ? swapf(v) : v;
+        }
+        const float2* r = transform(lv.ax[1], s.a, s.b, s.tw, L, pitch);
+        for (int e = threadIdx.x; e < L * n; e += blockDim.x) {
+            const int l = e & (L - 1), i = e >> sh;
+            const float2 v = r[l * pitch + spad(i)];
+            if (l < g.cols) grid[g.base + i * g.stride + l] = INVERSE ? swapf(v) : v;
+        }
     }
 }
 
@@ -981,12 +1075,13 @@ __global__ void __launch_bounds__(SEP_THREADS, 2) sep_fft_y_kernel(const __grid_
 // inverse along the last axis, cropped to r = 0 .. P (-r belongs to the pair (b, a)).  CROSS:
 // a and b may differ.  The next round's columns are loaded while the current one is transformed.
 template <bool CROSS>
-__global__ void __launch_bounds__(SEP_THREADS, CROSS ? 1 : 2)
+__global__ void __launch_bounds__(SEP_THREADS, CROSS ? 1 : COLOCC)
 sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
     __shared__ double dcs[SEP_THREADS / 2];
-    if (!enter<true>(tb, items, nitem, bk)) return;
+    if (!enter<true>(tb, items, nitem, bk, sep_smem, axis_last)) return;
     const SepLevel& lv = bk.lv;
+    float2* sm = sep_smem;
     const SepTier& t = tb.tier[bk.tier];
     int x0, y;
     const ColGroup g = last_axis(lv, bk.block, x0, y);
@@ -994,14 +1089,13 @@ sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict
     const bool dc_block = x0 == 0 && y == 0;
     const float2* Za = lv.Z + (int64_t)bk.a * lv.maxPairs * lv.N;
     const float2* Zb = lv.Z + (int64_t)bk.b * lv.maxPairs * lv.N;
+    float2* Zw = lv.Z;                       // one phase: the spectra are left for sep_mul
     const int pair = bk.a * lv.phases + bk.b;
     const int P = lv.n0 > 1 ? lv.P0 : lv.P1;
     // 3-D: U[r][y][x]; 2-D: V[r][x]
     float2* out = (lv.n0 > 1 ? lv.U : lv.V) + (int64_t)pair * (lv.n0 > 1 ? lv.strideU : lv.strideV) + g.base;
-    fill_twiddles(sep_smem, g.n);
     const bool cross = CROSS && bk.a != bk.b;
     if (ax.fast) {
-        __syncthreads();
         for_pow2(ax.fast, [&](auto cc) {
             constexpr int N = decltype(cc)::value, T = N / 8;
             constexpr int PAR1 = p2_exchanges(N) & 1;
@@ -1024,6 +1118,7 @@ sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict
                     if (p0 + c.slots < t.npair) load8<N>(Za + (int64_t)q * lv.N, g, c, q < t.npair, nx);
                     p2_fft<N, false, 0>(v, c.ln);
                     if (PAR1 != 0) __syncthreads();   // the next round starts in buffer 0 again
+                    if (lv.keep) store8<N>(Zw + (int64_t)p * lv.N, g, c, p < t.npair, v);
 #pragma unroll
                     for (int e = 0; e < 8; ++e) acc[e].x = fmaf(sg, fmaf(v[e].x, v[e].x, v[e].y * v[e].y), acc[e].x);
                     if (has_dc) dc += (double)sg * ((double)v[0].x * v[0].x + (double)v[0].y * v[0].y);
@@ -1082,7 +1177,7 @@ sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict
         return;
     }
     const int pitch = sep_pitch(g.n, g.L), sh = 31 - __clz(g.L), total = g.L * g.n;
-    const SepShared s = sep_shared(g.n, g.L, pitch);
+    const SepShared s = sep_shared(sm, g.n, g.L, pitch);
     float2 acc[SEP_OWN], za[SEP_OWN];
 #pragma unroll
     for (int q = 0; q < SEP_OWN; ++q) acc[q] = make_float2(0.f, 0.f);
@@ -1106,6 +1201,11 @@ sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict
             load_cols(Zb + (int64_t)p * lv.N, g, pitch, s.a);
             r = transform(ax, s.a, s.b, s.tw, g.L, pitch);
         }
+        if (lv.keep && !CROSS)
+            for (int e = threadIdx.x; e < total; e += blockDim.x) {
+                const int l = e & (g.L - 1), i = e >> sh;
+                if (l < g.cols) Zw[(int64_t)p * lv.N + g.base + i * g.stride + l] = r[l * pitch + spad(i)];
+            }
         own([&](int q, int at) {
             const float2 v = r[at], u = cross ? za[q] : v;
             acc[q].x = fmaf(sg, __fadd_rn(__fmul_rn(u.x, v.x), __fmul_rn(u.y, v.y)), acc[q].x);
@@ -1135,15 +1235,15 @@ template <bool DESC>
 __global__ void __launch_bounds__(SEP_THREADS, 2) sep_win_y_kernel(const __grid_constant__ SepTables tb,
                                                                    const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
-    if (!enter<true>(tb, items, nitem, bk)) return;
+    if (!enter<true>(tb, items, nitem, bk, sep_smem, axis_y)) return;
     const SepLevel& lv = bk.lv;
+    float2* sm = sep_smem;
     const int L = lv.colsY, n = lv.n1, P1 = lv.P1, wy = 2 * P1 + 1;
     const int xg = (lv.n2 + L - 1) / L, groups = xg * (lv.P0 + 1);
     const int slots = lv.ax[1].fast ? SEP_BLOCK_PTS / (L * n) : 1;
     const int pair = bk.a * lv.phases + bk.b;
     float2* U = lv.U + (int64_t)pair * lv.strideU;
     float2* V = lv.V + (int64_t)pair * lv.strideV;
-    fill_twiddles(sep_smem, n);
     auto window = [&](const float2* src, int i, int64_t stride) {
         // ry = i and ry = i - n (both at the aliased ry = +-n/2)
         float2 v = make_float2(0.f, 0.f);
@@ -1152,7 +1252,6 @@ __global__ void __launch_bounds__(SEP_THREADS, 2) sep_win_y_kernel(const __grid_
         return v;
     };
     if (lv.ax[1].fast) {
-        __syncthreads();
         for_pow2(lv.ax[1].fast, [&](auto cc) {
             constexpr int N = decltype(cc)::value, T = N / 8;
             const Cols<N> c(L);
@@ -1183,7 +1282,7 @@ __global__ void __launch_bounds__(SEP_THREADS, 2) sep_win_y_kernel(const __grid_
     }
     const int gi = bk.block, k = gi / xg, x0 = (gi % xg) * L, cols = min(L, lv.n2 - x0);
     const int pitch = sep_pitch(n, L), sh = 31 - __clz(L);
-    const SepShared s = sep_shared(n, L, pitch);
+    const SepShared s = sep_shared(sm, n, L, pitch);
     U += (int64_t)k * lv.n1 * lv.n2 + x0;
     V += (int64_t)k * wy * lv.n2 + x0;
     for (int e = threadIdx.x; e < L * n; e += blockDim.x) {
@@ -1238,60 +1337,132 @@ __device__ __forceinline__ int half_index(const SepLevel& lv, int rz, int ry, in
 }  // namespace
 
 // item: (level, phases a, b); blocks: groups of rowsW window rows.  Inverse along x: the
-// entries of block (a, b).
+// entries of block (a, b).  With lv.fuse (one phase, a loss and its gradient in one call) a row
+// goes straight on: its residuals D - D_des are G up to the loss' factor gscale, which sep_mul
+// applies, so they are embedded and transformed here (the rows of sep_gx), and the block leaves
+// its share of sum (D - D_des)^2 and sum D_des^2.
 __global__ void __launch_bounds__(SEP_THREADS, 2) sep_desc_kernel(const __grid_constant__ SepTables tb,
                                                                   const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
-    if (!enter<true>(tb, items, nitem, bk)) return;
+    __shared__ DF dsh[32];
+    if (!enter<true>(tb, items, nitem, bk, sep_smem, axis_x)) return;
     const SepLevel& lv = bk.lv;
+    float2* sm = sep_smem;
     const int n = lv.n2, P2 = lv.P2;
     const int R = window_rows(lv);
     const int row0 = bk.block * lv.rowsW, rows = min(lv.rowsW, R - row0);
     const int pair = bk.a * lv.phases + bk.b;
-    const float2* V = lv.V + (int64_t)pair * lv.strideV + (int64_t)row0 * n;
+    float2* V = lv.V + (int64_t)pair * lv.strideV + (int64_t)row0 * n;
     const double dc = lv.dc[pair];
     float* desc = lv.desc + (int64_t)pair * lv.Khalf;
+    // Kahan sums of this thread's residuals and targets
+    float r2 = 0.f, r2c = 0.f, t2 = 0.f, t2c = 0.f;
+    auto kahan = [](float& sum, float& comp, float v) {
+        const float y = v - comp, u = sum + y;
+        comp = (u - sum) - y;
+        sum = u;
+    };
+    // writes the entry of (row l, rx) and returns the residual (0 outside the half window,
+    // except at rx < 0 of row 0, the mirror of an entry of the same row)
     auto entry = [&](int l, int rx, float c) {
         int rz, ry;
         window_row(lv, row0 + l, rz, ry);
-        const int k = half_index(lv, rz, ry, rx);
-        if (k >= 0) desc[k] = (float)(((double)c + dc) * lv.scaleD);
+        int k = half_index(lv, rz, ry, rx);
+        const bool mirror = k < 0 && rz == 0 && ry == 0;
+        if (k < 0 && !(lv.fuse && mirror)) return 0.f;
+        if (mirror) k = -rx;
+        const float d = (float)(((double)c + dc) * lv.scaleD);
+        if (!mirror) desc[k] = d;
+        if (!lv.fuse) return 0.f;
+        const float t = lv.sub[k], rho = d - t;
+        if (!mirror) {
+            kahan(r2, r2c, rho * rho);
+            kahan(t2, t2c, t * t);
+        }
+        return lv.scaleG * (k == 0 ? rho + rho : rho);
     };
-    fill_twiddles(sep_smem, n);
+    // embedded coefficient of position i of the row (both ends at the aliased rx = +-n/2)
+    auto embedded = [&](int l, int i, float c) {
+        float gsum = 0.f;
+        if (i <= P2) gsum = entry(l, i, c);
+        if (i > 0 && n - i <= P2) gsum += entry(l, i - n, c);
+        return gsum;
+    };
+    // 3-D: row (0, -ry) holds the mirrored coefficients of (0, ry), i.e. the conjugate transform
+    auto mirror_row = [&](int l) {
+        int rz, ry;
+        window_row(lv, row0 + l, rz, ry);
+        return lv.n0 > 1 && rz == 0 && ry > 0 ? -2 * ry : 0;
+    };
+    auto skipped = [&](int l) {
+        int rz, ry;
+        window_row(lv, row0 + l, rz, ry);
+        return rz == 0 && ry < 0;
+    };
     if (lv.ax[2].fast) {
-        __syncthreads();
         for_pow2(lv.ax[2].fast, [&](auto cc) {
             constexpr int N = decltype(cc)::value, T = N / 8;
             constexpr bool WARP = T <= 32;
             const int line = threadIdx.x / T;
-            const Line<N> ln = row_line<N>(line, threadIdx.x % T, SEP_THREADS / T);
-            const bool in = line < rows;
+            const Line<N> ln = row_line<N>(sm, line, threadIdx.x % T, SEP_THREADS / T);
+            const bool in = line < rows && !skipped(line);
             float2 v[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) v[e] = in ? swapf(V[line * N + ln.t + e * T]) : make_float2(0.f, 0.f);
             p2_fft<N, WARP, 0>(v, ln);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float gv = in ? embedded(line, ln.t + e * T, v[e].y) : 0.f;
+                v[e] = make_float2(gv, 0.f);
+            }
+            if (!lv.fuse) return;
+            if (p2_exchanges(N) & 1) line_sync<WARP>();
+            p2_fft<N, WARP, 0>(v, ln);
             if (!in) return;
+            const int m = mirror_row(line);
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
                 const int i = ln.t + e * T;
-                if (i <= P2) entry(line, i, v[e].y);
-                if (i > 0 && N - i <= P2) entry(line, i - N, v[e].y);
+                V[line * N + i] = v[e];
+                if (m) V[(int64_t)(line + m) * N + i] = make_float2(v[e].x, -v[e].y);
             }
         });
-        return;
+    } else {
+        const int pitch = spad(n - 1) + 2, wx = 2 * P2 + 1;
+        const SepShared s = sep_shared(sm, n, lv.rowsW, pitch);
+        const float inv_n = 1.0f / (float)n;
+        for (int e = threadIdx.x; e < rows * n; e += blockDim.x) {
+            const int l = fdiv(e, inv_n), i = e - l * n;
+            s.a[l * pitch + spad(i)] = skipped(l) ? make_float2(0.f, 0.f) : swapf(V[e]);
+        }
+        float2* r = transform(lv.ax[2], s.a, s.b, s.tw, rows, pitch);
+        if (!lv.fuse) {
+            for (int e = threadIdx.x; e < rows * wx; e += blockDim.x) {
+                const int l = e / wx, rx = e - l * wx - P2;
+                entry(l, rx, r[l * pitch + spad(rx < 0 ? rx + n : rx)].y);
+            }
+        } else {
+            for (int e = threadIdx.x; e < rows * n; e += blockDim.x) {
+                const int l = fdiv(e, inv_n), i = e - l * n;
+                float2& x = r[l * pitch + spad(i)];
+                x = make_float2(skipped(l) ? 0.f : embedded(l, i, x.y), 0.f);
+            }
+            r = transform(lv.ax[2], r, r == s.a ? s.b : s.a, s.tw, rows, pitch);
+            for (int e = threadIdx.x; e < rows * n; e += blockDim.x) {
+                const int l = fdiv(e, inv_n), i = e - l * n;
+                if (skipped(l)) continue;
+                const float2 x = r[l * pitch + spad(i)];
+                const int m = mirror_row(l);
+                V[e] = x;
+                if (m) V[(int64_t)(l + m) * n + i] = make_float2(x.x, -x.y);
+            }
+        }
     }
-    const int pitch = spad(n - 1) + 2, wx = 2 * P2 + 1;
-    const SepShared s = sep_shared(n, lv.rowsW, pitch);
-    const float inv_n = 1.0f / (float)n;
-    for (int e = threadIdx.x; e < rows * n; e += blockDim.x) {
-        const int l = fdiv(e, inv_n), i = e - l * n;
-        s.a[l * pitch + spad(i)] = swapf(V[e]);
-    }
-    const float2* r = transform(lv.ax[2], s.a, s.b, s.tw, rows, pitch);
-    for (int e = threadIdx.x; e < rows * wx; e += blockDim.x) {
-        const int l = e / wx, rx = e - l * wx - P2;
-        entry(l, rx, r[l * pitch + spad(rx < 0 ? rx + n : rx)].y);
-    }
+    if (!lv.fuse) return;
+    // Kahan's (sum, comp) stands for sum - comp
+    const DF R2 = block_sum_df(df_two_sum(r2, -r2c), dsh);
+    const DF T2 = block_sum_df(df_two_sum(t2, -t2c), dsh);
+    if (threadIdx.x == 0) lv.sums[bk.block] = make_float4(R2.hi, R2.lo, T2.hi, T2.lo);
 }
 
 // item: (level, phases a, b); blocks: groups of rowsW window rows.  G(r) of the row (the
@@ -1299,13 +1470,13 @@ __global__ void __launch_bounds__(SEP_THREADS, 2) sep_desc_kernel(const __grid_c
 __global__ void __launch_bounds__(SEP_THREADS, 2) sep_gx_kernel(const __grid_constant__ SepTables tb,
                                                                 const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
-    if (!enter<true>(tb, items, nitem, bk)) return;
+    if (!enter<true>(tb, items, nitem, bk, sep_smem, axis_x)) return;
     const SepLevel& lv = bk.lv;
+    float2* sm = sep_smem;
     const int n = lv.n2, P2 = lv.P2;
     const int R = window_rows(lv);
     const int row0 = bk.block * lv.rowsW, rows = min(lv.rowsW, R - row0);
     const int pair = bk.a * lv.phases + bk.b;
-    fill_twiddles(sep_smem, n);
     const int64_t oab = (int64_t)pair * lv.Khalf, oba = ((int64_t)bk.b * lv.phases + bk.a) * lv.Khalf;
     const float scale = lv.scaleG * (lv.sc != nullptr ? lv.sc->gscale : 1.f);
     auto delta = [&](int64_t off, int k) {
@@ -1329,12 +1500,11 @@ __global__ void __launch_bounds__(SEP_THREADS, 2) sep_gx_kernel(const __grid_con
     };
     float2* V = lv.V + (int64_t)pair * lv.strideV + (int64_t)row0 * n;
     if (lv.ax[2].fast) {
-        __syncthreads();
         for_pow2(lv.ax[2].fast, [&](auto cc) {
             constexpr int N = decltype(cc)::value, T = N / 8;
             constexpr bool WARP = T <= 32;
             const int line = threadIdx.x / T;
-            const Line<N> ln = row_line<N>(line, threadIdx.x % T, SEP_THREADS / T);
+            const Line<N> ln = row_line<N>(sm, line, threadIdx.x % T, SEP_THREADS / T);
             const bool in = line < rows;
             float2 v[8];
 #pragma unroll
@@ -1347,7 +1517,7 @@ __global__ void __launch_bounds__(SEP_THREADS, 2) sep_gx_kernel(const __grid_con
         return;
     }
     const int pitch = spad(n - 1) + 2;
-    const SepShared s = sep_shared(n, lv.rowsW, pitch);
+    const SepShared s = sep_shared(sm, n, lv.rowsW, pitch);
     const float inv_n = 1.0f / (float)n;
     for (int e = threadIdx.x; e < rows * n; e += blockDim.x) {
         const int l = fdiv(e, inv_n), i = e - l * n;
@@ -1397,19 +1567,19 @@ struct GCols {
 // forward transform of the columns, the product sum_b conj(G^ab) Z^b and the inverse: Q^a, in
 // place of Z for a single phase (G is even then: a real spectrum).
 template <bool MULTI>
-__global__ void __launch_bounds__(SEP_THREADS, MULTI ? 1 : 2)
+__global__ void __launch_bounds__(SEP_THREADS, MULTI ? 1 : COLOCC)
 sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
-    if (!enter<true>(tb, items, nitem, bk)) return;
+    if (!enter<true>(tb, items, nitem, bk, sep_smem, axis_x)) return;
     const SepLevel& lv = bk.lv;
+    float2* sm = sep_smem;
     const SepTier& t = tb.tier[bk.tier];
     int x0, y;
     const ColGroup g = last_axis(lv, bk.block, x0, y);
     const SepAxis& ax = last_ax(lv);
-    const float norm = 1.0f / (float)lv.N;       // of the unnormalised inverse
-    fill_twiddles(sep_smem, g.n);
+    // of the unnormalised inverse; sep_desc's rows still lack the loss' factor
+    const float norm = (lv.fuse && lv.sc != nullptr ? lv.sc->gscale : 1.f) / (float)lv.N;
     if (ax.fast && (!MULTI || lv.phases <= SEP_FAST_PHASES)) {
-        __syncthreads();
         for_pow2(ax.fast, [&](auto cc) {
             constexpr int N = decltype(cc)::value, T = N / 8;
             constexpr int EX = p2_exchanges(N), PAR1 = EX & 1;
@@ -1442,10 +1612,14 @@ sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__
                     for (int e = 0; e < 8; ++e) v[e] = nx[e];
                     const int q = p + c.slots;
                     if (p0 + c.slots < t.npair) load8<N>(lv.Z + (int64_t)q * lv.N, g, c, q < t.npair, nx);
-                    p2_fft<N, false, 0>(v, c.ln);
+                    if (!lv.keep) {              // else sep_power left the spectra
+                        p2_fft<N, false, 0>(v, c.ln);
+                        if (PAR1) __syncthreads();
+                    }
 #pragma unroll
                     for (int e = 0; e < 8; ++e) v[e] = make_float2(gr[e] * v[e].y, gr[e] * v[e].x);
-                    p2_fft<N, false, PAR1>(v, c.ln);
+                    p2_fft<N, false, 0>(v, c.ln);
+                    if (PAR1) __syncthreads();
                 } else {
                     float2 acc[8];
 #pragma unroll
@@ -1473,7 +1647,7 @@ sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__
         return;
     }
     const int pitch = sep_pitch(g.n, g.L), sh = 31 - __clz(g.L), total = g.L * g.n;
-    const SepShared s = sep_shared(g.n, g.L, pitch);
+    const SepShared s = sep_shared(sm, g.n, g.L, pitch);
     float2* gs = s.b + g.L * pitch;              // the spectra of every b, own points
     auto own = [&](auto f) {
 #pragma unroll
@@ -1499,7 +1673,9 @@ sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__
         for (int b = 0; b < lv.phases; ++b) {
             __syncthreads();
             load_cols(lv.Z + ((int64_t)b * lv.maxPairs + p) * lv.N, g, pitch, s.a);
-            const float2* r = transform(ax, s.a, s.b, s.tw, g.L, pitch);
+            const float2* r = s.a;
+            if (MULTI || !lv.keep) r = transform(ax, s.a, s.b, s.tw, g.L, pitch);
+            else __syncthreads();
             own([&](int q, int e, int at) {
                 const float2 v = r[at], c = gs[b * total + e];
                 acc[q].x = fmaf(c.x, v.x, fmaf(-c.y, v.y, acc[q].x));
@@ -1521,73 +1697,84 @@ sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__
 
 // item: (level, phase a); blocks: groups of rows.  Inverse along x of every feature pair and
 // g(y) = sum_k s_k p_k'(M_y) Q_k(y), the slots' shares added in a fixed order.
-__global__ void __launch_bounds__(SEP_THREADS, 1) sep_grad_kernel(const __grid_constant__ SepTables tb,
-                                                                  const SepItem* __restrict__ items, int nitem) {
+__global__ void __launch_bounds__(SEP_ROW_THREADS, 3) sep_grad_kernel(const __grid_constant__ SepTables tb,
+                                                                      const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
-    __shared__ __align__(16) float2 cf[SEP_MAX_DEG * SEP_STRIDE];
-    if (!enter<true>(tb, items, nitem, bk)) return;
+    if (!enter<true>(tb, items, nitem, bk, sep_smem, axis_x)) return;
     const SepLevel& lv = bk.lv;
+    float2* sm = sep_smem;
     const SepTier& t = tb.tier[bk.tier];
-    load_coef<true>(tb, t, cf);
+    const float2* __restrict__ cf = tier_coef<true>(tb, t);
     const int rowsN = lv.n0 * lv.n1, n = lv.n2;
     const int row0 = bk.block * lv.rowsF, rows = min(lv.rowsF, rowsN - row0);
     const float* __restrict__ field = lv.field + (int64_t)bk.a * lv.N + (int64_t)row0 * n;
     const float2* __restrict__ Q = lv.Q + (int64_t)bk.a * lv.maxPairs * lv.N + (int64_t)row0 * n;
     float* __restrict__ part = lv.part + (int64_t)bk.a * lv.N + (int64_t)row0 * n;
-    fill_twiddles(sep_smem, n);
     __syncthreads();
     if (lv.ax[2].fast) {
         for_pow2(lv.ax[2].fast, [&](auto cc) {
             constexpr int N = decltype(cc)::value;
             using S = RowShape<N>;
-            const int line = threadIdx.x / S::T, p = line % S::SLOTS, row = line / S::SLOTS;
-            const Line<N> ln = row_line<N>(line, threadIdx.x % S::T, S::LINES);
-            const bool in = row < rows;
-            float g[8];
+            const int line = threadIdx.x / S::T, p = line % S::SLOTS, r0 = line / S::SLOTS;
+            const Line<N> ln = row_line<N>(sm, line, threadIdx.x % S::T, S::LINES);
+            float* red = reinterpret_cast<float*>(sm + N);      // over the line buffers: [slot][row][i]
+            for (int rb = 0; rb < lv.rowsF; rb += S::ROWS) {
+                const int row = rb + r0;
+                const bool in = row < rows;
+                float g[8];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) g[e] = 0.f;
-            for (int p0 = 0; p0 < t.npair; p0 += S::SLOTS) {
-                const bool live = in && p0 + p < t.npair;
-                float2 v[8];
-                const float2* src = Q + (int64_t)(p0 + p) * lv.N + row * N + ln.t;
+                for (int e = 0; e < 8; ++e) g[e] = 0.f;
+                for (int p0 = 0; p0 < t.npair; p0 += S::SLOTS) {
+                    const bool live = in && p0 + p < t.npair;
+                    float2 v[8];
+                    const float2* src = Q + (int64_t)(p0 + p) * lv.N + row * N + ln.t;
 #pragma unroll
-                for (int e = 0; e < 8; ++e) v[e] = live ? swapf(src[e * S::T]) : make_float2(0.f, 0.f);
-                p2_fft<N, S::WARP, 0>(v, ln);
-                if (live) {
-                    const float sg = p0 + p < t.npos ? t.inv_half : -t.inv_half;
-                    // four positions at a time: the series' state of eight does not fit the registers
+                    for (int e = 0; e < 8; ++e) v[e] = live ? swapf(src[e * S::T]) : make_float2(0.f, 0.f);
+                    p2_fft<N, S::WARP, 0>(v, ln);
+                    if (live) {
+                        const float sg = p0 + p < t.npos ? t.inv_half : -t.inv_half;
+                        // four positions at a time: the series' state of eight does not fit the registers
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        float x[4];
-                        float2 f[4];
+                        for (int h = 0; h < 2; ++h) {
+                            float x[4];
+                            float2 f[4];
 #pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            x[e] = (field[row * N + ln.t + (4 * h + e) * S::T] - t.mid) * t.inv_half;
-                        eval_features<true, 4>(cf + p0 + p, t.deg, x, f);
+                            for (int e = 0; e < 4; ++e)
+                                x[e] = (field[row * N + ln.t + (4 * h + e) * S::T] - t.mid) * t.inv_half;
+                            eval_features<true, 4>(cf + p0 + p, t.npair, t.deg, x, f);
 #pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            g[4 * h + e] = fmaf(sg, fmaf(f[e].x, v[4 * h + e].y, f[e].y * v[4 * h + e].x), g[4 * h + e]);
+                            for (int e = 0; e < 4; ++e)
+                                g[4 * h + e] =
+                                    fmaf(sg, fmaf(f[e].x, v[4 * h + e].y, f[e].y * v[4 * h + e].x), g[4 * h + e]);
+                        }
                     }
+                    if (p2_exchanges(N) & 1) line_sync<S::WARP>();
                 }
-                line_sync<S::WARP>();
-            }
-            // sum over the slots: red[slot][row][i]
-            __syncthreads();
-            float* red = reinterpret_cast<float*>(sep_smem + N);
+                if (S::SLOTS == 1) {
+                    if (in) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) red[(p * S::ROWS + row) * N + ln.t + e * S::T] = g[e];
-            __syncthreads();
-            for (int o = threadIdx.x; o < rows * N; o += SEP_THREADS) {
-                float s = red[o];
+                        for (int e = 0; e < 8; ++e) part[row * N + ln.t + e * S::T] = g[e];
+                    }
+                    continue;
+                }
+                __syncthreads();
 #pragma unroll
-                for (int k = 1; k < S::SLOTS; ++k) s += red[k * S::ROWS * N + o];
-                part[o] = s;
+                for (int e = 0; e < 8; ++e) red[(p * S::ROWS + r0) * N + ln.t + e * S::T] = g[e];
+                __syncthreads();
+                const int here = min(S::ROWS, rows - rb) * N;
+                for (int o = threadIdx.x; o < here; o += SEP_ROW_THREADS) {
+                    float s = red[o];
+#pragma unroll
+                    for (int k = 1; k < S::SLOTS; ++k) s += red[k * S::ROWS * N + o];
+                    part[rb * N + o] = s;
+                }
+                __syncthreads();
             }
         });
         return;
     }
     const int pitch = spad(n - 1) + 2;
-    const SepShared s = sep_shared(n, lv.rowsF * SEP_SLOTS, pitch);
+    const SepShared s = sep_shared(sm, n, lv.rowsF * SEP_SLOTS, pitch);
     const float inv_n = 1.0f / (float)n;
     float g[SEP_OWN];
 #pragma unroll
@@ -1603,13 +1790,13 @@ __global__ void __launch_bounds__(SEP_THREADS, 1) sep_grad_kernel(const __grid_c
         const float2* r = transform(lv.ax[2], s.a, s.b, s.tw, rows * nc, pitch);
 #pragma unroll
         for (int q = 0; q < SEP_OWN; ++q) {
-            const int e = threadIdx.x + q * SEP_THREADS;
+            const int e = threadIdx.x + q * SEP_ROW_THREADS;
             if (e < rows * n) {
                 const int l = fdiv(e, inv_n), i = e - l * n;
                 const float x[1] = {(field[e] - t.mid) * t.inv_half};
                 for (int c = 0; c < nc; ++c) {
                     float2 f[1];
-                    eval_features<true, 1>(cf + p0 + c, t.deg, x, f);
+                    eval_features<true, 1>(cf + p0 + c, t.npair, t.deg, x, f);
                     const float2 v = r[(l * nc + c) * pitch + spad(i)];
                     g[q] = fmaf(p0 + c < t.npos ? t.inv_half : -t.inv_half, fmaf(f[0].x, v.y, f[0].y * v.x), g[q]);
                 }
@@ -1618,7 +1805,7 @@ __global__ void __launch_bounds__(SEP_THREADS, 1) sep_grad_kernel(const __grid_c
     }
 #pragma unroll
     for (int q = 0; q < SEP_OWN; ++q) {
-        const int e = threadIdx.x + q * SEP_THREADS;
+        const int e = threadIdx.x + q * SEP_ROW_THREADS;
         if (e < rows * n) part[e] = g[q];
     }
 }
@@ -1628,21 +1815,22 @@ __global__ void __launch_bounds__(SEP_THREADS, 1) sep_grad_kernel(const __grid_c
 namespace {
 size_t bytes_of(int n, int lines, int pitch) { return (size_t)(((n + 1) & ~1) + 2 * lines * pitch) * sizeof(float2); }
 // power-of-two rows: the block's whole line capacity (row_pitch)
-size_t fast_row_bytes(int n) {
+size_t fast_row_bytes(int n, int threads) {
     int p = n - 1 + (n - 1) / 16 + 1;
     const int want = n >= 128 ? 0 : n / 8;
     while (p % 16 != want) ++p;
-    return bytes_of(n, SEP_BLOCK_PTS / n, p);
+    return bytes_of(n, 8 * threads / n, p);
 }
 }  // namespace
 
 size_t sep_smem_feat(const SepLevel& lv) {
     const int n = lv.n2;
-    return lv.ax[2].fast ? fast_row_bytes(n) : bytes_of(n, lv.rowsF * SEP_SLOTS, n - 1 + ((n - 1) >> 4) + 2);
+    return lv.ax[2].fast ? fast_row_bytes(n, SEP_ROW_THREADS)
+                         : bytes_of(n, lv.rowsF * SEP_SLOTS, n - 1 + ((n - 1) >> 4) + 2);
 }
 size_t sep_smem_window(const SepLevel& lv) {
     const int n = lv.n2;
-    return lv.ax[2].fast ? fast_row_bytes(n) : bytes_of(n, lv.rowsW, n - 1 + ((n - 1) >> 4) + 2);
+    return lv.ax[2].fast ? fast_row_bytes(n, SEP_THREADS) : bytes_of(n, lv.rowsW, n - 1 + ((n - 1) >> 4) + 2);
 }
 size_t sep_smem_y(const SepLevel& lv) {
     const int lines = lv.ax[1].fast ? SEP_BLOCK_PTS / lv.n1 : lv.colsY;
@@ -1666,19 +1854,18 @@ void launch_sep(SepKernel k, const SepTables& tb, const SepItem* items, int nite
     const unsigned b = (unsigned)blocks;
     constexpr int T = SEP_THREADS;
     switch (k) {
-        case SEP_RANGE: sep_range_kernel<<<b, 256, 0, s>>>(tb, items, nitem); break;
-        case SEP_FEAT: sep_feat_kernel<<<b, T, smem, s>>>(tb, items, nitem); break;
-        case SEP_FFT_Y: sep_fft_y_kernel<false><<<b, T, smem, s>>>(tb, items, nitem); break;
-        case SEP_POWER: sep_power_kernel<false><<<b, T, smem, s>>>(tb, items, nitem); break;
-        case SEP_POWER_PH: sep_power_kernel<true><<<b, T, smem, s>>>(tb, items, nitem); break;
-        case SEP_INV_Y: sep_win_y_kernel<true><<<b, T, smem, s>>>(tb, items, nitem); break;
-        case SEP_DESC: sep_desc_kernel<<<b, T, smem, s>>>(tb, items, nitem); break;
-        case SEP_GX: sep_gx_kernel<<<b, T, smem, s>>>(tb, items, nitem); break;
-        case SEP_GY: sep_win_y_kernel<false><<<b, T, smem, s>>>(tb, items, nitem); break;
-        case SEP_MUL: sep_mul_kernel<false><<<b, T, smem, s>>>(tb, items, nitem); break;
-        case SEP_MUL_PH: sep_mul_kernel<true><<<b, T, smem, s>>>(tb, items, nitem); break;
-        case SEP_IFFT_Y: sep_fft_y_kernel<true><<<b, T, smem, s>>>(tb, items, nitem); break;
-        case SEP_GRAD: sep_grad_kernel<<<b, T, smem, s>>>(tb, items, nitem); break;
+        case SEP_FEAT: launch_dep(sep_feat_kernel, b, SEP_ROW_THREADS, smem, s, tb, items, nitem); break;
+        case SEP_FFT_Y: launch_dep(sep_fft_y_kernel<false>, b, T, smem, s, tb, items, nitem); break;
+        case SEP_POWER: launch_dep(sep_power_kernel<false>, b, T, smem, s, tb, items, nitem); break;
+        case SEP_POWER_PH: launch_dep(sep_power_kernel<true>, b, T, smem, s, tb, items, nitem); break;
+        case SEP_INV_Y: launch_dep(sep_win_y_kernel<true>, b, T, smem, s, tb, items, nitem); break;
+        case SEP_DESC: launch_dep(sep_desc_kernel, b, T, smem, s, tb, items, nitem); break;
+        case SEP_GX: launch_dep(sep_gx_kernel, b, T, smem, s, tb, items, nitem); break;
+        case SEP_GY: launch_dep(sep_win_y_kernel<false>, b, T, smem, s, tb, items, nitem); break;
+        case SEP_MUL: launch_dep(sep_mul_kernel<false>, b, T, smem, s, tb, items, nitem); break;
+        case SEP_MUL_PH: launch_dep(sep_mul_kernel<true>, b, T, smem, s, tb, items, nitem); break;
+        case SEP_IFFT_Y: launch_dep(sep_fft_y_kernel<true>, b, T, smem, s, tb, items, nitem); break;
+        case SEP_GRAD: launch_dep(sep_grad_kernel, b, SEP_ROW_THREADS, smem, s, tb, items, nitem); break;
         default: break;
     }
 }
