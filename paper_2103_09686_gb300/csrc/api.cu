@@ -155,8 +155,13 @@ struct Plan {
     std::shared_ptr<const SepBasis> basis;
     int sep_tiers = 0, sep_pairs = 0;   // tiers worth running, feature pairs of the widest of them
     size_t o_tier = 0, o_tiers = 0, o_z[MAX_LEVELS] = {}, o_q[MAX_LEVELS] = {}, o_u[MAX_LEVELS] = {},
-           o_v[MAX_LEVELS] = {}, o_sdc[MAX_LEVELS] = {}, o_spart[MAX_LEVELS] = {}, o_excess = 0, o_sums = 0;
-    int sum_off[MAX_LEVELS] = {}, nsum = 0;   // residual sums of the sep_desc blocks per level
+           o_v[MAX_LEVELS] = {}, o_sdc[MAX_LEVELS] = {}, o_spart[MAX_LEVELS] = {};
+    // block sums of the loss, left by the descriptor kernels (two-point descriptor without FFT levels)
+    bool sums = false;
+    size_t o_excess = 0, o_sums = 0;
+    int red_off[MAX_LEVELS] = {}, nred = 0;   // fwd_reduce blocks: first of a level, all
+    int sep_off[MAX_LEVELS] = {}, nsep = 0;   // sep_desc blocks
+    int nexc = 0;                             // field blocks of fwd_reduce (direct path)
     size_t bytes = 0;
 };
 
@@ -188,7 +193,7 @@ size_t table_bound(const Plan& pl) {
     return sep + (size_t)levels *
                (pp * (sizeof(FwdSeg) + sizeof(RedSeg) + sizeof(GSeg) + sizeof(AdjSeg)) +
                 phases * sizeof(RestrictSeg) + 2 * sizeof(TildeSeg)) +
-           sizeof(PrepSeg) + sizeof(PenSeg) + sizeof(LossSeg) + phases * sizeof(FinalSeg) + sizeof(InitSeg);
+           sizeof(PrepSeg) + sizeof(PenSeg) + 2 * sizeof(LossSeg) + phases * sizeof(FinalSeg);
 }
 size_t table_slack(bool sep) { return (size_t)(16 + MAX_LEVELS + (sep ? 8 + SEP_KERNELS : 0)) * 16 + 256; }
 
@@ -519,23 +524,37 @@ dmcr_status validate_and_plan(const dmcr_params* p, Plan& pl) {
     }
     // workspace layout
     size_t o = 0;
+    // the scalars and the segment tables behind them are written by one upload per call
+    pl.o_scal = o; o = align_up(o + sizeof(Scalars));
     pl.tab_bytes = align_up(table_bound(pl) + table_slack(pl.sep));
     pl.o_tab = o; o += pl.tab_bytes;
-    pl.o_scal = o; o = align_up(o + sizeof(Scalars));
     pl.o_pen = o; o = align_up(o + 3 * NPEN_BLOCKS * sizeof(double));
     pl.o_desc = o; o = align_up(o + (size_t)pl.Ktot * sizeof(float));
     pl.o_tsum = o; o = align_up(o + (size_t)MAX_LEVELS * sizeof(float));
     if (pl.sep) {
         pl.o_tier = o; o = align_up(o + sizeof(int));
         pl.o_tiers = o; o = align_up(o + PREP_BLOCKS * sizeof(int));
-        pl.o_excess = o; o = align_up(o + PREP_BLOCKS * sizeof(float4));
+    }
+    pl.sums = pl.desc_kind == DMCR_DESC_S2 && !pl.any_fft;
+    if (pl.sums) {
+        const int64_t pp = (int64_t)pl.phases * pl.phases, Nall = pl.N1 * pl.phases;
+        int64_t nr = 0, ns = 0;
         for (int l = 0; l < pl.levels; ++l) {
-            SepLevel lv;
-            sep_shape(pl.g[l], pl.phases, pl.sep_pairs, lv);
-            pl.sum_off[l] = pl.nsum;
-            pl.nsum += (int)ceil_div(sep_v_rows(pl.g[l]), lv.rowsW);
+            pl.red_off[l] = (int)nr;
+            nr += pp * ceil_div(pl.g[l].Khalf, RED_K);
+            pl.sep_off[l] = (int)ns;
+            if (pl.sep) {
+                SepLevel lv;
+                sep_shape(pl.g[l], pl.phases, pl.sep_pairs, lv);
+                ns += pp * ceil_div(sep_v_rows(pl.g[l]), lv.rowsW);
+            }
         }
-        pl.o_sums = o; o = align_up(o + (size_t)pl.nsum * sizeof(float4));
+        if (nr > INT32_MAX || ns > INT32_MAX) return fail(DMCR_EINVAL, "window too large: the descriptor has too many blocks");
+        pl.nred = (int)nr;
+        pl.nsep = (int)ns;
+        pl.nexc = (int)std::min<int64_t>(NPEN_BLOCKS, ceil_div(Nall, 2048));
+        pl.o_excess = o; o = align_up(o + (size_t)std::max(pl.nexc, PREP_BLOCKS) * sizeof(float4));
+        pl.o_sums = o; o = align_up(o + (size_t)std::max(nr, ns) * sizeof(float4));
     }
     for (int l = 0; l < pl.levels; ++l) {
         const LevelGeom& g = pl.g[l];
@@ -559,8 +578,7 @@ dmcr_status validate_and_plan(const dmcr_params* p, Plan& pl) {
             pl.o_amax[l] = o; o = align_up(o + 2 * sizeof(float));
         } else if (pl.sep) {
             // gradient of the level and window means, then the buffers of the path that runs:
-            // spectra (separable) or partials and coefficients (direct, for fields outside the
-            // separable ranges) -- a call uses one of the two
+            // spectra (separable) or partials (direct, for fields outside the separable ranges) -- a call uses one of the two
             const size_t pp = ph * ph;
             pl.o_spart[l] = o; o = align_up(o + ph * g.N * sizeof(float));
             pl.o_sdc[l] = o; o = align_up(o + pp * sizeof(double));
@@ -572,15 +590,13 @@ dmcr_status validate_and_plan(const dmcr_params* p, Plan& pl) {
             pl.o_v[l] = o; o = align_up(o + pp * sep_v_rows(g) * g.n[2] * sizeof(float2));
             size_t d = start;
             pl.o_fwd[l] = d; d = align_up(d + ph * ph * g.fwdTiles * g.Khalf * sizeof(float));
-            pl.o_gd[l] = d; d = align_up(d + ph * ph * gd_floats(g) * sizeof(float));
             pl.o_adj[l] = d; d = align_up(d + ph * ph * g.nChunks * g.N * sizeof(float));
             o = std::max(o, d);
             continue;
         } else {
             pl.o_fwd[l] = o; o = align_up(o + ph * ph * g.fwdTiles * g.Khalf * sizeof(float));
         }
-        if (pl.desc_kind != DMCR_DESC_S3)
-            pl.o_gd[l] = o, o = align_up(o + ph * ph * gd_floats(g) * sizeof(float));
+        if (g.fft) pl.o_gd[l] = o, o = align_up(o + ph * ph * gd_floats(g) * sizeof(float));
         pl.o_adj[l] = o; o = align_up(o + ph * ph * g.nChunks * g.N * sizeof(float));
     }
     pl.bytes = o;
@@ -616,12 +632,13 @@ dmcr_status check_ws(const Plan& pl, void* ws, size_t ws_bytes) {
 //
 // Every entry point runs the same fused phases over a set of instances (one for the plain
 // calls, many for the batched ones).  The host fills one table buffer with the segment
-// arrays of every phase, writes it to the table region with blob_kernel (stream ordered,
-// no host synchronisation), then launches one kernel per phase:
-//   init -> restrict (per level index) -> corr_fwd -> fwd_reduce -> penalty -> loss
-//        -> gcoef -> corr_adj -> final (gradient assembly, optional Adam step).
+// arrays of every phase behind the instances' initial scalars, writes it to the upload region
+// with blob_kernel (stream ordered, no host synchronisation), then launches one kernel per phase:
+//   upload (scalars, tables) -> prep (pyramid, value range) -> corr_fwd -> fwd_reduce (and the
+//   loss, finished by its last block) -> corr_adj -> final (gradient assembly, optional Adam
+//   step); separable instances run the sep_* kernels instead (sep.cu), FFT and three-point
+//   ones theirs, with the statistics and the loss in two further launches.
 enum : unsigned {
-    F_INIT = 1u,     // reset the per-instance scalars (Adam step counters)
     F_FWD = 2u,      // pyramid + descriptor
     F_LOSS = 4u,     // penalty + loss
     F_BACK = 8u,     // adjoint coefficients + adjoint + gradient assembly
@@ -645,7 +662,7 @@ struct Inst {
     float* history = nullptr;
     bool use_done = false;         // kernels skip the instance once its done flag is set
     bool round_eval = false;       // reconstruction: evaluate the rounded result once more
-    int64_t step = 0;              // F_INIT: Adam steps taken before this call
+    int64_t step = 0;              // Adam steps taken before this call
     const float* lv[MAX_LEVELS] = {};
 };
 
@@ -660,7 +677,8 @@ struct TableBuf {
 };
 
 struct Prepared {
-    char* tab = nullptr;
+    char* tab = nullptr;           // device region: `nscal` Scalars, then the tables
+    size_t scal_bytes = 0;
     TableBuf tb;
     ThreshConst tc{};
     unsigned flags = 0;
@@ -671,14 +689,14 @@ struct Prepared {
     };
     std::vector<R> restricts;
     R fwd{0, 0, 0}, red{0, 0, 0}, pen{0, 0, 0}, loss{0, 0, 0}, gco{0, 0, 0}, adj{0, 0, 0}, fin{0, 0, 0},
-        fin_small{0, 0, 0}, init{0, 0, 0}, tmap{0, 0, 0}, tsum{0, 0, 0}, prep{0, 0, 0};
+        fin_small{0, 0, 0}, tmap{0, 0, 0}, tsum{0, 0, 0}, prep{0, 0, 0};
     size_t smem_fwd = 0, smem_adj = 0;
     // separable path, and the direct launches of its instances (run only where their gate opens)
     R sep[SEP_KERNELS] = {};
     size_t sep_smem[SEP_KERNELS] = {};
     SepTables sept{};
     size_t o_sep_level = 0, o_sep_coef = 0;
-    R gfwd{0, 0, 0}, gred{0, 0, 0}, ggco{0, 0, 0}, gadj{0, 0, 0};
+    R gfwd{0, 0, 0}, gred{0, 0, 0}, gadj{0, 0, 0};
     size_t smem_gfwd = 0, smem_gadj = 0;
     struct FftJob {
         LevelGeom g;
@@ -761,7 +779,7 @@ int prep_blocks(const Plan& pl) {
     return (int)std::min<int64_t>(PREP_BLOCKS, tiles);
 }
 
-// the separable kernels leave the loss' sums and the rows of G as they compute the descriptor
+// sep_desc goes straight on to the rows of G
 bool fused_loss(const Plan& pl, unsigned flags) {
     return pl.sep && pl.phases == 1 && pl.desc_kind == DMCR_DESC_S2 && (flags & F_FWD) && (flags & F_LOSS) &&
            (flags & F_BACK);
@@ -769,7 +787,7 @@ bool fused_loss(const Plan& pl, unsigned flags) {
 
 // Tables of the separable path: one SepLevel per (instance, level), one block range per
 // kernel and phase (pair), the basis' coefficients.
-void prepare_sep(const std::vector<Inst>& in, unsigned flags, Prepared& P) {
+void prepare_sep(const std::vector<Inst>& in, unsigned flags, const std::vector<const LossSeg*>& loss, Prepared& P) {
     std::vector<SepLevel> levels;
     std::vector<SepItem> items[SEP_KERNELS];
     const SepBasis* basis = nullptr;
@@ -787,7 +805,8 @@ void prepare_sep(const std::vector<Inst>& in, unsigned flags, Prepared& P) {
         P.sep_smem[k] = std::max(P.sep_smem[k], smem);
         items[k].push_back(it);
     };
-    for (const Inst& x : in) {
+    for (size_t xi = 0; xi < in.size(); ++xi) {
+        const Inst& x = in[xi];
         const Plan& pl = *x.pl;
         if (!pl.sep) continue;
         basis = pl.basis.get();
@@ -805,12 +824,16 @@ void prepare_sep(const std::vector<Inst>& in, unsigned flags, Prepared& P) {
             lv.tier = reinterpret_cast<int*>(x.ws + pl.o_tier);
             lv.tiers = reinterpret_cast<int*>(x.ws + pl.o_tiers);
             lv.ntiers = prep_blocks(pl);
-            lv.sums = reinterpret_cast<float4*>(x.ws + pl.o_sums) + pl.sum_off[l];
+            lv.loss = loss[xi];
+            lv.sums = reinterpret_cast<float4*>(x.ws + pl.o_sums);
+            lv.sumStart = pl.sep_off[l];
+            lv.arrive = pl.nsep;
             lv.fuse = fused_loss(pl, flags);
             lv.first = l == 0;
             lv.keep = pl.phases == 1 && (flags & F_FWD) && (flags & F_BACK);
             lv.desc = x.desc + pl.off[l];
             lv.scaleD = (double)pl.w[l] / ((double)g.N * (double)g.N);
+            if (flags & F_LOSS) lv.sub = x.target + pl.off[l];
             if (flags & F_BACK) {
                 lv.src = vjp ? x.target + pl.off[l] : x.desc + pl.off[l];
                 lv.sub = vjp ? nullptr : x.target + pl.off[l];
@@ -869,10 +892,28 @@ void prepare_sep(const std::vector<Inst>& in, unsigned flags, Prepared& P) {
     }
 }
 
-// Build every table of the requested phases; `tab`/`cap` is the device table region.
-dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap, Prepared& P) {
+// The scalars of an instance at the start of a call.
+Scalars initial_scalars(int64_t step, float beta1, float beta2) {
+    Scalars s;
+    memset(&s, 0, sizeof s);
+    s.adam_step = step;
+    s.b1t = pow((double)beta1, (double)step);
+    s.b2t = pow((double)beta2, (double)step);
+    return s;
+}
+
+// Build every table of the requested phases.  `tab` is the device region the upload writes
+// (`nscal` Scalars, padded to the alignment, then the tables), `cap` its size.
+dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap, int nscal, Prepared& P) {
     P.tab = tab;
     P.flags = flags;
+    P.scal_bytes = align_up((size_t)nscal * sizeof(Scalars));
+    P.tb.h.assign(P.scal_bytes, 0);
+    for (const Inst& x : in)
+        if (nscal > 0) {
+            const Scalars sc = initial_scalars(x.step, x.beta1, x.beta2);
+            memcpy(P.tb.h.data() + (reinterpret_cast<char*>(x.sc) - tab), &sc, sizeof sc);
+        }
     P.tc = in[0].pl->tc;
     int maxL = 0;
     for (Inst& x : in) {
@@ -890,11 +931,34 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
             if (x.pl->any_fft && !x.pl->tc.identity)
                 return fail(DMCR_ENOTSUP, "the FFT path of the soft threshold is exact for binary fields only: "
                                           "descriptor calls only (characterise targets with it)");
-    if (flags & F_INIT) {
-        std::vector<InitSeg> v;
-        for (const Inst& x : in)
-            v.push_back({x.sc, x.step, pow((double)x.beta1, (double)x.step), pow((double)x.beta2, (double)x.step)});
-        P.init = {push(P.tb, v), (int)v.size(), (int64_t)v.size()};
+    // losses finished by the descriptor kernels: one LossSeg per path of the instance
+    std::vector<const LossSeg*> loss_red(in.size(), nullptr), loss_sep(in.size(), nullptr);
+    if (flags & F_LOSS) {
+        std::vector<LossSeg> v;
+        std::vector<std::pair<size_t, bool>> who;
+        for (size_t i = 0; i < in.size(); ++i) {
+            const Inst& x = in[i];
+            const Plan& pl = *x.pl;
+            if (!pl.sums) continue;
+            LossSeg ls{};
+            ls.lp = x.lp;
+            ls.sums = reinterpret_cast<const float4*>(x.ws + pl.o_sums);
+            ls.excess = reinterpret_cast<const float4*>(x.ws + pl.o_excess);
+            ls.nsum = pl.nred;
+            ls.nexc = !x.lp.bc_on ? 0 : (pl.sep ? prep_blocks(pl) : pl.nexc);
+            ls.sc = x.sc;
+            ls.loss_out = x.loss_out;
+            ls.history = x.history;
+            v.push_back(ls);
+            who.push_back({i, false});
+            if (!pl.sep) continue;
+            ls.nsum = pl.nsep;
+            v.push_back(ls);
+            who.push_back({i, true});
+        }
+        const size_t off = push(P.tb, v);
+        for (size_t k = 0; k < who.size(); ++k)
+            (who[k].second ? loss_sep : loss_red)[who[k].first] = P.at<LossSeg>(off) + k;
     }
     if (need_pyr) {
         // levels the tiles of prep_kernel determine, then one restriction per deeper level
@@ -915,7 +979,7 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
                 p.tiers = reinterpret_cast<int*>(x.ws + pl.o_tiers);
                 p.ntier = pl.sep_tiers;
                 for (int t = 0; t < pl.sep_tiers; ++t) p.lo[t] = pl.basis->tier[t].lo, p.hi[t] = pl.basis->tier[t].hi;
-                if (fused_loss(pl, flags) && x.lp.bc_on) p.excess = reinterpret_cast<float4*>(x.ws + pl.o_excess);
+                if ((flags & F_LOSS) && pl.sums && x.lp.bc_on) p.excess = reinterpret_cast<float4*>(x.ws + pl.o_excess);
             }
             p.done = x.use_done ? &x.sc->done : nullptr;
             p.blockStart = pb;
@@ -952,7 +1016,11 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
         std::vector<Item> plain, gated;
         std::vector<RedSeg> rplain, rgated;
         int64_t rplain_b = 0, rgated_b = 0;
-        for (const Inst& x : in)
+        for (size_t xi = 0; xi < in.size(); ++xi) {
+            const Inst& x = in[xi];
+            const LossSeg* loss = loss_red[xi];
+            // the box excess of a separable instance comes with its value range (prep_kernel)
+            const int nexc = loss != nullptr && !x.pl->sep && x.lp.bc_on ? x.pl->nexc : 0;
             for (int l = 0; l < x.pl->levels; ++l) {
                 const LevelGeom& g = x.pl->g[l];
                 // an instance on the separable path keeps the direct kernels for fields outside its ranges
@@ -991,12 +1059,27 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
                         r.done = it.f.done;
                         r.gate = gate;
                         r.scale = (float)((double)x.pl->w[l] / (double)g.N);
+                        const int64_t own = ceil_div(g.Khalf, RED_K);
+                        if (loss != nullptr) {
+                            r.loss = loss;
+                            r.target = x.target + x.pl->off[l] + blk * g.Khalf;
+                            r.sums = reinterpret_cast<float4*>(x.ws + x.pl->o_sums) + x.pl->red_off[l] + blk * own;
+                            r.arrive = x.pl->nred + nexc;
+                            if (l == 0 && blk == 0 && nexc > 0) {
+                                r.nexc = nexc;
+                                r.excess = reinterpret_cast<float4*>(x.ws + x.pl->o_excess);
+                                r.field = x.field;
+                                r.fieldN = x.pl->N1 * x.pl->phases;
+                                r.excChunk = ceil_div(r.fieldN, nexc);
+                            }
+                        }
                         r.blockStart = rb;
-                        rb += ceil_div(g.Khalf, RED_K);
+                        rb += own + r.nexc;
                         rv.push_back(r);
                     }
                 smem = std::max(smem, fwd_smem_bytes(g));
             }
+        }
         // heaviest blocks first: the tail of the launch is made of the light ones
         auto table = [&](std::vector<Item>& items) {
             std::stable_sort(items.begin(), items.end(), [](const Item& a, const Item& b) { return a.work > b.work; });
@@ -1036,25 +1119,15 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
         std::vector<LossSeg> lvv;
         int maxblk = 0;
         for (const Inst& x : in) {
+            if (x.pl->sums) continue;      // its descriptor kernels finish the loss
             double* pen = reinterpret_cast<double*>(x.ws + x.pl->o_pen);
             const int64_t Nall = x.pl->N1 * x.pl->phases;
             const int nblk = stats_blocks(x.pl->Ktot, x.lp.bc_on ? Nall : 0);
             maxblk = std::max(maxblk, nblk);
-            const bool fuse = fused_loss(*x.pl, flags);
-            const int* gate = fuse ? reinterpret_cast<const int*>(x.ws + x.pl->o_tier) : nullptr;
-            pv.push_back({gate, x.lp.bc_on ? x.field : nullptr, Nall, x.desc, x.target, x.pl->Ktot, pen,
+            pv.push_back({x.lp.bc_on ? x.field : nullptr, Nall, x.desc, x.target, x.pl->Ktot, pen,
                           x.use_done ? &x.sc->done : nullptr, nblk});
             LossSeg ls{};
-            if (fuse) {
-                ls.tier = gate;
-                ls.sums = reinterpret_cast<const float4*>(x.ws + x.pl->o_sums);
-                ls.nsum = x.pl->nsum;
-                ls.excess = reinterpret_cast<const float4*>(x.ws + x.pl->o_excess);
-                ls.nexc = x.lp.bc_on ? prep_blocks(*x.pl) : 0;
-            }
             ls.lp = x.lp;
-            ls.desc = x.desc;
-            ls.target = x.target;
             ls.pen = pen;
             ls.nblk = nblk;
             ls.sc = x.sc;
@@ -1071,20 +1144,18 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
             int64_t work, blocks;
         };
         std::vector<Item> plain, gated;
-        std::vector<GSeg> gplain, ggated;
+        std::vector<GSeg> gv;
         std::vector<TildeSeg> tsv;
         // gradient assembly: a small field has few positions for many chunk partials and its
         // segments go to the launch with FIN_SUB threads per position; the others to the one
         // with one thread per position
         std::vector<FinalSeg> fv, fvs;
-        int64_t gplain_b = 0, ggated_b = 0, fb = 0, fbs = 0;
+        int64_t gb = 0, fb = 0, fbs = 0;
         const bool vjp = !(flags & F_LOSS);
         for (const Inst& x : in) {
             const int nph = x.pl->phases;
             const int* gate = x.pl->sep ? reinterpret_cast<const int*>(x.ws + x.pl->o_tier) : nullptr;
             std::vector<Item>& items = gate ? gated : plain;
-            std::vector<GSeg>& gv = gate ? ggated : gplain;
-            int64_t& gb = gate ? ggated_b : gplain_b;
             size_t& smem = gate ? P.smem_gadj : P.smem_adj;
             FinalSeg fs{};
             FinalArgs& fa = fs.a;
@@ -1111,34 +1182,36 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
                 for (int pa = 0; pa < nph; ++pa)
                     for (int pb = 0; pb < nph; ++pb) {
                         const int64_t blk = (int64_t)pa * nph + pb, mir = (int64_t)pb * nph + pa;
-                        float* Gd = reinterpret_cast<float*>(x.ws + x.pl->o_gd[l]) + blk * gd_floats(g);
-                        GSeg gs{};
-                        gs.g = g;
-                        gs.src = src + blk * g.Khalf;
-                        gs.sub = sub ? sub + blk * g.Khalf : nullptr;
-                        gs.src2 = src + mir * g.Khalf;
-                        gs.sub2 = sub ? sub + mir * g.Khalf : nullptr;
-                        gs.sc = vjp ? nullptr : x.sc;
-                        gs.scale = gcoef_scale(g, x.pl->tc, x.pl->w[l]);
-                        gs.Gd = Gd;
-                        gs.done = x.use_done ? &x.sc->done : nullptr;
-                        gs.gate = gate;
+                        const int* done = x.use_done ? &x.sc->done : nullptr;
+                        CoefSrc cs{};
+                        cs.src = src + blk * g.Khalf;
+                        cs.sub = sub ? sub + blk * g.Khalf : nullptr;
+                        cs.src2 = src + mir * g.Khalf;
+                        cs.sub2 = sub ? sub + mir * g.Khalf : nullptr;
+                        cs.sc = vjp ? nullptr : x.sc;
+                        cs.scale = gcoef_scale(g, x.pl->tc, x.pl->w[l]);
                         if (x.pl->desc_kind == DMCR_DESC_S2_TILDE) {
                             TildeSeg t{};
-                            t.src = gs.src;
-                            t.sub = gs.sub;
+                            t.src = cs.src;
+                            t.sub = cs.sub;
                             t.tsum = reinterpret_cast<float*>(x.ws + x.pl->o_tsum) + l;
                             t.K = g.Khalf;
-                            t.done = gs.done;
+                            t.done = done;
                             tsv.push_back(t);
-                            gs.tsum = t.tsum;
-                            gs.q = x.pl->q_tilde;
+                            cs.tsum = t.tsum;
+                            cs.q = x.pl->q_tilde;
                         }
-                        gs.blockStart = gb;
-                        gb += ceil_div((int64_t)(2 * g.P[0] + 1) * (2 * g.P[1] + 1) * g.NB * T, GCOEF_TH);
-                        gv.push_back(gs);
                         float* pblk = part + blk * g.nChunks * g.N;
                         if (g.fft) {
+                            float* Gd = reinterpret_cast<float*>(x.ws + x.pl->o_gd[l]) + blk * gd_floats(g);
+                            GSeg gs{};
+                            gs.g = g;
+                            gs.c = cs;
+                            gs.Gd = Gd;
+                            gs.done = done;
+                            gs.blockStart = gb;
+                            gb += ceil_div((int64_t)(2 * g.P[0] + 1) * (2 * g.P[1] + 1) * g.NB * T, GCOEF_TH);
+                            gv.push_back(gs);
                             Prepared::FftJob j = fft_job(x, l);
                             j.Gd = Gd;
                             j.part = pblk;
@@ -1149,9 +1222,9 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
                         it.a.g = g;
                         it.a.field = x.lv[l] + pa * g.N;
                         it.a.tip = x.lv[l] + pb * g.N;
-                        it.a.Gd = Gd;
+                        it.a.c = cs;
                         it.a.part = pblk;
-                        it.a.done = gs.done;
+                        it.a.done = done;
                         it.a.gate = gate;
                         it.work = (int64_t)g.RZ * g.RY * g.NBc;
                         it.blocks = g.adjTiles * g.nChunks;
@@ -1213,15 +1286,14 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
             }
             return Prepared::R{push(P.tb, av), (int)av.size(), ab};
         };
-        P.gco = {push(P.tb, gplain), (int)gplain.size(), gplain_b};
+        P.gco = {push(P.tb, gv), (int)gv.size(), gb};
         P.tsum = {push(P.tb, tsv), (int)tsv.size(), (int64_t)tsv.size()};
         P.adj = table(plain);
-        P.ggco = {push(P.tb, ggated), (int)ggated.size(), ggated_b};
         P.gadj = table(gated);
         P.fin = {push(P.tb, fv), (int)fv.size(), fb};
         P.fin_small = {push(P.tb, fvs), (int)fvs.size(), fbs};
     }
-    if (need_pyr) prepare_sep(in, flags, P);
+    if (need_pyr) prepare_sep(in, flags, loss_sep, P);
     if (P.tb.h.size() > cap) return fail(DMCR_ENOMEM, "segment tables (%zu bytes) exceed their region", P.tb.h.size());
     // every fused launch indexes its blocks with a 1-D grid
     int64_t most = std::max({P.fwd.blocks, P.red.blocks, P.gco.blocks, P.adj.blocks, P.fin.blocks, P.fin_small.blocks,
@@ -1321,10 +1393,6 @@ void run_sep(const Prepared& P, SepKernel k, const char* name, cudaStream_t s) {
 }
 
 void run(const Prepared& P, cudaStream_t s) {
-    if (P.flags & F_INIT) {
-        ProfScope ps("scalars_init", -1, s);
-        launch_scalars_init(P.at<InitSeg>(P.init.off), P.init.nseg, s);
-    }
     if (P.prep.blocks > 0) {
         ProfScope ps("pyramid", -1, s);
         launch_prep(P.at<PrepSeg>(P.prep.off), P.prep.nseg, P.prep.blocks, s);
@@ -1368,7 +1436,7 @@ void run(const Prepared& P, cudaStream_t s) {
             launch_tilde_map(P.at<TildeSeg>(P.tmap.off), P.tmap.nseg, P.tmap.blocks, s);
         }
     }
-    if (P.flags & F_LOSS) {
+    if ((P.flags & F_LOSS) && P.loss.nseg > 0) {
         {
             ProfScope ps("loss_stats", -1, s);
             launch_penalty(P.at<PenSeg>(P.pen.off), P.pen.nseg, (int)P.pen.blocks, s);
@@ -1389,7 +1457,6 @@ void run(const Prepared& P, cudaStream_t s) {
         run_sep(P, SEP_GRAD, "sep_grad", s);
         if (P.gadj.nseg > 0) {
             ProfScope ps("corr_adj_gated", -1, s);
-            launch_gcoef_gated(P.at<GSeg>(P.ggco.off), P.ggco.nseg, P.ggco.blocks, P.tc, s);
             launch_corr_adj_gated(P.at<AdjSeg>(P.gadj.off), P.gadj.nseg, P.gadj.blocks, P.smem_gadj, P.tc, s);
         }
         if (P.gco.nseg > 0) {
@@ -1435,12 +1502,14 @@ Inst single(const Plan& pl, void* ws) {
     return x;
 }
 
-char* table_region(const Plan& pl, void* ws) { return static_cast<char*>(ws) + pl.o_tab; }
+// the region one upload writes: scalars and tables
+char* upload_region(const Plan& pl, void* ws) { return static_cast<char*>(ws) + pl.o_scal; }
+size_t upload_bytes(const Plan& pl) { return pl.o_tab + pl.tab_bytes - pl.o_scal; }
 
 dmcr_status exec_single(Inst& x, unsigned flags, cudaStream_t s, const char* what) {
     std::vector<Inst> in{x};
     Prepared P;
-    DMCR_TRY(prepare(in, flags, table_region(*x.pl, x.ws), x.pl->tab_bytes, P));
+    DMCR_TRY(prepare(in, flags, upload_region(*x.pl, x.ws), upload_bytes(*x.pl), x.sc != nullptr ? 1 : 0, P));
     upload(P, s);
     run(P, s);
     return cuda_check(cudaGetLastError(), what);
@@ -1454,11 +1523,12 @@ dmcr_status check_loss_opts(const dmcr_loss_opts* o) {
 
 // ---------------------------------------------------------------------------- batches
 //
-// Batch workspace: [segment tables][count x Scalars][instance workspaces (Plan layouts)].
+// Batch workspace: [count x Scalars][segment tables][instance workspaces (Plan layouts)].
 struct BatchLayout {
     std::vector<Plan> plans;
     std::vector<size_t> o_inst;
     size_t o_tab = 0, tab_bytes = 0, o_scal = 0, bytes = 0;
+    size_t upload_bytes() const { return o_tab + tab_bytes - o_scal; }
 };
 
 dmcr_status batch_layout(int count, const dmcr_params* params, BatchLayout& B) {
@@ -1471,11 +1541,11 @@ dmcr_status batch_layout(int count, const dmcr_params* params, BatchLayout& B) {
         tb += table_bound(B.plans[i]) + 32;
     }
     size_t o = 0;
+    B.o_scal = o;
+    o = align_up(o + (size_t)count * sizeof(Scalars));
     B.o_tab = o;
     B.tab_bytes = align_up(tb);
     o += B.tab_bytes;
-    B.o_scal = o;
-    o = align_up(o + (size_t)count * sizeof(Scalars));
     for (int i = 0; i < count; ++i) {
         B.o_inst.push_back(o);
         o = align_up(o + B.plans[i].bytes);
@@ -1507,7 +1577,7 @@ std::vector<Inst> batch_insts(const BatchLayout& B, void* ws) {
 dmcr_status exec_batch(const BatchLayout& B, void* ws, std::vector<Inst>& in, unsigned flags, cudaStream_t s,
                        const char* what) {
     Prepared P;
-    DMCR_TRY(prepare(in, flags, static_cast<char*>(ws) + B.o_tab, B.tab_bytes, P));
+    DMCR_TRY(prepare(in, flags, static_cast<char*>(ws) + B.o_scal, B.upload_bytes(), (int)in.size(), P));
     upload(P, s);
     run(P, s);
     return cuda_check(cudaGetLastError(), what);
@@ -1543,8 +1613,8 @@ std::string prepared_key(const Prepared& P) {
     add(&P.flags, sizeof P.flags);
     add(&P.tc, sizeof P.tc);
     for (const Prepared::R& r : P.restricts) add(&r, sizeof r);
-    for (const Prepared::R* r : {&P.fwd, &P.red, &P.pen, &P.loss, &P.gco, &P.adj, &P.fin, &P.fin_small, &P.init,
-                                   &P.tmap, &P.tsum, &P.prep, &P.gfwd, &P.gred, &P.ggco, &P.gadj})
+    for (const Prepared::R* r : {&P.fwd, &P.red, &P.pen, &P.loss, &P.gco, &P.adj, &P.fin, &P.fin_small,
+                                   &P.tmap, &P.tsum, &P.prep, &P.gfwd, &P.gred, &P.gadj})
         add(r, sizeof *r);
     add(P.sep, sizeof P.sep);
     add(P.sep_smem, sizeof P.sep_smem);
@@ -1563,7 +1633,7 @@ std::string prepared_key(const Prepared& P) {
         add(&n, sizeof n);
         if (n) add(v->data(), n * sizeof((*v)[0]));
     }
-    add(P.tb.h.data(), P.tb.h.size());
+    add(P.tb.h.data() + P.scal_bytes, P.tb.h.size() - P.scal_bytes);   // not the step counts in front
     return k;
 }
 
@@ -1638,12 +1708,8 @@ dmcr_status reconstruct_insts(std::vector<Inst>& in, char* tab, size_t tab_cap, 
         if ((st = cuda_check(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "cudaEventCreate"))) break;
         if ((st = cuda_check(cudaEventRecord(ev, caller), "cudaEventRecord"))) break;
         if ((st = cuda_check(cudaStreamWaitEvent(s, ev, 0), "cudaStreamWaitEvent"))) break;
-        Prepared P0;
-        if ((st = prepare(in, F_INIT, tab, tab_cap, P0))) break;
-        upload(P0, s);
-        run(P0, s);
         Prepared P;
-        if ((st = prepare(in, F_FWD | F_LOSS | F_BACK | F_ADAM, tab, tab_cap, P))) break;
+        if ((st = prepare(in, F_FWD | F_LOSS | F_BACK | F_ADAM, tab, tab_cap, count, P))) break;
         upload(P, s);
         const std::string key = prepared_key(P);
         cached = recon_graph_acquire(key);
@@ -1712,7 +1778,7 @@ dmcr_status reconstruct_insts(std::vector<Inst>& in, char* tab, size_t tab_cap, 
             y.lp.recon = 0;
         }
         Prepared PR;
-        if ((st = prepare(rin, F_FWD | F_LOSS, tab, tab_cap, PR))) break;
+        if ((st = prepare(rin, F_FWD | F_LOSS, tab, tab_cap, count, PR))) break;
         upload(PR, s);
         run(PR, s);
         if ((st = cuda_check(cudaMemcpyAsync(hs.data(), scal_base, count * sizeof(Scalars), cudaMemcpyDeviceToHost, s),
@@ -1767,9 +1833,9 @@ void recon_inst(Inst& x, const dmcr_recon_opts* o, const float* target, float* f
 // dmcr_adam_step(_batched) is called once per iteration with the same arguments over and
 // over; for small problems its ten launches, the planning and the table building cost more
 // than the arithmetic.  The first call with a given set of arguments therefore captures the
-// iteration (table upload + every kernel) into a CUDA graph on a private stream and keeps
-// the instantiated graph; a later call with the same arguments launches one small kernel
-// that sets the Adam step scalars of this call (passed by value) and the graph.  The key is
+// iteration's kernels into a CUDA graph on a private stream and keeps the instantiated graph
+// and the table bytes; a later call with the same arguments uploads the tables with this
+// call's Adam step scalars in front (passed by value, one small kernel) and launches the graph.  The key is
 // every argument that shapes the launch sequence or that the tables point to: the params
 // and options field by field, all pointers, the workspace size and the device.  Calls made
 // while the stream is being captured by the caller, or while the library's per-kernel
@@ -1797,7 +1863,9 @@ struct StepGraph {
     std::string key;
     cudaGraphExec_t exec = nullptr;
     cudaEvent_t done = nullptr;     // recorded after every replay: eviction waits for it
-    std::vector<Scalars*> sc;       // per instance
+    std::vector<unsigned char> up;  // scalars (of the last call) and tables
+    char* tab = nullptr;            // where they go
+    size_t count = 0;               // instances
     float beta1 = 0.9f, beta2 = 0.999f;
     uint64_t used = 0;
 };
@@ -1834,12 +1902,12 @@ bool replay_step_graph(const std::string& key, const int64_t* steps, cudaStream_
     for (StepGraph& g : graph_cache())
         if (g.key == key) {
             g.used = ++g_graph_clock;
-            std::vector<InitSeg> init;
-            for (size_t i = 0; i < g.sc.size(); ++i)
-                init.push_back({g.sc[i], steps[i], pow((double)g.beta1, (double)steps[i]),
-                                pow((double)g.beta2, (double)steps[i])});
-            launch_scalars_set(init.data(), (int)init.size(), s);
-            *st = cuda_check(cudaGetLastError(), "scalars set");
+            for (size_t i = 0; i < g.count; ++i) {
+                const Scalars sc = initial_scalars(steps[i], g.beta1, g.beta2);
+                memcpy(g.up.data() + i * sizeof(Scalars), &sc, sizeof sc);
+            }
+            launch_blob(g.up.data(), g.up.size(), g.tab, s);
+            *st = cuda_check(cudaGetLastError(), "scalars and tables upload");
             if (*st == DMCR_OK) *st = cuda_check(cudaGraphLaunch(g.exec, s), "cudaGraphLaunch (cached iteration)");
             if (*st == DMCR_OK) *st = cuda_check(cudaEventRecord(g.done, s), "cudaEventRecord (cached iteration)");
             return true;
@@ -1847,8 +1915,8 @@ bool replay_step_graph(const std::string& key, const int64_t* steps, cudaStream_
     return false;
 }
 
-// Capture the prepared iteration (tables + kernels, no scalar initialisation) into a graph
-// and store it under `key`.  Returns false (and leaves no error pending) if anything fails.
+// Capture the prepared iteration's kernels into a graph and store it under `key`, with the
+// tables to upload before each replay.  Returns false (and leaves no error pending) if anything fails.
 bool capture_step_graph(const std::string& key, const Prepared& P, const std::vector<Inst>& in) {
     cudaStream_t cs = nullptr;
     cudaGraph_t graph = nullptr;
@@ -1856,7 +1924,6 @@ bool capture_step_graph(const std::string& key, const Prepared& P, const std::ve
     bool ok = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess;
     if (ok) ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
     if (ok) {
-        upload(P, cs);
         run(P, cs);
         ok = cudaStreamEndCapture(cs, &graph) == cudaSuccess && graph != nullptr;
     }
@@ -1874,7 +1941,9 @@ bool capture_step_graph(const std::string& key, const Prepared& P, const std::ve
     g.key = key;
     g.exec = exec;
     g.done = done;
-    for (const Inst& x : in) g.sc.push_back(x.sc);
+    g.up = P.tb.h;
+    g.tab = P.tab;
+    g.count = in.size();
     g.beta1 = in[0].beta1;
     g.beta2 = in[0].beta2;
     std::lock_guard<std::mutex> lk(g_graph_mu);
@@ -1902,13 +1971,9 @@ dmcr_status adam_iteration(const std::string& key, std::vector<Inst>& in, char* 
     for (const Inst& x : in) steps.push_back(x.step);
     dmcr_status st = DMCR_OK;
     if (graphs && replay_step_graph(key, steps.data(), s, &st)) return st;
-    if (graphs) {
-        Prepared P;
-        DMCR_TRY(prepare(in, F_FWD | F_LOSS | F_BACK | F_ADAM, tab, tab_cap, P));
-        if (capture_step_graph(key, P, in) && replay_step_graph(key, steps.data(), s, &st)) return st;
-    }
     Prepared P;
-    DMCR_TRY(prepare(in, F_INIT | F_FWD | F_LOSS | F_BACK | F_ADAM, tab, tab_cap, P));
+    DMCR_TRY(prepare(in, F_FWD | F_LOSS | F_BACK | F_ADAM, tab, tab_cap, (int)in.size(), P));
+    if (graphs && capture_step_graph(key, P, in) && replay_step_graph(key, steps.data(), s, &st)) return st;
     upload(P, s);
     run(P, s);
     return cuda_check(cudaGetLastError(), what);
@@ -2053,7 +2118,7 @@ dmcr_status dmcr_adam_step(const dmcr_params* p, const dmcr_recon_opts* o, const
     one.check_every = 1;
     recon_inst(in[0], &one, target_desc, field, state, nullptr);
     in[0].loss_out = loss_out;
-    DMCR_TRY(adam_iteration(k.b, in, table_region(pl, ws), pl.tab_bytes, s, "dmcr_adam_step launch"));
+    DMCR_TRY(adam_iteration(k.b, in, upload_region(pl, ws), upload_bytes(pl), s, "dmcr_adam_step launch"));
     state->step += 1;
     return DMCR_OK;
 }
@@ -2074,7 +2139,7 @@ dmcr_status dmcr_reconstruct(const dmcr_params* p, const dmcr_recon_opts* o, con
     if (o->init == DMCR_INIT_UNIFORM_SEEDED) launch_init_uniform(field, pl.N1 * pl.phases, o->seed, s);
     std::vector<Inst> in{single(pl, ws)};
     recon_inst(in[0], o, target_desc, field, state, history);
-    const dmcr_status st = reconstruct_insts(in, table_region(pl, ws), pl.tab_bytes, in[0].sc, {o->max_iters},
+    const dmcr_status st = reconstruct_insts(in, upload_region(pl, ws), upload_bytes(pl), in[0].sc, {o->max_iters},
                                              o->check_every, report, state, s, false);
     report->status = st;
     return st;
@@ -2191,7 +2256,7 @@ dmcr_status dmcr_adam_step_batched(int count, const dmcr_params* params, const d
         recon_inst(in[i], &one, targets[i], fields[i], &states[i], nullptr);
         in[i].loss_out = loss_out != nullptr ? loss_out + (size_t)DMCR_OUT_COUNT * i : nullptr;
     }
-    DMCR_TRY(adam_iteration(k.b, in, static_cast<char*>(ws) + B.o_tab, B.tab_bytes, s,
+    DMCR_TRY(adam_iteration(k.b, in, static_cast<char*>(ws) + B.o_scal, B.upload_bytes(), s,
                             "dmcr_adam_step_batched launch"));
     for (int i = 0; i < count; ++i) states[i].step += 1;
     return DMCR_OK;
@@ -2221,7 +2286,7 @@ dmcr_status dmcr_reconstruct_batched(int count, const dmcr_params* params, const
     for (int i = 0; i < count; ++i)
         if (opts[i].init == DMCR_INIT_UNIFORM_SEEDED)
             launch_init_uniform(fields[i], B.plans[i].N1 * B.plans[i].phases, opts[i].seed, s);
-    return reconstruct_insts(in, static_cast<char*>(ws) + B.o_tab, B.tab_bytes,
+    return reconstruct_insts(in, static_cast<char*>(ws) + B.o_scal, B.upload_bytes(),
                              reinterpret_cast<Scalars*>(static_cast<char*>(ws) + B.o_scal), iters, poll, reports,
                              states, s, true);
 }
@@ -2305,7 +2370,8 @@ extern "C" dmcr_status dmcr_descriptor_noalloc(const dmcr_params* p, const float
     // compact layout: segment tables, pyramid levels 2.. and the forward partials of every level
     Plan cp = pl;
     cp.sep = false;            // the spectra of the separable path do not fit
-    cp.tab_bytes = align_up(table_bound(cp) + table_slack(false));
+    cp.tab_bytes = align_up((size_t)cp.levels * (sizeof(FwdSeg) + sizeof(RedSeg) + sizeof(RestrictSeg)) +
+                            sizeof(PrepSeg) + table_slack(false));      // the forward's tables only
     size_t o = 0;
     cp.o_tab = o;
     o += cp.tab_bytes;

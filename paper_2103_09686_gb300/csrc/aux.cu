@@ -7,6 +7,7 @@
 #include <string.h>
 
 #include "common.cuh"
+#include "loss.cuh"
 
 namespace dmcr {
 
@@ -43,11 +44,6 @@ __global__ void restrict_kernel(const RestrictSeg* __restrict__ segs, int nseg) 
 
 // --------------------------------------------------------------------- pyramid
 
-// Box excess of Sec. 3.1: (M-1) H(M-1) - M H(-M), H(0) = 0.
-__device__ __forceinline__ float box_excess(float M) {
-    return M > 1.f ? M - 1.f : (M < 0.f ? -M : 0.f);
-}
-
 // All coarser levels of a tile in one pass over the finest field (each the mean of its 2^d
 // children, summed as restrict_one does), with the tier of the values' range and the box
 // excess, which need the same pass.  A thread reads a 2^d block; the coarser means go through
@@ -66,9 +62,7 @@ __device__ __forceinline__ void prep_tiles(const PrepSeg& sg, int blk, float* sh
         lo = fminf(lo, v);
         hi = fmaxf(hi, v);
         const float ex = box_excess(v);
-        const float y = ex * ex - e2c, u = e2 + y;
-        e2c = (u - e2) - y;
-        e2 = u;
+        kahan_add(e2, e2c, ex * ex);
     };
     for (int64_t tile = blk; tile < tiles; tile += sg.nblk) {
         const int x0 = (int)(tile % t2) * TILE, y0 = (int)(tile / t2 % t1) * TILE;
@@ -223,7 +217,6 @@ __global__ void stats_kernel(const PenSeg* __restrict__ segs) {
     const PenSeg& sg = segs[blockIdx.y];
     if (sg.done != nullptr && *sg.done) return;
     if ((int)blockIdx.x >= sg.nblk) return;
-    if (sg.gate != nullptr && *sg.gate < SEP_TIERS) return;
     __shared__ DF sh[32];
     const int64_t stride = (int64_t)sg.nblk * blockDim.x;
     const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -231,12 +224,6 @@ __global__ void stats_kernel(const PenSeg* __restrict__ segs) {
     // this part and a thread sums only about 8 terms (stats_blocks) -- then a double-float
     // (two-sum) tree across the block
     float r2 = 0.f, r2c = 0.f, t2 = 0.f, t2c = 0.f, e2 = 0.f, e2c = 0.f;
-    auto kahan = [](float& sum, float& comp, float v) {
-        const float y = v - comp;
-        const float t = sum + y;
-        comp = (t - sum) - y;
-        sum = t;
-    };
     // the terms of this thread in order; their loads issued four at a time (the same sums)
     int64_t k = i0;
     for (; k + 3 * stride < sg.K; k += 4 * stride) {
@@ -249,15 +236,15 @@ __global__ void stats_kernel(const PenSeg* __restrict__ segs) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const float r = dv[u] - tv[u];
-            kahan(r2, r2c, r * r);
-            kahan(t2, t2c, tv[u] * tv[u]);
+            kahan_add(r2, r2c, r * r);
+            kahan_add(t2, t2c, tv[u] * tv[u]);
         }
     }
     for (; k < sg.K; k += stride) {
         const float t = sg.target[k];
         const float r = sg.desc[k] - t;
-        kahan(r2, r2c, r * r);
-        kahan(t2, t2c, t * t);
+        kahan_add(r2, r2c, r * r);
+        kahan_add(t2, t2c, t * t);
     }
     if (sg.field != nullptr) {
         int64_t i = i0;
@@ -268,12 +255,12 @@ __global__ void stats_kernel(const PenSeg* __restrict__ segs) {
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const float e = box_excess(fv[u]);
-                kahan(e2, e2c, e * e);
+                kahan_add(e2, e2c, e * e);
             }
         }
         for (; i < sg.N; i += stride) {
             const float e = box_excess(sg.field[i]);
-            kahan(e2, e2c, e * e);
+            kahan_add(e2, e2c, e * e);
         }
     }
     // Kahan's (sum, comp) stands for sum - comp
@@ -339,84 +326,23 @@ void launch_tilde_sum(const TildeSeg* segs, int nseg, cudaStream_t s) {
     launch_dep(tilde_sum_kernel, nseg, 256, 0, s, segs);
 }
 
-// One block per instance: sums the stats partials in a fixed tree, then E, E^2, E_bc,
-// lambda, L, rel_err and the gradient scalars; in a reconstruction also the stopping test
-// and the Adam step bookkeeping.
+// One block per instance whose statistics came from stats_kernel (three-point and corrected
+// descriptors, FFT levels): sums the partials in a fixed tree and finishes the loss.
 __global__ void __launch_bounds__(NPEN_BLOCKS) loss_kernel(const LossSeg* __restrict__ segs) {
     dep_wait();
     dep_trigger();
     const LossSeg& sg = segs[blockIdx.x];
-    const LossParams lp = sg.lp;
-    const double* __restrict__ pen = sg.pen;
-    Scalars* sc = sg.sc;
-    float* loss_out = sg.loss_out;
-    float* history = sg.history;
-    if (lp.recon && sc->done) return;
+    if (sg.lp.recon && sg.sc->done) return;
     __shared__ DF sh[32];
     // the instance's nblk double-float partials (the remaining threads add zeros)
     const int b = threadIdx.x;
-    const float2* part = reinterpret_cast<const float2*>(pen);
+    const float2* part = reinterpret_cast<const float2*>(sg.pen);
     const DF zero{0.f, 0.f};
-    DF r2 = zero, t2 = zero, x2 = zero;
-    if (sg.tier != nullptr && *sg.tier < SEP_TIERS) {
-        // the separable kernels left their own block sums
-        for (int i = b; i < sg.nsum; i += NPEN_BLOCKS) {
-            const float4 v = sg.sums[i];
-            r2 = df_add(r2, DF{v.x, v.y});
-            t2 = df_add(t2, DF{v.z, v.w});
-        }
-        for (int i = b; i < sg.nexc; i += NPEN_BLOCKS) x2 = df_add(x2, DF{sg.excess[i].x, sg.excess[i].y});
-    } else if (b < sg.nblk) {
-        r2 = DF{part[3 * b].x, part[3 * b].y};
-        t2 = DF{part[3 * b + 1].x, part[3 * b + 1].y};
-        x2 = DF{part[3 * b + 2].x, part[3 * b + 2].y};
-    }
-    const DF e2s = block_sum_df(r2, sh);
-    const DF t2s = block_sum_df(t2, sh);
-    const DF x2s = block_sum_df(x2, sh);
-    if (threadIdx.x != 0) return;
-    // the scalars in FP64 on this one thread (a few dozen FP64 operations once per
-    // evaluation): the double-float sums keep about 48 bits, and the square roots and
-    // quotients below keep them, so E, rel_err and L reach the output rounded once to FP32
-    const double E2 = (double)e2s.hi + (double)e2s.lo;
-    const double T2 = (double)t2s.hi + (double)t2s.lo;
-    const double ex2 = (double)x2s.hi + (double)x2s.lo;
-    const double N = (double)lp.N;
-    const double lam0 = lp.bc_on ? (double)lp.lambda0 : 0.0;
-    const double E = sqrt(E2);
-    const double Ebc = ex2 / (N * N);
-    const double phi = lp.mode == 0 ? E : E2;
-    const double lam = lam0 * phi;
-    const double L = phi + lam * Ebc;
-    const double rel = T2 > 0.0 ? E / sqrt(T2) : (double)INFINITY;
-    const float out[6] = {(float)E, (float)E2, (float)Ebc, (float)lam, (float)L, (float)rel};
-    for (int i = 0; i < 6; ++i) sc->loss[i] = out[i];
-    if (loss_out != nullptr)
-        for (int i = 0; i < 6; ++i) loss_out[i] = out[i];
-    // dL/dD = phi'(E) (1 + lam0 E_bc) dE/dD ;  dL/dM (penalty) = lam0 phi dE_bc/dM
-    double gs;
-    if (lp.mode == 0) gs = E > 0.0 ? (1.0 + lam0 * Ebc) / E : 0.0;
-    else gs = 2.0 * (1.0 + lam0 * Ebc);
-    sc->gscale = (float)gs;
-    sc->pen_coef = (float)(2.0 * lam0 * phi / (N * N));
-    if (!lp.recon) return;
-    const int it = sc->iter;
-    if (history != nullptr && it < lp.max_iters) {
-        history[3 * it + 0] = out[0];
-        history[3 * it + 1] = out[4];
-        history[3 * it + 2] = out[5];
-    }
-    sc->iter = it + 1;
-    if (!isfinite(out[4])) { sc->done = 2; return; }
-    if (lp.tol_rel > 0.f && (it % lp.check_every) == 0 && out[5] < lp.tol_rel) { sc->done = 1; return; }
-    if (it + 1 > lp.max_iters) { sc->done = 3; return; }
-    sc->adam_step = sc->adam_step + 1;
-    // beta^t products stay FP64: they are multiplied once per step over many steps
-    const double b1t = sc->b1t * (double)lp.beta1;
-    const double b2t = sc->b2t * (double)lp.beta2;
-    sc->b1t = b1t;
-    sc->b2t = b2t;
-    sc->lr_t = (float)((double)lp.lr * sqrt(1.0 - b2t) / (1.0 - b1t));
+    auto get = [&](int q) { return b < sg.nblk ? DF{part[3 * b + q].x, part[3 * b + q].y} : zero; };
+    const DF e2s = block_sum_df(get(0), sh);
+    const DF t2s = block_sum_df(get(1), sh);
+    const DF x2s = block_sum_df(get(2), sh);
+    if (threadIdx.x == 0) loss_scalars(sg, e2s, t2s, x2s);
 }
 
 void launch_loss(const LossSeg* segs, int nseg, cudaStream_t s) {
@@ -515,60 +441,6 @@ void launch_final(const FinalSeg* segs, int nseg, int64_t blocks, int sub, cudaS
         launch_dep(final_kernel<1>, (unsigned)blocks, ELEM_TH, 0, s, segs, nseg);
     else
         launch_dep(final_kernel<FIN_SUB>, (unsigned)blocks, ELEM_TH, 0, s, segs, nseg);
-}
-
-__device__ __forceinline__ void scalars_init_one(const InitSeg& g) {
-    Scalars* sc = g.sc;
-    for (int k = 0; k < 6; ++k) sc->loss[k] = 0.f;
-    sc->gscale = 0.f;
-    sc->pen_coef = 0.f;
-    sc->lr_t = 0.f;
-    sc->done = 0;
-    sc->iter = 0;
-    sc->adam_step = g.step;
-    sc->b1t = g.b1t;
-    sc->b2t = g.b2t;
-    sc->err = 0;
-}
-
-__global__ void scalars_init_kernel(const InitSeg* __restrict__ segs, int nseg) {
-    dep_wait();
-    dep_trigger();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nseg) return;
-    scalars_init_one(segs[i]);
-}
-
-void launch_scalars_init(const InitSeg* segs, int nseg, cudaStream_t s) {
-    if (nseg <= 0) return;
-    launch_dep(scalars_init_kernel, (nseg + 127) / 128, 128, 0, s, segs, nseg);
-}
-
-// The same initialisation with the segments passed by value (no table in device memory):
-// used before a replay of a cached iteration graph, whose captured tables cannot carry the
-// Adam step count of the current call.
-constexpr int SET_MAX = 960;
-struct InitBatch {
-    int n;
-    InitSeg seg[SET_MAX];
-};
-
-__global__ void scalars_set_kernel(const InitBatch b) {
-    dep_wait();
-    dep_trigger();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= b.n) return;
-    scalars_init_one(b.seg[i]);
-}
-
-void launch_scalars_set(const InitSeg* segs, int nseg, cudaStream_t s) {
-    static thread_local InitBatch b;
-    for (int off = 0; off < nseg; off += SET_MAX) {
-        const int k = nseg - off < SET_MAX ? nseg - off : SET_MAX;
-        b.n = k;
-        memcpy(b.seg, segs + off, (size_t)k * sizeof(InitSeg));
-        launch_dep(scalars_set_kernel, (k + 127) / 128, 128, 0, s, b);
-    }
 }
 
 // Writes up to BLOB_BYTES of host data, passed by value as a kernel parameter, to device

@@ -160,6 +160,17 @@ struct FinalArgs {
 // A fused launch covers several (instance, level) segments; every segment owns the
 // contiguous block range [blockStart, next blockStart) of a 1-D grid and the kernels find
 // their segment by binary search.  Tables live in device memory (written by blob_kernel).
+struct LossSeg {
+    LossParams lp;
+    const double* pen;          // stats_kernel's partials (nblk blocks) ...
+    int nblk;
+    const float4* sums;         // ... or the descriptor blocks' sum (D - D_des)^2, sum D_des^2 (hi, lo each)
+    const float4* excess;       // and the field blocks' sum of squared box excess (hi, lo)
+    int nsum, nexc;
+    Scalars* sc;
+    float* loss_out;
+    float* history;
+};
 struct FwdSeg {
     LevelGeom g;
     const float* field;     // tails of the pairs (x)
@@ -176,31 +187,47 @@ struct RedSeg {
     const int* gate;        // gated launches only: run when *gate >= SEP_TIERS
     const int* done;
     float scale;             // w_l / N_l
+    // loss: this segment's target, its block sums (one per block), the instance's loss and the
+    // number of blocks that leave sums for it; null: no loss, or statistics by stats_kernel
+    const float* target;
+    float4* sums;
+    const LossSeg* loss;
+    int arrive;
+    // box excess of the field in `nexc` extra blocks of this segment (0: elsewhere or none)
+    int nexc;
+    float4* excess;
+    const float* field;
+    int64_t fieldN, excChunk;
     int64_t blockStart;
 };
-struct AdjSeg {
-    LevelGeom g;
-    const float* field;     // own positions y (the gradient's field)
-    const float* tip;       // partners y + r: the same field, or another phase's
-    const float* Gd;
-    float* part;
-    const int* gate;        // gated launches only: run when *gate >= SEP_TIERS
-    const int* done;
-    int64_t blockStart;
-};
-struct GSeg {
-    LevelGeom g;
+// Gradient coefficients of one level and phase pair: G(r) from the residuals or the upstream
+// gradient (see coef_value in corr.cu).
+struct CoefSrc {
     const float* src;       // dL/dS (or S - S_des) of the block (a, b), shifts r of the half window
     const float* sub;
     const float* src2;      // the block (b, a), which holds -r; src2 = src, sub2 = sub for a = b
     const float* sub2;
     const Scalars* sc;
     float scale;
-    float* Gd;
-    const int* gate;
-    const int* done;
     const float* tsum;      // corrected descriptor: sum_{k >= 1} (src - sub) of the block, else null
     float q;                // corrected descriptor: 2 f(1/2)^2
+};
+struct AdjSeg {
+    LevelGeom g;
+    const float* field;     // own positions y (the gradient's field)
+    const float* tip;       // partners y + r: the same field, or another phase's
+    CoefSrc c;
+    float* part;
+    const int* gate;        // gated launches only: run when *gate >= SEP_TIERS
+    const int* done;
+    int64_t blockStart;
+};
+// dense coefficient grid of an FFT level
+struct GSeg {
+    LevelGeom g;
+    CoefSrc c;
+    float* Gd;
+    const int* done;
     int64_t blockStart;
 };
 // Corrected two-point descriptor (App. A, Eq. s2rfroms2rbar), one (instance, level) block:
@@ -243,7 +270,6 @@ struct PrepSeg {
     int64_t blockStart;
 };
 struct PenSeg {
-    const int* gate;         // separable path with fused sums: run only when *gate >= SEP_TIERS
     const float* field;      // null: no box penalty
     int64_t N;
     const float* desc;
@@ -253,32 +279,11 @@ struct PenSeg {
     const int* done;
     int nblk;                // blocks of this instance: a function of its own sizes only
 };
-struct LossSeg {
-    // separable path with fused residual sums: used while *tier < SEP_TIERS (else `pen`)
-    const int* tier;
-    const float4* sums;         // nsum entries: sum (D - D_des)^2, sum D_des^2 (hi, lo each)
-    const float4* excess;       // nexc entries: sum of squared box excess (hi, lo)
-    int nsum, nexc;
-    LossParams lp;
-    const float* desc;
-    const float* target;
-    const double* pen;
-    int nblk;
-    Scalars* sc;
-    float* loss_out;
-    float* history;
-};
 struct FinalSeg {
     FinalArgs a;
     const int* done;
     int64_t blockStart;
 };
-struct InitSeg {
-    Scalars* sc;
-    int64_t step;
-    double b1t, b2t;
-};
-
 // Three-point descriptor, one (instance, level) (gram.cu).  K = half-window shifts, Kpad =
 // K rounded up to 256, Npad = the level's position count rounded up to 128.
 struct S3Job {
@@ -387,7 +392,9 @@ struct SepLevel {
     const float* tsum;        // corrected descriptor
     float q, scaleG;
     int fuse;                 // one phase, loss and gradient in one call: sep_desc goes on to the rows of G
-    float4* sums;             // fuse: per sep_desc block sum (D - D_des)^2 and sum D_des^2 (hi, lo each)
+    const LossSeg* loss;      // sep_desc leaves the loss' sums (`sums`, one per block of the instance) and
+    float4* sums;             //   its last block finishes the loss; null: no loss, or statistics elsewhere
+    int sumStart, arrive;     // this level's first block sum of phase pair 0; blocks in all
     float* part;              // this level's gradient, one field per phase
     const int* done;
 };
@@ -439,7 +446,6 @@ void launch_fwd_reduce(const RedSeg* segs, int nseg, int64_t blocks, cudaStream_
 void launch_corr_fwd_gated(const FwdSeg* segs, int nseg, int64_t blocks, size_t smem, const ThreshConst& tc,
                            cudaStream_t s);
 void launch_fwd_reduce_gated(const RedSeg* segs, int nseg, int64_t blocks, cudaStream_t s);
-void launch_gcoef_gated(const GSeg* segs, int nseg, int64_t blocks, const ThreshConst& tc, cudaStream_t s);
 void launch_corr_adj_gated(const AdjSeg* segs, int nseg, int64_t blocks, size_t smem, const ThreshConst& tc,
                            cudaStream_t s);
 void launch_penalty(const PenSeg* segs, int nseg, int maxblk, cudaStream_t s);
@@ -454,8 +460,6 @@ void launch_corr_adj(const AdjSeg* segs, int nseg, int64_t blocks, size_t smem, 
 void launch_final(const FinalSeg* segs, int nseg, int64_t blocks, int sub, cudaStream_t s);
 void launch_init_uniform(float* field, int64_t count, uint64_t seed, cudaStream_t s);
 void launch_round_field(const float* src, float* dst, int64_t count, cudaStream_t s);
-void launch_scalars_init(const InitSeg* segs, int nseg, cudaStream_t s);
-void launch_scalars_set(const InitSeg* host_segs, int nseg, cudaStream_t s);   // segments by value
 void set_kernel_attributes();
 void set_gram_attributes();
 size_t gemm_smem_bytes();

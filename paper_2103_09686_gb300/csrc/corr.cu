@@ -30,6 +30,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "loss.cuh"
 
 namespace dmcr {
 
@@ -561,20 +562,30 @@ corr_fwd_gated_kernel(const FwdSeg* __restrict__ segs, int nseg, int64_t total, 
 // Fixed-order sum over tiles, scaled by w_l / N_l.  A block owns 32 consecutive shifts (one
 // per lane, coalesced rows); warp w sums the tiles t = w (mod 8) in order (Kahan, FP32) and
 // the 8 warp sums are combined in a fixed order as double-floats.
+// With a loss to evaluate the block also leaves its shifts' sums, extra blocks sum the box
+// excess of the field, and the instance's last block finishes the loss.
 __device__ __forceinline__ void fwd_reduce_block(const RedSeg& sg, int64_t local) {
     const int64_t Khalf = sg.g.Khalf, tiles = sg.g.fwdTiles;
     __shared__ DF sh[8][RED_K];
+    __shared__ DF dsh[32];
+    const int64_t own = (Khalf + RED_K - 1) / RED_K;
+    if (local >= own) {
+        const int64_t i0 = (local - own) * sg.excChunk, i1 = min(i0 + sg.excChunk, sg.fieldN);
+        float e2 = 0.f, e2c = 0.f;
+        for (int64_t i = i0 + threadIdx.x; i < i1; i += 256) {
+            const float ex = box_excess(sg.field[i]);
+            kahan_add(e2, e2c, ex * ex);
+        }
+        const DF E = block_sum_df(df_two_sum(e2, -e2c), dsh);
+        if (threadIdx.x == 0) sg.excess[local - own] = make_float4(E.hi, E.lo, 0.f, 0.f);
+        loss_arrive(*sg.loss, sg.arrive, dsh);
+        return;
+    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t k = local * RED_K + lane;
     // compensated (Kahan) FP32 sum over this warp's tiles, then a double-float (two-sum)
     // combination of the 8 warps
     float sum = 0.f, comp = 0.f;
-    auto kahan = [&](float v) {
-        const float y = v - comp;
-        const float u = sum + y;
-        comp = (u - sum) - y;
-        sum = u;
-    };
     if (k < Khalf) {
         // this warp's tiles in order, their loads issued four at a time
         int64_t t = warp;
@@ -583,17 +594,29 @@ __device__ __forceinline__ void fwd_reduce_block(const RedSeg& sg, int64_t local
 #pragma unroll
             for (int u = 0; u < 4; ++u) v[u] = sg.partial[(t + 8 * u) * Khalf + k];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) kahan(v[u]);
+            for (int u = 0; u < 4; ++u) kahan_add(sum, comp, v[u]);
         }
-        for (; t < tiles; t += 8) kahan(sg.partial[t * Khalf + k]);
+        for (; t < tiles; t += 8) kahan_add(sum, comp, sg.partial[t * Khalf + k]);
     }
     sh[warp][lane] = df_two_sum(sum, -comp);
     __syncthreads();
-    if (warp == 0 && k < Khalf) {
+    if (warp == 0) {
         DF tot = sh[0][lane];
         for (int w = 1; w < 8; ++w) tot = df_add(tot, sh[w][lane]);
-        sg.desc[k] = (tot.hi + tot.lo) * sg.scale;
+        const float d = (tot.hi + tot.lo) * sg.scale;
+        if (k < Khalf) sg.desc[k] = d;
+        if (sg.loss != nullptr) {
+            // the residual and target squares of the block's 32 shifts, one per lane
+            const float t = k < Khalf ? sg.target[k] : 0.f, r = k < Khalf ? d - t : 0.f;
+            DF R2{r * r, 0.f}, T2{t * t, 0.f};
+            for (int o = 16; o > 0; o >>= 1) {
+                R2 = df_add(R2, DF{__shfl_xor_sync(0xffffffffu, R2.hi, o), __shfl_xor_sync(0xffffffffu, R2.lo, o)});
+                T2 = df_add(T2, DF{__shfl_xor_sync(0xffffffffu, T2.hi, o), __shfl_xor_sync(0xffffffffu, T2.lo, o)});
+            }
+            if (lane == 0) sg.sums[local] = make_float4(R2.hi, R2.lo, T2.hi, T2.lo);
+        }
     }
+    if (sg.loss != nullptr) loss_arrive(*sg.loss, sg.arrive, dsh);
 }
 
 __global__ void __launch_bounds__(256) fwd_reduce_kernel(const RedSeg* __restrict__ segs, int nseg) {
@@ -611,6 +634,41 @@ __global__ void __launch_bounds__(256) fwd_reduce_gated_kernel(const RedSeg* __r
 }
 
 // ------------------------------------------------------------------------- adjoint
+
+// Coefficient of the full-window shift r = (rz, ry, rx) of one level and phase pair (a, b):
+//   G(r) = scale * (src[k] - sub[k]) for r in the half window (k its canonical index),
+//   G(r) = scale * (src2[k] - sub2[k]) for -r in it (k the index of -r),
+//   G(0) = scale * ((src - sub) + (src2 - sub2))[0]   (2 (src - sub)[0] for one field),
+//   scale = weight * (gscale from the loss, or 1) * (c1 alpha / N_l, or 1 / N_l for f(x)=x),
+// zero where rx > P2 (padding of the last rx block).
+__device__ __forceinline__ float coef_value(const CoefSrc& c, const LevelGeom& g, int rz, int ry, int rx) {
+    if (rx > g.P[2]) return 0.f;
+    // dL/dS of one block entry; corrected descriptor: dL/dS_bar = A^T dL/dS_tilde (App. A
+    // map, transposed)
+    auto delta = [&](const float* src, const float* sub, int64_t k) {
+        float d = src[k] - (sub != nullptr ? sub[k] : 0.f);
+        if (c.tsum != nullptr) d = k == 0 ? d - c.q / (1.f - c.q) * *c.tsum : d / (1.f - c.q);
+        return d;
+    };
+    // r of the half window: block (a, b); -r of it: block (b, a) at r; r = 0 pairs the
+    // position with itself in both blocks (2 dL/dS(0) for a = b)
+    const int64_t k = canon_index(g, rz, ry, rx);
+    float d;
+    if (k == 0) d = delta(c.src, c.sub, 0) + delta(c.src2, c.sub2, 0);
+    else if (k > 0) d = delta(c.src, c.sub, k);
+    else d = delta(c.src2, c.sub2, canon_index(g, -rz, -ry, -rx));
+    return c.scale * (c.sc != nullptr ? c.sc->gscale : 1.f) * d;
+}
+
+// (A, B, C) = (-c1 G, (c1 - c3) G, c3 G) (f(x) = x: (G, 0, 0)) of shift m of a block of 8: a
+// block of GBLOCK = 48 floats stores (A, A, B, B) for m = 0..7 and then (C_m, C_m, C_m+1, C_m+1)
+// for even m, so that both halves of a packed pair get the same coefficient.
+template <bool IDENT>
+__device__ __forceinline__ void store_coef(const ThreshConst& tc, float v, float* blk, int m) {
+    const float A = IDENT ? v : -tc.c1 * v, B = IDENT ? 0.f : (tc.c1 - tc.c3) * v, C = IDENT ? 0.f : tc.c3 * v;
+    *reinterpret_cast<float4*>(blk + 4 * m) = make_float4(A, A, B, B);
+    *reinterpret_cast<float2*>(blk + gblock_c(m)) = make_float2(C, C);
+}
 
 // lastValid: shifts of the chunk's last rx block inside the window (T unless the chunk ends
 // the row and 2 P2 + 1 is not a multiple of T); block-uniform
@@ -640,7 +698,6 @@ __device__ __forceinline__ void corr_adj_block(const AdjSeg& sg, const int64_t l
     const LevelGeom g = sg.g;
     const float* __restrict__ field = sg.field;
     const float* __restrict__ tipf = sg.tip;
-    const float* __restrict__ Gd = sg.Gd;
     float* __restrict__ part = sg.part;
     extern __shared__ __align__(16) float smem[];
     const int lane = threadIdx.x & 31, strip = threadIdx.x >> 5;
@@ -694,7 +751,7 @@ __device__ __forceinline__ void corr_adj_block(const AdjSeg& sg, const int64_t l
         const int pairRows = 32 + ryN - 1;
         __syncthreads();
         const int64_t gz = wrap1(z + rz, n0);
-        // raw halo (pair rows i, i + 32) and the chunk's coefficient rows, copied asynchronously
+        // raw halo (pair rows i, i + 32) copied asynchronously; the chunk's coefficients meanwhile
         for (int i = warp; i < pairRows; i += NW) {
             const float* srcA = tipf + (gz * n1 + wrap1(y0 + ryS + i, n1)) * n2;
             const float* srcB = tipf + (gz * n1 + wrap1(y0 + ryS + i + 32, n1)) * n2;
@@ -707,10 +764,10 @@ __device__ __forceinline__ void corr_adj_block(const AdjSeg& sg, const int64_t l
                 while (gx >= n2) gx -= n2;
             }
         }
-        const float* grow0 = Gd + (((int64_t)(rz + g.P[0]) * (2 * g.P[1] + 1) + (ryS + g.P[1])) * g.NB + bbA) * GBLOCK;
-        for (int i = threadIdx.x; i < ryN * (rowG / 4); i += ADJ_THREADS) {
-            const int r = i / (rowG / 4), c = i - r * (rowG / 4);
-            cp_async16(Gs + r * rowG + 4 * c, grow0 + (int64_t)r * g.NB * GBLOCK + 4 * c);
+        for (int i = threadIdx.x; i < ryN * nbb * T; i += ADJ_THREADS) {
+            const int r = i / (nbb * T), c = i - r * (nbb * T);
+            const float v = coef_value(sg.c, g, rz, ryS + r, T * bbA + c - g.P[2]);
+            store_coef<IDENT>(tc, v, Gs + r * rowG + (c / T) * GBLOCK, c % T);
         }
         cp_async_wait_own();
         // every thread transforms the halo entries it copied
@@ -794,65 +851,24 @@ corr_adj_gated_kernel(const AdjSeg* __restrict__ segs, int nseg, int64_t total, 
     run_gated(segs, nseg, total, [&](const AdjSeg& sg, int64_t local) { corr_adj_block<false>(sg, local, tc); });
 }
 
-// Dense full-window coefficient grid of one level (one phase pair (a, b)), in adjoint order:
-//   G(r) = scale * (src[k] - sub[k]) for r in the half window (k its canonical index),
-//   G(r) = scale * (src2[k] - sub2[k]) for -r in it (k the index of -r),
-//   G(0) = scale * ((src - sub) + (src2 - sub2))[0]   (2 (src - sub)[0] for one field),
-//   scale = weight * (gscale from the loss, or 1) * (c1 alpha / N_l, or 1 / N_l for f(x)=x),
-//   (A, B, C) = (-c1 G, (c1 - c3) G, c3 G)   (f(x) = x: (G, 0, 0)),
-// zero where rx > P2 (padding of the last rx block).  Row (rz, ry) holds NB blocks of 8
-// shifts; a block of GBLOCK = 48 floats stores (A, A, B, B) for m = 0..7 and then
-// (C_m, C_m, C_m+1, C_m+1) for even m: both halves of a packed pair get the same coefficient.
-__device__ __forceinline__ void gcoef_block(const GSeg& sg, int64_t local, const ThreshConst& tc) {
-    const LevelGeom& g = sg.g;
-    const int WB = g.NB * T;
-    const int64_t total = (int64_t)(2 * g.P[0] + 1) * (2 * g.P[1] + 1) * WB;
-    const int64_t i = local * GCOEF_TH + threadIdx.x;
-    if (i >= total) return;
-    const int col = (int)(i % WB);
-    const int64_t row = i / WB;
-    const int ryi = (int)(row % (2 * g.P[1] + 1));
-    const int rzi = (int)(row / (2 * g.P[1] + 1));
-    const int rz = rzi - g.P[0], ry = ryi - g.P[1], rx = col - g.P[2];
-    float v = 0.f;
-    if (rx <= g.P[2]) {
-        // dL/dS of one block entry; corrected descriptor: dL/dS_bar = A^T dL/dS_tilde (App. A
-        // map, transposed)
-        auto delta = [&](const float* src, const float* sub, int64_t k) {
-            float d = src[k] - (sub != nullptr ? sub[k] : 0.f);
-            if (sg.tsum != nullptr) d = k == 0 ? d - sg.q / (1.f - sg.q) * *sg.tsum : d / (1.f - sg.q);
-            return d;
-        };
-        // r of the half window: block (a, b); -r of it: block (b, a) at r; r = 0 pairs the
-        // position with itself in both blocks (2 dL/dS(0) for a = b)
-        const int64_t k = canon_index(g, rz, ry, rx);
-        float d;
-        if (k == 0) d = delta(sg.src, sg.sub, 0) + delta(sg.src2, sg.sub2, 0);
-        else if (k > 0) d = delta(sg.src, sg.sub, k);
-        else d = delta(sg.src2, sg.sub2, canon_index(g, -rz, -ry, -rx));
-        v = sg.scale * (sg.sc != nullptr ? sg.sc->gscale : 1.f) * d;
-    }
-    const int b = col / T, m = col % T;
-    float A, B, C;
-    if (tc.identity) { A = v; B = 0.f; C = 0.f; }
-    else { A = -tc.c1 * v; B = (tc.c1 - tc.c3) * v; C = tc.c3 * v; }
-    float* blk = sg.Gd + (row * g.NB + b) * GBLOCK;
-    *reinterpret_cast<float4*>(blk + 4 * m) = make_float4(A, A, B, B);
-    *reinterpret_cast<float2*>(blk + gblock_c(m)) = make_float2(C, C);
-}
-
+// Dense full-window coefficient grid of an FFT level, row (rz, ry) holding NB blocks of 8 shifts.
 __global__ void gcoef_kernel(const GSeg* __restrict__ segs, int nseg, ThreshConst tc) {
     dep_wait();
     dep_trigger();
     const GSeg& sg = segs[find_segment(segs, nseg, (int64_t)blockIdx.x)];
     if (sg.done != nullptr && *sg.done) return;
-    gcoef_block(sg, (int64_t)blockIdx.x - sg.blockStart, tc);
-}
-
-__global__ void gcoef_gated_kernel(const GSeg* __restrict__ segs, int nseg, int64_t total, ThreshConst tc) {
-    dep_wait();
-    dep_trigger();
-    run_gated(segs, nseg, total, [&](const GSeg& sg, int64_t local) { gcoef_block(sg, local, tc); });
+    const LevelGeom& g = sg.g;
+    const int WB = g.NB * T;
+    const int64_t total = (int64_t)(2 * g.P[0] + 1) * (2 * g.P[1] + 1) * WB;
+    const int64_t i = ((int64_t)blockIdx.x - sg.blockStart) * GCOEF_TH + threadIdx.x;
+    if (i >= total) return;
+    const int col = (int)(i % WB);
+    const int64_t row = i / WB;
+    const int ryi = (int)(row % (2 * g.P[1] + 1)), rzi = (int)(row / (2 * g.P[1] + 1));
+    const float v = coef_value(sg.c, g, rzi - g.P[0], ryi - g.P[1], col - g.P[2]);
+    float* blk = sg.Gd + (row * g.NB + col / T) * GBLOCK;
+    if (tc.identity) store_coef<true>(tc, v, blk, col % T);
+    else store_coef<false>(tc, v, blk, col % T);
 }
 
 // ------------------------------------------------------------------------- launchers
@@ -895,7 +911,8 @@ void launch_corr_adj(const AdjSeg* segs, int nseg, int64_t blocks, size_t smem, 
     else launch_dep(corr_adj_kernel<false>, (unsigned)blocks, ADJ_THREADS, smem, s, segs, nseg, tc);
 }
 
-// resident blocks of a gated launch: as many as run at once (4 per SM; the small kernels 2)
+// blocks of a gated launch at most: enough for the hardware to balance them when the gate is
+// open, few enough to be dismissed in a few microseconds when it is not
 constexpr int64_t GATED_BLOCKS = 8192, GATED_SMALL = 8192;
 
 void launch_corr_fwd_gated(const FwdSeg* segs, int nseg, int64_t blocks, size_t smem, const ThreshConst& tc,
@@ -907,11 +924,6 @@ void launch_corr_fwd_gated(const FwdSeg* segs, int nseg, int64_t blocks, size_t 
 void launch_fwd_reduce_gated(const RedSeg* segs, int nseg, int64_t blocks, cudaStream_t s) {
     if (blocks <= 0) return;
     launch_dep(fwd_reduce_gated_kernel, (unsigned)std::min(blocks, GATED_SMALL), 256, 0, s, segs, nseg, blocks);
-}
-
-void launch_gcoef_gated(const GSeg* segs, int nseg, int64_t blocks, const ThreshConst& tc, cudaStream_t s) {
-    if (blocks <= 0) return;
-    launch_dep(gcoef_gated_kernel, (unsigned)std::min(blocks, GATED_SMALL), GCOEF_TH, 0, s, segs, nseg, blocks, tc);
 }
 
 void launch_corr_adj_gated(const AdjSeg* segs, int nseg, int64_t blocks, size_t smem, const ThreshConst& tc,

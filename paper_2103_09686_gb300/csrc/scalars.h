@@ -19,6 +19,7 @@ struct Scalars {
     int64_t adam_step;    // Adam steps taken (global, for bias correction)
     double b1t, b2t;      // beta1^adam_step, beta2^adam_step (running products)
     int err;              // set when a bounded tensor-core wait timed out (any kernel of the instance)
+    unsigned ticket;      // descriptor blocks finished so far (the last one finishes the loss, then resets it)
 };
 
 // Status of one instance after a run: a timed-out bounded wait outranks a non-finite loss

@@ -36,6 +36,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "loss.cuh"
 
 namespace dmcr {
 
@@ -1337,10 +1338,10 @@ __device__ __forceinline__ int half_index(const SepLevel& lv, int rz, int ry, in
 }  // namespace
 
 // item: (level, phases a, b); blocks: groups of rowsW window rows.  Inverse along x: the
-// entries of block (a, b).  With lv.fuse (one phase, a loss and its gradient in one call) a row
-// goes straight on: its residuals D - D_des are G up to the loss' factor gscale, which sep_mul
-// applies, so they are embedded and transformed here (the rows of sep_gx), and the block leaves
-// its share of sum (D - D_des)^2 and sum D_des^2.
+// entries of block (a, b); with a loss to evaluate, its share of the loss' sums too.  With
+// lv.fuse (one phase, a loss and its gradient in one call) a row goes straight on: its residuals
+// D - D_des are G up to the loss' factor gscale, which sep_mul applies, so they are embedded and
+// transformed here (the rows of sep_gx).
 __global__ void __launch_bounds__(SEP_THREADS, 2) sep_desc_kernel(const __grid_constant__ SepTables tb,
                                                                   const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
@@ -1357,11 +1358,6 @@ __global__ void __launch_bounds__(SEP_THREADS, 2) sep_desc_kernel(const __grid_c
     float* desc = lv.desc + (int64_t)pair * lv.Khalf;
     // Kahan sums of this thread's residuals and targets
     float r2 = 0.f, r2c = 0.f, t2 = 0.f, t2c = 0.f;
-    auto kahan = [](float& sum, float& comp, float v) {
-        const float y = v - comp, u = sum + y;
-        comp = (u - sum) - y;
-        sum = u;
-    };
     // writes the entry of (row l, rx) and returns the residual (0 outside the half window,
     // except at rx < 0 of row 0, the mirror of an entry of the same row)
     auto entry = [&](int l, int rx, float c) {
@@ -1373,11 +1369,11 @@ __global__ void __launch_bounds__(SEP_THREADS, 2) sep_desc_kernel(const __grid_c
         if (mirror) k = -rx;
         const float d = (float)(((double)c + dc) * lv.scaleD);
         if (!mirror) desc[k] = d;
-        if (!lv.fuse) return 0.f;
-        const float t = lv.sub[k], rho = d - t;
+        if (lv.loss == nullptr) return 0.f;
+        const float t = lv.sub[(int64_t)pair * lv.Khalf + k], rho = d - t;
         if (!mirror) {
-            kahan(r2, r2c, rho * rho);
-            kahan(t2, t2c, t * t);
+            kahan_add(r2, r2c, rho * rho);
+            kahan_add(t2, t2c, t * t);
         }
         return lv.scaleG * (k == 0 ? rho + rho : rho);
     };
@@ -1458,11 +1454,13 @@ __global__ void __launch_bounds__(SEP_THREADS, 2) sep_desc_kernel(const __grid_c
             }
         }
     }
-    if (!lv.fuse) return;
+    if (lv.loss == nullptr) return;
     // Kahan's (sum, comp) stands for sum - comp
     const DF R2 = block_sum_df(df_two_sum(r2, -r2c), dsh);
     const DF T2 = block_sum_df(df_two_sum(t2, -t2c), dsh);
-    if (threadIdx.x == 0) lv.sums[bk.block] = make_float4(R2.hi, R2.lo, T2.hi, T2.lo);
+    const int blocks = (R + lv.rowsW - 1) / lv.rowsW;
+    if (threadIdx.x == 0) lv.sums[lv.sumStart + pair * blocks + bk.block] = make_float4(R2.hi, R2.lo, T2.hi, T2.lo);
+    loss_arrive(*lv.loss, lv.arrive, dsh);
 }
 
 // item: (level, phases a, b); blocks: groups of rowsW window rows.  G(r) of the row (the
