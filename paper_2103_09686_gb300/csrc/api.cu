@@ -314,6 +314,7 @@ int64_t sep_v_rows(const LevelGeom& g) {
 // shape of one level for sep.cu (no pointers)
 bool sep_shape(const LevelGeom& g, int phases, int max_pairs, SepLevel& lv) {
     lv = SepLevel{};
+    if (g.N > SEP_MAX_POINTS) return false;
     for (int a = 0; a < 3; ++a)
         if (!sep_axis(g.n[a], lv.ax[a])) return false;
     lv.n0 = (int)g.n[0], lv.n1 = (int)g.n[1], lv.n2 = (int)g.n[2];
@@ -326,8 +327,8 @@ bool sep_shape(const LevelGeom& g, int phases, int max_pairs, SepLevel& lv) {
     lv.strideV = sep_v_rows(g) * g.n[2];
     lv.rowsF = sep_feature_rows(lv.ax[2], (int64_t)lv.n0 * lv.n1);
     lv.rowsW = sep_window_rows(lv.ax[2]);
-    lv.colsY = sep_cols(lv.ax[1], true);
-    lv.colsL = lv.n0 > 1 ? sep_cols(lv.ax[0], true) : sep_cols(lv.ax[1], false);
+    lv.colsY = sep_cols(lv.ax[1], true, phases);
+    lv.colsL = lv.n0 > 1 ? sep_cols(lv.ax[0], true, phases) : sep_cols(lv.ax[1], false, phases);
     return std::max(sep_smem_last(lv, true), sep_smem_feat(lv)) <= (size_t)SEP_MAX_SMEM;
 }
 
@@ -581,7 +582,7 @@ dmcr_status validate_and_plan(const dmcr_params* p, Plan& pl) {
             // spectra (separable) or partials (direct, for fields outside the separable ranges) -- a call uses one of the two
             const size_t pp = ph * ph;
             pl.o_spart[l] = o; o = align_up(o + ph * g.N * sizeof(float));
-            pl.o_sdc[l] = o; o = align_up(o + pp * sizeof(double));
+            pl.o_sdc[l] = o; o = align_up(o + pp * sizeof(float2));
             const size_t start = o;
             pl.o_z[l] = o; o = align_up(o + ph * pl.sep_pairs * g.N * sizeof(float2));
             pl.o_q[l] = pl.o_z[l];
@@ -820,7 +821,7 @@ void prepare_sep(const std::vector<Inst>& in, unsigned flags, const std::vector<
             lv.Q = reinterpret_cast<float2*>(x.ws + pl.o_q[l]);
             lv.U = reinterpret_cast<float2*>(x.ws + pl.o_u[l]);
             lv.V = reinterpret_cast<float2*>(x.ws + pl.o_v[l]);
-            lv.dc = reinterpret_cast<double*>(x.ws + pl.o_sdc[l]);
+            lv.dc = reinterpret_cast<float2*>(x.ws + pl.o_sdc[l]);
             lv.tier = reinterpret_cast<int*>(x.ws + pl.o_tier);
             lv.tiers = reinterpret_cast<int*>(x.ws + pl.o_tiers);
             lv.ntiers = prep_blocks(pl);

@@ -331,10 +331,11 @@ constexpr int SEP_BLOCK_PTS = 8 * SEP_THREADS;   // points a block holds in regi
 constexpr int SEP_ROW_THREADS = 256;   // threads of the feature and gradient kernels
 constexpr int SEP_SLOTS = 8;        // feature pairs a row block holds side by side at most
 constexpr int SEP_FAST_PHASES = 3;  // phases whose spectra fit behind the line buffers of sep_mul
-constexpr int SEP_MAX_DEG = 128;    // Chebyshev coefficients per feature at most
+constexpr int SEP_SEG = 8;          // segments of the value range per unit
+constexpr int SEP_MAX_NC = 14;      // coefficients of a feature in one segment at most
 constexpr int SEP_MAX_N = 2048;     // longest axis
+constexpr int64_t SEP_MAX_POINTS = 1 << 28;   // points of one grid (32-bit offsets)
 constexpr int SEP_MAX_RAD = 12;
-constexpr int COLOCC = 2;
 constexpr int SEP_OWN = 8;          // points of a column group one thread owns (at most 4096 per block)
 constexpr int SEP_MAX_SMEM = 222 * 1024;
 
@@ -353,8 +354,9 @@ __host__ __device__ inline int sep_pitch(int n, int L) {
 }
 
 struct SepTier {
-    float lo, hi, mid, inv_half;
-    int deg, npair, npos;     // coefficients per feature, packed pairs, the first npos of them with s = +1
+    float lo, hi;
+    int seg0, nseg, nc;       // first segment, segments, coefficients per segment
+    int npair, npos;          // packed pairs of features, the first npos of them with s = +1
     int coef;                 // offset of this tier's coefficients
 };
 
@@ -377,7 +379,7 @@ struct SepLevel {
     float2 *Z, *Q;            // spectra of the features, products: phases x maxPairs grids (one phase: Q = Z)
     float2 *U, *V;            // window spectra (3-D: [r0][y][x]; [row][x]), one per ordered phase pair
     int64_t strideU, strideV;
-    double* dc;               // sum_k s_k conj(Z^a_k(0)) Z^b_k(0) per phase pair
+    float2* dc;               // scaleD sum_k s_k conj(Z^a_k(0)) Z^b_k(0) per phase pair (hi, lo)
     int* tiers;               // tiers of the range blocks
     int ntiers;
     int* tier;                // the instance's tier
@@ -421,7 +423,7 @@ std::shared_ptr<const SepBasis> sep_basis(float alpha);
 const float2* sep_device_coef(const SepBasis& b);
 bool sep_axis(int64_t n, SepAxis& ax);
 double sep_axis_cost(const SepAxis& ax);
-int sep_cols(const SepAxis& ax, bool wide);
+int sep_cols(const SepAxis& ax, bool wide, int phases);
 int sep_window_rows(const SepAxis& ax);
 int sep_feature_rows(const SepAxis& ax, int64_t rows);
 size_t sep_smem_feat(const SepLevel& lv);

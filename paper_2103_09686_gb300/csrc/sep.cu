@@ -95,11 +95,13 @@ void jacobi_eigen(std::vector<double>& A, std::vector<double>& V, int n) {
     }
 }
 
-// One tier: eigenfunctions of F on [lo, hi], discretised at Chebyshev nodes, as Chebyshev
-// series.  False when SEP_MAX_PAIRS packed pairs of at most SEP_MAX_DEG coefficients do not
-// reach the tolerances (largest error of F and of dF/du over the range).
-bool build_tier(const PairFn& fn, double lo, double hi, double tolF, double tolFu, SepTier& t,
+// One tier: eigenfunctions of F on the range of the segments k0 .. k1 (segment k holds the
+// values within half a segment of k / SEP_SEG), discretised at Chebyshev nodes, as one short
+// polynomial per segment.  False when SEP_MAX_PAIRS packed pairs, or polynomials of SEP_MAX_NC
+// coefficients, do not reach the tolerances (largest error of F and of dF/du over the range).
+bool build_tier(const PairFn& fn, int k0, int k1, double tolF, double tolFu, SepTier& t,
                 std::vector<float2>& coef) {
+    const double lo = (k0 - 0.5) / SEP_SEG, hi = (k1 + 0.5) / SEP_SEG;
     const double mid = 0.5 * (lo + hi), half = 0.5 * (hi - lo);
     // nodes: the degree grows with the range measured in widths of the sigmoid
     const int n = (int)std::min(160.0, std::max(48.0, 24.0 + 2.6 * (hi - lo) * fn.a));
@@ -223,39 +225,72 @@ bool build_tier(const PairFn& fn, double lo, double hi, double tolF, double tolF
         if (eF < tolF && eD < tolFu) ok = true;
     }
     if (!ok) return false;
-    int deg = 4;
-    for (const auto* side : {&pos, &neg})
-        for (const auto& c : *side)
-            for (int j = 0; j < n; ++j)
-                if (fabs(c[j]) > 3e-10) deg = std::max(deg, j + 1);
-    if (deg > SEP_MAX_DEG) return false;
+    // local polynomials in u = SEP_SEG M - k, |u| <= 1/2: interpolation at SEP_MAX_NC + 4
+    // Chebyshev points, cut where the rest is below the rounding of the largest terms
+    constexpr int m = SEP_MAX_NC + 4;
+    const int nseg = k1 - k0 + 1, npos = (int)(pos.size() + 1) / 2, npair = npos + (int)(neg.size() + 1) / 2;
+    std::vector<double> local((size_t)2 * npair * nseg * m, 0.0);       // [feature][segment][power]
+    int nc = 4;
+    for (int side = 0; side < 2; ++side)
+        for (size_t k = 0; k < (side ? neg : pos).size(); ++k) {
+            const std::vector<double>& c = (side ? neg : pos)[k];
+            const size_t feature = (side ? 2 * npos : 0) + k;
+            for (int sg = 0; sg < nseg; ++sg) {
+                double y[m], ch[m];
+                for (int i = 0; i < m; ++i) {
+                    const double M = (k0 + sg + 0.5 * cos((i + 0.5) * M_PI / m)) / SEP_SEG, xx = (M - mid) / half;
+                    double b1 = 0.0, b2 = 0.0;                          // Clenshaw
+                    for (int q = n - 1; q >= 1; --q) {
+                        const double b0 = c[q] + 2.0 * xx * b1 - b2;
+                        b2 = b1, b1 = b0;
+                    }
+                    y[i] = c[0] + xx * b1 - b2;
+                }
+                for (int q = 0; q < m; ++q) {
+                    double v = 0.0;
+                    for (int i = 0; i < m; ++i) v += y[i] * cos(q * (i + 0.5) * M_PI / m);
+                    ch[q] = v * (q == 0 ? 1.0 : 2.0) / m;
+                    if (q < SEP_MAX_NC + 1 && fabs(ch[q]) > 3e-9) nc = std::max(nc, q + 1);
+                }
+                if (nc > SEP_MAX_NC) return false;
+                // Chebyshev in 2 u to powers of u, terms up to nc of this and later features alike
+                std::vector<double> t0(m, 0.0), t1(m, 0.0), pw(m, 0.0);
+                t0[0] = 1.0;
+                t1[1] = 2.0;
+                for (int q = 0; q < SEP_MAX_NC; ++q) {
+                    if (fabs(ch[q]) > 1e-13)
+                        for (int e = 0; e <= q; ++e) pw[e] += ch[q] * t0[e];
+                    std::vector<double> t2(m, 0.0);
+                    for (int e = 0; e + 1 < m; ++e) t2[e + 1] += 4.0 * t1[e];
+                    for (int e = 0; e < m; ++e) t2[e] -= t0[e];
+                    t0 = t1, t1 = t2;
+                }
+                for (int e = 0; e < m; ++e) local[(feature * nseg + sg) * m + e] = pw[e];
+            }
+        }
     t.lo = (float)lo;
     t.hi = (float)hi;
-    t.mid = (float)mid;
-    t.inv_half = (float)(1.0 / half);
-    t.deg = deg;
-    t.npos = (int)(pos.size() + 1) / 2;
-    t.npair = t.npos + (int)(neg.size() + 1) / 2;
+    t.seg0 = k0;
+    t.nseg = nseg;
+    t.nc = nc;
+    t.npos = npos;
+    t.npair = npair;
     t.coef = (int)coef.size();
-    // coefficients [deg][npair]: (feature 2p, feature 2p + 1); then j times them, the series of
-    // the derivatives in U_{j-1}
-    for (int der = 0; der < 2; ++der)
-        for (int j = 0; j < deg; ++j)
-            for (int p = 0; p < t.npair; ++p) {
-                const auto& side = p < t.npos ? pos : neg;
-                const size_t k = 2 * (size_t)(p < t.npos ? p : p - t.npos);
-                const double f = der ? (double)j : 1.0;
-                coef.push_back(make_float2((float)(f * side[k][j]), k + 1 < side.size() ? (float)(f * side[k + 1][j]) : 0.f));
-            }
+    // coefficients [power][pair][segment] of the features (2p, 2p + 1)
+    for (int e = 0; e < nc; ++e)
+        for (int p = 0; p < npair; ++p)
+            for (int sg = 0; sg < nseg; ++sg)
+                coef.push_back(make_float2((float)local[((size_t)(2 * p) * nseg + sg) * m + e],
+                                           (float)local[((size_t)(2 * p + 1) * nseg + sg) * m + e]));
     return true;
 }
 
 }  // namespace
 
-// The basis of one alpha.  The first range is a field between the phases with the overshoot of
-// a few optimiser steps; the penalty weakens as the loss falls, so fields of long runs spread
-// over the wider ones (measured over 3000 Adam steps: [-1.7, 1.9]).  A wider range needs more
-// features: 8, 10, 13, 15, 19, 25 packed pairs at alpha = 10.
+// The basis of one alpha.  The first range, [-1/16, 17/16], is a field between the phases with
+// the overshoot of an optimiser step or two; the penalty weakens as the loss falls, so fields of
+// long runs spread over the wider ones, up to [-2.3, 2.6] (measured over 3000 Adam steps:
+// [-1.7, 1.9]).  A wider range needs more features: 7 .. 25 packed pairs at alpha = 10.
 std::shared_ptr<const SepBasis> sep_basis(float alpha) {
     static std::mutex mu;
     static std::vector<std::shared_ptr<const SepBasis>>* cache = new std::vector<std::shared_ptr<const SepBasis>>();
@@ -269,8 +304,7 @@ std::shared_ptr<const SepBasis> sep_basis(float alpha) {
     auto b = std::make_shared<SepBasis>();
     b->alpha = alpha;
     const PairFn fn((double)alpha);
-    const double ranges[SEP_TIERS][2] = {{-0.0625, 1.0625}, {-0.25, 1.25}, {-0.5, 1.5},
-                                         {-1.0, 1.625},     {-1.5, 2.0},   {-2.25, 2.5}};
+    const int ranges[SEP_TIERS][2] = {{0, 8}, {-2, 10}, {-4, 12}, {-8, 13}, {-12, 16}, {-18, 20}};   // segments
     for (int t = 0; t < SEP_TIERS; ++t) {
         // below the FP32 rounding of a pair's value and derivative
         if (!build_tier(fn, ranges[t][0], ranges[t][1], t == 0 ? 1.5e-9 : 1e-8, 3e-7, b->tier[t],
@@ -288,7 +322,7 @@ std::shared_ptr<const SepBasis> sep_basis(float alpha) {
 // another stream is being captured); slots are never rewritten, so kernels and graphs may keep
 // reading them.  Null when there is no slot: the call uploads the coefficients with its tables.
 namespace {
-constexpr int SEP_SLOTS_DEV = 16, SEP_SLOT_LEN = 16384;
+constexpr int SEP_SLOTS_DEV = 8, SEP_SLOT_LEN = 24576;
 __device__ float2 g_sep_coef[SEP_SLOTS_DEV][SEP_SLOT_LEN];
 }  // namespace
 
@@ -380,14 +414,16 @@ int pow2_floor(int v) {
 }  // namespace
 
 // Adjacent columns of a strided axis per block.  A block holds SEP_BLOCK_PTS points of a power
-// of two: its remaining factor goes to feature pairs (or planes).  2-D grids stay in L2, where
-// 32-byte segments (4 columns) cost nothing and the narrow groups give more blocks; 3-D grids
-// stream from DRAM in 128-byte lines.
-int sep_cols(const SepAxis& ax, bool wide) {
+// of two: its remaining factor goes to feature pairs (or planes).  3-D grids take 16 columns
+// (128-byte lines).  2-D grids trade the width of their segments against the number of blocks:
+// 8 columns (64 bytes) where those fill the device -- long columns, several phases -- and 4
+// otherwise (256^2: sep_power 16.7 us with 4, 20.6 us with 8; nine phase pairs of 512^2: 213 and
+// 148 us; two columns, half a sector, took 43 us where four took 31).
+int sep_cols(const SepAxis& ax, bool wide, int phases) {
     const int n = ax.n;
     if (ax.fast) {
         const int lines = SEP_BLOCK_PTS / n;
-        const int narrow = std::max(4, lines / 8);       // at most 8 pairs side by side
+        const int narrow = std::max(n >= 512 || phases > 1 ? 8 : 4, lines / 8);   // at most 8 pairs side by side
         return std::min(std::min(lines, 16), wide ? 16 : narrow);
     }
     if (n > 1024) return 2;
@@ -538,6 +574,18 @@ template <bool WARP>
 __device__ __forceinline__ void line_sync() {
     if (WARP) __syncwarp();
     else __syncthreads();
+}
+
+// Hides a value from the optimiser: a loop over rounds recomputes the few addresses derived from
+// it instead of keeping dozens of them in registers (the column kernels spilled 800 bytes).
+__device__ __forceinline__ int opaque(int v) {
+    asm volatile("" : "+r"(v));
+    return v;
+}
+template <int N>
+__device__ __forceinline__ Line<N> opaque(Line<N> ln) {
+    ln.t = opaque(ln.t);
+    return ln;
 }
 
 template <int N, int Ns, bool WARP, int PAR>
@@ -760,69 +808,42 @@ __device__ __forceinline__ void for_pow2(int k, F&& body) {
 
 namespace {
 
-// The coefficients are read from global memory: all threads of a line read the same ones, and
-// the few kilobytes of a tier stay in L1.
-template <bool DERIV>
-__device__ __forceinline__ const float2* tier_coef(const SepTables& tb, const SepTier& t) {
-    return tb.coef + t.coef + (DERIV ? t.deg * t.npair : 0);
+// C values M of one line: their segments (offsets into the coefficient tables) and positions
+// u = SEP_SEG M - k in them, both exact.
+template <int C>
+__device__ __forceinline__ void locate(const SepTier& t, const float (&M)[C], int (&seg)[C], float (&u)[C]) {
+#pragma unroll
+    for (int e = 0; e < C; ++e) {
+        const float y = (float)SEP_SEG * M[e];
+        seg[e] = min(max(__float2int_rn(y) - t.seg0, 0), t.nseg - 1);
+        u[e] = y - (float)(seg[e] + t.seg0);
+    }
 }
 
-// One packed pair of features (DERIV: of their derivatives) at C normalised values:
-// sum_j c_j W_j(x), W = T_j (DERIV: U_{j-1}), both W_{j+1} = 2 x W_j - W_{j-1}.  The terms from
-// j = 4 on are summed first and the four large ones last, so that the small terms are not
-// lost against them.  Bound by the FP32 pipe: per term one FFMA2 and one FFMA.
+// One packed pair of features (DERIV: of their derivatives) at C located values: a polynomial
+// of nc coefficients per value, the coefficients of its segment gathered from global memory
+// (`cf`: those of the pair; step: from one power to the next).  The tables of a tier stay in
+// L1, a gather touches one or two lines, and the cost does not grow with the range.  Against
+// one Chebyshev series over the whole range (35 .. 127 terms) this takes 8 gathers and 7 FFMA2
+// per pair: the row kernels' instructions per point fell from 156 to about 75.
 template <bool DERIV, int C>
-__device__ __forceinline__ void eval_features(const float2* __restrict__ cf, int stride, int deg, const float (&x)[C],
-                                              float2 (&out)[C]) {
-    float x2[C], w0[C], w1[C];
+__device__ __forceinline__ void eval_features(const float2* __restrict__ cf, int step, int nc, const int (&seg)[C],
+                                              const float (&u)[C], float2 (&out)[C]) {
+    const float2* c = cf + (nc - 1) * step;
 #pragma unroll
     for (int e = 0; e < C; ++e) {
-        x2[e] = 2.f * x[e];
-        out[e] = make_float2(0.f, 0.f);
-        // W_3 and W_4
-        if (DERIV) {
-            w0[e] = fmaf(x2[e], x2[e], -1.f);               // U_2
-            w1[e] = fmaf(x2[e], w0[e], -x2[e]);             // U_3
-        } else {
-            const float t2 = fmaf(x2[e], x[e], -1.f);
-            w0[e] = fmaf(x2[e], t2, -x[e]);                 // T_3
-            w1[e] = fmaf(x2[e], w0[e], -t2);                // T_4
-        }
+        out[e] = __ldg(c + seg[e]);
+        if (DERIV) out[e] = __fmul2_rn(out[e], make_float2((float)(nc - 1), (float)(nc - 1)));
     }
-    const float2* c = cf + 4 * stride;
-    int j = 4;
-    for (; j + 1 < deg; j += 2, c += 2 * stride) {
-        const float2 ca = __ldg(c), cb = __ldg(c + stride);
+    for (int j = nc - 2; j >= (DERIV ? 1 : 0); --j) {
+        c -= step;
+        const float2 f = make_float2((float)j, (float)j);
 #pragma unroll
         for (int e = 0; e < C; ++e) {
-            out[e] = __ffma2_rn(ca, make_float2(w1[e], w1[e]), out[e]);
-            w0[e] = fmaf(x2[e], w1[e], -w0[e]);
-            out[e] = __ffma2_rn(cb, make_float2(w0[e], w0[e]), out[e]);
-            w1[e] = fmaf(x2[e], w0[e], -w1[e]);
+            float2 k = __ldg(c + seg[e]);
+            if (DERIV) k = __fmul2_rn(k, f);
+            out[e] = __ffma2_rn(out[e], make_float2(u[e], u[e]), k);
         }
-    }
-    if (j < deg) {
-        const float2 ca = __ldg(c);
-#pragma unroll
-        for (int e = 0; e < C; ++e) out[e] = __ffma2_rn(ca, make_float2(w1[e], w1[e]), out[e]);
-    }
-    const float2 c0 = __ldg(cf), c1 = __ldg(cf + stride), c2 = __ldg(cf + 2 * stride), c3 = __ldg(cf + 3 * stride);
-#pragma unroll
-    for (int e = 0; e < C; ++e) {
-        float a1, a2, a3;
-        if (DERIV) {
-            a1 = 1.f;
-            a2 = x2[e];
-            a3 = fmaf(x2[e], x2[e], -1.f);
-        } else {
-            a1 = x[e];
-            a2 = fmaf(x2[e], x[e], -1.f);
-            a3 = fmaf(x2[e], a2, -x[e]);
-        }
-        out[e] = __ffma2_rn(c3, make_float2(a3, a3), out[e]);
-        out[e] = __ffma2_rn(c2, make_float2(a2, a2), out[e]);
-        out[e] = __ffma2_rn(c1, make_float2(a1, a1), out[e]);
-        if (!DERIV) out[e] = __fadd2_rn(c0, out[e]);
     }
 }
 
@@ -871,7 +892,8 @@ __global__ void __launch_bounds__(SEP_ROW_THREADS, 4) sep_feat_kernel(const __gr
     if (lv.first && bk.a == 0 && bk.block == 0 && threadIdx.x == 0) *lv.tier = tier;
     if (tier >= SEP_TIERS) return;
     const SepTier& t = tb.tier[tier];
-    const float2* __restrict__ cf = tier_coef<false>(tb, t);
+    const float2* __restrict__ cf = tb.coef + t.coef;
+    const int step = t.npair * t.nseg;
     const int row0 = bk.block * lv.rowsF, rows = min(lv.rowsF, rowsN - row0);
     const float* __restrict__ field = lv.field + (int64_t)bk.a * lv.N + (int64_t)row0 * n;
     float2* __restrict__ Z = lv.Z + (int64_t)bk.a * lv.maxPairs * lv.N + (int64_t)row0 * n;
@@ -883,15 +905,16 @@ __global__ void __launch_bounds__(SEP_ROW_THREADS, 4) sep_feat_kernel(const __gr
             const Line<N> ln = row_line<N>(sm, line, threadIdx.x % S::T, S::LINES);
             for (int row = line / S::SLOTS; row < lv.rowsF; row += S::ROWS) {
                 const bool in = row < rows;
-                float x[8];
+                float x[8], u[8];
+                int seg[8];
 #pragma unroll
-                for (int e = 0; e < 8; ++e)
-                    x[e] = in ? (field[row * N + ln.t + e * S::T] - t.mid) * t.inv_half : 0.f;
+                for (int e = 0; e < 8; ++e) x[e] = in ? field[row * N + ln.t + e * S::T] : 0.f;
+                locate<8>(t, x, seg, u);
                 for (int p0 = 0; p0 < t.npair; p0 += S::SLOTS) {
                     const bool live = in && p0 + p < t.npair;
                     float2 v[8];
-                    if (live) eval_features<false, 8>(cf + p0 + p, t.npair, t.deg, x, v);
-                    p2_fft<N, S::WARP, 0>(v, ln);
+                    if (live) eval_features<false, 8>(cf + (p0 + p) * t.nseg, step, t.nc, seg, u, v);
+                    p2_fft<N, S::WARP, 0>(v, opaque(ln));
                     if (live) {
                         float2* out = Z + (int64_t)(p0 + p) * lv.N + row * N + ln.t;
 #pragma unroll
@@ -913,9 +936,12 @@ __global__ void __launch_bounds__(SEP_ROW_THREADS, 4) sep_feat_kernel(const __gr
         for (int e = threadIdx.x; e < rows * nc * n; e += blockDim.x) {
             const int q = fdiv(e, inv_n), i = e - q * n;        // q = l nc + c
             const int l = q / nc, c = q - l * nc;
-            const float x[1] = {(field[l * n + i] - t.mid) * t.inv_half};
+            const float x[1] = {field[l * n + i]};
+            float u[1];
+            int seg[1];
+            locate<1>(t, x, seg, u);
             float2 f[1];
-            eval_features<false, 1>(cf + p0 + c, t.npair, t.deg, x, f);
+            eval_features<false, 1>(cf + (p0 + c) * t.nseg, step, t.nc, seg, u, f);
             s.a[q * pitch + spad(i)] = f[0];
         }
         const float2* r = transform(lv.ax[2], s.a, s.b, s.tw, rows * nc, pitch);
@@ -974,11 +1000,13 @@ __device__ __forceinline__ ColGroup last_axis(const SepLevel& lv, int block, int
 
 __device__ __forceinline__ const SepAxis& last_ax(const SepLevel& lv) { return lv.n0 > 1 ? lv.ax[0] : lv.ax[1]; }
 
+// A thread's eight points of one grid.  Element offsets within a grid fit 32 bits (at most
+// SEP_MAX_POINTS points).
 template <int N>
 __device__ __forceinline__ void load8(const float2* __restrict__ src, const ColGroup& g, const Cols<N>& c, bool on,
                                       float2 (&v)[8]) {
-    const float2* p = src + g.base + c.ln.t * g.stride + c.l;
-    const int64_t step = (N / 8) * g.stride;
+    const int stride = opaque((int)g.stride), step = (N / 8) * stride;
+    const float2* p = src + (int)g.base + (c.ln.t * stride + c.l);
 #pragma unroll
     for (int e = 0; e < 8; ++e) v[e] = on && c.l < g.cols ? p[e * step] : make_float2(0.f, 0.f);
 }
@@ -986,8 +1014,8 @@ __device__ __forceinline__ void load8(const float2* __restrict__ src, const ColG
 template <int N>
 __device__ __forceinline__ void store8(float2* __restrict__ dst, const ColGroup& g, const Cols<N>& c, bool on,
                                        const float2 (&v)[8]) {
-    float2* p = dst + g.base + c.ln.t * g.stride + c.l;
-    const int64_t step = (N / 8) * g.stride;
+    const int stride = opaque((int)g.stride), step = (N / 8) * stride;
+    float2* p = dst + (int)g.base + (c.ln.t * stride + c.l);
     if (on && c.l < g.cols) {
 #pragma unroll
         for (int e = 0; e < 8; ++e) p[e * step] = v[e];
@@ -1009,7 +1037,7 @@ __device__ __forceinline__ void load_cols(const float2* __restrict__ src, const 
 // (level, phase a); blocks: groups of planes' columns (x fastest, then z).  A block walks the
 // feature pairs, loading the next pair's columns while it transforms the current ones.
 template <bool INVERSE>
-__global__ void __launch_bounds__(SEP_THREADS, COLOCC) sep_fft_y_kernel(const __grid_constant__ SepTables tb,
+__global__ void __launch_bounds__(SEP_THREADS, 2) sep_fft_y_kernel(const __grid_constant__ SepTables tb,
                                                                    const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
     if (!enter<true>(tb, items, nitem, bk, sep_smem, axis_y)) return;
@@ -1043,7 +1071,7 @@ __global__ void __launch_bounds__(SEP_THREADS, COLOCC) sep_fft_y_kernel(const __
 #pragma unroll
                 for (int e = 0; e < 8; ++e) v[e] = INVERSE ? swapf(nx[e]) : nx[e];
                 if (p + 1 < npair) load8<N>(grid + (int64_t)(p + 1) * lv.N, g, c, on, nx);
-                p2_fft<N, false, 0>(v, c.ln);
+                p2_fft<N, false, 0>(v, opaque(c.ln));
                 if (p2_exchanges(N) & 1) __syncthreads();
                 if (INVERSE) swap8(v);
                 store8<N>(grid + (int64_t)p * lv.N, g, c, on, v);
@@ -1072,11 +1100,19 @@ __global__ void __launch_bounds__(SEP_THREADS, COLOCC) sep_fft_y_kernel(const __
 
 // ------------------------------------------------------------------------- last axis: power
 
+namespace {
+// FP64 value as an FP32 pair
+__device__ __forceinline__ float2 split(double v) {
+    const float hi = (float)v;
+    return make_float2(hi, (float)(v - (double)hi));
+}
+}  // namespace
+
 // item: (level, phases a, b).  Sums s_k conj(Z^a_k) Z^b_k over the feature pairs and writes the
 // inverse along the last axis, cropped to r = 0 .. P (-r belongs to the pair (b, a)).  CROSS:
-// a and b may differ.  The next round's columns are loaded while the current one is transformed.
+// a and b may differ.
 template <bool CROSS>
-__global__ void __launch_bounds__(SEP_THREADS, CROSS ? 1 : COLOCC)
+__global__ void __launch_bounds__(SEP_THREADS, CROSS ? 1 : 2)
 sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
     __shared__ double dcs[SEP_THREADS / 2];
@@ -1101,34 +1137,43 @@ sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict
             constexpr int N = decltype(cc)::value, T = N / 8;
             constexpr int PAR1 = p2_exchanges(N) & 1;
             const Cols<N> c(g.L);
+            // one phase: the eight sums of a thread wait in shared memory (its own words), which
+            // keeps the transform's 64 registers free of spills
+            float* own = reinterpret_cast<float*>(sm + N + 2 * c.slots * c.L * sep_pitch(N, c.L)) + threadIdx.x;
             float2 acc[8];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) acc[e] = make_float2(0.f, 0.f);
+            for (int e = 0; e < 8; ++e) {
+                if (CROSS) acc[e] = make_float2(0.f, 0.f);
+                else own[e * SEP_THREADS] = 0.f;
+            }
             double dc = 0.0;
             const bool has_dc = dc_block && c.l == 0 && c.ln.t == 0;
-            float2 nx[8];
-            load8<N>(Za + (int64_t)c.slot * lv.N, g, c, c.slot < t.npair, nx);
             for (int p0 = 0; p0 < t.npair; p0 += c.slots) {
                 const int p = p0 + c.slot;
                 const float sg = p < t.npos ? 1.f : -1.f;
                 float2 v[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) v[e] = nx[e];
-                if (!cross) {
-                    const int q = p + c.slots;
-                    if (p0 + c.slots < t.npair) load8<N>(Za + (int64_t)q * lv.N, g, c, q < t.npair, nx);
-                    p2_fft<N, false, 0>(v, c.ln);
+                load8<N>(Za + (int64_t)p * lv.N, g, c, p < t.npair, v);
+                if (!CROSS) {
+                    p2_fft<N, false, 0>(v, opaque(c.ln));
                     if (PAR1 != 0) __syncthreads();   // the next round starts in buffer 0 again
                     if (lv.keep) store8<N>(Zw + (int64_t)p * lv.N, g, c, p < t.npair, v);
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) acc[e].x = fmaf(sg, fmaf(v[e].x, v[e].x, v[e].y * v[e].y), acc[e].x);
+                    for (int e = 0; e < 8; ++e)
+                        own[e * SEP_THREADS] = fmaf(sg, fmaf(v[e].x, v[e].x, v[e].y * v[e].y), own[e * SEP_THREADS]);
+                    if (has_dc) dc += (double)sg * ((double)v[0].x * v[0].x + (double)v[0].y * v[0].y);
+                } else if (!cross) {
+                    p2_fft<N, false, 0>(v, opaque(c.ln));
+                    if (PAR1 != 0) __syncthreads();
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        acc[e].x = fmaf(sg, __fadd_rn(__fmul_rn(v[e].x, v[e].x), __fmul_rn(v[e].y, v[e].y)), acc[e].x);
                     if (has_dc) dc += (double)sg * ((double)v[0].x * v[0].x + (double)v[0].y * v[0].y);
                 } else {
                     float2 u[8];
                     load8<N>(Zb + (int64_t)p * lv.N, g, c, p < t.npair, u);
-                    p2_fft<N, false, 0>(v, c.ln);
+                    p2_fft<N, false, 0>(v, opaque(c.ln));
                     if (PAR1 != 0) __syncthreads();
-                    p2_fft<N, false, 0>(u, c.ln);
+                    p2_fft<N, false, 0>(u, opaque(c.ln));
                     if (PAR1 != 0) __syncthreads();
                     // conj(v) u; the imaginary part as a difference of rounded products, so that
                     // exchanging a and b gives exactly the conjugate
@@ -1138,9 +1183,11 @@ sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict
                         acc[e].y = fmaf(sg, __fsub_rn(__fmul_rn(v[e].x, u[e].y), __fmul_rn(v[e].y, u[e].x)), acc[e].y);
                     }
                     if (has_dc) dc += (double)sg * ((double)v[0].x * u[0].x + (double)v[0].y * u[0].y);
-                    const int q = p + c.slots;
-                    if (p0 + c.slots < t.npair) load8<N>(Za + (int64_t)q * lv.N, g, c, q < t.npair, nx);
                 }
+            }
+            if (!CROSS) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) acc[e] = make_float2(own[e * SEP_THREADS], 0.f);
             }
             // sum over the slots in a fixed order; the mean's power goes on in FP64
             if (has_dc) dcs[c.slot] = dc;
@@ -1162,11 +1209,11 @@ sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict
             if (has_dc && c.slot == 0) {
                 double s = dcs[0];
                 for (int k = 1; k < c.slots; ++k) s += dcs[k];
-                lv.dc[pair] = s;
+                lv.dc[pair] = split(s * lv.scaleD);
             }
             if (has_dc) acc[0] = make_float2(0.f, 0.f);
             swap8(acc);
-            p2_fft<N, false, 0>(acc, c.ln);
+            p2_fft<N, false, 0>(acc, opaque(c.ln));
             if (c.slot == 0 && c.l < g.cols) {
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
@@ -1215,7 +1262,7 @@ sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict
         });
     }
     if (has_dc) {
-        lv.dc[pair] = dc;
+        lv.dc[pair] = split(dc * lv.scaleD);
         acc[0] = make_float2(0.f, 0.f);
     }
     __syncthreads();
@@ -1266,7 +1313,7 @@ __global__ void __launch_bounds__(SEP_THREADS, 2) sep_win_y_kernel(const __grid_
                 const int i = c.ln.t + e * T;
                 v[e] = !on ? make_float2(0.f, 0.f) : (DESC ? swapf(u[(int64_t)i * lv.n2]) : window(w, i, lv.n2));
             }
-            p2_fft<N, false, 0>(v, c.ln);
+            p2_fft<N, false, 0>(v, opaque(c.ln));
             if (!on) return;
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
@@ -1354,7 +1401,8 @@ __global__ void __launch_bounds__(SEP_THREADS, 2) sep_desc_kernel(const __grid_c
     const int row0 = bk.block * lv.rowsW, rows = min(lv.rowsW, R - row0);
     const int pair = bk.a * lv.phases + bk.b;
     float2* V = lv.V + (int64_t)pair * lv.strideV + (int64_t)row0 * n;
-    const double dc = lv.dc[pair];
+    const float2 dc = lv.dc[pair];
+    const float scaleD = (float)lv.scaleD;
     float* desc = lv.desc + (int64_t)pair * lv.Khalf;
     // Kahan sums of this thread's residuals and targets
     float r2 = 0.f, r2c = 0.f, t2 = 0.f, t2c = 0.f;
@@ -1367,7 +1415,7 @@ __global__ void __launch_bounds__(SEP_THREADS, 2) sep_desc_kernel(const __grid_c
         const bool mirror = k < 0 && rz == 0 && ry == 0;
         if (k < 0 && !(lv.fuse && mirror)) return 0.f;
         if (mirror) k = -rx;
-        const float d = (float)(((double)c + dc) * lv.scaleD);
+        const float d = dc.x + fmaf(c, scaleD, dc.y);
         if (!mirror) desc[k] = d;
         if (lv.loss == nullptr) return 0.f;
         const float t = lv.sub[(int64_t)pair * lv.Khalf + k], rho = d - t;
@@ -1565,7 +1613,7 @@ struct GCols {
 // forward transform of the columns, the product sum_b conj(G^ab) Z^b and the inverse: Q^a, in
 // place of Z for a single phase (G is even then: a real spectrum).
 template <bool MULTI>
-__global__ void __launch_bounds__(SEP_THREADS, MULTI ? 1 : COLOCC)
+__global__ void __launch_bounds__(SEP_THREADS, MULTI ? 1 : 2)
 sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
     if (!enter<true>(tb, items, nitem, bk, sep_smem, axis_x)) return;
@@ -1584,21 +1632,19 @@ sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__
             const Cols<N> c(g.L);
             // MULTI: every phase's spectrum, this thread's points, behind the line buffers
             float2* gs = sep_smem + N + 2 * c.slots * c.L * sep_pitch(N, c.L) + threadIdx.x;
-            float gr[8];
-            float2 nx[8];
-            if (!MULTI) load8<N>(lv.Z + (int64_t)c.slot * lv.N, g, c, c.slot < t.npair, nx);
+            float* gr = reinterpret_cast<float*>(sm + N + 2 * c.slots * c.L * sep_pitch(N, c.L)) + threadIdx.x;
             for (int b = 0; b < lv.phases; ++b) {
                 const GCols gc(lv, bk.a, b, g);
                 float2 v[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e)
                     v[e] = c.l < g.cols ? gc.at(c.ln.t + e * T, c.l) : make_float2(0.f, 0.f);
-                p2_fft<N, false, 0>(v, c.ln);
+                p2_fft<N, false, 0>(v, opaque(c.ln));
                 if (PAR1) __syncthreads();
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     if (MULTI) gs[(b * 8 + e) * SEP_THREADS] = make_float2(norm * v[e].x, -norm * v[e].y);
-                    else gr[e] = norm * v[e].x;
+                    else gr[e * SEP_THREADS] = norm * v[e].x;
                 }
             }
             for (int p0 = 0; p0 < t.npair; p0 += c.slots) {
@@ -1606,17 +1652,17 @@ sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__
                 const bool on = p < t.npair;
                 float2 v[8];
                 if (!MULTI) {
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) v[e] = nx[e];
-                    const int q = p + c.slots;
-                    if (p0 + c.slots < t.npair) load8<N>(lv.Z + (int64_t)q * lv.N, g, c, q < t.npair, nx);
+                    load8<N>(lv.Z + (int64_t)p * lv.N, g, c, on, v);
                     if (!lv.keep) {              // else sep_power left the spectra
-                        p2_fft<N, false, 0>(v, c.ln);
+                        p2_fft<N, false, 0>(v, opaque(c.ln));
                         if (PAR1) __syncthreads();
                     }
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) v[e] = make_float2(gr[e] * v[e].y, gr[e] * v[e].x);
-                    p2_fft<N, false, 0>(v, c.ln);
+                    for (int e = 0; e < 8; ++e) {
+                        const float w = gr[e * SEP_THREADS];
+                        v[e] = make_float2(w * v[e].y, w * v[e].x);
+                    }
+                    p2_fft<N, false, 0>(v, opaque(c.ln));
                     if (PAR1) __syncthreads();
                 } else {
                     float2 acc[8];
@@ -1624,7 +1670,7 @@ sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__
                     for (int e = 0; e < 8; ++e) acc[e] = make_float2(0.f, 0.f);
                     for (int b = 0; b < lv.phases; ++b) {
                         load8<N>(lv.Z + ((int64_t)b * lv.maxPairs + p) * lv.N, g, c, on, v);
-                        p2_fft<N, false, 0>(v, c.ln);
+                        p2_fft<N, false, 0>(v, opaque(c.ln));
                         if (PAR1) __syncthreads();
 #pragma unroll
                         for (int e = 0; e < 8; ++e) {
@@ -1635,7 +1681,7 @@ sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__
                     }
 #pragma unroll
                     for (int e = 0; e < 8; ++e) v[e] = swapf(acc[e]);
-                    p2_fft<N, false, 0>(v, c.ln);
+                    p2_fft<N, false, 0>(v, opaque(c.ln));
                     if (PAR1) __syncthreads();
                 }
                 swap8(v);
@@ -1702,7 +1748,8 @@ __global__ void __launch_bounds__(SEP_ROW_THREADS, 3) sep_grad_kernel(const __gr
     const SepLevel& lv = bk.lv;
     float2* sm = sep_smem;
     const SepTier& t = tb.tier[bk.tier];
-    const float2* __restrict__ cf = tier_coef<true>(tb, t);
+    const float2* __restrict__ cf = tb.coef + t.coef;
+    const int step = t.npair * t.nseg;
     const int rowsN = lv.n0 * lv.n1, n = lv.n2;
     const int row0 = bk.block * lv.rowsF, rows = min(lv.rowsF, rowsN - row0);
     const float* __restrict__ field = lv.field + (int64_t)bk.a * lv.N + (int64_t)row0 * n;
@@ -1728,22 +1775,23 @@ __global__ void __launch_bounds__(SEP_ROW_THREADS, 3) sep_grad_kernel(const __gr
                     const float2* src = Q + (int64_t)(p0 + p) * lv.N + row * N + ln.t;
 #pragma unroll
                     for (int e = 0; e < 8; ++e) v[e] = live ? swapf(src[e * S::T]) : make_float2(0.f, 0.f);
-                    p2_fft<N, S::WARP, 0>(v, ln);
+                    p2_fft<N, S::WARP, 0>(v, opaque(ln));
                     if (live) {
-                        const float sg = p0 + p < t.npos ? t.inv_half : -t.inv_half;
-                        // four positions at a time: the series' state of eight does not fit the registers
+                        const float sg = p0 + p < t.npos ? (float)SEP_SEG : -(float)SEP_SEG;
+                        // four positions at a time, located anew in every round: the state of eight
+                        // does not fit the registers
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            float x[4];
+                        for (int h = 0; h < 8; h += 4) {
+                            float x[4], u[4];
+                            int seg[4];
                             float2 f[4];
 #pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                x[e] = (field[row * N + ln.t + (4 * h + e) * S::T] - t.mid) * t.inv_half;
-                            eval_features<true, 4>(cf + p0 + p, t.npair, t.deg, x, f);
+                            for (int e = 0; e < 4; ++e) x[e] = field[row * N + ln.t + (h + e) * S::T];
+                            locate<4>(t, x, seg, u);
+                            eval_features<true, 4>(cf + (p0 + p) * t.nseg, step, t.nc, seg, u, f);
 #pragma unroll
                             for (int e = 0; e < 4; ++e)
-                                g[4 * h + e] =
-                                    fmaf(sg, fmaf(f[e].x, v[4 * h + e].y, f[e].y * v[4 * h + e].x), g[4 * h + e]);
+                                g[h + e] = fmaf(sg, fmaf(f[e].x, v[h + e].y, f[e].y * v[h + e].x), g[h + e]);
                         }
                     }
                     if (p2_exchanges(N) & 1) line_sync<S::WARP>();
@@ -1791,12 +1839,15 @@ __global__ void __launch_bounds__(SEP_ROW_THREADS, 3) sep_grad_kernel(const __gr
             const int e = threadIdx.x + q * SEP_ROW_THREADS;
             if (e < rows * n) {
                 const int l = fdiv(e, inv_n), i = e - l * n;
-                const float x[1] = {(field[e] - t.mid) * t.inv_half};
+                const float x[1] = {field[e]};
+                float u[1];
+                int seg[1];
+                locate<1>(t, x, seg, u);
                 for (int c = 0; c < nc; ++c) {
                     float2 f[1];
-                    eval_features<true, 1>(cf + p0 + c, t.npair, t.deg, x, f);
+                    eval_features<true, 1>(cf + (p0 + c) * t.nseg, step, t.nc, seg, u, f);
                     const float2 v = r[(l * nc + c) * pitch + spad(i)];
-                    g[q] = fmaf(p0 + c < t.npos ? t.inv_half : -t.inv_half, fmaf(f[0].x, v.y, f[0].y * v.x), g[q]);
+                    g[q] = fmaf(p0 + c < t.npos ? (float)SEP_SEG : -(float)SEP_SEG, fmaf(f[0].x, v.y, f[0].y * v.x), g[q]);
                 }
             }
         }
@@ -1838,6 +1889,7 @@ size_t sep_smem_last(const SepLevel& lv, bool mul) {
     const SepAxis& ax = lv.n0 > 1 ? lv.ax[0] : lv.ax[1];
     const int lines = ax.fast ? SEP_BLOCK_PTS / ax.n : lv.colsL;
     size_t b = bytes_of(ax.n, lines, sep_pitch(ax.n, lv.colsL));
+    if (ax.fast && lv.phases == 1) b += (size_t)SEP_BLOCK_PTS * sizeof(float);      // a thread's own eight values
     if (mul) {
         if (!ax.fast || lv.phases > SEP_FAST_PHASES) b = bytes_of(ax.n, lv.colsL, sep_pitch(ax.n, lv.colsL)) +
                                                          (size_t)lv.phases * lv.colsL * ax.n * sizeof(float2);
