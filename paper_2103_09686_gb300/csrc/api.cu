@@ -335,36 +335,45 @@ bool sep_shape(const LevelGeom& g, int phases, int max_pairs, SepLevel& lv) {
 // The separable path for the soft threshold's two-point descriptor: when a basis of this
 // alpha exists, every axis of every level can be transformed, its buffers stay moderate and
 // the direct kernels are estimated to be slower in each of the three kinds of call.  All levels
-// of an instance or none.  Seconds, fitted to GB300 measurements of both paths (2-D 64^2 ..
-// 2048^2, 3-D 32^3 .. 160^3, windows 2 .. 64; captured calls, GPU time): e.g. loss and gradient
-// at 256^2, +-32, 3 levels 201 us direct and 82 us separable, 64^2, +-16: 45 and 57 us;
-// 128^3, +-4: 883 and 575 us, 128^3, +-2: 530 and 572 us; 600^2 (8 * 3 * 5^2), +-16: 211 and
-// 321 us.  The separable cost of a tier grows with its feature pairs (7 in the narrowest), so
-// wide ranges are left to the direct kernels where the window is small.
+// of an instance or none, and one path for every kind of call (the loss of a field that equals
+// its target is exactly 0).  Seconds, fitted to GB300 measurements of both paths (2-D 16^2 ..
+// 2048^2, 3-D 16^3 .. 160^3, windows 2 .. 64; captured calls, GPU time), the direct kernels with
+// the padding of their 64 x 32 (adjoint) and 32-wide (forward) tiles.  Loss and gradient, direct
+// and separable: 64^2, +-16: 41 and 49 us; 128^2, +-32, 2 levels: 112 and 57 us; 512^2, +-8: 118
+// and 126 us; 512^2, +-16: 160 and 127 us; 48^3, +-8: 413 and 232 us; 128^3, +-2: 525 and 502 us
+// (its VJP 187 and 407 us); 600^2 (8 * 3 * 5^2), +-16: 207 and 326 us, +-48: 1032 and 328 us.  The
+// separable cost of a tier grows with its feature pairs (7 in the narrowest), so wide ranges
+// are left to the direct kernels where the window is small.
 bool choose_sep(const dmcr_params* p, Plan& pl) {
     if (p->path != DMCR_PATH_AUTO || p->threshold != DMCR_SOFT || pl.desc_kind == DMCR_DESC_S3) return false;
     const double ph = pl.phases;
-    double pairs = 0.0, bytes = 0.0, points = 0.0, N = 0.0;
+    double fwd = 0.0, adj = 0.0, bytes = 0.0, points = 0.0, N = 0.0;
+    bool fast = true;
     for (int l = 0; l < pl.levels; ++l) {
         const LevelGeom& g = pl.g[l];
         SepLevel lv;
         if (!sep_shape(g, pl.phases, SEP_MAX_PAIRS, lv)) return false;
-        pairs += ph * ph * (double)g.N * (double)g.Khalf;
+        const double pairs = ph * ph * (double)g.N * (double)g.Khalf;
+        const double padx = (double)(g.tilesX * TX) / (double)g.n[2];
+        fwd += pairs * padx;
+        adj += pairs * padx * (double)(g.adjTilesY * ADJ_ROWS) / (double)g.n[1];
         bytes += 8.0 * (double)g.N * ph * (pl.phases > 1 ? 2 : 1);
         double per = 0.0;
         for (int a = 0; a < 3; ++a)
-            if (g.n[a] > 1) per += sep_axis_cost(lv.ax[a]);
+            if (g.n[a] > 1) per += sep_axis_cost(lv.ax[a]), fast = fast && lv.ax[a].fast;
         points += ph * (double)g.N * per;
         N += ph * ph * (double)g.N;
     }
     const bool d3 = pl.g[0].n[0] > 1;
-    const double direct_lg = 4.0e-5 + 5.7e-13 * pairs + (d3 ? 2.2e-10 : 1.2e-10) * N;
-    const double direct_d = 1.4e-5 + 1.55e-13 * pairs + (d3 ? 1.2e-10 : 0.8e-10) * N;
-    const double direct_v = 2.4e-5 + 4.1e-13 * pairs + 0.6e-10 * N;
+    const double direct_lg = 4.0e-5 + 1.55e-13 * fwd + 4.15e-13 * adj + (d3 ? 2.2e-10 : 1.2e-10) * N;
+    const double direct_d = 1.4e-5 + 1.55e-13 * fwd + (d3 ? 1.2e-10 : 0.8e-10) * N;
+    const double direct_v = 2.2e-5 + 4.15e-13 * adj + 0.6e-10 * N;
+    // start-up of the chain of kernels; lengths that are no power of two run more, slower stages
+    const double start = fast ? 1.0 : 2.2;
     auto worth = [&](int npair) {
         const double w = points * npair / 7.0;
-        return bytes * npair <= 16e9 && direct_lg > 1.1 * (5.5e-5 + w) && direct_d > 2.8e-5 + 0.45 * w &&
-               direct_v > 3.7e-5 + 0.8 * w;
+        return bytes * npair <= 16e9 && direct_lg > 1.03 * (4.9e-5 * start + w) && direct_d > 2.5e-5 * start + 0.5 * w &&
+               direct_v > 3.3e-5 * start + 0.8 * w;
     };
     if (!worth(1)) return false;
     pl.basis = sep_basis(p->alpha);

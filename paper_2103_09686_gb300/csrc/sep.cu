@@ -1616,7 +1616,7 @@ template <bool MULTI>
 __global__ void __launch_bounds__(SEP_THREADS, MULTI ? 1 : 2)
 sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
-    if (!enter<true>(tb, items, nitem, bk, sep_smem, axis_x)) return;
+    if (!enter<true>(tb, items, nitem, bk, sep_smem, axis_last)) return;
     const SepLevel& lv = bk.lv;
     float2* sm = sep_smem;
     const SepTier& t = tb.tier[bk.tier];
