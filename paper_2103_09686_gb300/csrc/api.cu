@@ -384,7 +384,7 @@ bool choose_sep(const dmcr_params* p, Plan& pl) {
     return pl.sep_tiers > 0;
 }
 
-dmcr_status validate_and_plan(const dmcr_params* p, Plan& pl) {
+dmcr_status make_plan(const dmcr_params* p, Plan& pl) {
     if (p == nullptr) return fail(DMCR_EINVAL, "params is NULL");
     if (p->ndim != 2 && p->ndim != 3) return fail(DMCR_EINVAL, "ndim must be 2 or 3 (got %d)", p->ndim);
     if (p->levels < 1 || p->levels > MAX_LEVELS)
@@ -610,6 +610,49 @@ dmcr_status validate_and_plan(const dmcr_params* p, Plan& pl) {
         pl.o_adj[l] = o; o = align_up(o + ph * ph * g.nChunks * g.N * sizeof(float));
     }
     pl.bytes = o;
+    return DMCR_OK;
+}
+
+// Plans of the last few problems of this thread, by the parameters' values: a call plans the
+// same problem two or three times (descriptor length, workspace size, the call itself), and
+// programs alternate between few problems.  A plan holds sizes and offsets only; a rejected
+// problem is planned anew every time.  (4 us per planning on the host.)
+dmcr_status validate_and_plan(const dmcr_params* p, Plan& pl) {
+    struct Entry {
+        dmcr_params key;
+        Plan plan;
+        uint64_t used = 0;
+    };
+    constexpr size_t KEEP = 8;
+    static thread_local std::vector<Entry> cache;
+    static thread_local uint64_t clock = 0;
+    if (p == nullptr) return make_plan(p, pl);
+    // field by field: the struct has padding, and a NaN never equals itself
+    auto same = [](const dmcr_params& a, const dmcr_params& b) {
+        bool eq = a.ndim == b.ndim && a.levels == b.levels && a.threshold == b.threshold && a.alpha == b.alpha &&
+                  a.level_weight_exp == b.level_weight_exp && a.path == b.path && a.descriptor == b.descriptor &&
+                  a.phases == b.phases;
+        for (int i = 0; i < 3; ++i) eq = eq && a.n[i] == b.n[i] && a.window[i] == b.window[i];
+        for (int i = 0; i < 4; ++i) eq = eq && a.tune[i] == b.tune[i];
+        return eq;
+    };
+    for (Entry& e : cache)
+        if (same(e.key, *p)) {
+            e.used = ++clock;
+            pl = e.plan;
+            return DMCR_OK;
+        }
+    DMCR_TRY(make_plan(p, pl));
+    Entry* slot = nullptr;
+    if (cache.size() < KEEP) {
+        cache.emplace_back();
+        slot = &cache.back();
+    } else {
+        slot = &*std::min_element(cache.begin(), cache.end(), [](const Entry& a, const Entry& b) { return a.used < b.used; });
+    }
+    slot->key = *p;
+    slot->plan = pl;
+    slot->used = ++clock;
     return DMCR_OK;
 }
 
