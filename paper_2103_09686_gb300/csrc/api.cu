@@ -139,7 +139,8 @@ struct Plan {
     // workspace offsets (bytes)
     size_t o_tab = 0, tab_bytes = 0, o_scal = 0, o_pen = 0, o_desc = 0, o_pyr[MAX_LEVELS] = {},
            o_fwd[MAX_LEVELS] = {}, o_gd[MAX_LEVELS] = {}, o_adj[MAX_LEVELS] = {};
-    // FFT levels: two complex FP64 grids, twiddles of the three axes, one FP64 scalar
+    // FFT levels: the field's FP64 half spectrum, the window's planes and rows, twiddles of the
+    // three axes, scalars
     size_t o_fx[MAX_LEVELS] = {}, o_fh[MAX_LEVELS] = {}, o_tw[MAX_LEVELS] = {}, o_dc[MAX_LEVELS] = {};
     bool any_fft = false;
     double fh2 = 0.0;          // f(1/2)^2 of the soft threshold (App. A mapping of the FFT path)
@@ -182,6 +183,29 @@ bool fft_cheaper(const LevelGeom& g) {
     const double t_direct = (double)g.N * kfull * 1.481e-13 + (double)g.N * 1.266e-10 + 1.506e-4;
     const double t_fft = (double)g.N * 7.577e-10 + 1.568e-4;
     return t_fft < t_direct;
+}
+
+// sizes of one FFT level (no pointers)
+FftArgs fft_shape(const LevelGeom& g) {
+    FftArgs a;
+    memset(&a, 0, sizeof a);       // padding too: the arguments are part of the graph keys
+    a.n0 = (int)g.n[0], a.n1 = (int)g.n[1], a.n2 = (int)g.n[2];
+    a.nh = a.n2 / 2 + 1;
+    a.P0 = g.P[0], a.P1 = g.P[1], a.P2 = g.P[2];
+    a.NB = g.NB;
+    a.N = g.N;
+    fft_axis(a.n0, a.ax[0]);
+    fft_axis(a.n1, a.ax[1]);
+    fft_axis(a.n2, a.ax[2]);
+    a.Lx = fft_lines_per_block(a.n2, false);
+    a.Ly = fft_lines_per_block(a.n1, true);
+    a.Ll = fft_lines_per_block(a.n0 > 1 ? a.n0 : a.n1, true);
+    a.nsq = fft_row_blocks(a);
+    return a;
+}
+int64_t fft_u_len(const FftArgs& a) { return a.n0 > 1 ? (int64_t)(a.P0 + 1) * a.n1 * a.nh : 0; }
+int64_t fft_v_len(const FftArgs& a) {
+    return (a.n0 > 1 ? (int64_t)(a.P0 + 1) * (2 * a.P1 + 1) : a.P1 + 1) * (int64_t)a.nh;
 }
 
 // Upper bound of the segment-table bytes of one instance (every phase, 16-B aligned arrays).
@@ -571,10 +595,11 @@ dmcr_status make_plan(const dmcr_params* p, Plan& pl) {
         const size_t ph = (size_t)pl.phases;
         if (l > 0) { pl.o_pyr[l] = o; o = align_up(o + ph * g.N * sizeof(float)); }
         if (g.fft) {
-            pl.o_fx[l] = o; o = align_up(o + (size_t)g.N * 16);
-            pl.o_fh[l] = o; o = align_up(o + (size_t)g.N * 16);
+            const FftArgs a = fft_shape(g);
+            pl.o_fx[l] = o; o = align_up(o + (size_t)g.n[0] * g.n[1] * a.nh * 16);
+            pl.o_fh[l] = o; o = align_up(o + (size_t)(fft_u_len(a) + fft_v_len(a)) * 16);
             pl.o_tw[l] = o; o = align_up(o + (size_t)(g.n[0] + g.n[1] + g.n[2]) * 16);
-            pl.o_dc[l] = o; o = align_up(o + 16);
+            pl.o_dc[l] = o; o = align_up(o + 16 + (size_t)a.nsq * sizeof(double));
         } else if (pl.desc_kind == DMCR_DESC_S3) {
             const size_t Kp = (size_t)pl.s3Kpad, Np = (size_t)pl.s3Npad[l];
             // FP16 operand pairs, FP32 W^T, two scale sources
@@ -751,21 +776,7 @@ struct Prepared {
     size_t o_sep_level = 0, o_sep_coef = 0;
     R gfwd{0, 0, 0}, gred{0, 0, 0}, gadj{0, 0, 0};
     size_t smem_gfwd = 0, smem_gadj = 0;
-    struct FftJob {
-        LevelGeom g;
-        const float* field;
-        double2* X;
-        double2* H;
-        double2* tw;
-        double* dc;
-        float* desc;
-        float weight;
-        int mode;
-        double fh2;
-        const float* Gd;
-        float* part;
-    };
-    std::vector<FftJob> fftf, fftb;
+    std::vector<FftArgs> fftf, fftb;
     std::vector<S3Job> s3f, s3b;
     template <typename S>
     const S* at(size_t off) const { return reinterpret_cast<const S*>(tab + off); }
@@ -780,20 +791,24 @@ bool same_thresh(const ThreshConst& a, const ThreshConst& b) {
     return a.identity == b.identity && a.kappa == b.kappa && a.cexp == b.cexp && a.c1 == b.c1 && a.c3 == b.c3;
 }
 
-Prepared::FftJob fft_job(const Inst& x, int l) {
+FftArgs fft_job(const Inst& x, int l) {
     const Plan& pl = *x.pl;
-    Prepared::FftJob j{};
-    j.g = pl.g[l];
-    j.field = x.lv[l];
-    j.X = reinterpret_cast<double2*>(x.ws + pl.o_fx[l]);
-    j.H = reinterpret_cast<double2*>(x.ws + pl.o_fh[l]);
-    j.tw = reinterpret_cast<double2*>(x.ws + pl.o_tw[l]);
-    j.dc = reinterpret_cast<double*>(x.ws + pl.o_dc[l]);
-    j.desc = x.desc + pl.off[l];
-    j.weight = pl.w[l];
-    j.mode = pl.tc.identity ? 0 : 1;
-    j.fh2 = pl.fh2;
-    return j;
+    FftArgs a = fft_shape(pl.g[l]);
+    a.field = x.lv[l];
+    a.X = reinterpret_cast<double2*>(x.ws + pl.o_fx[l]);
+    a.U = reinterpret_cast<double2*>(x.ws + pl.o_fh[l]);
+    a.V = a.U + fft_u_len(a);
+    double2* tw = reinterpret_cast<double2*>(x.ws + pl.o_tw[l]);
+    a.ax[0].tw = tw;
+    a.ax[1].tw = tw + a.n0;
+    a.ax[2].tw = tw + a.n0 + a.n1;
+    a.dc = reinterpret_cast<double*>(x.ws + pl.o_dc[l]);
+    a.sq = a.dc + 2;
+    a.desc = x.desc + pl.off[l];
+    a.weight = pl.w[l];
+    a.mode = pl.tc.identity ? 0 : 1;
+    a.fh2 = pl.fh2;
+    return a;
 }
 
 S3Job s3_job(const Inst& x, int l, bool loss) {
@@ -1265,9 +1280,10 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
                             gs.blockStart = gb;
                             gb += ceil_div((int64_t)(2 * g.P[0] + 1) * (2 * g.P[1] + 1) * g.NB * T, GCOEF_TH);
                             gv.push_back(gs);
-                            Prepared::FftJob j = fft_job(x, l);
+                            FftArgs j = fft_job(x, l);
                             j.Gd = Gd;
                             j.part = pblk;
+                            j.x_ready = (flags & F_FWD) != 0;
                             P.fftb.push_back(j);
                             continue;
                         }
@@ -1359,80 +1375,6 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
     return DMCR_OK;
 }
 
-// Axis passes of one grid (last axis first); the first forward pass may read the real field.
-void fft_grid(const Prepared::FftJob& j, double2* data, const float* real_in, int sign, cudaStream_t s) {
-    const double two_pi = 6.283185307179586476925;
-    for (int axis = 2; axis >= 0; --axis) {
-        const int len = (int)j.g.n[axis];
-        const int64_t tw_off = axis == 2 ? 0 : (axis == 1 ? j.g.n[2] : j.g.n[2] + j.g.n[1]);
-        if (len == 1) continue;
-        FftPass p{};
-        p.data = data;
-        p.real_in = real_in;
-        real_in = nullptr;
-        for (int a = 0; a < 3; ++a) p.n[a] = j.g.n[a];
-        p.axis = axis;
-        p.sign = sign;
-        p.len = len;
-        p.L = fft_lines_per_block(len);
-        int m = len;
-        p.nrad = 0;
-        while (m % 4 == 0) { p.rad[p.nrad++] = 4; m /= 4; }
-        while (m % 2 == 0) { p.rad[p.nrad++] = 2; m /= 2; }
-        while (m % 3 == 0) { p.rad[p.nrad++] = 3; m /= 3; }
-        while (m % 5 == 0) { p.rad[p.nrad++] = 5; m /= 5; }
-        p.tw = j.tw + tw_off;
-        for (int t = 0; t < 3; ++t) p.om3[t] = make_double2(cos(two_pi * t / 3), -sin(two_pi * t / 3));
-        for (int t = 0; t < 5; ++t) p.om5[t] = make_double2(cos(two_pi * t / 5), -sin(two_pi * t / 5));
-        launch_fft_pass(p, s);
-    }
-    if (real_in != nullptr) {
-        // a 1 x 1 x 1 grid has no pass: copy the value in through a trivial pass of length 1
-        FftPass p{};
-        p.data = data;
-        p.real_in = real_in;
-        for (int a = 0; a < 3; ++a) p.n[a] = j.g.n[a];
-        p.axis = 2;
-        p.sign = sign;
-        p.len = 1;
-        p.L = 1;
-        p.nrad = 0;
-        p.tw = j.tw;
-        launch_fft_pass(p, s);
-    }
-}
-
-void fft_twiddles(const Prepared::FftJob& j, cudaStream_t s) {
-    int64_t off = 0;
-    for (int axis = 2; axis >= 0; --axis) {
-        if (j.g.n[axis] > 1) launch_fft_twiddles(j.tw + off, (int)j.g.n[axis], s);
-        off += j.g.n[axis];
-    }
-}
-
-// X = DFT(M) stays in the workspace; the power spectrum and its inverse go to H
-void fft_descriptor(const Prepared::FftJob& j, cudaStream_t s) {
-    fft_twiddles(j, s);
-    fft_grid(j, j.X, j.field, -1, s);
-    launch_fft_power(j.X, j.H, j.g.N, s);
-    fft_grid(j, j.H, nullptr, +1, s);
-    launch_fft_sample(j.g, j.H, j.weight, j.mode, j.fh2, j.desc, s);
-}
-
-// x_ready: the descriptor of the same call left X = DFT(M) (and the twiddles) in place
-void fft_vjp(const Prepared::FftJob& j, bool x_ready, cudaStream_t s) {
-    if (!x_ready) {
-        fft_twiddles(j, s);
-        fft_grid(j, j.X, j.field, -1, s);
-    }
-    launch_fft_embed(j.g, j.Gd, j.H, s);
-    fft_grid(j, j.H, nullptr, -1, s);
-    launch_fft_dc(j.H, j.dc, s);
-    launch_fft_xcorr(j.X, j.H, j.g.N, s);
-    fft_grid(j, j.H, nullptr, +1, s);
-    launch_fft_vjp_combine(j.g.N, j.field, j.H, j.dc, j.part, s);
-}
-
 void upload(const Prepared& P, cudaStream_t s) {
     if (P.tb.h.empty()) return;
     ProfScope ps("tables", -1, s);
@@ -1478,7 +1420,7 @@ void run(const Prepared& P, cudaStream_t s) {
         }
         if (!P.fftf.empty()) {
             ProfScope ps("fft_descriptor", -1, s);
-            for (const Prepared::FftJob& j : P.fftf) fft_descriptor(j, s);
+            for (const FftArgs& j : P.fftf) launch_fft_descriptor(j, s);
         }
         if (!P.s3f.empty()) {
             ProfScope ps("s3_gram", -1, s);
@@ -1522,7 +1464,7 @@ void run(const Prepared& P, cudaStream_t s) {
         }
         if (!P.fftb.empty()) {
             ProfScope ps("fft_vjp", -1, s);
-            for (const Prepared::FftJob& j : P.fftb) fft_vjp(j, (P.flags & F_FWD) != 0, s);
+            for (const FftArgs& j : P.fftb) launch_fft_vjp(j, s);
         }
         if (!P.s3b.empty()) {
             ProfScope ps("s3_adjoint", -1, s);

@@ -308,19 +308,30 @@ struct S3Job {
     int* err;               // set on a tensor-core wait timeout
 };
 
-// One mixed-radix Stockham pass over the lines of one axis (fft.cu).
-struct FftPass {
-    double2* data;            // complex grid, transformed in place
-    const float* real_in;     // non-null: read the real input from here instead of `data`
-    int64_t n[3];
-    int axis;                 // 0, 1, 2
-    int sign;                 // -1 forward, +1 inverse (unnormalised)
-    int len;                  // n[axis]
-    int L;                    // lines per block
-    int nrad;
-    int rad[16];
-    const double2* tw;        // tw[t] = exp(-2 pi i t / len)
-    double2 om3[3], om5[5];   // exp(-2 pi i t / 3), exp(-2 pi i t / 5)
+// FFT path, one (instance, level) (fft.cu).
+struct FftAxis {
+    int n, nrad;
+    unsigned char rad[16];
+    double2* tw;              // tw[t] = exp(-2 pi i t / n)
+};
+struct FftArgs {
+    int n0, n1, n2, nh;       // sizes; nh = n2 / 2 + 1 columns of the half spectrum
+    int P0, P1, P2, NB;
+    int64_t N;
+    FftAxis ax[3];
+    int Lx, Ly, Ll;           // lines per block: rows (row pairs), middle axis, last axis
+    const float* field;
+    double2 *X, *U, *V;       // half spectrum of the field; window planes (3-D) and rows
+    double* sq;               // sum M^2 of the row blocks
+    int nsq;
+    double* dc;               // sum_r A(r)
+    const float* Gd;          // dense coefficient grid (plane 0 is A)
+    float weight;
+    int mode;                 // 0 identity threshold, 1 soft threshold of a binary field
+    double fh2;               // f(1/2)^2
+    float* desc;
+    float* part;
+    int x_ready;              // X holds the whole transform (the descriptor ran in this call)
 };
 
 // ---------------------------------------------------------------- separable path (sep.cu)
@@ -469,18 +480,11 @@ bool gram_ready();   // the TMA tensor-map encoder is available
 void launch_s3_forward(const S3Job& j, const ThreshConst& tc, int* err, cudaStream_t s);
 void launch_s3_backward(const S3Job& j, const ThreshConst& tc, int* err, cudaStream_t s);
 void set_fft_attributes();
-size_t fft_smem_bytes(int len, int L);
-int fft_lines_per_block(int len);
-void launch_fft_pass(const FftPass& p, cudaStream_t s);
-void launch_fft_twiddles(double2* tw, int len, cudaStream_t s);
-void launch_fft_power(const double2* X, double2* P, int64_t N, cudaStream_t s);
-void launch_fft_xcorr(const double2* X, double2* H, int64_t N, cudaStream_t s);
-void launch_fft_sample(const LevelGeom& g, const double2* X, float weight, int mode, double fh2, float* desc,
-                       cudaStream_t s);
-void launch_fft_embed(const LevelGeom& g, const float* Gd, double2* H, cudaStream_t s);
-void launch_fft_dc(const double2* H, double* out, cudaStream_t s);
-void launch_fft_vjp_combine(int64_t N, const float* M, const double2* Z, const double* sumA, float* part,
-                            cudaStream_t s);
+void fft_axis(int len, FftAxis& ax);
+int fft_lines_per_block(int len, bool strided);
+int fft_row_blocks(const FftArgs& g);
+void launch_fft_descriptor(const FftArgs& g, cudaStream_t s);
+void launch_fft_vjp(const FftArgs& g, cudaStream_t s);
 size_t fwd_smem_bytes(const LevelGeom& g);
 size_t adj_smem_bytes(const LevelGeom& g);
 float gcoef_scale(const LevelGeom& g, const ThreshConst& tc, float weight);

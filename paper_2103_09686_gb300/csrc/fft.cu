@@ -8,292 +8,550 @@
 //     used to characterise binary targets;
 // and the identity-threshold adjoint as one cross-correlation,
 //         g(y) = ( M_y sum_r A(r) + sum_r A(r) M_{y+r} ) / 2,
-//         sum_r A(r) M_{y+r} = (1/N) IDFT( DFT(M) conj(DFT(A_embedded)) )(y).
-// Transforms are hand-written: mixed-radix (2, 3, 4, 5) Stockham passes over one axis per
-// launch, a block transforming L lines in shared memory, in FP64 complex arithmetic (the
-// descriptor needs ~1e-7 relative accuracy; an FP32 transform of 2^20 points is not there).
+//         sum_r A(r) M_{y+r} = (1/N) IDFT( DFT(M) DFT(A) )(y)       (A even: DFT(A) real).
+// Hand-written mixed-radix (8, 4, 2, 3, 5) Stockham transforms in FP64 (the descriptor needs
+// ~1e-7 relative accuracy on C(r)).
+//
+// The path is bound by the FP64 pipe (1.7 operations per SM and clock), so it computes only what
+// is used: the field and A are real, so two rows share one complex transform along x and only the
+// n2/2 + 1 columns of the half spectrum go on; the correlation is needed on the window alone, so
+// after the inverse along the last axis (z in 3-D, y in 2-D) only r = 0 .. P planes are kept, and
+// A's transform starts from the same few rows; the power spectrum and the product are formed
+// where the last axis is transformed, without a pass of their own.
+//   fft_rows    rows of M in pairs -> X[z][y][kx]; sum M^2
+//   fft_y       3-D: transform along y, in place
+//   fft_last    last axis: transform (X stays), |X|^2, inverse, cropped
+//   fft_win_y   3-D: inverse along y cropped to the window / A's rows embedded and transformed
+//   fft_desc    inverse along x, two window rows at a time: the descriptor
+//   fft_coef    rows of A in pairs along x
+//   fft_mul     last axis: transform of A, product with X, inverse
+//   fft_grad    inverse along x, two rows at a time: the gradient
+// 128^3, +-24, loss and gradient: 1715 us with twelve full complex passes of 130 us and seven
+// elementwise kernels, 603 us so.
 #include "common.cuh"
 
 namespace dmcr {
 
+namespace {
+
+constexpr int FFT_THREADS = 256;
+
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
-    return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+    return make_double2(fma(a.x, b.x, -(a.y * b.y)), fma(a.x, b.y, a.y * b.x));
 }
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
-// multiply by -i (forward radix-4) or +i (inverse)
-__device__ __forceinline__ double2 mul_i(double2 a, int sign) {
-    return sign < 0 ? make_double2(a.y, -a.x) : make_double2(-a.y, a.x);
+__device__ __forceinline__ double2 cswap(double2 a) { return make_double2(a.y, a.x); }
+__device__ __forceinline__ double2 conj2(double2 a) { return make_double2(a.x, -a.y); }
+// multiply by -i
+__device__ __forceinline__ double2 mul_mi(double2 a) { return make_double2(a.y, -a.x); }
+
+__device__ __forceinline__ void bfly4(double2& a, double2& b, double2& c, double2& d) {
+    const double2 s0 = cadd(a, c), d0 = csub(a, c), s1 = cadd(b, d), d1 = mul_mi(csub(b, d));
+    a = cadd(s0, s1);
+    b = cadd(d0, d1);
+    c = csub(s0, s1);
+    d = csub(d0, d1);
 }
 
-// Line geometry of one pass: lines along `axis` of an (n0, n1, n2) grid.
-struct LineMap {
-    int64_t base;
-    int64_t stride;
-    bool valid;
-};
-
-__device__ __forceinline__ LineMap line_of(const FftPass& p, int l) {
-    LineMap m;
-    const int64_t n0 = p.n[0], n1 = p.n[1], n2 = p.n[2];
-    if (p.axis == 2) {
-        const int64_t li = (int64_t)blockIdx.x * p.L + l;
-        m.valid = li < n0 * n1;
-        m.base = li * n2;
-        m.stride = 1;
-    } else {
-        const int64_t nb2 = (n2 + p.L - 1) / p.L;
-        const int64_t pidx = blockIdx.x / nb2;
-        const int64_t i2 = (blockIdx.x % nb2) * p.L + l;
-        m.valid = i2 < n2;
-        if (p.axis == 1) {
-            m.base = pidx * n1 * n2 + i2;
-            m.stride = n2;
-        } else {
-            m.base = pidx * n2 + i2;
-            m.stride = n1 * n2;
-        }
-    }
-    return m;
-}
-
-// One Stockham stage of radix R over the L lines in shared memory (src -> dst): every
-// butterfly reads R values n/R apart, multiplies by the twiddles of its offset k within the
-// current sub-transform length Ns, and writes R values Ns apart.  R is a template parameter so
-// that the butterfly's values stay in registers.
+// One forward Stockham stage of radix R over `lines` lines of n points in shared memory
+// (src -> dst): every butterfly reads R values n/R apart, multiplies by the twiddles of its
+// offset k within the current sub-transform length Ns, and writes R values Ns apart.
 template <int R>
-__device__ __forceinline__ void fft_stage(const FftPass& p, const double2* __restrict__ src, double2* __restrict__ dst,
-                                          int Ns) {
-    const int n = p.len, L = p.L;
-    const int nR = n / R;
-    const int tstep = n / (Ns * R);
-    for (int t = threadIdx.x; t < L * nR; t += blockDim.x) {
+__device__ __forceinline__ void fft_stage(const FftAxis& ax, const double2* __restrict__ src,
+                                          double2* __restrict__ dst, int lines, int Ns) {
+    const int n = ax.n, nR = n / R, tstep = nR / Ns;
+    for (int t = threadIdx.x; t < lines * nR; t += FFT_THREADS) {
         const int l = t / nR, j = t - l * nR;
         const int k = j % Ns;
         const double2* in = src + l * n;
         double2 v[R];
-        v[0] = in[j];
 #pragma unroll
-        for (int r = 1; r < R; ++r) {
-            double2 w = p.tw[(k * r) * tstep];
-            if (p.sign > 0) w.y = -w.y;
-            v[r] = cmul(in[j + r * nR], w);
+        for (int r = 0; r < R; ++r) v[r] = in[j + r * nR];
+        if (Ns > 1) {
+#pragma unroll
+            for (int r = 1; r < R; ++r) v[r] = cmul(v[r], ax.tw[k * r * tstep]);
         }
         double2 V[R];
-        if (R == 2) {
+        if constexpr (R == 2) {
             V[0] = cadd(v[0], v[1]);
             V[1] = csub(v[0], v[1]);
-        } else if (R == 4) {
-            const double2 a = cadd(v[0], v[2]), b = csub(v[0], v[2]);
-            const double2 c = cadd(v[1], v[3]), d = mul_i(csub(v[1], v[3]), p.sign);
-            V[0] = cadd(a, c);
-            V[1] = cadd(b, d);
-            V[2] = csub(a, c);
-            V[3] = csub(b, d);
+        } else if constexpr (R == 4) {
+            bfly4(v[0], v[1], v[2], v[3]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) V[q] = v[q];
+        } else if constexpr (R == 8) {
+            bfly4(v[0], v[2], v[4], v[6]);
+            bfly4(v[1], v[3], v[5], v[7]);
+            constexpr double h = 0.70710678118654752440;
+            const double2 w1 = make_double2(v[3].x + v[3].y, v[3].y - v[3].x);     // odd 1 times (1 - i)
+            const double2 w2 = mul_mi(v[5]);
+            const double2 w3 = make_double2(v[7].y - v[7].x, -v[7].x - v[7].y);    // odd 3 times -(1 + i)
+            V[0] = cadd(v[0], v[1]);
+            V[4] = csub(v[0], v[1]);
+            V[1] = make_double2(fma(h, w1.x, v[2].x), fma(h, w1.y, v[2].y));
+            V[5] = make_double2(fma(-h, w1.x, v[2].x), fma(-h, w1.y, v[2].y));
+            V[2] = cadd(v[4], w2);
+            V[6] = csub(v[4], w2);
+            V[3] = make_double2(fma(h, w3.x, v[6].x), fma(h, w3.y, v[6].y));
+            V[7] = make_double2(fma(-h, w3.x, v[6].x), fma(-h, w3.y, v[6].y));
         } else {
-            // radix 3 and 5: V[q] = sum_r v[r] omega^(r q),  omega = exp(sign 2 pi i / R)
-#pragma unroll
-            for (int q = 0; q < R; ++q) {
-                double2 acc = v[0];
-#pragma unroll
-                for (int r = 1; r < R; ++r) {
-                    double2 w = R == 3 ? p.om3[(r * q) % 3] : p.om5[(r * q) % 5];
-                    if (p.sign > 0) w.y = -w.y;
-                    acc = cadd(acc, cmul(v[r], w));
-                }
-                V[q] = acc;
+            // radix 3 and 5: V[q] = sum_r v[r] exp(-2 pi i r q / R), r paired with R - r
+            constexpr double c3 = -0.5, s3 = 0.86602540378443864676;
+            constexpr double c51 = 0.30901699437494742410, c52 = -0.80901699437494742410,
+                             s51 = 0.95105651629515357212, s52 = 0.58778525229247312917;
+            if constexpr (R == 3) {
+                const double2 p = cadd(v[1], v[2]), m = mul_mi(csub(v[1], v[2]));
+                const double2 a = make_double2(fma(c3, p.x, v[0].x), fma(c3, p.y, v[0].y));
+                V[0] = cadd(v[0], p);
+                V[1] = make_double2(fma(s3, m.x, a.x), fma(s3, m.y, a.y));
+                V[2] = make_double2(fma(-s3, m.x, a.x), fma(-s3, m.y, a.y));
+            } else {
+                const double2 p1 = cadd(v[1], v[4]), m1 = mul_mi(csub(v[1], v[4]));
+                const double2 p2 = cadd(v[2], v[3]), m2 = mul_mi(csub(v[2], v[3]));
+                V[0] = cadd(v[0], cadd(p1, p2));
+                const double2 a1 = make_double2(fma(c51, p1.x, fma(c52, p2.x, v[0].x)), fma(c51, p1.y, fma(c52, p2.y, v[0].y)));
+                const double2 a2 = make_double2(fma(c52, p1.x, fma(c51, p2.x, v[0].x)), fma(c52, p1.y, fma(c51, p2.y, v[0].y)));
+                const double2 b1 = make_double2(fma(s51, m1.x, s52 * m2.x), fma(s51, m1.y, s52 * m2.y));
+                const double2 b2 = make_double2(fma(s52, m1.x, -(s51 * m2.x)), fma(s52, m1.y, -(s51 * m2.y)));
+                V[1] = cadd(a1, b1);
+                V[4] = csub(a1, b1);
+                V[2] = cadd(a2, b2);
+                V[3] = csub(a2, b2);
             }
         }
-        double2* out = dst + l * n + (j / Ns) * Ns * R + k;
+        double2* out = dst + l * n + (j - k) * R + k;
 #pragma unroll
         for (int q = 0; q < R; ++q) out[q * Ns] = V[q];
     }
 }
 
-__global__ void __launch_bounds__(256) fft_pass_kernel(FftPass p) {
-    extern __shared__ __align__(16) double2 sbuf[];
-    const int n = p.len, L = p.L;
-    double2* src = sbuf;
-    double2* dst = sbuf + (size_t)L * n;
-    const int total = L * n;
-    // load L lines (lanes along the contiguous axis when the lines are strided)
-    for (int e = threadIdx.x; e < total; e += blockDim.x) {
-        int l, i;
-        if (p.axis == 2) { l = e / n; i = e - l * n; }
-        else { i = e / L; l = e - i * L; }
-        const LineMap m = line_of(p, l);
-        double2 v = make_double2(0.0, 0.0);
-        if (m.valid) {
-            const int64_t g = m.base + (int64_t)i * m.stride;
-            v = p.real_in != nullptr ? make_double2((double)p.real_in[g], 0.0) : p.data[g];
-        }
-        src[l * n + i] = v;
-    }
+// Forward transform of `lines` lines from `a`, through `b` and back; returns the buffer that holds
+// the result.  Begins and ends with a barrier.  An inverse exchanges real and imaginary parts
+// of its input and output.
+__device__ __noinline__ double2* fft_lines(const FftAxis& ax, double2* a, double2* b, int lines) {
     int Ns = 1;
-    for (int s = 0; s < p.nrad; ++s) {
-        const int R = p.rad[s];
-        __syncthreads();
+    __syncthreads();
+    for (int s = 0; s < ax.nrad; ++s) {
+        const int R = ax.rad[s];
         switch (R) {
-            case 2: fft_stage<2>(p, src, dst, Ns); break;
-            case 3: fft_stage<3>(p, src, dst, Ns); break;
-            case 4: fft_stage<4>(p, src, dst, Ns); break;
-            default: fft_stage<5>(p, src, dst, Ns); break;
+            case 8: fft_stage<8>(ax, a, b, lines, Ns); break;
+            case 4: fft_stage<4>(ax, a, b, lines, Ns); break;
+            case 2: fft_stage<2>(ax, a, b, lines, Ns); break;
+            case 3: fft_stage<3>(ax, a, b, lines, Ns); break;
+            default: fft_stage<5>(ax, a, b, lines, Ns); break;
         }
-        double2* tmp = src;
-        src = dst;
-        dst = tmp;
         Ns *= R;
+        double2* x = a;
+        a = b;
+        b = x;
+        __syncthreads();
+    }
+    return a;
+}
+
+extern __shared__ __align__(16) double2 fft_smem[];
+
+// Canonical half-window index of (rz, ry, rx), -1 if it is not in the half window.
+__device__ __forceinline__ int64_t fft_half_index(const FftArgs& g, int rz, int ry, int rx) {
+    const int Px = g.P2, Py = g.P1;
+    if (rz == 0 && ry == 0) return rx >= 0 ? rx : -1;
+    if (rz == 0) return ry > 0 ? (Px + 1) + (int64_t)(ry - 1) * (2 * Px + 1) + (rx + Px) : -1;
+    if (rz < 0) return -1;
+    return (Px + 1) + (int64_t)Py * (2 * Px + 1) + ((int64_t)(rz - 1) * (2 * Py + 1) + (ry + Py)) * (2 * Px + 1) +
+           (rx + Px);
+}
+
+// rows kept of the window -> (rz, ry): 3-D rz = 0 .. P0 and every ry, 2-D ry = 0 .. P1
+__device__ __forceinline__ void fft_window_row(const FftArgs& g, int row, int& rz, int& ry) {
+    if (g.n0 > 1) {
+        const int wy = 2 * g.P1 + 1;
+        rz = row / wy;
+        ry = row - rz * wy - g.P1;
+    } else {
+        rz = 0;
+        ry = row;
+    }
+}
+__device__ __forceinline__ int fft_window_rows(const FftArgs& g) {
+    return g.n0 > 1 ? (g.P0 + 1) * (2 * g.P1 + 1) : g.P1 + 1;
+}
+
+// fixed-order sum over the block (FFT_THREADS threads); valid in every thread
+__device__ __forceinline__ double block_sum(double v, double* sh) {
+    __syncthreads();
+    sh[threadIdx.x] = v;
+    for (int w = FFT_THREADS / 2; w > 0; w >>= 1) {
+        __syncthreads();
+        if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < total; e += blockDim.x) {
-        int l, i;
-        if (p.axis == 2) { l = e / n; i = e - l * n; }
-        else { i = e / L; l = e - i * L; }
-        const LineMap m = line_of(p, l);
-        if (m.valid) p.data[m.base + (int64_t)i * m.stride] = src[l * n + i];
+    return sh[0];
+}
+
+// Half spectra of two real lines from the transform Z of (first + i second).
+__device__ __forceinline__ void unpack(const double2* r, int n, int k, double2& A, double2& B) {
+    const double2 z = r[k], y = r[k == 0 ? 0 : n - k];
+    A = make_double2(0.5 * (z.x + y.x), 0.5 * (z.y - y.y));
+    B = make_double2(0.5 * (z.y + y.y), 0.5 * (y.x - z.x));
+}
+// The transform of (first + i second) at k from their half spectra, exchanged for an inverse.
+__device__ __forceinline__ double2 pack_swapped(const double2* A, const double2* B, int n, int nh, int k) {
+    double2 a, b;
+    if (k < nh) {
+        a = A[k];
+        b = B != nullptr ? B[k] : make_double2(0.0, 0.0);
+    } else {
+        a = conj2(A[n - k]);
+        b = B != nullptr ? conj2(B[n - k]) : make_double2(0.0, 0.0);
+    }
+    return make_double2(a.y + b.x, a.x - b.y);       // swapped (a.x - b.y, a.y + b.x)
+}
+
+}  // namespace
+
+// tw[t] = exp(-2 pi i t / len) of the three axes, one block column per axis
+__global__ void fft_twiddle_kernel(FftArgs g) {
+    dep_wait();
+    dep_trigger();
+    const FftAxis& ax = g.ax[blockIdx.y];
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= ax.n) return;
+    double sv, cv;
+    sincospi(2.0 * (double)t / (double)ax.n, &sv, &cv);
+    ax.tw[t] = make_double2(cv, -sv);
+}
+
+// Row pairs of the field along x; the block's share of sum M^2.
+__global__ void __launch_bounds__(FFT_THREADS, 3) fft_rows_kernel(const __grid_constant__ FftArgs g) {
+    dep_wait();
+    dep_trigger();
+    __shared__ double sh[FFT_THREADS];
+    const int n = g.n2, nh = g.nh, L = g.Lx;
+    const int64_t rows = (int64_t)g.n0 * g.n1, q0 = (int64_t)blockIdx.x * L;
+    const int lines = (int)min((int64_t)L, (rows + 1) / 2 - q0);
+    double2 *a = fft_smem, *b = fft_smem + L * n;
+    double sq = 0.0;
+    for (int e = threadIdx.x; e < lines * n; e += FFT_THREADS) {
+        const int l = e / n, i = e - l * n;
+        const int64_t row = 2 * (q0 + l);
+        const float u = g.field[row * n + i], v = row + 1 < rows ? g.field[(row + 1) * n + i] : 0.f;
+        a[e] = make_double2((double)u, (double)v);
+        sq = fma((double)u, (double)u, fma((double)v, (double)v, sq));
+    }
+    const double2* r = fft_lines(g.ax[2], a, b, lines);
+    for (int e = threadIdx.x; e < lines * nh; e += FFT_THREADS) {
+        const int l = e / nh, k = e - l * nh;
+        const int64_t row = 2 * (q0 + l);
+        double2 A, B;
+        unpack(r + l * n, n, k, A, B);
+        g.X[row * nh + k] = A;
+        if (row + 1 < rows) g.X[(row + 1) * nh + k] = B;
+    }
+    sq = block_sum(sq, sh);
+    if (threadIdx.x == 0) g.sq[blockIdx.x] = sq;
+}
+
+// columns of one block along a strided axis: L adjacent kx
+struct FftCols {
+    int n, L, cols;
+    int64_t base, stride;
+};
+
+__device__ __forceinline__ void fft_load(const double2* __restrict__ src, const FftCols& c, bool swap, double2* a) {
+    for (int e = threadIdx.x; e < c.L * c.n; e += FFT_THREADS) {
+        const int i = e / c.L, l = e - i * c.L;
+        const double2 v = l < c.cols ? src[c.base + i * c.stride + l] : make_double2(0.0, 0.0);
+        a[l * c.n + i] = swap ? cswap(v) : v;
     }
 }
 
-size_t fft_smem_bytes(int len, int L) { return (size_t)2 * L * len * sizeof(double2); }
-
-int fft_lines_per_block(int len) {
-    int L = 4096 / len;
-    if (L > 16) L = 16;
-    return L < 1 ? 1 : L;
+// Middle axis of 3-D, in place.
+template <bool INVERSE>
+__global__ void __launch_bounds__(FFT_THREADS, 3) fft_y_kernel(const __grid_constant__ FftArgs g) {
+    dep_wait();
+    dep_trigger();
+    const int xg = (g.nh + g.Ly - 1) / g.Ly, x0 = (int)(blockIdx.x % xg) * g.Ly, z = (int)(blockIdx.x / xg);
+    const FftCols c{g.n1, g.Ly, min(g.Ly, g.nh - x0), (int64_t)z * g.n1 * g.nh + x0, g.nh};
+    double2 *a = fft_smem, *b = fft_smem + c.L * c.n;
+    fft_load(g.X, c, INVERSE, a);
+    const double2* r = fft_lines(g.ax[1], a, b, c.L);
+    for (int e = threadIdx.x; e < c.L * c.n; e += FFT_THREADS) {
+        const int i = e / c.L, l = e - i * c.L;
+        if (l < c.cols) g.X[c.base + i * c.stride + l] = INVERSE ? cswap(r[l * c.n + i]) : r[l * c.n + i];
+    }
 }
 
-void launch_fft_pass(const FftPass& p, cudaStream_t s) {
-    int64_t blocks;
-    if (p.axis == 2) blocks = (p.n[0] * p.n[1] + p.L - 1) / p.L;
-    else blocks = (p.axis == 1 ? p.n[0] : p.n[1]) * ((p.n[2] + p.L - 1) / p.L);
-    fft_pass_kernel<<<(unsigned)blocks, 256, fft_smem_bytes(p.len, p.L), s>>>(p);
+__device__ __forceinline__ FftCols fft_last_cols(const FftArgs& g) {
+    const int xg = (g.nh + g.Ll - 1) / g.Ll, x0 = (int)(blockIdx.x % xg) * g.Ll, y = (int)(blockIdx.x / xg);
+    const bool d3 = g.n0 > 1;
+    return FftCols{d3 ? g.n0 : g.n1, g.Ll, min(g.Ll, g.nh - x0), (int64_t)y * g.nh + x0,
+                   d3 ? (int64_t)g.n1 * g.nh : (int64_t)g.nh};
 }
 
-// P <- |X|^2 (X is kept: the adjoint of the same call reuses the transform of the field)
-__global__ void fft_power_kernel(const double2* __restrict__ X, double2* __restrict__ P, int64_t N) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const double2 v = X[i];
-    P[i] = make_double2(v.x * v.x + v.y * v.y, 0.0);
+// Last axis: X's transform (left in place), the power spectrum and its inverse, rows 0 .. P.
+__global__ void __launch_bounds__(FFT_THREADS, 3) fft_last_kernel(const __grid_constant__ FftArgs g) {
+    dep_wait();
+    dep_trigger();
+    const FftCols c = fft_last_cols(g);
+    const FftAxis& ax = g.n0 > 1 ? g.ax[0] : g.ax[1];
+    double2 *a = fft_smem, *b = fft_smem + c.L * c.n;
+    fft_load(g.X, c, false, a);
+    double2* r = fft_lines(ax, a, b, c.L);
+    for (int e = threadIdx.x; e < c.L * c.n; e += FFT_THREADS) {
+        const int i = e / c.L, l = e - i * c.L;
+        const double2 v = r[l * c.n + i];
+        if (l < c.cols) g.X[c.base + i * c.stride + l] = v;
+        r[l * c.n + i] = make_double2(0.0, fma(v.x, v.x, v.y * v.y));      // exchanged
+    }
+    const double2* o = fft_lines(ax, r, r == a ? b : a, c.L);
+    const int P = g.n0 > 1 ? g.P0 : g.P1;
+    double2* out = g.n0 > 1 ? g.U : g.V;
+    for (int e = threadIdx.x; e < c.L * (P + 1); e += FFT_THREADS) {
+        const int i = e / c.L, l = e - i * c.L;
+        if (l < c.cols) out[c.base + i * c.stride + l] = cswap(o[l * c.n + i]);
+    }
 }
 
-// H <- X conj(H)
-__global__ void fft_xcorr_kernel(const double2* __restrict__ X, double2* __restrict__ H, int64_t N) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const double2 a = X[i], b = H[i];
-    H[i] = make_double2(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
-}
-
-__device__ __forceinline__ int64_t wrapn(int64_t v, int64_t n) {
-    const int64_t m = v % n;
-    return m < 0 ? m + n : m;
-}
-
-// Canonical half-window index k -> (rz, ry, rx).
-__device__ __forceinline__ void canon_decode(const LevelGeom& g, int64_t k, int& rz, int& ry, int& rx) {
-    const int Px = g.P[2], Py = g.P[1];
-    const int64_t wx = 2 * Px + 1, wy = 2 * Py + 1;
-    if (k <= Px) { rz = 0; ry = 0; rx = (int)k; return; }
-    k -= Px + 1;
-    if (k < (int64_t)Py * wx) { rz = 0; ry = 1 + (int)(k / wx); rx = (int)(k % wx) - Px; return; }
-    k -= (int64_t)Py * wx;
-    rz = 1 + (int)(k / (wy * wx));
-    const int64_t rem = k % (wy * wx);
-    ry = (int)(rem / wx) - Py;
-    rx = (int)(rem % wx) - Px;
-}
-
-// desc[k] = w * S_bar(r_k) from the unnormalised inverse transform X = N^2 C (mode 0:
-// identity threshold; mode 1: soft threshold of a binary field, App. A with fh2 = f(1/2)^2).
-__global__ void fft_sample_kernel(LevelGeom g, const double2* __restrict__ X, float weight, int mode, double fh2,
-                                  float* __restrict__ desc) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= g.Khalf) return;
-    int rz, ry, rx;
-    canon_decode(g, k, rz, ry, rx);
-    const double invN2 = 1.0 / ((double)g.N * (double)g.N);
-    const double C0 = X[0].x * invN2;
-    const double Cr = X[(wrapn(rz, g.n[0]) * g.n[1] + wrapn(ry, g.n[1])) * g.n[2] + wrapn(rx, g.n[2])].x * invN2;
-    double s;
-    if (mode == 0) s = 0.5 * (C0 + Cr);
-    else s = (k == 0) ? C0 : (1.0 - 2.0 * fh2) * Cr + 2.0 * fh2 * C0;
-    desc[k] = (float)((double)weight * s);
-}
-
-// H[u] = sum of the window coefficients A(r) with r = u (mod n), gathered over the at most
-// two preimages per axis (windows are at most half a period); A is plane 0 of the dense
-// coefficient grid (quad layout of gcoef_kernel).
-__global__ void fft_embed_kernel(LevelGeom g, const float* __restrict__ Gd, double2* __restrict__ H) {
-    const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (u >= g.N) return;
-    const int64_t ux = u % g.n[2], uy = (u / g.n[2]) % g.n[1], uz = u / (g.n[1] * g.n[2]);
-    const int64_t cz[2] = {uz, uz - g.n[0]}, cy[2] = {uy, uy - g.n[1]}, cx[2] = {ux, ux - g.n[2]};
-    double acc = 0.0;
-    const int wy = 2 * g.P[1] + 1;
-    for (int a = 0; a < 2; ++a) {
-        const int64_t rz = cz[a];
-        if (rz < -g.P[0] || rz > g.P[0] || (a == 1 && cz[1] == cz[0])) continue;
-        for (int b = 0; b < 2; ++b) {
-            const int64_t ry = cy[b];
-            if (ry < -g.P[1] || ry > g.P[1]) continue;
-            for (int c = 0; c < 2; ++c) {
-                const int64_t rx = cx[c];
-                if (rx < -g.P[2] || rx > g.P[2]) continue;
-                const int64_t row = (rz + g.P[0]) * wy + (ry + g.P[1]);
-                const int col = (int)(rx + g.P[2]);
-                const int blk = col / T, m = col % T;
-                acc += (double)Gd[(row * g.NB + blk) * GBLOCK + 4 * m];
+// 3-D: middle axis of the window.  DESC: U -> V, inverse cropped to -P1 .. P1.  Otherwise V -> U:
+// A's rows embedded (both ends at the aliased +-n/2) and transformed.
+template <bool DESC>
+__global__ void __launch_bounds__(FFT_THREADS, 3) fft_win_y_kernel(const __grid_constant__ FftArgs g) {
+    dep_wait();
+    dep_trigger();
+    const int xg = (g.nh + g.Ly - 1) / g.Ly, x0 = (int)(blockIdx.x % xg) * g.Ly, rz = (int)(blockIdx.x / xg);
+    const int n = g.n1, L = g.Ly, cols = min(L, g.nh - x0), wy = 2 * g.P1 + 1;
+    double2 *a = fft_smem, *b = fft_smem + L * n;
+    double2* U = g.U + (int64_t)rz * g.n1 * g.nh + x0;
+    double2* V = g.V + (int64_t)rz * wy * g.nh + x0;
+    for (int e = threadIdx.x; e < L * n; e += FFT_THREADS) {
+        const int i = e / L, l = e - i * L;
+        double2 v = make_double2(0.0, 0.0);
+        if (l < cols) {
+            if (DESC) {
+                v = cswap(U[(int64_t)i * g.nh + l]);
+            } else {
+                if (i <= g.P1) v = V[(int64_t)(i + g.P1) * g.nh + l];
+                if (i > 0 && n - i <= g.P1) v = cadd(v, V[(int64_t)(i - n + g.P1) * g.nh + l]);
             }
         }
+        a[l * n + i] = v;
     }
-    H[u] = make_double2(acc, 0.0);
+    const double2* r = fft_lines(g.ax[1], a, b, L);
+    for (int e = threadIdx.x; e < L * (DESC ? wy : n); e += FFT_THREADS) {
+        const int i = e / L, l = e - i * L;
+        if (l >= cols) continue;
+        if (DESC) {
+            const int ry = i - g.P1;
+            V[(int64_t)i * g.nh + l] = cswap(r[l * n + (ry < 0 ? ry + n : ry)]);
+        } else {
+            U[(int64_t)i * g.nh + l] = r[l * n + i];
+        }
+    }
 }
 
-// part[y] = ( M_y sum_r A(r) + Re(Z[y]) / N ) / 2,  sum_r A(r) = Re(DFT(H)[0]) read before the product.
-__global__ void fft_vjp_combine_kernel(int64_t N, const float* __restrict__ M, const double2* __restrict__ Z,
-                                       const double* __restrict__ sumA, float* __restrict__ part) {
-    const int64_t y = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (y >= N) return;
-    part[y] = (float)(0.5 * ((double)M[y] * (*sumA) + Z[y].x / (double)N));
+// Pairs of window rows, inverse along x: desc[k] = w S_bar(r_k) (mode 0: identity threshold;
+// mode 1: soft threshold of a binary field, App. A with fh2 = f(1/2)^2).
+__global__ void __launch_bounds__(FFT_THREADS, 3) fft_desc_kernel(const __grid_constant__ FftArgs g) {
+    dep_wait();
+    dep_trigger();
+    __shared__ double sh[FFT_THREADS];
+    const int n = g.n2, nh = g.nh, L = g.Lx, R = fft_window_rows(g), q0 = blockIdx.x * L;
+    const int lines = min(L, (R + 1) / 2 - q0);
+    double2 *a = fft_smem, *b = fft_smem + L * n;
+    double s = 0.0;
+    for (int i = threadIdx.x; i < g.nsq; i += FFT_THREADS) s += g.sq[i];
+    const double C0 = block_sum(s, sh) / (double)g.N;
+    for (int e = threadIdx.x; e < lines * n; e += FFT_THREADS) {
+        const int l = e / n, k = e - l * n, row = 2 * (q0 + l);
+        const double2* A = g.V + (int64_t)row * nh;
+        a[e] = pack_swapped(A, row + 1 < R ? A + nh : nullptr, n, nh, k);
+    }
+    const double2* r = fft_lines(g.ax[2], a, b, lines);
+    const double invN2 = 1.0 / ((double)g.N * (double)g.N);
+    const int wx = 2 * g.P2 + 1;
+    for (int e = threadIdx.x; e < 2 * lines * wx; e += FFT_THREADS) {
+        const int h = e / wx, rx = e - h * wx - g.P2, row = 2 * q0 + h;
+        if (row >= R) continue;
+        int rz, ry;
+        fft_window_row(g, row, rz, ry);
+        const int64_t k = fft_half_index(g, rz, ry, rx);
+        if (k < 0) continue;
+        const double2 v = r[(h / 2) * n + (rx < 0 ? rx + n : rx)];
+        const double Cr = (h & 1 ? v.x : v.y) * invN2;       // exchanged: the first row is the imaginary part
+        double S;
+        if (g.mode == 0) S = k == 0 ? C0 : 0.5 * (C0 + Cr);
+        else S = k == 0 ? C0 : (1.0 - 2.0 * g.fh2) * Cr + 2.0 * g.fh2 * C0;
+        g.desc[k] = (float)((double)g.weight * S);
+    }
 }
 
-__global__ void fft_dc_kernel(const double2* __restrict__ H, double* __restrict__ out) { *out = H[0].x; }
-
-// tw[t] = exp(-2 pi i t / len), from the library's sincospi (double)
-__global__ void fft_twiddle_kernel(double2* __restrict__ tw, int len) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= len) return;
-    double sv, cv;
-    sincospi(2.0 * (double)t / (double)len, &sv, &cv);
-    tw[t] = make_double2(cv, -sv);
+// Pairs of window rows of A (plane 0 of the dense coefficient grid) embedded along x.
+__global__ void __launch_bounds__(FFT_THREADS, 3) fft_coef_kernel(const __grid_constant__ FftArgs g) {
+    dep_wait();
+    dep_trigger();
+    const int n = g.n2, nh = g.nh, L = g.Lx, R = fft_window_rows(g), q0 = blockIdx.x * L;
+    const int lines = min(L, (R + 1) / 2 - q0);
+    double2 *a = fft_smem, *b = fft_smem + L * n;
+    auto A = [&](int row, int i) {
+        if (row >= R) return 0.0;
+        int rz, ry;
+        fft_window_row(g, row, rz, ry);
+        const float* p = g.Gd + ((int64_t)(rz + g.P0) * (2 * g.P1 + 1) + (ry + g.P1)) * g.NB * GBLOCK;
+        double v = 0.0;
+        if (i <= g.P2) v = (double)p[((i + g.P2) / T) * GBLOCK + 4 * ((i + g.P2) % T)];
+        if (i > 0 && n - i <= g.P2) v += (double)p[((i - n + g.P2) / T) * GBLOCK + 4 * ((i - n + g.P2) % T)];
+        return v;
+    };
+    for (int e = threadIdx.x; e < lines * n; e += FFT_THREADS) {
+        const int l = e / n, i = e - l * n, row = 2 * (q0 + l);
+        a[e] = make_double2(A(row, i), A(row + 1, i));
+    }
+    const double2* r = fft_lines(g.ax[2], a, b, lines);
+    for (int e = threadIdx.x; e < lines * nh; e += FFT_THREADS) {
+        const int l = e / nh, k = e - l * nh, row = 2 * (q0 + l);
+        double2 u, v;
+        unpack(r + l * n, n, k, u, v);
+        g.V[(int64_t)row * nh + k] = u;
+        if (row + 1 < R) g.V[(int64_t)(row + 1) * nh + k] = v;
+    }
 }
 
-void launch_fft_twiddles(double2* tw, int len, cudaStream_t s) {
-    fft_twiddle_kernel<<<(len + 255) / 256, 256, 0, s>>>(tw, len);
+// Last axis: transform of A (real, since A is even: row -r is the conjugate of row r), product
+// with X (transformed here first when no descriptor of the same call left it so), inverse, in
+// place; sum_r A(r) = DFT(A)(0).
+__global__ void __launch_bounds__(FFT_THREADS, 3) fft_mul_kernel(const __grid_constant__ FftArgs g) {
+    dep_wait();
+    dep_trigger();
+    const FftCols c = fft_last_cols(g);
+    const FftAxis& ax = g.n0 > 1 ? g.ax[0] : g.ax[1];
+    const int P = g.n0 > 1 ? g.P0 : g.P1;
+    const double2* src = g.n0 > 1 ? g.U : g.V;
+    double2 *a = fft_smem, *b = fft_smem + c.L * c.n;
+    double* w = reinterpret_cast<double*>(b + c.L * c.n);
+    for (int e = threadIdx.x; e < c.L * c.n; e += FFT_THREADS) {
+        const int i = e / c.L, l = e - i * c.L;
+        double2 v = make_double2(0.0, 0.0);
+        if (l < c.cols) {
+            if (i <= P) v = src[c.base + i * c.stride + l];
+            if (i > 0 && c.n - i <= P) v = cadd(v, conj2(src[c.base + (c.n - i) * c.stride + l]));
+        }
+        a[l * c.n + i] = v;
+    }
+    double2* r = fft_lines(ax, a, b, c.L);
+    for (int e = threadIdx.x; e < c.L * c.n; e += FFT_THREADS) w[e] = r[e].x;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *g.dc = r[0].x;
+    __syncthreads();
+    fft_load(g.X, c, false, a);
+    r = a;
+    if (!g.x_ready) r = fft_lines(ax, a, b, c.L);
+    else __syncthreads();
+    for (int e = threadIdx.x; e < c.L * c.n; e += FFT_THREADS) {
+        const double2 v = r[e];
+        r[e] = make_double2(w[e] * v.y, w[e] * v.x);         // exchanged
+    }
+    const double2* o = fft_lines(ax, r, r == a ? b : a, c.L);
+    for (int e = threadIdx.x; e < c.L * c.n; e += FFT_THREADS) {
+        const int i = e / c.L, l = e - i * c.L;
+        if (l < c.cols) g.X[c.base + i * c.stride + l] = cswap(o[l * c.n + i]);
+    }
 }
 
-void launch_fft_power(const double2* X, double2* P, int64_t N, cudaStream_t s) {
-    fft_power_kernel<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(X, P, N);
+// Row pairs, inverse along x: part[y] = ( M_y sum_r A(r) + Z[y] / N ) / 2.
+__global__ void __launch_bounds__(FFT_THREADS, 3) fft_grad_kernel(const __grid_constant__ FftArgs g) {
+    dep_wait();
+    dep_trigger();
+    const int n = g.n2, nh = g.nh, L = g.Lx;
+    const int64_t rows = (int64_t)g.n0 * g.n1, q0 = (int64_t)blockIdx.x * L;
+    const int lines = (int)min((int64_t)L, (rows + 1) / 2 - q0);
+    double2 *a = fft_smem, *b = fft_smem + L * n;
+    for (int e = threadIdx.x; e < lines * n; e += FFT_THREADS) {
+        const int l = e / n, k = e - l * n;
+        const int64_t row = 2 * (q0 + l);
+        const double2* A = g.X + row * nh;
+        a[e] = pack_swapped(A, row + 1 < rows ? A + nh : nullptr, n, nh, k);
+    }
+    const double2* r = fft_lines(g.ax[2], a, b, lines);
+    const double half_sum = 0.5 * *g.dc, scale = 0.5 / (double)g.N;
+    for (int e = threadIdx.x; e < lines * n; e += FFT_THREADS) {
+        const int l = e / n, i = e - l * n;
+        const int64_t row = 2 * (q0 + l), y = row * n + i;
+        g.part[y] = (float)fma((double)g.field[y], half_sum, r[e].y * scale);
+        if (row + 1 < rows) g.part[y + n] = (float)fma((double)g.field[y + n], half_sum, r[e].x * scale);
+    }
 }
-void launch_fft_xcorr(const double2* X, double2* H, int64_t N, cudaStream_t s) {
-    fft_xcorr_kernel<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(X, H, N);
+
+// ------------------------------------------------------------------------- launchers
+
+void fft_axis(int len, FftAxis& ax) {
+    ax.n = len;
+    ax.nrad = 0;
+    int m = len;
+    for (int r : {8, 4, 2, 3, 5})
+        while (m % r == 0) {
+            ax.rad[ax.nrad++] = (unsigned char)r;
+            m /= r;
+        }
 }
-void launch_fft_sample(const LevelGeom& g, const double2* X, float weight, int mode, double fh2, float* desc,
-                       cudaStream_t s) {
-    fft_sample_kernel<<<(unsigned)((g.Khalf + 255) / 256), 256, 0, s>>>(g, X, weight, mode, fh2, desc);
+
+// Lines of `len` points per block: about 1024 points (2 x 16 KB of shared memory and room for
+// three blocks per SM), at most 16, at least 4 adjacent columns (64 bytes) of a strided axis.
+int fft_lines_per_block(int len, bool strided) {
+    int L = 1024 / len;
+    if (L > 16) L = 16;
+    const int least = strided ? (len > 2048 ? 1 : (len > 1024 ? 2 : 4)) : 1;
+    return L < least ? least : L;
 }
-void launch_fft_embed(const LevelGeom& g, const float* Gd, double2* H, cudaStream_t s) {
-    fft_embed_kernel<<<(unsigned)((g.N + 255) / 256), 256, 0, s>>>(g, Gd, H);
+
+int fft_row_blocks(const FftArgs& g) { return (int)(((int64_t)g.n0 * g.n1 + 1) / 2 + g.Lx - 1) / g.Lx; }
+
+namespace {
+size_t row_smem(const FftArgs& g) { return (size_t)2 * g.Lx * g.n2 * sizeof(double2); }
+size_t y_smem(const FftArgs& g) { return (size_t)2 * g.Ly * g.n1 * sizeof(double2); }
+size_t last_smem(const FftArgs& g, bool mul) {
+    const size_t pts = (size_t)g.Ll * (g.n0 > 1 ? g.n0 : g.n1);
+    return 2 * pts * sizeof(double2) + (mul ? pts * sizeof(double) : 0);
 }
-void launch_fft_dc(const double2* H, double* out, cudaStream_t s) { fft_dc_kernel<<<1, 1, 0, s>>>(H, out); }
-void launch_fft_vjp_combine(int64_t N, const float* M, const double2* Z, const double* sumA, float* part,
-                            cudaStream_t s) {
-    fft_vjp_combine_kernel<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(N, M, Z, sumA, part);
+unsigned win_blocks(const FftArgs& g) {
+    const int R = g.n0 > 1 ? (g.P0 + 1) * (2 * g.P1 + 1) : g.P1 + 1;
+    return (unsigned)(((R + 1) / 2 + g.Lx - 1) / g.Lx);
+}
+unsigned last_blocks(const FftArgs& g) { return (unsigned)((g.nh + g.Ll - 1) / g.Ll) * (g.n0 > 1 ? g.n1 : 1); }
+unsigned y_blocks(const FftArgs& g, int planes) { return (unsigned)((g.nh + g.Ly - 1) / g.Ly) * planes; }
+
+// twiddles, rows and the middle axis of the field
+void field_spectrum(const FftArgs& g, cudaStream_t s) {
+    const int longest = g.n0 > g.n1 ? (g.n0 > g.n2 ? g.n0 : g.n2) : (g.n1 > g.n2 ? g.n1 : g.n2);
+    launch_dep(fft_twiddle_kernel, dim3((longest + 127) / 128, 3), 128, 0, s, g);
+    launch_dep(fft_rows_kernel, (unsigned)fft_row_blocks(g), FFT_THREADS, row_smem(g), s, g);
+    if (g.n0 > 1) launch_dep(fft_y_kernel<false>, y_blocks(g, g.n0), FFT_THREADS, y_smem(g), s, g);
+}
+}  // namespace
+
+void launch_fft_descriptor(const FftArgs& g, cudaStream_t s) {
+    field_spectrum(g, s);
+    launch_dep(fft_last_kernel, last_blocks(g), FFT_THREADS, last_smem(g, false), s, g);
+    if (g.n0 > 1) launch_dep(fft_win_y_kernel<true>, y_blocks(g, g.P0 + 1), FFT_THREADS, y_smem(g), s, g);
+    launch_dep(fft_desc_kernel, win_blocks(g), FFT_THREADS, row_smem(g), s, g);
+}
+
+// g.x_ready: the descriptor of the same call left X (and the twiddles) in place
+void launch_fft_vjp(const FftArgs& g, cudaStream_t s) {
+    if (!g.x_ready) field_spectrum(g, s);
+    launch_dep(fft_coef_kernel, win_blocks(g), FFT_THREADS, row_smem(g), s, g);
+    if (g.n0 > 1) launch_dep(fft_win_y_kernel<false>, y_blocks(g, g.P0 + 1), FFT_THREADS, y_smem(g), s, g);
+    launch_dep(fft_mul_kernel, last_blocks(g), FFT_THREADS, last_smem(g, true), s, g);
+    if (g.n0 > 1) launch_dep(fft_y_kernel<true>, y_blocks(g, g.n0), FFT_THREADS, y_smem(g), s, g);
+    launch_dep(fft_grad_kernel, (unsigned)fft_row_blocks(g), FFT_THREADS, row_smem(g), s, g);
 }
 
 void set_fft_attributes() {
-    cudaFuncSetAttribute(fft_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
+    const void* ks[] = {(const void*)fft_rows_kernel,         (const void*)fft_y_kernel<false>,
+                        (const void*)fft_y_kernel<true>,      (const void*)fft_last_kernel,
+                        (const void*)fft_win_y_kernel<true>,  (const void*)fft_win_y_kernel<false>,
+                        (const void*)fft_desc_kernel,         (const void*)fft_coef_kernel,
+                        (const void*)fft_mul_kernel,          (const void*)fft_grad_kernel};
+    for (const void* k : ks) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
 }
 
 }  // namespace dmcr
