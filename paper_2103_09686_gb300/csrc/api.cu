@@ -562,7 +562,7 @@ dmcr_status make_plan(const dmcr_params* p, Plan& pl) {
     pl.o_scal = o; o = align_up(o + sizeof(Scalars));
     pl.tab_bytes = align_up(table_bound(pl) + table_slack(pl.sep));
     pl.o_tab = o; o += pl.tab_bytes;
-    pl.o_pen = o; o = align_up(o + 3 * NPEN_BLOCKS * sizeof(double));
+    pl.o_pen = o; o = align_up(o + 2 * NPEN_BLOCKS * sizeof(float4));
     pl.o_desc = o; o = align_up(o + (size_t)pl.Ktot * sizeof(float));
     pl.o_tsum = o; o = align_up(o + (size_t)MAX_LEVELS * sizeof(float));
     if (pl.sep) {
@@ -766,7 +766,7 @@ struct Prepared {
         int64_t blocks;
     };
     std::vector<R> restricts;
-    R fwd{0, 0, 0}, red{0, 0, 0}, pen{0, 0, 0}, loss{0, 0, 0}, gco{0, 0, 0}, adj{0, 0, 0}, fin{0, 0, 0},
+    R fwd{0, 0, 0}, red{0, 0, 0}, pen{0, 0, 0}, gco{0, 0, 0}, adj{0, 0, 0}, fin{0, 0, 0},
         fin_small{0, 0, 0}, tmap{0, 0, 0}, tsum{0, 0, 0}, prep{0, 0, 0};
     size_t smem_fwd = 0, smem_adj = 0;
     // separable path, and the direct launches of its instances (run only where their gate opens)
@@ -1188,23 +1188,25 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
         int maxblk = 0;
         for (const Inst& x : in) {
             if (x.pl->sums) continue;      // its descriptor kernels finish the loss
-            double* pen = reinterpret_cast<double*>(x.ws + x.pl->o_pen);
+            float4* sums = reinterpret_cast<float4*>(x.ws + x.pl->o_pen);
             const int64_t Nall = x.pl->N1 * x.pl->phases;
             const int nblk = stats_blocks(x.pl->Ktot, x.lp.bc_on ? Nall : 0);
             maxblk = std::max(maxblk, nblk);
-            pv.push_back({x.lp.bc_on ? x.field : nullptr, Nall, x.desc, x.target, x.pl->Ktot, pen,
-                          x.use_done ? &x.sc->done : nullptr, nblk});
+            pv.push_back({x.lp.bc_on ? x.field : nullptr, Nall, x.desc, x.target, x.pl->Ktot, sums, sums + NPEN_BLOCKS,
+                          nullptr, x.use_done ? &x.sc->done : nullptr, nblk});
             LossSeg ls{};
             ls.lp = x.lp;
-            ls.pen = pen;
-            ls.nblk = nblk;
+            ls.sums = sums;
+            ls.excess = sums + NPEN_BLOCKS;
+            ls.nsum = ls.nexc = nblk;
             ls.sc = x.sc;
             ls.loss_out = x.loss_out;
             ls.history = x.history;
             lvv.push_back(ls);
         }
+        const size_t off = push(P.tb, lvv);
+        for (size_t k = 0; k < pv.size(); ++k) pv[k].loss = P.at<LossSeg>(off) + k;
         P.pen = {push(P.tb, pv), (int)pv.size(), (int64_t)maxblk};
-        P.loss = {push(P.tb, lvv), (int)lvv.size(), (int64_t)lvv.size()};
     }
     if (flags & F_BACK) {
         struct Item {
@@ -1431,13 +1433,9 @@ void run(const Prepared& P, cudaStream_t s) {
             launch_tilde_map(P.at<TildeSeg>(P.tmap.off), P.tmap.nseg, P.tmap.blocks, s);
         }
     }
-    if ((P.flags & F_LOSS) && P.loss.nseg > 0) {
-        {
-            ProfScope ps("loss_stats", -1, s);
-            launch_penalty(P.at<PenSeg>(P.pen.off), P.pen.nseg, (int)P.pen.blocks, s);
-        }
-        ProfScope ps("loss", -1, s);
-        launch_loss(P.at<LossSeg>(P.loss.off), P.loss.nseg, s);
+    if ((P.flags & F_LOSS) && P.pen.nseg > 0) {
+        ProfScope ps("loss_stats", -1, s);
+        launch_penalty(P.at<PenSeg>(P.pen.off), P.pen.nseg, (int)P.pen.blocks, s);
     }
     if (P.flags & F_BACK) {
         if (P.tsum.nseg > 0) {
@@ -1608,7 +1606,7 @@ std::string prepared_key(const Prepared& P) {
     add(&P.flags, sizeof P.flags);
     add(&P.tc, sizeof P.tc);
     for (const Prepared::R& r : P.restricts) add(&r, sizeof r);
-    for (const Prepared::R* r : {&P.fwd, &P.red, &P.pen, &P.loss, &P.gco, &P.adj, &P.fin, &P.fin_small,
+    for (const Prepared::R* r : {&P.fwd, &P.red, &P.pen, &P.gco, &P.adj, &P.fin, &P.fin_small,
                                    &P.tmap, &P.tsum, &P.prep, &P.gfwd, &P.gred, &P.gadj})
         add(r, sizeof *r);
     add(P.sep, sizeof P.sep);

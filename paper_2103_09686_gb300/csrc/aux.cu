@@ -206,12 +206,13 @@ __device__ __forceinline__ double block_sum_d(double v, double* sh) {
     return r;
 }
 
-// grid (max nblk, instances): double-float partial sums of one loss evaluation over the
+// Loss of the instances whose descriptor kernels do not finish it (three-point and corrected
+// descriptors, FFT levels), grid (max nblk, instances): double-float partial sums over the
 // instance's own nblk blocks (a fixed grid per problem size) -- sum (D - D_des)^2 and
 // sum D_des^2 over the descriptor, and sum ex^2 of the box excess over the field (when the
-// penalty is on).
-// partials[3 b + {0, 1, 2}] for block b.
-__global__ void stats_kernel(const PenSeg* __restrict__ segs) {
+// penalty is on); its last block sums the partials in a fixed order and finishes the loss
+// (a launch of its own: 9 us more).
+__global__ void __launch_bounds__(256) stats_kernel(const PenSeg* __restrict__ segs) {
     dep_wait();
     dep_trigger();
     const PenSeg& sg = segs[blockIdx.y];
@@ -224,17 +225,18 @@ __global__ void stats_kernel(const PenSeg* __restrict__ segs) {
     // this part and a thread sums only about 8 terms (stats_blocks) -- then a double-float
     // (two-sum) tree across the block
     float r2 = 0.f, r2c = 0.f, t2 = 0.f, t2c = 0.f, e2 = 0.f, e2c = 0.f;
-    // the terms of this thread in order; their loads issued four at a time (the same sums)
+    // the terms of this thread in order; their loads issued eight at a time (the same sums)
     int64_t k = i0;
-    for (; k + 3 * stride < sg.K; k += 4 * stride) {
-        float tv[4], dv[4];
+    constexpr int U = 8;
+    for (; k + (U - 1) * stride < sg.K; k += U * stride) {
+        float tv[U], dv[U];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < U; ++u) {
             tv[u] = sg.target[k + u * stride];
             dv[u] = sg.desc[k + u * stride];
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < U; ++u) {
             const float r = dv[u] - tv[u];
             kahan_add(r2, r2c, r * r);
             kahan_add(t2, t2c, tv[u] * tv[u]);
@@ -268,11 +270,10 @@ __global__ void stats_kernel(const PenSeg* __restrict__ segs) {
     const DF T2 = block_sum_df(df_two_sum(t2, -t2c), sh);
     const DF E2 = block_sum_df(df_two_sum(e2, -e2c), sh);
     if (threadIdx.x == 0) {
-        float2* part = reinterpret_cast<float2*>(sg.partials);
-        part[3 * blockIdx.x + 0] = make_float2(R2.hi, R2.lo);
-        part[3 * blockIdx.x + 1] = make_float2(T2.hi, T2.lo);
-        part[3 * blockIdx.x + 2] = make_float2(E2.hi, E2.lo);
+        sg.sums[blockIdx.x] = make_float4(R2.hi, R2.lo, T2.hi, T2.lo);
+        sg.excess[blockIdx.x] = make_float4(E2.hi, E2.lo, 0.f, 0.f);
     }
+    loss_arrive(*sg.loss, sg.nblk, sh);
 }
 
 void launch_penalty(const PenSeg* segs, int nseg, int maxblk, cudaStream_t s) {
@@ -324,30 +325,6 @@ __global__ void tilde_sum_kernel(const TildeSeg* __restrict__ segs) {
 void launch_tilde_sum(const TildeSeg* segs, int nseg, cudaStream_t s) {
     if (nseg <= 0) return;
     launch_dep(tilde_sum_kernel, nseg, 256, 0, s, segs);
-}
-
-// One block per instance whose statistics came from stats_kernel (three-point and corrected
-// descriptors, FFT levels): sums the partials in a fixed tree and finishes the loss.
-__global__ void __launch_bounds__(NPEN_BLOCKS) loss_kernel(const LossSeg* __restrict__ segs) {
-    dep_wait();
-    dep_trigger();
-    const LossSeg& sg = segs[blockIdx.x];
-    if (sg.lp.recon && sg.sc->done) return;
-    __shared__ DF sh[32];
-    // the instance's nblk double-float partials (the remaining threads add zeros)
-    const int b = threadIdx.x;
-    const float2* part = reinterpret_cast<const float2*>(sg.pen);
-    const DF zero{0.f, 0.f};
-    auto get = [&](int q) { return b < sg.nblk ? DF{part[3 * b + q].x, part[3 * b + q].y} : zero; };
-    const DF e2s = block_sum_df(get(0), sh);
-    const DF t2s = block_sum_df(get(1), sh);
-    const DF x2s = block_sum_df(get(2), sh);
-    if (threadIdx.x == 0) loss_scalars(sg, e2s, t2s, x2s);
-}
-
-void launch_loss(const LossSeg* segs, int nseg, cudaStream_t s) {
-    if (nseg <= 0) return;
-    launch_dep(loss_kernel, nseg, NPEN_BLOCKS, 0, s, segs);
 }
 
 // --------------------------------------------------------------------- gradient + Adam

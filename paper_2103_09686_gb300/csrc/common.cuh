@@ -162,10 +162,8 @@ struct FinalArgs {
 // their segment by binary search.  Tables live in device memory (written by blob_kernel).
 struct LossSeg {
     LossParams lp;
-    const double* pen;          // stats_kernel's partials (nblk blocks) ...
-    int nblk;
-    const float4* sums;         // ... or the descriptor blocks' sum (D - D_des)^2, sum D_des^2 (hi, lo each)
-    const float4* excess;       // and the field blocks' sum of squared box excess (hi, lo)
+    const float4* sums;         // block sums of (D - D_des)^2 and D_des^2 (hi, lo each)
+    const float4* excess;       // block sums of the squared box excess (hi, lo)
     int nsum, nexc;
     Scalars* sc;
     float* loss_out;
@@ -275,7 +273,8 @@ struct PenSeg {
     const float* desc;
     const float* target;
     int64_t K;
-    double* partials;        // 3 x nblk
+    float4 *sums, *excess;   // nblk each
+    const LossSeg* loss;
     const int* done;
     int nblk;                // blocks of this instance: a function of its own sizes only
 };
@@ -463,7 +462,6 @@ void launch_corr_adj_gated(const AdjSeg* segs, int nseg, int64_t blocks, size_t 
                            cudaStream_t s);
 void launch_penalty(const PenSeg* segs, int nseg, int maxblk, cudaStream_t s);
 int stats_blocks(int64_t K, int64_t N);
-void launch_loss(const LossSeg* segs, int nseg, cudaStream_t s);
 void launch_gcoef(const GSeg* segs, int nseg, int64_t blocks, const ThreshConst& tc, cudaStream_t s);
 void launch_tilde_map(const TildeSeg* segs, int nseg, int64_t blocks, cudaStream_t s);
 void launch_tilde_sum(const TildeSeg* segs, int nseg, cudaStream_t s);

@@ -236,6 +236,8 @@ __global__ void __launch_bounds__(GemmShape<BN>::THREADS, 1) tc_gemm_kernel(cons
     constexpr int GN = BN, GSTAGES = S::STAGES, STAGE_BYTES = S::STAGE_BYTES, B_TILE = S::B_TILE;
     constexpr int EPI_WARPS = S::EPI_WARPS, FLUSH = S::FLUSH;
     constexpr uint32_t TMEM_COLS = S::TMEM_COLS;
+    dep_wait();
+    dep_trigger();
     if (g.done != nullptr && *g.done) return;
     extern __shared__ __align__(1024) uint8_t gsm_raw[];
     // the swizzle atoms need 1024-byte aligned tiles
@@ -452,12 +454,6 @@ __device__ __forceinline__ int wrap_add(int v, int d, int n) {
     return w < 0 ? w + n : w;
 }
 
-// linear index of p + (rz, ry, rx), periodic
-__device__ __forceinline__ int64_t partner(const LevelGeom& g, const Pos3& p, int rz, int ry, int rx) {
-    const int n0 = (int)g.n[0], n1 = (int)g.n[1], n2 = (int)g.n[2];
-    return ((int64_t)wrap_add(p.z, rz, n0) * n1 + wrap_add(p.y, ry, n1)) * n2 + wrap_add(p.c, rx, n2);
-}
-
 // s = sigma(alpha (a - 0.75)) for a = (u + v) / 2, exact form (any finite range)
 __device__ __forceinline__ float sig_pair(const ThreshConst& tc, float u, float v) {
     float e;
@@ -467,94 +463,154 @@ __device__ __forceinline__ float sig_pair(const ThreshConst& tc, float u, float 
     return s;
 }
 
-// one block: 64 positions x 32 shifts.  Thread (tx, ty) owns positions x0 + 2 tx and
-// x0 + 2 tx + 1 and shifts k0 + ty + 8 i (i = 0..3).  E^T rows (shift-major) are written as
-// pairs of positions, one 32-bit word per thread (128-byte lines per warp); E rows
-// (position-major) go through a shared transpose and are written as pairs of shifts.
-// Padding entries are 0.
-__global__ void __launch_bounds__(256) ens_kernel(S3Job j, ThreshConst tc) {
+// One block: 128 positions x 64 shifts; a lane owns four consecutive positions and a warp eight
+// consecutive shifts, whose partners it reaches by stepping along rx (the row is found again only
+// where (rz, ry) changes).  E^T rows (shift-major) are written as 8 bytes per lane, 256 per warp;
+// E rows (position-major) go through shared memory, 16-byte chunks of eight shifts stored at
+// chunk ^ (position / 4 % 8) (conflict-free both ways), and are written as 128-byte lines.
+// Padding entries are 0.  Bound by the instruction rate and, close to it, by the stores
+// (8 bytes an entry): 16384 x 1985: 52 us
+// (5.2 TB/s; 64 x 32 blocks with an index computed per entry: 116 us).
+constexpr int ENS_X = 128, ENS_K = 64;
+
+// the pair (a, b) split into FP16 hi and lo words (a in the lower half)
+__device__ __forceinline__ void split_pair(float a, float b, uint32_t& hi, uint32_t& lo) {
+    const __half2 h = __floats2half2_rn(a, b);
+    const float2 f = __half22float2(h);
+    const __half2 l = __floats2half2_rn(a - f.x, b - f.y);
+    hi = *reinterpret_cast<const uint32_t*>(&h);
+    lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+
+template <bool IDENTITY>
+__global__ void __launch_bounds__(256, 3) ens_kernel(const __grid_constant__ S3Job j, const __grid_constant__ ThreshConst tc) {
+    dep_wait();
+    dep_trigger();
     if (j.done != nullptr && *j.done) return;
-    __shared__ uint16_t th[64][34], tl[64][34];
-    __shared__ int3 shifts[32];
+    __shared__ uint4 th[ENS_X * 8], tl[ENS_X * 8];
     const LevelGeom& g = j.g;
+    if (blockIdx.x == 0 && threadIdx.x == 0) j.amax[0] = 0.f;     // max |G| starts here
     // f(x) = x: e is bounded by max |M|, scaled into [-1, 1); the soft f is bounded by ~1.03
-    const float sE = ldexpf(1.f, -(tc.identity ? scale_exp(j.amax + 1) : 0));
-    const int64_t x0 = (int64_t)(blockIdx.x % (j.Npad / 64)) * 64;
-    const int64_t k0 = (int64_t)(blockIdx.x / (j.Npad / 64)) * 32;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
-    if (threadIdx.x < 32 && k0 + threadIdx.x < j.K) {
-        int rz, ry, rx;
-        decode_shift(g, (int)(k0 + threadIdx.x), rz, ry, rx);
-        shifts[threadIdx.x] = make_int3(rz, ry, rx);
-    }
-    __syncthreads();
-    const int64_t xa = x0 + 2 * tx;
-    const bool ina = xa < g.N, inb = xa + 1 < g.N;
-    const Pos3 pa = pos_of(g, ina ? xa : 0), pb = pos_of(g, inb ? xa + 1 : 0);
-    const float ua = ina ? j.field[xa] : 0.f, ub = inb ? j.field[xa + 1] : 0.f;
-    uint32_t* Eth = reinterpret_cast<uint32_t*>(j.Eth);
-    uint32_t* Etl = reinterpret_cast<uint32_t*>(j.Etl);
+    const float sE = IDENTITY ? ldexpf(1.f, -scale_exp(j.amax + 1)) : 1.f;
+    const unsigned xb = (unsigned)(j.Npad / ENS_X);
+    const int64_t x0 = (int64_t)(blockIdx.x % xb) * ENS_X, k0 = (int64_t)(blockIdx.x / xb) * ENS_K;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n0 = (int)g.n[0], n1 = (int)g.n[1], n2 = (int)g.n[2];
+    const int64_t xa = x0 + 4 * lane;
+    const int64_t ka = k0 + 8 * warp;
+    const float* __restrict__ field = j.field;
+    bool in[4];
+    float u[4];
+    Pos3 p[4];
+    int row[4], col[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int kk = ty + 8 * i;
-        const int64_t k = k0 + kk;
-        float ea = 0.f, eb = 0.f;
-        if (k < j.K) {
-            const int3 r = shifts[kk];
-            if (ina) {
-                const float v = j.field[partner(g, pa, r.x, r.y, r.z)];
-                ea = tc.identity ? 0.5f * (ua + v) : fmaf(tc.c1, sig_pair(tc, ua, v), tc.c3);
+    for (int q = 0; q < 4; ++q) {
+        in[q] = xa + q < g.N;
+        p[q] = pos_of(g, in[q] ? xa + q : 0);
+        u[q] = in[q] ? field[xa + q] : 0.f;
+    }
+    int rz = 0, ry = 0, rx = 0;
+    if (ka < j.K) decode_shift(g, (int)ka, rz, ry, rx);
+    auto start_row = [&]() {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            row[q] = (wrap_add(p[q].z, rz, n0) * n1 + wrap_add(p[q].y, ry, n1)) * n2;
+            col[q] = wrap_add(p[q].c, rx, n2);
+        }
+    };
+    start_row();
+    uint32_t hw[4][4], lw[4][4];        // [position][pair of shifts]
+    uint32_t ph[2], pl[2];              // the pair's first shift, positions in pairs
+    uint2* Eth = reinterpret_cast<uint2*>(j.Eth + ka * j.Npad + xa);
+    uint2* Etl = reinterpret_cast<uint2*>(j.Etl + ka * j.Npad + xa);
+    const int64_t step = j.Npad / 4;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        float e[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            e[q] = 0.f;
+            if (ka + i < j.K) {
+                const float v = field[row[q] + col[q]];
+                e[q] = IDENTITY ? 0.5f * (u[q] + v) * sE : fmaf(tc.c1, sig_pair(tc, u[q], v), tc.c3);
+                if (!in[q]) e[q] = 0.f;
             }
-            if (inb) {
-                const float v = j.field[partner(g, pb, r.x, r.y, r.z)];
-                eb = tc.identity ? 0.5f * (ub + v) : fmaf(tc.c1, sig_pair(tc, ub, v), tc.c3);
+            const unsigned c = (unsigned)col[q] + 1u;
+            col[q] = (int)min(c, c - (unsigned)n2);
+        }
+        if (++rx > g.P[2]) {
+            rx = -g.P[2];
+            if (++ry > g.P[1]) {
+                ry = -g.P[1];
+                ++rz;
+            }
+            if (ka + i + 1 < j.K) start_row();
+        }
+        uint32_t h[2], l[2];
+        split_pair(e[0], e[1], h[0], l[0]);
+        split_pair(e[2], e[3], h[1], l[1]);
+        Eth[i * step] = make_uint2(h[0], h[1]);
+        Etl[i * step] = make_uint2(l[0], l[1]);
+        if (i % 2 == 0) {
+            ph[0] = h[0], ph[1] = h[1], pl[0] = l[0], pl[1] = l[1];
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const unsigned sel = q % 2 ? 0x7632u : 0x5410u;
+                hw[q][i / 2] = __byte_perm(ph[q / 2], h[q / 2], sel);
+                lw[q][i / 2] = __byte_perm(pl[q / 2], l[q / 2], sel);
             }
         }
-        uint16_t ha, la, hb, lb;
-        split_f16(ea * sE, ha, la);
-        split_f16(eb * sE, hb, lb);
-        // the lower address holds the lower 16 bits (little endian)
-        Eth[(k * j.Npad + xa) / 2] = (uint32_t)ha | ((uint32_t)hb << 16);
-        Etl[(k * j.Npad + xa) / 2] = (uint32_t)la | ((uint32_t)lb << 16);
-        th[2 * tx][kk] = ha;
-        th[2 * tx + 1][kk] = hb;
-        tl[2 * tx][kk] = la;
-        tl[2 * tx + 1][kk] = lb;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int o = (4 * lane + q) * 8 + (warp ^ (lane & 7));
+        th[o] = make_uint4(hw[q][0], hw[q][1], hw[q][2], hw[q][3]);
+        tl[o] = make_uint4(lw[q][0], lw[q][1], lw[q][2], lw[q][3]);
     }
     __syncthreads();
-    // E rows: 64 positions x 16 words of shift pairs
-    uint32_t* Eh = reinterpret_cast<uint32_t*>(j.Eh);
-    uint32_t* El = reinterpret_cast<uint32_t*>(j.El);
-    const int w = threadIdx.x & 15;
-    for (int pp = threadIdx.x >> 4; pp < 64; pp += 16) {
-        const int64_t o = ((x0 + pp) * j.Kpad + k0) / 2 + w;
-        Eh[o] = (uint32_t)th[pp][2 * w] | ((uint32_t)th[pp][2 * w + 1] << 16);
-        El[o] = (uint32_t)tl[pp][2 * w] | ((uint32_t)tl[pp][2 * w + 1] << 16);
+    // E rows: 128 positions x 8 chunks
+    const int c = threadIdx.x & 7;
+    for (int pp = threadIdx.x >> 3; pp < ENS_X; pp += 32) {
+        const int64_t o = (x0 + pp) * j.Kpad + k0 + 8 * c;
+        const int t = pp * 8 + (c ^ ((pp >> 2) & 7));
+        *reinterpret_cast<uint4*>(j.Eh + o) = th[t];
+        *reinterpret_cast<uint4*>(j.El + o) = tl[t];
     }
 }
 
 // G(a, b) = w * gscale * sym(D3 - D3_des) on the level's K x K block; d<G, E^T E>/dE =
 // E (G + G^T), so G is symmetrised (the loss gradient already is symmetric).  A block holds
 // a 32 x 32 tile; the transposed entries come through shared memory, so both reads are
-// coalesced.  Returns v(a0 + i, b0 + tx) for i = ty, ty + 8, ... in v[4] (0 outside K x K).
+// coalesced, and v is symmetric: a block covers the tiles (ta, tb) and (tb, ta), ta <= tb, from
+// one read of both.  Returns v(a0 + i, b0 + tx) for i = ty, ty + 8, ... in v[4] (0 outside K x K).
 __device__ __forceinline__ float g3_delta(const S3Job& j, int64_t a, int64_t b) {
     return j.src[a * j.K + b] - (j.sub != nullptr ? j.sub[a * j.K + b] : 0.f);
 }
 
-__device__ __forceinline__ void g3_tile(const S3Job& j, int64_t a0, int64_t b0, float (&v)[4]) {
-    __shared__ float tt[32][33];
+__device__ __forceinline__ void g3_tile(const S3Job& j, int64_t a0, int64_t b0, float (*tt)[33], float (&v)[4]) {
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    for (int i = ty; i < 32; i += 8) {
-        const int64_t b = b0 + i, a = a0 + tx;
-        tt[tx][i] = (a < j.K && b < j.K) ? g3_delta(j, b, a) : 0.f;   // tt[a - a0][b - b0] = d(b, a)
+    float d[4], m[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int64_t i = ty + 8 * q;
+        d[q] = (a0 + i < j.K && b0 + tx < j.K) ? g3_delta(j, a0 + i, b0 + tx) : 0.f;
+        m[q] = (b0 + i < j.K && a0 + tx < j.K) ? g3_delta(j, b0 + i, a0 + tx) : 0.f;
     }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) tt[tx][ty + 8 * q] = m[q];
     __syncthreads();
     const float sc = j.weight * (j.sc != nullptr ? j.sc->gscale : 1.f);
-    for (int q = 0; q < 4; ++q) {
-        const int i = ty + 8 * q;
-        const int64_t a = a0 + i, b = b0 + tx;
-        v[q] = (a < j.K && b < j.K) ? sc * 0.5f * (g3_delta(j, a, b) + tt[i][tx]) : 0.f;
-    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = sc * 0.5f * (d[q] + tt[ty + 8 * q][tx]);
+}
+
+// block -> tile pair (ta <= tb) of the upper triangle, columns in order: tb (tb + 1) / 2 + ta
+__device__ __forceinline__ void g3_pair(int64_t t, int64_t& ta, int64_t& tb) {
+    tb = (int64_t)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+    while (tb * (tb + 1) / 2 > t) --tb;
+    while ((tb + 1) * (tb + 2) / 2 <= t) ++tb;
+    ta = t - tb * (tb + 1) / 2;
 }
 
 // max |v| of a block's values into *out (non-negative floats order like their bit patterns;
@@ -570,19 +626,25 @@ __device__ __forceinline__ void block_absmax(float m, float* out) {
     }
 }
 
-// one 32 x 32 tile of G per block
-__global__ void __launch_bounds__(256) g3_absmax_kernel(S3Job j) {
+// one pair of 32 x 32 tiles of G per block (K = 1985: 12 us; each tile on its own 18)
+__global__ void __launch_bounds__(256) g3_absmax_kernel(const __grid_constant__ S3Job j) {
+    dep_wait();
+    dep_trigger();
     if (j.done != nullptr && *j.done) return;
-    const int64_t tiles = (j.K + 31) / 32;
+    __shared__ float tt[32][33];
+    int64_t ta, tb;
+    g3_pair(blockIdx.x, ta, tb);
     float v[4];
-    g3_tile(j, (blockIdx.x / tiles) * 32, (blockIdx.x % tiles) * 32, v);
+    g3_tile(j, ta * 32, tb * 32, tt, v);
     float m = 0.f;
     for (int q = 0; q < 4; ++q) m = fmaxf(m, fabsf(v[q]));
     block_absmax(m, j.amax);
 }
 
 // f(x) = x: max |M| of the level's field, the bound of |e|
-__global__ void __launch_bounds__(256) field_absmax_kernel(S3Job j) {
+__global__ void __launch_bounds__(256) field_absmax_kernel(const __grid_constant__ S3Job j) {
+    dep_wait();
+    dep_trigger();
     if (j.done != nullptr && *j.done) return;
     float m = 0.f;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < j.g.N; i += (int64_t)gridDim.x * blockDim.x)
@@ -590,99 +652,117 @@ __global__ void __launch_bounds__(256) field_absmax_kernel(S3Job j) {
     block_absmax(m, j.amax + 1);
 }
 
-// G scaled by 2^-eG (max |G| into [1/2, 1)) and split into FP16 hi + lo, one 32 x 32 tile of
-// Kpad x Kpad per block (zero padding)
-__global__ void __launch_bounds__(256) g3_split_kernel(S3Job j) {
+// G scaled by 2^-eG (max |G| into [1/2, 1)) and split into FP16 hi + lo, one pair of 32 x 32
+// tiles of Kpad x Kpad per block (zero padding; K = 1985: 14 us, each tile on its own 20)
+__global__ void __launch_bounds__(256) g3_split_kernel(const __grid_constant__ S3Job j) {
+    dep_wait();
+    dep_trigger();
     if (j.done != nullptr && *j.done) return;
-    const int64_t tiles = j.Kpad / 32;
-    const int64_t a0 = (blockIdx.x / tiles) * 32, b0 = (blockIdx.x % tiles) * 32;
+    __shared__ float tt[32][33];
+    int64_t ta, tb;
+    g3_pair(blockIdx.x, ta, tb);
     float v[4];
-    g3_tile(j, a0, b0, v);
+    g3_tile(j, ta * 32, tb * 32, tt, v);
     const int eG = scale_exp(j.amax);
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    // the second tile is the transpose of the first
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) tt[tx][ty + 8 * q] = v[q];
+    __syncthreads();
+#pragma unroll
     for (int q = 0; q < 4; ++q) {
-        const int64_t i = (a0 + ty + 8 * q) * j.Kpad + b0 + tx;
+        const int r = ty + 8 * q;
         uint16_t hi, lo;
         split_f16(ldexpf(v[q], -eG), hi, lo);
+        const int64_t i = (ta * 32 + r) * j.Kpad + tb * 32 + tx;
         j.Gh[i] = hi;
         j.Gl[i] = lo;
+        split_f16(ldexpf(tt[r][tx], -eG), hi, lo);
+        const int64_t t = (tb * 32 + r) * j.Kpad + ta * 32 + tx;
+        j.Gh[t] = hi;
+        j.Gl[t] = lo;
     }
 }
 
 // g_y = sum_k c_k [W(k, y) f'(a_y(r_k)) + W(k, y - r_k) f'(a_{y - r_k}(r_k))], c_0 = 1/2 (the two
 // terms coincide at r = 0), c_k = 1/2 otherwise; f' = c1 alpha s (1 - s), or 1 for f(x) = x.
 // Block (position block, shift chunk of S3_SHIFTS): per-chunk partials, summed in a fixed order
-// by the gradient assembly.
-__global__ void __launch_bounds__(256) s3_gather_kernel(S3Job j, ThreshConst tc) {
+// by the gradient assembly.  The chunk's shifts come in canonical order (rx fastest, then ry,
+// then rz): the partner columns are stepped along rx, the rows rebuilt where (rz, ry) changes;
+// four shifts per step, their loads issued together.  Bound by the instruction rate (four
+// special-function operations a term): 16384 x 1985 61 us, 127 with 64-bit indexes.
+template <bool IDENTITY>
+__global__ void __launch_bounds__(256, 5) s3_gather_kernel(const __grid_constant__ S3Job j, const __grid_constant__ ThreshConst tc) {
+    dep_wait();
+    dep_trigger();
     if (j.done != nullptr && *j.done) return;
     const LevelGeom& g = j.g;
-    const int64_t y = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     if (y >= g.N) return;
-    const int64_t kA = (int64_t)blockIdx.y * S3_SHIFTS;
-    const int64_t kB = min(kA + (int64_t)S3_SHIFTS, j.K);
-    const float c1a = tc.c1 * tc.alpha;
-    const float my = j.field[y];
-    const Pos3 py = pos_of(g, y);
-    float acc = 0.f;
-    // the chunk's shifts in canonical order: rx fastest, then ry, then rz (decoded once); the
-    // partner indices y + r and y - r are stepped along rx and rebuilt when (rz, ry) changes;
-    // four shifts per step, their loads issued together
-    int rz, ry, rx;
-    decode_shift(g, (int)kA, rz, ry, rx);
+    const int kA = (int)blockIdx.y * S3_SHIFTS;
+    const int nk = (int)min((int64_t)S3_SHIFTS, j.K - kA);
     const float* __restrict__ field = j.field;
-    const float* __restrict__ W = j.W;
+    const float* __restrict__ W = j.W + (int64_t)kA * j.Npad;
     const int n0 = (int)g.n[0], n1 = (int)g.n[1], n2 = (int)g.n[2];
-    int64_t rowp = 0, rowm = 0;
-    int cp = 0, cm = 0;
+    const float my = field[y];
+    const Pos3 py = pos_of(g, y);
+    int rz, ry, rx, rowp, rowm, cp, cm;
+    decode_shift(g, kA, rz, ry, rx);
     auto rows = [&]() {
-        rowp = ((int64_t)wrap_add(py.z, rz, n0) * n1 + wrap_add(py.y, ry, n1)) * n2;
-        rowm = ((int64_t)wrap_add(py.z, -rz, n0) * n1 + wrap_add(py.y, -ry, n1)) * n2;
+        rowp = (wrap_add(py.z, rz, n0) * n1 + wrap_add(py.y, ry, n1)) * n2;
+        rowm = (wrap_add(py.z, -rz, n0) * n1 + wrap_add(py.y, -ry, n1)) * n2;
+        cp = wrap_add(py.c, rx, n2);
+        cm = wrap_add(py.c, -rx, n2);
     };
     rows();
-    cp = wrap_add(py.c, rx, n2);
-    cm = wrap_add(py.c, -rx, n2);
+    auto next = [&]() {
+        if (++rx > g.P[2]) {
+            rx = -g.P[2];
+            if (++ry > g.P[1]) {
+                ry = -g.P[1];
+                ++rz;
+            }
+            rows();
+        } else {
+            const unsigned c = (unsigned)cp + 1u;
+            cp = (int)min(c, c - (unsigned)n2);
+            cm = cm == 0 ? n2 - 1 : cm - 1;
+        }
+    };
+    // W f' without the constant factor c1 alpha
+    auto term = [&](float w, float u, float v) {
+        if (IDENTITY) return w;
+        const float s = sig_pair(tc, u, v);
+        return w * fmaf(-s, s, s);
+    };
+    float acc = 0.f;
     constexpr int U = 4;
-    for (int64_t k0 = kA; k0 < kB; k0 += U) {
-        int64_t ym[U];
+    int k = 0;
+    for (; k + U <= nk; k += U, W += U * j.Npad) {
         float vp[U], vm[U], w1[U], w2[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const bool in = k0 + u < kB;
-            const int64_t k = in ? k0 + u : kA;
-            const int64_t yp = rowp + cp;                       // y + r
-            ym[u] = rowm + cm;                                  // y - r
-            vp[u] = field[yp];
-            vm[u] = field[ym[u]];
-            w1[u] = in ? W[k * j.Npad + y] : 0.f;
-            w2[u] = in ? W[k * j.Npad + ym[u]] : 0.f;
-            if (++rx > g.P[2]) {
-                rx = -g.P[2];
-                if (++ry > g.P[1]) {
-                    ry = -g.P[1];
-                    ++rz;
-                }
-                rows();
-                cp = wrap_add(py.c, rx, n2);
-                cm = wrap_add(py.c, -rx, n2);
-            } else {
-                cp = cp + 1 == n2 ? 0 : cp + 1;
-                cm = cm == 0 ? n2 - 1 : cm - 1;
-            }
+            const int ym = rowm + cm;                           // y - r
+            vp[u] = IDENTITY ? 0.f : field[rowp + cp];          // y + r
+            vm[u] = IDENTITY ? 0.f : field[ym];
+            w1[u] = W[u * j.Npad + y];
+            w2[u] = W[u * j.Npad + ym];
+            next();
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            float d1 = 1.f, d2 = 1.f;
-            if (!tc.identity) {
-                const float s1 = sig_pair(tc, my, vp[u]);
-                const float s2 = sig_pair(tc, vm[u], my);
-                d1 = c1a * s1 * (1.f - s1);
-                d2 = c1a * s2 * (1.f - s2);
-            }
-            acc = fmaf(0.5f * w1[u], d1, acc);
-            acc = fmaf(0.5f * w2[u], d2, acc);
+            acc += term(w1[u], my, vp[u]);
+            acc += term(w2[u], vm[u], my);
         }
     }
-    j.part[(int64_t)blockIdx.y * g.N + y] = acc;
+    for (; k < nk; ++k, W += j.Npad) {
+        const int ym = rowm + cm;
+        acc += term(W[y], my, field[rowp + cp]);
+        acc += term(W[ym], field[ym], my);
+        next();
+    }
+    j.part[(int64_t)blockIdx.y * g.N + y] = IDENTITY ? 0.5f * acc : 0.5f * tc.c1 * tc.alpha * acc;
 }
 
 // ------------------------------------------------------------------------- launchers
@@ -695,6 +775,8 @@ void set_gram_attributes() {
 }
 
 __global__ void set_flag_kernel(int* flag, int v) {
+    dep_wait();
+    dep_trigger();
     if (flag != nullptr) *flag = v;
 }
 
@@ -740,7 +822,7 @@ void launch_tc_gemm(const GemmOperands& o, cudaStream_t s) {
                     make_map(&a.tb_hi, o.Bh, o.N, o.K, o.ldb, BN) && make_map(&a.tb_lo, o.Bl, o.N, o.K, o.ldb, BN);
     if (!ok) {
         // no valid tensor map: never launch TMA on it; report through the error word
-        set_flag_kernel<<<1, 1, 0, s>>>(o.err, 2);
+        launch_dep(set_flag_kernel, 1, 1, 0, s, o.err, 2);
         return;
     }
     a.M = o.M; a.N = o.N; a.K = o.K;
@@ -754,21 +836,24 @@ void launch_tc_gemm(const GemmOperands& o, cudaStream_t s) {
     a.done = o.done;
     a.err = o.err;
     if (BN == 128)
-        tc_gemm_kernel<128><<<(unsigned)blocks, GemmShape<128>::THREADS, GemmShape<128>::SMEM, s>>>(a);
+        launch_dep(tc_gemm_kernel<128>, (unsigned)blocks, GemmShape<128>::THREADS, GemmShape<128>::SMEM, s, a);
     else
-        tc_gemm_kernel<256><<<(unsigned)blocks, GemmShape<256>::THREADS, GemmShape<256>::SMEM, s>>>(a);
+        launch_dep(tc_gemm_kernel<256>, (unsigned)blocks, GemmShape<256>::THREADS, GemmShape<256>::SMEM, s, a);
 }
 
 constexpr int ABSMAX_BLOCKS = 512;
 
 // E and E^T of one level (f(x) = x: after the bound of |e|)
 void launch_ensemble(const S3Job& j, const ThreshConst& tc, cudaStream_t s) {
+    const unsigned blocks = (unsigned)((j.Npad / ENS_X) * (j.Kpad / ENS_K));
     if (tc.identity) {
-        set_flag_kernel<<<1, 1, 0, s>>>(reinterpret_cast<int*>(j.amax + 1), 0);
-        const int64_t blocks = std::min<int64_t>(ABSMAX_BLOCKS, (j.g.N + 255) / 256);
-        field_absmax_kernel<<<(unsigned)blocks, 256, 0, s>>>(j);
+        launch_dep(set_flag_kernel, 1, 1, 0, s, reinterpret_cast<int*>(j.amax + 1), 0);
+        const int64_t fb = std::min<int64_t>(ABSMAX_BLOCKS, (j.g.N + 255) / 256);
+        launch_dep(field_absmax_kernel, (unsigned)fb, 256, 0, s, j);
+        launch_dep(ens_kernel<true>, blocks, 256, 0, s, j, tc);
+    } else {
+        launch_dep(ens_kernel<false>, blocks, 256, 0, s, j, tc);
     }
-    ens_kernel<<<(unsigned)((j.Npad / 64) * (j.Kpad / 32)), 256, 0, s>>>(j, tc);
 }
 
 void launch_s3_forward(const S3Job& j, const ThreshConst& tc, int* err, cudaStream_t s) {
@@ -791,10 +876,9 @@ void launch_s3_forward(const S3Job& j, const ThreshConst& tc, int* err, cudaStre
 
 void launch_s3_backward(const S3Job& j, const ThreshConst& tc, int* err, cudaStream_t s) {
     if (j.ens) launch_ensemble(j, tc, s);
-    set_flag_kernel<<<1, 1, 0, s>>>(reinterpret_cast<int*>(j.amax), 0);
-    const int64_t tk = (j.K + 31) / 32;
-    g3_absmax_kernel<<<(unsigned)(tk * tk), 256, 0, s>>>(j);
-    g3_split_kernel<<<(unsigned)((j.Kpad / 32) * (j.Kpad / 32)), 256, 0, s>>>(j);
+    const int64_t tk = (j.K + 31) / 32, tp = j.Kpad / 32;
+    launch_dep(g3_absmax_kernel, (unsigned)(tk * (tk + 1) / 2), 256, 0, s, j);
+    launch_dep(g3_split_kernel, (unsigned)(tp * (tp + 1) / 2), 256, 0, s, j);
     GemmOperands a{};
     a.Ah = j.Eh; a.Al = j.El; a.Bh = j.Gh; a.Bl = j.Gl;
     a.amaxA = tc.identity ? j.amax + 1 : nullptr;
@@ -814,7 +898,8 @@ void launch_s3_backward(const S3Job& j, const ThreshConst& tc, int* err, cudaStr
     a.err = err;
     launch_tc_gemm(a, s);
     const dim3 grid((unsigned)((j.g.N + 255) / 256), (unsigned)((j.K + S3_SHIFTS - 1) / S3_SHIFTS));
-    s3_gather_kernel<<<grid, 256, 0, s>>>(j, tc);
+    if (tc.identity) launch_dep(s3_gather_kernel<true>, grid, 256, 0, s, j, tc);
+    else launch_dep(s3_gather_kernel<false>, grid, 256, 0, s, j, tc);
 }
 
 }  // namespace dmcr
