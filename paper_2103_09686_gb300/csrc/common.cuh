@@ -473,7 +473,6 @@ void launch_init_uniform(float* field, int64_t count, uint64_t seed, cudaStream_
 void launch_round_field(const float* src, float* dst, int64_t count, cudaStream_t s);
 void set_kernel_attributes();
 void set_gram_attributes();
-size_t gemm_smem_bytes();
 bool gram_ready();   // the TMA tensor-map encoder is available
 void launch_s3_forward(const S3Job& j, const ThreshConst& tc, int* err, cudaStream_t s);
 void launch_s3_backward(const S3Job& j, const ThreshConst& tc, int* err, cudaStream_t s);

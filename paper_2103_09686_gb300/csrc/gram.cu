@@ -15,10 +15,9 @@
 //                   product), operands staged by TMA (128-byte swizzled K-major layout), one
 //                   thread issues the MMAs and commits them to an mbarrier per stage; the
 //                   epilogue undoes the operands' scales exactly;
-//                   Gram:  S_bar3 = Et Et^T w/N (upper-triangle 128 x 128 tiles, mirrored,
-//                          three 64 KB stages);
-//                   W:     W^T = (2/N) G E^T  as  E G^T with a transposed epilogue (128 x 256
-//                          tiles, two 96 KB stages);
+//                   S_bar3 = Et Et^T w/N (upper-triangle 128 x 128 tiles, mirrored);
+//   tc_gemm_pair_kernel  the same for W^T = (2/N) G E^T as E G^T with a transposed epilogue:
+//                   256 x 256 tiles, each on a pair of SMs (cta_group::2);
 //   g3_split_kernel G = w * gscale * (D3 - D3_des) symmetrised (or the upstream gradient),
 //                   scaled by the power of two that brings max |G| (g3_absmax_kernel) into
 //                   [1/2, 1), split like E;
@@ -46,7 +45,6 @@ struct GemmArgs {
     const float* amaxB;
     float* C;
     int64_t ldc;
-    int mode;               // 1 symmetric Gram (upper tiles, mirrored), 2 C[n][m]
     int Mvalid, Nvalid;
     const int* done;
     int* err;
@@ -62,7 +60,7 @@ struct GemmOperands {
     const float* amaxB;
     float* C;
     int64_t ldc;
-    int mode;
+    int mode;               // 1 symmetric Gram (upper tiles, mirrored), 2 C[n][m]
     int Mvalid, Nvalid;
     const int* done;
     int* err;
@@ -70,34 +68,29 @@ struct GemmOperands {
 
 namespace {
 
-// Tiles of GM x BN outputs, BN = 128 or 256 (kernel template); GK reduction steps per stage.
+// A CTA holds 128 rows of a tile; GK reduction steps per stage, three stages.  Both kernels stage
+// 128 rows of A and of B, hi and lo, 64 KB.
 constexpr int GM = 128, GK = 64;
-constexpr int A_TILE = GM * GK * 2;                    // one FP16 A tile (128 rows of 128 bytes), 16 KB
-template <int BN>
-struct GemmShape {
-    static constexpr int B_TILE = BN * GK * 2;                   // one FP16 B tile
-    static constexpr int STAGE_BYTES = 2 * A_TILE + 2 * B_TILE;  // A hi, A lo, B hi, B lo
-    static constexpr int STAGES = BN == 128 ? 3 : 2;             // 192 KB of stages
-    static constexpr int EPI_WARPS = BN / 32;                    // 128 columns of one lane quadrant each
-    static constexpr int THREADS = 32 * (EPI_WARPS + 2);         // epilogue warps, then TMA, then MMA
-    // 128-wide tiles keep the small cross terms hi*lo + lo*hi in an accumulator of their own
-    // (FLUSH 8 k-blocks: 32 MMAs per accumulator); 256-wide tiles add all three products into
-    // one accumulator (TMEM holds two buffers of 256 columns) and drain twice as often
-    static constexpr bool SPLIT = BN == 128;
-    static constexpr int FLUSH = SPLIT ? 8 : 4;
-    static constexpr uint32_t BUF_COLS = SPLIT ? 2 * BN : BN;     // one buffer: main (+ cross)
-    static constexpr uint32_t TMEM_COLS = 2 * BUF_COLS;          // 512 columns, 128 lanes
-    // instruction descriptor, kind::f16: D F32 (bits 4-5 = 1), A and B F16 (bits 7-9, 10-12 = 0),
-    // both K-major (bits 15, 16 = 0), N >> 3 at bits 17-22, M >> 4 at bits 24-28
-    static constexpr uint32_t IDESC = (1u << 4) | (0u << 7) | (0u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                                      ((uint32_t)(GM >> 4) << 24);
-    static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024 + 256;
-};
+constexpr int OP_TILE = GM * GK * 2;                   // one FP16 operand tile (128 rows of 128 bytes), 16 KB
+constexpr int STAGE_BYTES = 4 * OP_TILE;               // A hi, A lo, B hi, B lo
+constexpr int GSTAGES = 3;
+constexpr size_t GEMM_SMEM = (size_t)GSTAGES * STAGE_BYTES + 1024 + 256;
+constexpr uint32_t BUF_COLS = 256, TMEM_COLS = 512;    // two accumulator buffers
+constexpr int EC = 128;                                // accumulator columns of one epilogue thread
+// Gram: 4 epilogue warps; a buffer holds hi*hi and, 128 columns further, the small cross terms
+// hi*lo + lo*hi.  Pair: 8 epilogue warps; a buffer holds all three products of 256 columns and
+// is drained twice as often.
+constexpr int GRAM_EPI = 4, GRAM_FLUSH = 8;
+constexpr int PAIR_EPI = 8, PAIR_FLUSH = 4;
+// instruction descriptor, kind::f16: D F32 (bits 4-5 = 1), A and B F16 (bits 7-9, 10-12 = 0),
+// both K-major (bits 15, 16 = 0), N >> 3 at bits 17-22, M >> 4 at bits 24-28
+__host__ __device__ constexpr uint32_t idesc_f16(int m, int n) { return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24); }
 // The tensor core adds into its FP32 accumulator without round-to-nearest: over a long
 // reduction the error is biased toward zero (~4e-8 relative per accumulation measured on
-// GB300).  So TMEM accumulates at most FLUSH k-blocks (GemmShape) before the partial sums are
-// added, rounded to nearest, into FP32 registers.
+// GB300).  So TMEM accumulates at most FLUSH k-blocks before the partial sums are added,
+// rounded to nearest, into FP32 registers.
 constexpr uint32_t WAIT_LIMIT = 1u << 22;
+constexpr unsigned long long WAIT_NS = 4000000000ull;
 
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -122,34 +115,79 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
 
-// bounded wait for the completion of the mbarrier phase with the given parity
+// bounded wait (tries, and WAIT_NS of time) for the completion of the mbarrier phase with the
+// given parity; CLUSTER: the other CTA of the pair arrives on it
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
     const uint32_t addr = smem_u32(bar);
+    unsigned long long start = 0;
     for (uint32_t i = 0; i < WAIT_LIMIT; ++i) {
         uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.b32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(addr), "r"(parity)
-            : "memory");
+        if constexpr (CLUSTER)
+            asm volatile(
+                "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                "selp.b32 %0, 1, 0, p;\n\t}"
+                : "=r"(ok)
+                : "r"(addr), "r"(parity)
+                : "memory");
+        else
+            asm volatile(
+                "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                "selp.b32 %0, 1, 0, p;\n\t}"
+                : "=r"(ok)
+                : "r"(addr), "r"(parity)
+                : "memory");
         if (ok) return true;
+        if (i % 1024 == 1023) {
+            unsigned long long now;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+            if (start == 0) start = now;
+            else if (now - start > WAIT_NS) return false;
+        }
     }
     return false;
+}
+// arrive on the barrier at the same place in the pair's first CTA
+__device__ __forceinline__ void mbar_arrive_first(uint64_t* bar) {
+    asm volatile(
+        "{\n\t.reg .b32 ra;\n\tmapa.shared::cluster.u32 ra, %0, 0;\n\t"
+        "mbarrier.arrive.release.cluster.shared::cluster.b64 _, [ra];\n\t}" ::"r"(smem_u32(bar))
+        : "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
 }
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// whole warp: allocate TMEM columns, address written to shared memory
-__device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t ncols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)),
-                 "r"(ncols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+// whole warp: allocate all TMEM columns, address written to shared memory; PAIR: one warp of each
+// CTA of the pair
+template <bool PAIR>
+__device__ __forceinline__ void tmem_alloc(uint32_t* slot) {
+    if constexpr (PAIR) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)),
+                     "r"(TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)),
+                     "r"(TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
 }
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+template <bool PAIR>
+__device__ __forceinline__ void tmem_dealloc(uint32_t taddr) {
+    if constexpr (PAIR)
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(TMEM_COLS) : "memory");
+    else
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(TMEM_COLS) : "memory");
 }
 
 // shared-memory matrix descriptor, K-major with the 128-byte swizzle: each operand row is
@@ -162,18 +200,36 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
            (2ull << 61);
 }
 
+template <bool PAIR>
 __device__ __forceinline__ void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
-        : "memory");
+    if constexpr (PAIR)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+            "l"(a), "l"(b), "r"(idesc), "r"(acc)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+            "l"(a), "l"(b), "r"(idesc), "r"(acc)
+            : "memory");
 }
 
+// arrive on the barrier (PAIR: at the same place in both CTAs) when every earlier MMA of this
+// thread has completed
+template <bool PAIR>
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                     smem_u32(bar))
-                 : "memory");
+    if constexpr (PAIR)
+        asm volatile(
+            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+                smem_u32(bar)),
+            "h"((uint16_t)3)
+            : "memory");
+    else
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                         smem_u32(bar))
+                     : "memory");
 }
 
 // 32 lanes x 16 columns of 32 bits: thread i of the warp gets lane (lane base + i)
@@ -214,31 +270,53 @@ __device__ __forceinline__ int scale_exp(const float* amax) {
 // ------------------------------------------------------------------------- GEMM
 
 // C = scale 2^(eA + eB) A B^T with A (M x K) and B (N x K) row-major (K contiguous), each given
-// as FP16 hi + lo through four TMA tensor maps (boxes 64 x 128 for A, 64 x BN for B, 128-byte
-// swizzle).  M a multiple of 128, N of BN, K of 64.  Tiles are 128 x BN.  mode 1 (Gram, A = B,
-// square tiles, BN = 128): only tiles bn >= bm, written to C[m][n] and C[n][m]; mode 2:
-// C[n][m].  Entries with m >= Mvalid or n >= Nvalid are not written.
+// as FP16 hi + lo through four TMA tensor maps (boxes 64 x 128, 128-byte swizzle; rows past the
+// end read as zero).  K a multiple of 64.
 //
-// The single issuing thread spends about 400 cycles per stage besides the MMAs (barrier
-// wait, commit, loop): 128 x 256 tiles (twice the MMA work per stage) keep the tensor pipe
-// fed where the grid is large (the W GEMM); the Gram, whose upper triangle holds few tiles,
-// keeps 128 x 128 tiles so that it fills the SMs.
-//
-// Warp roles: warp EPI (one lane) loads the stages with TMA; warp EPI + 1 (one lane) issues
-// the MMAs and commits them; warps 0 .. EPI - 1 drain the TMEM accumulators every FLUSH
-// k-blocks into FP32 registers (warp w reads TMEM lanes 32 (w % 4) .. + 31 and columns
-// 128 (w / 4) .. + 127; TMEM is double-buffered, two periods of BN columns) and write the
-// tile.  Barriers: full[s] (TMA bytes landed), empty[s] (MMAs done reading stage s),
-// tfull[b] (period finished in TMEM buffer b), tempty[b] (buffer b read).
-template <int BN>
-__global__ void __launch_bounds__(GemmShape<BN>::THREADS, 1) tc_gemm_kernel(const __grid_constant__ GemmArgs g) {
-    using S = GemmShape<BN>;
-    constexpr int GN = BN, GSTAGES = S::STAGES, STAGE_BYTES = S::STAGE_BYTES, B_TILE = S::B_TILE;
-    constexpr int EPI_WARPS = S::EPI_WARPS, FLUSH = S::FLUSH;
-    constexpr uint32_t TMEM_COLS = S::TMEM_COLS;
-    dep_wait();
-    dep_trigger();
-    if (g.done != nullptr && *g.done) return;
+// Warp roles of both kernels: warp EPI (one lane) loads the stages with TMA; warp EPI + 1 (one
+// lane) issues the MMAs and commits them; warps 0 .. EPI - 1 drain the TMEM accumulators every
+// FLUSH k-blocks into FP32 registers (warp w reads TMEM lanes 32 (w % 4) .. + 31 and columns
+// 128 (w / 4) .. + 127; TMEM is double-buffered) and write the tile.  Barriers: full[s] (TMA
+// bytes landed), empty[s] (MMAs done reading stage s), tfull[b] (period finished in TMEM buffer
+// b), tempty[b] (buffer b read), mdone (every MMA finished).
+
+// all k-blocks of one tile into the stages; kb0 counts the k-blocks of the CTA's earlier tiles
+__device__ __forceinline__ bool load_tile(const GemmArgs& g, uint8_t* gsm, uint64_t* full, uint64_t* empty, int nk,
+                                          int row_a, int row_b, int64_t kb0, int64_t& issued) {
+    for (int kb = 0; kb < nk; ++kb) {
+        const int64_t q = kb0 + kb;
+        const int s = (int)(q % GSTAGES);
+        if (q >= GSTAGES && !mbar_wait(&empty[s], (uint32_t)((q / GSTAGES) - 1) & 1)) return false;
+        uint8_t* st = gsm + s * STAGE_BYTES;
+        mbar_expect_tx(&full[s], STAGE_BYTES);
+        const int k0 = kb * GK;
+        tma_load_2d(st, &g.ta_hi, k0, row_a, &full[s]);
+        tma_load_2d(st + OP_TILE, &g.ta_lo, k0, row_a, &full[s]);
+        tma_load_2d(st + 2 * OP_TILE, &g.tb_hi, k0, row_b, &full[s]);
+        tma_load_2d(st + 3 * OP_TILE, &g.tb_lo, k0, row_b, &full[s]);
+        issued = q + 1;
+    }
+    return true;
+}
+
+// No copy of a CTA may still be in flight when it exits, after a give-up as well: wait (bounded)
+// for the bytes of the stages it actually started.  Each stage's barrier has begun no phase after
+// the one waited on here, so the parity is unambiguous.
+__device__ __forceinline__ bool drain_loads(uint64_t* full, int64_t issued) {
+    bool ok = true;
+    for (int64_t q = issued > GSTAGES ? issued - GSTAGES : 0; q < issued; ++q)
+        if (!mbar_wait(&full[q % GSTAGES], (uint32_t)(q / GSTAGES) & 1)) ok = false;
+    return ok;
+}
+
+// The Gram: A = B, M = N, only tiles bn >= bm of 128 x 128, written to C[m][n] and C[n][m] where
+// m, n < Mvalid.  One tile a CTA: the upper triangle holds few (136 at 1985 shifts).  Bound by
+// what an SM reads from L2 and shared memory (64 KB a stage for 768 cycles of MMA), so hi*hi and
+// hi*lo are one MMA of 256 columns over the adjacent hi and lo tiles of B: A is read twice per
+// k-step, not three times.  The tile goes through shared memory on its way to the rows of C, so
+// both halves of the matrix are written in lines.  2048 x 2048 over 16384 / 4096 positions: 143 / 45
+// us (75 / 63 % of the tensor pipe; three MMAs of 128 columns and rows written by lane: 170 / 62).
+__global__ void __launch_bounds__(32 * (GRAM_EPI + 2), 1) tc_gemm_kernel(const __grid_constant__ GemmArgs g) {
     extern __shared__ __align__(1024) uint8_t gsm_raw[];
     // the swizzle atoms need 1024-byte aligned tiles
     uint8_t* gsm = gsm_raw + ((1024 - (smem_u32(gsm_raw) & 1023)) & 1023);
@@ -246,26 +324,9 @@ __global__ void __launch_bounds__(GemmShape<BN>::THREADS, 1) tc_gemm_kernel(cons
     uint64_t* empty = full + GSTAGES;
     uint64_t* tfull = empty + GSTAGES;
     uint64_t* tempty = tfull + 2;
-    uint64_t* mdone = tempty + 2;   // every MMA of this CTA finished (the last commit)
+    uint64_t* mdone = tempty + 2;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(mdone + 1);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tilesM = g.M / GM, tilesN = g.N / GN;
-    int bm, bn;
-    if (g.mode == 1) {
-        // the upper triangle in square tiles (the launcher takes BN = GM), row by row: (bm, bn >= bm)
-        int t = (int)blockIdx.x;
-        bm = 0;
-        while (t >= tilesN - bm) {
-            t -= tilesN - bm;
-            ++bm;
-        }
-        bn = bm + t;
-    } else {
-        // B tiles fastest: the CTAs in flight share a few A row blocks and sweep the whole of
-        // B (the W GEMM's G, Kpad x Kpad, stays in L2), so A streams from DRAM once
-        bn = (int)(blockIdx.x % tilesN);
-        bm = (int)(blockIdx.x / tilesN);
-    }
     if (tid == 0) {
         for (int s = 0; s < GSTAGES; ++s) {
             mbar_init(&full[s], 1);
@@ -273,86 +334,71 @@ __global__ void __launch_bounds__(GemmShape<BN>::THREADS, 1) tc_gemm_kernel(cons
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&tfull[b], 1);
-            mbar_init(&tempty[b], EPI_WARPS * 32);
+            mbar_init(&tempty[b], GRAM_EPI * 32);
         }
         mbar_init(mdone, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == EPI_WARPS + 1) tmem_alloc(tslot, TMEM_COLS);
+    if (warp == GRAM_EPI + 1) tmem_alloc<false>(tslot);
+    // the upper triangle row by row: (bm, bn >= bm)
+    const int tiles = g.N / GM;
+    int bm = 0, t = (int)blockIdx.x;
+    while (t >= tiles - bm) {
+        t -= tiles - bm;
+        ++bm;
+    }
+    const int bn = bm + t;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
-    const int nk = g.K / GK;
-    const int nper = (nk + FLUSH - 1) / FLUSH;
+    dep_wait();
+    dep_trigger();
+    const bool skip = g.done != nullptr && *g.done;
+    const int nk = skip ? 0 : g.K / GK;
+    const int nper = (nk + GRAM_FLUSH - 1) / GRAM_FLUSH;
     bool ok = true;
 
-    if (warp == EPI_WARPS) {
-        // ---- TMA producer
+    if (warp == GRAM_EPI) {
         if (lane == 0) {
-            int issued = 0;   // stages whose copies were started
-            for (int kb = 0; kb < nk; ++kb) {
-                const int s = kb % GSTAGES;
-                if (kb >= GSTAGES) ok = mbar_wait(&empty[s], ((kb / GSTAGES) - 1) & 1);
-                if (!ok) break;
-                uint8_t* st = gsm + s * STAGE_BYTES;
-                mbar_expect_tx(&full[s], STAGE_BYTES);
-                const int k0 = kb * GK;
-                tma_load_2d(st, &g.ta_hi, k0, bm * GM, &full[s]);
-                tma_load_2d(st + A_TILE, &g.ta_lo, k0, bm * GM, &full[s]);
-                tma_load_2d(st + 2 * A_TILE, &g.tb_hi, k0, bn * GN, &full[s]);
-                tma_load_2d(st + 2 * A_TILE + B_TILE, &g.tb_lo, k0, bn * GN, &full[s]);
-                issued = kb + 1;
-            }
-            // no copy of this CTA may still be in flight when it exits, after a give-up as
-            // well: wait (bounded) for the bytes of the stages it actually started.  Each
-            // stage's barrier has begun no phase after the one waited on here, so the
-            // parity is unambiguous.
-            for (int kb = issued > GSTAGES ? issued - GSTAGES : 0; kb < issued; ++kb)
-                if (!mbar_wait(&full[kb % GSTAGES], (kb / GSTAGES) & 1)) ok = false;
+            int64_t issued = 0;
+            ok = load_tile(g, gsm, full, empty, nk, bm * GM, bn * GM, 0, issued);
+            if (!drain_loads(full, issued)) ok = false;
         }
         __syncwarp();
-    } else if (warp == EPI_WARPS + 1) {
+    } else if (warp == GRAM_EPI + 1) {
         // ---- MMA issuer
         if (lane == 0) {
             for (int kb = 0; kb < nk; ++kb) {
                 const int s = kb % GSTAGES;
-                const int p = kb / FLUSH, buf = p & 1;
+                const int p = kb / GRAM_FLUSH, buf = p & 1;
                 // TMEM buffer buf was last used by period p - 2: wait until it was read
-                if (kb % FLUSH == 0 && p >= 2) ok = mbar_wait(&tempty[buf], ((p / 2) - 1) & 1);
+                if (kb % GRAM_FLUSH == 0 && p >= 2) ok = mbar_wait(&tempty[buf], ((p / 2) - 1) & 1);
                 if (ok) ok = mbar_wait(&full[s], (kb / GSTAGES) & 1);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t st = smem_u32(gsm + s * STAGE_BYTES);
-                const uint32_t t_acc = tmem + (uint32_t)buf * S::BUF_COLS;
-                const uint32_t t_cross = S::SPLIT ? t_acc + GN : t_acc;
+                const uint32_t t_acc = tmem + (uint32_t)buf * BUF_COLS;
 #pragma unroll
                 for (int ks = 0; ks < GK / 16; ++ks) {
                     const uint32_t off = ks * 32;   // 16 FP16 = 32 bytes per k-step
-                    const uint64_t ah = smem_desc_sw128(st + off);
-                    const uint64_t al = smem_desc_sw128(st + A_TILE + off);
-                    const uint64_t bh = smem_desc_sw128(st + 2 * A_TILE + off);
-                    const uint64_t bl = smem_desc_sw128(st + 2 * A_TILE + B_TILE + off);
-                    const uint32_t more = (kb % FLUSH != 0) || ks != 0;
-                    mma_f16(t_acc, ah, bh, S::IDESC, more);
-                    mma_f16(t_cross, ah, bl, S::IDESC, S::SPLIT ? more : 1u);
-                    mma_f16(t_cross, al, bh, S::IDESC, 1);
+                    const uint64_t ah = smem_desc_sw128(st + off), al = smem_desc_sw128(st + OP_TILE + off);
+                    const uint64_t b = smem_desc_sw128(st + 2 * OP_TILE + off);   // hi, then lo: 256 rows
+                    mma_f16<false>(t_acc, ah, b, idesc_f16(GM, 256), (kb % GRAM_FLUSH != 0) || ks != 0);
+                    mma_f16<false>(t_acc + GM, al, b, idesc_f16(GM, GM), 1);
                 }
-                mma_commit(&empty[s]);
-                if (kb % FLUSH == FLUSH - 1 || kb == nk - 1) mma_commit(&tfull[buf]);
+                mma_commit<false>(&empty[s]);
+                if (kb % GRAM_FLUSH == GRAM_FLUSH - 1 || kb == nk - 1) mma_commit<false>(&tfull[buf]);
             }
             // TMEM is freed below: first every MMA issued above (all of them, also after a
             // give-up of this thread or of another role) must have finished writing it.  A
             // commit tracks every earlier tcgen05 operation of this thread.
-            mma_commit(mdone);
+            mma_commit<false>(mdone);
             if (!mbar_wait(mdone, 0)) ok = false;
         }
         __syncwarp();
     } else {
-        // ---- epilogue: warp w owns TMEM lanes 32 (w % 4) .. + 31 (tile rows) and the 128
-        // columns from 128 (w / 4)
-        constexpr int EC = 128;
-        const int quad = warp & 3, half = warp >> 2;
+        // ---- epilogue
         float acc[EC];
 #pragma unroll
         for (int c = 0; c < EC; ++c) acc[c] = 0.f;
@@ -362,40 +408,41 @@ __global__ void __launch_bounds__(GemmShape<BN>::THREADS, 1) tc_gemm_kernel(cons
             ok = __all_sync(0xffffffffu, mbar_wait(&tfull[buf], (p / 2) & 1));
             if (!ok) break;
             tc_fence_after();
-            const uint32_t t_acc =
-                tmem + (uint32_t)buf * S::BUF_COLS + (uint32_t)(EC * half) + ((uint32_t)(32 * quad) << 16);
+            const uint32_t t_acc = tmem + (uint32_t)buf * BUF_COLS + ((uint32_t)(32 * warp) << 16);
 #pragma unroll
             for (int c = 0; c < EC; c += 16) {
-                float v[16];
+                float v[16], w[16];
                 tmem_ld16(t_acc + (uint32_t)c, v);
-                if (S::SPLIT) {
-                    float w[16];
-                    tmem_ld16(t_acc + GN + (uint32_t)c, w);
+                tmem_ld16(t_acc + GM + (uint32_t)c, w);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) acc[c + j] += v[j] + w[j];
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) acc[c + j] += v[j];
-                }
+                for (int j = 0; j < 16; ++j) acc[c + j] += v[j] + w[j];
             }
             tc_fence_before();
             mbar_arrive(&tempty[buf]);
         }
-        const int m = bm * GM + 32 * quad + lane;
-        // undo the operands' power-of-two scales together with the output scale (exact)
-        const float scale = ldexpf(g.scale, scale_exp(g.amaxA) + scale_exp(g.amaxB));
-        if (ok && m < g.Mvalid) {
+        if (!skip) {
+            const int r = 32 * warp + lane, m = bm * GM + r;
+            // undo the operands' power-of-two scales together with the output scale (exact)
+            const float scale = ldexpf(g.scale, scale_exp(g.amaxA) + scale_exp(g.amaxB));
+            // the last period's barrier: every stage has been read, its memory is free (given up
+            // on: this warp's part of it is not used)
+            float* tile = reinterpret_cast<float*>(gsm);
+            if (ok) {
 #pragma unroll
-            for (int c = 0; c < EC; ++c) {
-                const int n = bn * GN + EC * half + c;
-                if (n >= g.Nvalid) continue;
-                const float x = scale * acc[c];
-                if (g.mode == 2) {
-                    g.C[(int64_t)n * g.ldc + m] = x;
-                } else {
-                    // Gram: a diagonal tile holds both halves; the others are mirrored
-                    g.C[(int64_t)m * g.ldc + n] = x;
-                    if (bm != bn) g.C[(int64_t)n * g.ldc + m] = x;
+                for (int c = 0; c < EC; ++c) {
+                    const int n = bn * GM + c;
+                    const float x = scale * acc[c];
+                    tile[r * (GM + 1) + c] = x;
+                    if (bm != bn && m < g.Mvalid && n < g.Nvalid) g.C[(int64_t)n * g.ldc + m] = x;
+                }
+                __syncwarp();
+                for (int q = 0; q < 32; ++q) {
+                    const int mr = 32 * warp + q;
+                    if (bm * GM + mr >= g.Mvalid) break;
+                    float* C = g.C + (int64_t)(bm * GM + mr) * g.ldc + bn * GM;
+#pragma unroll
+                    for (int c = lane; c < GM; c += 32)
+                        if (bn * GM + c < g.Nvalid) C[c] = tile[mr * (GM + 1) + c];
                 }
             }
         }
@@ -405,7 +452,170 @@ __global__ void __launch_bounds__(GemmShape<BN>::THREADS, 1) tc_gemm_kernel(cons
     // wait for it ran out), and the epilogue warps after their last TMEM read
     tc_fence_before();
     __syncthreads();
-    if (warp == EPI_WARPS + 1) tmem_dealloc(tmem, TMEM_COLS);
+    if (warp == GRAM_EPI + 1) tmem_dealloc<false>(tmem);
+}
+
+// C[n][m] = scale A B^T where m < Mvalid and n < Nvalid; N a multiple of 256.  A pair of CTAs
+// (one cluster, two SMs) owns a 256 x 256 tile: each holds 128 rows of A, half of B's rows and
+// the accumulators of its 128 rows, and the first CTA's MMAs (cta_group::2) work on both.  Per
+// SM a stage of 64 KB feeds 1536 cycles of MMA (one CTA alone on 128 x 256 needs 96 KB for them,
+// what L2 can deliver to an SM at best).  The kernel is persistent: the pairs walk the tiles (B
+// tiles fastest: the pairs in flight share a few row blocks of A and sweep the whole of B, which
+// stays in L2), and while the epilogue warps write a tile the next one's stages and first
+// periods are under way.  16384 / 4096 x 2048 over 2048: 231 / 72 us (80 / 74 % of the tensor
+// pipe; one CTA on a 128 x 256 tile, one tile a CTA: 306 / 100).
+// The copies signal each CTA's own barriers; the second CTA's MMA warp passes its full[s] on to
+// the first CTA's pfull[s].  Commits arrive in both CTAs; tempty[b] of the first CTA counts the
+// epilogue warps of both.
+__global__ void __launch_bounds__(32 * (PAIR_EPI + 2), 1) tc_gemm_pair_kernel(const __grid_constant__ GemmArgs g) {
+    extern __shared__ __align__(1024) uint8_t gsm_raw[];
+    uint8_t* gsm = gsm_raw + ((1024 - (smem_u32(gsm_raw) & 1023)) & 1023);
+    uint64_t* full = reinterpret_cast<uint64_t*>(gsm + GSTAGES * STAGE_BYTES);
+    uint64_t* empty = full + GSTAGES;
+    uint64_t* pfull = empty + GSTAGES;
+    uint64_t* tfull = pfull + GSTAGES;
+    uint64_t* tempty = tfull + 2;
+    uint64_t* mdone = tempty + 2;
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(mdone + 1);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = (int)cluster_rank();
+    if (tid == 0) {
+        for (int s = 0; s < GSTAGES; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+            mbar_init(&pfull[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&tfull[b], 1);
+            mbar_init(&tempty[b], 2 * PAIR_EPI);
+        }
+        mbar_init(mdone, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == PAIR_EPI + 1) tmem_alloc<true>(tslot);
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();
+    tc_fence_after();
+    const uint32_t tmem = *tslot;
+    dep_wait();
+    dep_trigger();
+    const bool skip = g.done != nullptr && *g.done;
+    const int nk = g.K / GK;
+    const int nper = (nk + PAIR_FLUSH - 1) / PAIR_FLUSH;
+    const int tilesN = g.N / 256;
+    const int tiles = skip ? 0 : (g.M + 255) / 256 * tilesN;
+    const int first = (int)(blockIdx.x / 2), pairs = (int)(gridDim.x / 2);
+    bool ok = true;
+
+    if (warp == PAIR_EPI) {
+        // ---- TMA producer
+        if (lane == 0) {
+            int64_t issued = 0, kb0 = 0;
+            for (int t = first; ok && t < tiles; t += pairs, kb0 += nk)
+                ok = load_tile(g, gsm, full, empty, nk, t / tilesN * 256 + rank * GM, t % tilesN * 256 + rank * GM, kb0,
+                               issued);
+            if (!drain_loads(full, issued)) ok = false;
+            // the commits that arrive here from the first CTA have to land before the exit, too
+            for (int64_t q = issued > GSTAGES ? issued - GSTAGES : 0; q < issued; ++q)
+                if (!mbar_wait(&empty[q % GSTAGES], (uint32_t)(q / GSTAGES) & 1)) ok = false;
+        }
+        __syncwarp();
+    } else if (warp == PAIR_EPI + 1) {
+        if (lane == 0 && rank == 0) {
+            // ---- MMA issuer
+            int64_t q = 0, p = 0;      // k-blocks and periods so far
+            for (int t = first; ok && t < tiles; t += pairs) {
+                for (int kb = 0; kb < nk; ++kb, ++q) {
+                    const int s = (int)(q % GSTAGES), buf = (int)(p & 1);
+                    const uint32_t par = (uint32_t)(q / GSTAGES) & 1;
+                    // TMEM buffer buf was last used by period p - 2: wait until both CTAs read it
+                    if (kb % PAIR_FLUSH == 0 && p >= 2) ok = mbar_wait<true>(&tempty[buf], (uint32_t)((p / 2) - 1) & 1);
+                    if (ok) ok = mbar_wait(&full[s], par);
+                    if (ok) ok = mbar_wait<true>(&pfull[s], par);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t st = smem_u32(gsm + s * STAGE_BYTES);
+                    const uint32_t t_acc = tmem + (uint32_t)buf * BUF_COLS;
+#pragma unroll
+                    for (int ks = 0; ks < GK / 16; ++ks) {
+                        const uint32_t off = ks * 32;   // 16 FP16 = 32 bytes per k-step
+                        const uint64_t ah = smem_desc_sw128(st + off), al = smem_desc_sw128(st + OP_TILE + off);
+                        const uint64_t bh = smem_desc_sw128(st + 2 * OP_TILE + off);
+                        const uint64_t bl = smem_desc_sw128(st + 3 * OP_TILE + off);
+                        mma_f16<true>(t_acc, ah, bh, idesc_f16(256, 256), (kb % PAIR_FLUSH != 0) || ks != 0);
+                        mma_f16<true>(t_acc, ah, bl, idesc_f16(256, 256), 1);
+                        mma_f16<true>(t_acc, al, bh, idesc_f16(256, 256), 1);
+                    }
+                    mma_commit<true>(&empty[s]);
+                    if (kb % PAIR_FLUSH == PAIR_FLUSH - 1 || kb == nk - 1) {
+                        mma_commit<true>(&tfull[buf]);
+                        ++p;
+                    }
+                }
+            }
+            // as in the Gram: every MMA issued above must have finished before the exit
+            mma_commit<true>(mdone);
+            if (!mbar_wait(mdone, 0)) ok = false;
+        } else if (lane == 0) {
+            // ---- the second CTA's stages are announced to the first
+            int64_t q = 0;
+            for (int t = first; ok && t < tiles; t += pairs)
+                for (int kb = 0; kb < nk; ++kb, ++q) {
+                    const int s = (int)(q % GSTAGES);
+                    ok = mbar_wait(&full[s], (uint32_t)(q / GSTAGES) & 1);
+                    if (!ok) break;
+                    mbar_arrive_first(&pfull[s]);
+                }
+            if (!mbar_wait(mdone, 0)) ok = false;
+        }
+        __syncwarp();
+    } else {
+        // ---- epilogue
+        const int quad = warp & 3, half = warp >> 2;
+        // undo the operands' power-of-two scales together with the output scale (exact)
+        const float scale = ldexpf(g.scale, scale_exp(g.amaxA) + scale_exp(g.amaxB));
+        int64_t p = 0;
+        for (int t = first; ok && t < tiles; t += pairs) {
+            float acc[EC];
+#pragma unroll
+            for (int c = 0; c < EC; ++c) acc[c] = 0.f;
+            for (int i = 0; i < nper; ++i, ++p) {
+                const int buf = (int)(p & 1);
+                ok = __all_sync(0xffffffffu, mbar_wait(&tfull[buf], (uint32_t)(p / 2) & 1));
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t t_acc =
+                    tmem + (uint32_t)buf * BUF_COLS + (uint32_t)(EC * half) + ((uint32_t)(32 * quad) << 16);
+#pragma unroll
+                for (int c = 0; c < EC; c += 16) {
+                    float v[16];
+                    tmem_ld16(t_acc + (uint32_t)c, v);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) acc[c + j] += v[j];
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_first(&tempty[buf]);
+            }
+            const int m = t / tilesN * 256 + rank * GM + 32 * quad + lane;
+            const int n0 = t % tilesN * 256 + EC * half;
+            if (ok && m < g.Mvalid) {
+                float* C = g.C + (int64_t)n0 * g.ldc + m;
+#pragma unroll
+                for (int c = 0; c < EC; ++c, C += g.ldc)
+                    if (n0 + c < g.Nvalid) *C = scale * acc[c];
+            }
+        }
+    }
+    if (!ok && g.err != nullptr) atomicExch(g.err, 1);
+    // neither CTA frees its TMEM, or exits, before both are through
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();
+    tc_fence_after();
+    if (warp == PAIR_EPI + 1) tmem_dealloc<true>(tmem);
+    cluster_sync();
 }
 
 // ------------------------------------------------------------------------- ensemble
@@ -767,11 +977,9 @@ __global__ void __launch_bounds__(256, 5) s3_gather_kernel(const __grid_constant
 
 // ------------------------------------------------------------------------- launchers
 
-size_t gemm_smem_bytes() { return std::max(GemmShape<128>::SMEM, GemmShape<256>::SMEM); }
-
 void set_gram_attributes() {
-    cudaFuncSetAttribute(tc_gemm_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GemmShape<128>::SMEM);
-    cudaFuncSetAttribute(tc_gemm_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GemmShape<256>::SMEM);
+    cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GEMM_SMEM);
+    cudaFuncSetAttribute(tc_gemm_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GEMM_SMEM);
 }
 
 __global__ void set_flag_kernel(int* flag, int v) {
@@ -810,16 +1018,33 @@ bool make_map(CUtensorMap* m, const uint16_t* base, int64_t rows, int64_t cols, 
 
 bool gram_ready() { return tensor_map_encoder() != nullptr; }
 
-// BN = 128 for the Gram (mode 1), 256 otherwise
+// Pairs of CTAs that are resident at once (one CTA an SM; an SM without a partner stays out): the
+// persistent kernel's grid, since a pair that had to wait would run its tiles after all others.
+int resident_pairs(cudaLaunchConfig_t cfg) {
+    static std::mutex mu;
+    static int known[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
+    std::lock_guard<std::mutex> lk(mu);
+    if (known[dev] == 0) {
+        int n = 0;
+        cfg.gridDim = dim3(2);
+        if (cudaOccupancyMaxActiveClusters(&n, tc_gemm_pair_kernel, &cfg) != cudaSuccess || n < 1) {
+            cudaGetLastError();
+            n = 32;
+        }
+        known[dev] = n;
+    }
+    return known[dev];
+}
+
+// mode 1: the Gram (A = B, M = N multiples of 128); mode 2: C[n][m] on pairs of SMs
 void launch_tc_gemm(const GemmOperands& o, cudaStream_t s) {
-    const int BN = o.mode == 1 ? 128 : 256;
-    const int64_t tm = o.M / GM, tn = o.N / BN;
-    int64_t blocks = tm * tn;
-    if (o.mode == 1) blocks = tm * (tm + 1) / 2;   // square tiles: BN = 128, M = N
-    if (blocks <= 0) return;
+    const int64_t tm = o.M / GM;
+    if (tm <= 0 || o.N <= 0) return;
     GemmArgs a{};
     const bool ok = make_map(&a.ta_hi, o.Ah, o.M, o.K, o.lda, GM) && make_map(&a.ta_lo, o.Al, o.M, o.K, o.lda, GM) &&
-                    make_map(&a.tb_hi, o.Bh, o.N, o.K, o.ldb, BN) && make_map(&a.tb_lo, o.Bl, o.N, o.K, o.ldb, BN);
+                    make_map(&a.tb_hi, o.Bh, o.N, o.K, o.ldb, GM) && make_map(&a.tb_lo, o.Bl, o.N, o.K, o.ldb, GM);
     if (!ok) {
         // no valid tensor map: never launch TMA on it; report through the error word
         launch_dep(set_flag_kernel, 1, 1, 0, s, o.err, 2);
@@ -831,14 +1056,30 @@ void launch_tc_gemm(const GemmOperands& o, cudaStream_t s) {
     a.amaxB = o.amaxB;
     a.C = o.C;
     a.ldc = o.ldc;
-    a.mode = o.mode;
     a.Mvalid = o.Mvalid; a.Nvalid = o.Nvalid;
     a.done = o.done;
     a.err = o.err;
-    if (BN == 128)
-        launch_dep(tc_gemm_kernel<128>, (unsigned)blocks, GemmShape<128>::THREADS, GemmShape<128>::SMEM, s, a);
-    else
-        launch_dep(tc_gemm_kernel<256>, (unsigned)blocks, GemmShape<256>::THREADS, GemmShape<256>::SMEM, s, a);
+    if (o.mode == 1) {
+        launch_dep(tc_gemm_kernel, (unsigned)(tm * (tm + 1) / 2), 32 * (GRAM_EPI + 2), GEMM_SMEM, s, a);
+        return;
+    }
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.blockDim = dim3(32 * (PAIR_EPI + 2));
+    cfg.dynamicSmemBytes = GEMM_SMEM;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const int64_t tiles = (tm + 1) / 2 * (o.N / 256);
+    const int64_t pairs = std::min<int64_t>(tiles, resident_pairs(cfg));
+    cfg.gridDim = dim3((unsigned)(2 * pairs));
+    cfg.numAttrs = 2;
+    cudaLaunchKernelEx(&cfg, tc_gemm_pair_kernel, a);
 }
 
 constexpr int ABSMAX_BLOCKS = 512;
