@@ -212,7 +212,7 @@ __device__ __forceinline__ double block_sum_d(double v, double* sh) {
 // sum D_des^2 over the descriptor, and sum ex^2 of the box excess over the field (when the
 // penalty is on); its last block sums the partials in a fixed order and finishes the loss
 // (a launch of its own: 9 us more).
-__global__ void __launch_bounds__(256) stats_kernel(const PenSeg* __restrict__ segs) {
+__global__ void __launch_bounds__(256, 5) stats_kernel(const PenSeg* __restrict__ segs) {
     dep_wait();
     dep_trigger();
     const PenSeg& sg = segs[blockIdx.y];
@@ -225,15 +225,16 @@ __global__ void __launch_bounds__(256) stats_kernel(const PenSeg* __restrict__ s
     // this part and a thread sums only about 8 terms (stats_blocks) -- then a double-float
     // (two-sum) tree across the block
     float r2 = 0.f, r2c = 0.f, t2 = 0.f, t2c = 0.f, e2 = 0.f, e2c = 0.f;
-    // the terms of this thread in order; their loads issued eight at a time (the same sums)
-    int64_t k = i0;
+    // the terms of this thread in order, their loads issued eight at a time, the last ones too
+    // (terms past the end are zeros: one by one they took as long as all the others)
     constexpr int U = 8;
-    for (; k + (U - 1) * stride < sg.K; k += U * stride) {
+    for (int64_t k = i0; k < sg.K; k += U * stride) {
         float tv[U], dv[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            tv[u] = sg.target[k + u * stride];
-            dv[u] = sg.desc[k + u * stride];
+            const bool in = k + u * stride < sg.K;
+            tv[u] = in ? sg.target[k + u * stride] : 0.f;
+            dv[u] = in ? sg.desc[k + u * stride] : 0.f;
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -242,27 +243,16 @@ __global__ void __launch_bounds__(256) stats_kernel(const PenSeg* __restrict__ s
             kahan_add(t2, t2c, tv[u] * tv[u]);
         }
     }
-    for (; k < sg.K; k += stride) {
-        const float t = sg.target[k];
-        const float r = sg.desc[k] - t;
-        kahan_add(r2, r2c, r * r);
-        kahan_add(t2, t2c, t * t);
-    }
     if (sg.field != nullptr) {
-        int64_t i = i0;
-        for (; i + 3 * stride < sg.N; i += 4 * stride) {
-            float fv[4];
+        for (int64_t i = i0; i < sg.N; i += U * stride) {
+            float fv[U];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) fv[u] = sg.field[i + u * stride];
+            for (int u = 0; u < U; ++u) fv[u] = i + u * stride < sg.N ? sg.field[i + u * stride] : 0.f;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < U; ++u) {
                 const float e = box_excess(fv[u]);
                 kahan_add(e2, e2c, e * e);
             }
-        }
-        for (; i < sg.N; i += stride) {
-            const float e = box_excess(sg.field[i]);
-            kahan_add(e2, e2c, e * e);
         }
     }
     // Kahan's (sum, comp) stands for sum - comp
@@ -335,13 +325,27 @@ void launch_tilde_sum(const TildeSeg* segs, int nseg, cudaStream_t s) {
 // their loads issued eight at a time.
 template <int SUB>
 __device__ __forceinline__ float chunk_sums(const FinalArgs& a, int64_t i, int q) {
-    const int64_t x = i % a.n1[2], y = (i / a.n1[2]) % a.n1[1], z = i / (a.n1[1] * a.n1[2]);
+    // coordinates only where a coarser level needs them, in 32 bits where they fit (the 64-bit
+    // divisions: 22 us for 128^3, one level, 9 so)
+    int64_t x = i, y = 0, z = 0;
+    if (a.levels > 1) {
+        if (a.n1[0] * a.n1[1] * a.n1[2] <= 0x7fffffff) {
+            const unsigned n2 = (unsigned)a.n1[2], n1 = (unsigned)a.n1[1], row = (unsigned)i / n2;
+            x = (unsigned)i - row * n2;
+            z = row / n1;
+            y = row - (unsigned)z * n1;
+        } else {
+            x = i % a.n1[2];
+            y = (i / a.n1[2]) % a.n1[1];
+            z = i / (a.n1[1] * a.n1[2]);
+        }
+    }
     float g = 0.f, scale = 1.f;
     const float step = a.ndim == 2 ? 0.25f : 0.125f;
     const bool sep = a.tier != nullptr && *a.tier < SEP_TIERS;
     for (int l = 0; l < a.levels; ++l) {
         const int64_t lz = a.ndim == 2 ? 0 : (z >> l);
-        const int64_t li = (lz * a.nl[l][1] + (y >> l)) * a.nl[l][2] + (x >> l);
+        const int64_t li = l == 0 ? i : (lz * a.nl[l][1] + (y >> l)) * a.nl[l][2] + (x >> l);
         const int64_t jump = SUB * a.Nl[l];
         const float* p = (sep ? a.sparts[l] : a.parts[l]) + li + q * a.Nl[l];
         const int nc = sep ? 1 : a.nChunks[l];
@@ -366,49 +370,58 @@ __device__ __forceinline__ float chunk_sums(const FinalArgs& a, int64_t i, int q
 // (a small field: few positions for many chunk partials): thread (q, p) -- q = threadIdx.x /
 // positions, so a warp still reads consecutive positions of one chunk -- sums the chunks
 // c = q (mod FIN_SUB) and the FIN_SUB partials are added in a fixed order through shared
-// memory.  Two instantiations, so that SUB = 1 keeps the 32 registers with which 8 blocks
-// stay resident per SM (a 512^2 field is one wave).
+// memory.
+// The segment's arguments (written at least two launches earlier) and the field and moments at
+// the thread's position are read before the adjoint kernels' end is waited for.
 template <int SUB>
 __global__ void __launch_bounds__(ELEM_TH) final_kernel(const FinalSeg* __restrict__ segs, int nseg) {
-    dep_wait();
-    dep_trigger();
-    const int si = find_segment(segs, nseg, (int64_t)blockIdx.x);
-    const FinalSeg& sg = segs[si];
-    if (sg.done != nullptr && *sg.done) return;
+    constexpr int NPOS = ELEM_TH / SUB;
+    __shared__ FinalSeg sg;
+    static_assert(sizeof(FinalSeg) % 4 == 0 && sizeof(FinalSeg) / 4 <= ELEM_TH, "one word a thread");
+    const FinalSeg* src = segs + find_segment(segs, nseg, (int64_t)blockIdx.x);
+    if (threadIdx.x < sizeof(FinalSeg) / 4)
+        reinterpret_cast<uint32_t*>(&sg)[threadIdx.x] = reinterpret_cast<const uint32_t*>(src)[threadIdx.x];
+    __syncthreads();
     const FinalArgs& a = sg.a;
     const int64_t N1 = a.n1[0] * a.n1[1] * a.n1[2];
-    const int64_t b = (int64_t)blockIdx.x - sg.blockStart;
-    int64_t i;
-    float g;
-    if constexpr (SUB == 1) {
-        i = b * ELEM_TH + threadIdx.x;
-        if (i >= N1) return;
-        g = chunk_sums<1>(a, i, 0);
-    } else {
-        static_assert(SUB == 4, "the combine below adds four partials");
-        constexpr int NPOS = ELEM_TH / SUB;
-        __shared__ float part[SUB][NPOS];
-        const int q = threadIdx.x / NPOS, pl = threadIdx.x % NPOS;
-        i = b * NPOS + pl;
-        const bool valid = i < N1;
-        part[q][pl] = valid ? chunk_sums<SUB>(a, i, q) : 0.f;
-        __syncthreads();
-        if (q != 0 || !valid) return;
-        g = (part[0][pl] + part[1][pl]) + (part[2][pl] + part[3][pl]);
+    const int q = threadIdx.x / NPOS, pl = threadIdx.x % NPOS;
+    const int64_t i = ((int64_t)blockIdx.x - sg.blockStart) * NPOS + pl;
+    const bool valid = i < N1;
+    float M = 0.f, m0 = 0.f, v0 = 0.f;
+    if (valid && q == 0) {
+        if (a.M != nullptr) {
+            M = a.M[i];
+            m0 = a.m[i];
+            v0 = a.v[i];
+        } else if (a.sc != nullptr && a.field != nullptr) {
+            M = a.field[i];
+        }
     }
+    dep_wait();
+    dep_trigger();
+    if (sg.done != nullptr && *sg.done) return;
+    float g = valid ? chunk_sums<SUB>(a, i, q) : 0.f;
+    if constexpr (SUB > 1) {
+        __shared__ float part[SUB][NPOS];
+        part[q][pl] = g;
+        __syncthreads();
+        if (q != 0) return;
+        for (int u = 1; u < SUB; ++u) g += part[u][pl];
+    }
+    if (!valid) return;
     if (a.sc != nullptr && a.field != nullptr) {
-        const float M = a.field[i];
-        const float ex = box_excess(M);
-        const float dex = M > 1.f ? 1.f : (M < 0.f ? -1.f : 0.f);
+        const float f = a.M != nullptr && a.M != a.field ? a.field[i] : M;
+        const float ex = box_excess(f);
+        const float dex = f > 1.f ? 1.f : (f < 0.f ? -1.f : 0.f);
         g = fmaf(a.sc->pen_coef * ex, dex, g);
     }
     if (a.grad_out != nullptr) a.grad_out[i] = g;
     if (a.M != nullptr) {
-        const float m = fmaf(a.beta1, a.m[i], (1.f - a.beta1) * g);
-        const float v = fmaf(a.beta2, a.v[i], (1.f - a.beta2) * g * g);
+        const float m = fmaf(a.beta1, m0, (1.f - a.beta1) * g);
+        const float v = fmaf(a.beta2, v0, (1.f - a.beta2) * g * g);
         a.m[i] = m;
         a.v[i] = v;
-        a.M[i] = a.M[i] - a.sc->lr_t * m / (sqrtf(v) + a.eps);
+        a.M[i] = M - a.sc->lr_t * m / (sqrtf(v) + a.eps);
     }
 }
 

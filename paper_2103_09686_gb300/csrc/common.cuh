@@ -489,8 +489,8 @@ float gcoef_scale(const LevelGeom& g, const ThreshConst& tc, float weight);
 constexpr int RED_K = 32;      // shifts per fwd_reduce block
 constexpr int GCOEF_TH = 256;  // entries per gcoef block
 constexpr int ELEM_TH = 256;   // pixels per restrict block; threads per final block
-constexpr int FIN_SUB = 4;     // gradient assembly of a small field: threads per position (each sums
-                               // every 4th chunk; the combine adds exactly four partials)
+constexpr int FIN_SUB = 8;     // gradient assembly of a small field: threads per position (each sums
+                               // every 8th chunk)
 constexpr int64_t FIN_SUB_BELOW = 1 << 16;   // fields of fewer positions use FIN_SUB threads each
 
 // Segment of linear block b: the last segment whose blockStart <= b.
