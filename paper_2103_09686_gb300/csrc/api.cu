@@ -162,6 +162,7 @@ struct Plan {
     size_t o_excess = 0, o_sums = 0;
     int red_off[MAX_LEVELS] = {}, nred = 0;   // fwd_reduce blocks: first of a level, all
     int sep_off[MAX_LEVELS] = {}, nsep = 0;   // sep_desc blocks
+    int sep_parts[MAX_LEVELS] = {};           // shares of the pairs in sep_power
     int nexc = 0;                             // field blocks of fwd_reduce (direct path)
     size_t bytes = 0;
 };
@@ -355,6 +356,40 @@ bool sep_shape(const LevelGeom& g, int phases, int max_pairs, SepLevel& lv) {
     lv.colsL = lv.n0 > 1 ? sep_cols(lv.ax[0], true, phases) : sep_cols(lv.ax[1], false, phases);
     return std::max(sep_smem_last(lv, true), sep_smem_feat(lv)) <= (size_t)SEP_MAX_SMEM;
 }
+
+// sep_power and sep_mul where the groups of columns are few (2-D, a small problem): their blocks
+// walk the feature pairs, a long level's several times as often as a short level's, on a part of
+// the chip.  The range of blocks that takes the most rounds (`width` pairs each) gets another block
+// for every group, at the price of a transform more, while all still fit two to an SM and more
+// than two rounds are left.  512^2, three levels, 11 pairs: sep_mul 160 blocks of up to 11 rounds
+// -> 288 of up to 4, sep_power (at most two shares: sep_desc adds them) 224 of up to 6.
+struct PairShare {
+    int64_t blocks;
+    int width, parts;
+};
+void share_pairs(std::vector<PairShare>& v, int pairs, int most_parts) {
+    int64_t total = 0;
+    for (const PairShare& s : v) total += s.blocks;
+    for (;;) {
+        PairShare* most = nullptr;
+        int64_t rounds = 2;
+        for (PairShare& s : v) {
+            const int64_t r = ceil_div(pairs, (int64_t)s.parts * s.width);
+            if (r > rounds) rounds = r, most = &s;
+        }
+        if (most == nullptr || most->parts == most_parts || total + most->blocks > 2 * SMS) return;
+        ++most->parts;
+        total += most->blocks;
+    }
+}
+// column groups of the last axis, and the pairs in flight in one block
+PairShare last_groups(const SepLevel& lv) {
+    const bool d3 = lv.n0 > 1;
+    const SepAxis& ax = lv.ax[d3 ? 0 : 1];
+    return {ceil_div(lv.n2, lv.colsL) * (d3 ? lv.n1 : 1), ax.fast ? SEP_BLOCK_PTS / (lv.colsL * ax.n) : 1, 1};
+}
+// the pairs of a field a little beyond [0, 1]
+int usual_pairs(const SepBasis& b) { return std::max(b.tier[0].npair, b.tier[1].npair); }
 
 // The separable path for the soft threshold's two-point descriptor: when a basis of this
 // alpha exists, every axis of every level can be transformed, its buffers stay moderate and
@@ -568,6 +603,15 @@ dmcr_status make_plan(const dmcr_params* p, Plan& pl) {
     if (pl.sep) {
         pl.o_tier = o; o = align_up(o + sizeof(int));
         pl.o_tiers = o; o = align_up(o + PREP_BLOCKS * sizeof(int));
+        std::vector<PairShare> power;
+        for (int l = 0; l < pl.levels; ++l) {
+            SepLevel lv;
+            sep_shape(pl.g[l], pl.phases, pl.sep_pairs, lv);
+            power.push_back(last_groups(lv));
+        }
+        // 3-D planes and phase pairs are many as they are
+        if (pl.phases == 1 && pl.ndim == 2) share_pairs(power, usual_pairs(*pl.basis), 2);
+        for (int l = 0; l < pl.levels; ++l) pl.sep_parts[l] = power[l].parts;
     }
     pl.sums = pl.desc_kind == DMCR_DESC_S2 && !pl.any_fft;
     if (pl.sums) {
@@ -616,13 +660,13 @@ dmcr_status make_plan(const dmcr_params* p, Plan& pl) {
             // spectra (separable) or partials (direct, for fields outside the separable ranges) -- a call uses one of the two
             const size_t pp = ph * ph;
             pl.o_spart[l] = o; o = align_up(o + ph * g.N * sizeof(float));
-            pl.o_sdc[l] = o; o = align_up(o + pp * sizeof(float2));
+            pl.o_sdc[l] = o; o = align_up(o + pp * pl.sep_parts[l] * sizeof(float2));
             const size_t start = o;
             pl.o_z[l] = o; o = align_up(o + ph * pl.sep_pairs * g.N * sizeof(float2));
             pl.o_q[l] = pl.o_z[l];
             if (ph > 1) { pl.o_q[l] = o; o = align_up(o + ph * pl.sep_pairs * g.N * sizeof(float2)); }
             pl.o_u[l] = o; o = align_up(o + pp * sep_u_len(g) * sizeof(float2));
-            pl.o_v[l] = o; o = align_up(o + pp * sep_v_rows(g) * g.n[2] * sizeof(float2));
+            pl.o_v[l] = o; o = align_up(o + pp * pl.sep_parts[l] * sep_v_rows(g) * g.n[2] * sizeof(float2));
             size_t d = start;
             pl.o_fwd[l] = d; d = align_up(d + ph * ph * g.fwdTiles * g.Khalf * sizeof(float));
             pl.o_adj[l] = d; d = align_up(d + ph * ph * g.nChunks * g.N * sizeof(float));
@@ -859,17 +903,19 @@ void prepare_sep(const std::vector<Inst>& in, unsigned flags, const std::vector<
     std::vector<SepLevel> levels;
     std::vector<SepItem> items[SEP_KERNELS];
     const SepBasis* basis = nullptr;
+    std::vector<PairShare> mul;
     const bool vjp = !(flags & F_LOSS);
     const int *lv_tier = nullptr, *lv_done = nullptr;
-    auto add = [&](SepKernel k, int a, int b, int64_t blocks, size_t smem) {
+    auto add = [&](SepKernel k, int a, int b, int64_t blocks, size_t smem, int parts = 1) {
         SepItem it{};
         it.level = (int)levels.size();
         it.a = a;
         it.b = b;
+        it.parts = parts;
         it.blockStart = P.sep[k].blocks;
         it.tier = lv_tier;
         it.done = lv_done;
-        P.sep[k].blocks += blocks;
+        P.sep[k].blocks += blocks * parts;
         P.sep_smem[k] = std::max(P.sep_smem[k], smem);
         items[k].push_back(it);
     };
@@ -883,6 +929,7 @@ void prepare_sep(const std::vector<Inst>& in, unsigned flags, const std::vector<
             SepLevel lv;
             sep_shape(g, pl.phases, pl.sep_pairs, lv);
             lv.ntier = pl.sep_tiers;
+            lv.parts = pl.sep_parts[l];
             lv.field = x.lv[l];
             lv.Z = reinterpret_cast<float2*>(x.ws + pl.o_z[l]);
             lv.Q = reinterpret_cast<float2*>(x.ws + pl.o_q[l]);
@@ -928,13 +975,14 @@ void prepare_sep(const std::vector<Inst>& in, unsigned flags, const std::vector<
                 if (d3) add(SEP_FFT_Y, a, 0, ceil_div(xy * lv.n0, side), sy);
                 if (flags & F_BACK) {
                     add(pl.phases > 1 ? SEP_MUL_PH : SEP_MUL, a, 0, last, sep_smem_last(lv, true));
+                    if (pl.phases == 1) mul.push_back(last_groups(lv));
                     if (d3) add(SEP_IFFT_Y, a, 0, ceil_div(xy * lv.n0, side), sy);
                     add(SEP_GRAD, a, 0, fgroups, sf);
                 }
                 for (int b = 0; b < pl.phases; ++b) {
                     const int64_t kept = lv.P0 + 1, wrows = sep_v_rows(g);
                     if (flags & F_FWD) {
-                        add(pl.phases > 1 ? SEP_POWER_PH : SEP_POWER, a, b, last, sep_smem_last(lv, false));
+                        add(pl.phases > 1 ? SEP_POWER_PH : SEP_POWER, a, b, last, sep_smem_last(lv, false), lv.parts);
                         if (d3) add(SEP_INV_Y, a, b, ceil_div(xy * kept, side), sy);
                         add(SEP_DESC, a, b, ceil_div(wrows, lv.rowsW), sw);
                     }
@@ -948,6 +996,14 @@ void prepare_sep(const std::vector<Inst>& in, unsigned flags, const std::vector<
         }
     }
     if (levels.empty()) return;
+    share_pairs(mul, usual_pairs(*basis), 4);
+    int64_t mb = 0;
+    for (size_t i = 0; i < mul.size(); ++i) {
+        items[SEP_MUL][i].parts = mul[i].parts;
+        items[SEP_MUL][i].blockStart = mb;
+        mb += mul[i].blocks * mul[i].parts;
+    }
+    P.sep[SEP_MUL].blocks = mb;
     P.o_sep_level = push(P.tb, levels);
     const float2* coef = sep_device_coef(*basis);
     if (coef == nullptr) P.o_sep_coef = push(P.tb, basis->coef);

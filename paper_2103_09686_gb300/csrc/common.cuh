@@ -84,6 +84,7 @@ inline void launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
 }
 
 constexpr int MAX_DYN_SMEM = 200 * 1024;   // dynamic shared memory limit of the correlation kernels
+constexpr int SMS = 152;           // what the splits of work that depend on the free part of the chip aim at
 constexpr int MAX_PHASES = 8;      // phase fields of one problem (their ordered pairs each get a block)
 
 // One multigrid level, every field handled as 3-D (2-D fields have n[0] = 1, P[0] = 0).
@@ -396,6 +397,7 @@ struct SepLevel {
     int first;                // finest level: writes *tier
     int keep;                 // one phase, forward and backward in one call: sep_power leaves its spectra in Z
     int rowsF, rowsW, colsY, colsL;
+    int parts;                // sums of sep_power (over a share of the pairs each) that sep_desc adds, strideV apart
     float* desc;
     double scaleD;            // w / N^2
     const float* src;         // gradient coefficients: scaleG (gscale) (src - sub)
@@ -412,7 +414,8 @@ struct SepLevel {
 };
 
 struct SepItem {
-    int level, a, b, pad;
+    int level, a, b;
+    int parts;                // sep_power, sep_mul: blocks that share the pairs of one group of columns
     int64_t blockStart;
     const int* tier;
     const int* done;

@@ -746,7 +746,7 @@ __device__ __forceinline__ SepShared sep_shared(float2* sm, int n, int lines, in
 
 struct SepBlock {
     SepLevel lv;
-    int a, b, block, tier;
+    int a, b, block, part, parts, tier;      // block: group of lines; part of parts: its share of the pairs
 };
 
 // Before the wait for the predecessor: finds the block's item (every thread looks at one),
@@ -769,7 +769,10 @@ __device__ __forceinline__ bool enter(const SepTables& tb, const SepItem* __rest
     if (threadIdx.x == 0) {
         bk.a = it.a;
         bk.b = it.b;
-        bk.block = (int)((int64_t)blockIdx.x - it.blockStart);
+        const int local = (int)((int64_t)blockIdx.x - it.blockStart);
+        bk.block = local / it.parts;
+        bk.part = local - bk.block * it.parts;
+        bk.parts = it.parts;
     }
     const int *tier = it.tier, *done = it.done;
     __syncthreads();
@@ -1130,7 +1133,7 @@ sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict
     const int pair = bk.a * lv.phases + bk.b;
     const int P = lv.n0 > 1 ? lv.P0 : lv.P1;
     // 3-D: U[r][y][x]; 2-D: V[r][x]
-    float2* out = (lv.n0 > 1 ? lv.U : lv.V) + (int64_t)pair * (lv.n0 > 1 ? lv.strideU : lv.strideV) + g.base;
+    float2* out = (lv.n0 > 1 ? lv.U : lv.V) + (int64_t)(pair + bk.part) * (lv.n0 > 1 ? lv.strideU : lv.strideV) + g.base;
     const bool cross = CROSS && bk.a != bk.b;
     if (ax.fast) {
         for_pow2(ax.fast, [&](auto cc) {
@@ -1148,7 +1151,7 @@ sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict
             }
             double dc = 0.0;
             const bool has_dc = dc_block && c.l == 0 && c.ln.t == 0;
-            for (int p0 = 0; p0 < t.npair; p0 += c.slots) {
+            for (int p0 = bk.part * c.slots; p0 < t.npair; p0 += bk.parts * c.slots) {
                 const int p = p0 + c.slot;
                 const float sg = p < t.npos ? 1.f : -1.f;
                 float2 v[8];
@@ -1209,7 +1212,7 @@ sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict
             if (has_dc && c.slot == 0) {
                 double s = dcs[0];
                 for (int k = 1; k < c.slots; ++k) s += dcs[k];
-                lv.dc[pair] = split(s * lv.scaleD);
+                lv.dc[pair + bk.part] = split(s * lv.scaleD);
             }
             if (has_dc) acc[0] = make_float2(0.f, 0.f);
             swap8(acc);
@@ -1238,7 +1241,7 @@ sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict
             if (e < total) f(q, (e & (g.L - 1)) * pitch + spad(e >> sh));
         }
     };
-    for (int p = 0; p < t.npair; ++p) {
+    for (int p = bk.part; p < t.npair; p += bk.parts) {
         const float sg = p < t.npos ? 1.f : -1.f;
         __syncthreads();
         load_cols(Za + (int64_t)p * lv.N, g, pitch, s.a);
@@ -1262,7 +1265,7 @@ sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict
         });
     }
     if (has_dc) {
-        lv.dc[pair] = split(dc * lv.scaleD);
+        lv.dc[pair + bk.part] = split(dc * lv.scaleD);
         acc[0] = make_float2(0.f, 0.f);
     }
     __syncthreads();
@@ -1401,7 +1404,17 @@ __global__ void __launch_bounds__(SEP_THREADS, 2) sep_desc_kernel(const __grid_c
     const int row0 = bk.block * lv.rowsW, rows = min(lv.rowsW, R - row0);
     const int pair = bk.a * lv.phases + bk.b;
     float2* V = lv.V + (int64_t)pair * lv.strideV + (int64_t)row0 * n;
-    const float2 dc = lv.dc[pair];
+    float2 dc = lv.dc[pair];
+    for (int q = 1; q < lv.parts; ++q) {
+        const DF d = df_add(DF{dc.x, dc.y}, DF{lv.dc[q].x, lv.dc[q].y});
+        dc = make_float2(d.hi, d.lo);
+    }
+    // the window spectra, summed over sep_power's shares of the pairs
+    auto spectrum = [&](int64_t e) {
+        float2 v = V[e];
+        for (int q = 1; q < lv.parts; ++q) v = caddf(v, V[e + q * lv.strideV]);
+        return swapf(v);
+    };
     const float scaleD = (float)lv.scaleD;
     float* desc = lv.desc + (int64_t)pair * lv.Khalf;
     // Kahan sums of this thread's residuals and targets
@@ -1452,7 +1465,7 @@ __global__ void __launch_bounds__(SEP_THREADS, 2) sep_desc_kernel(const __grid_c
             const bool in = line < rows && !skipped(line);
             float2 v[8];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = in ? swapf(V[line * N + ln.t + e * T]) : make_float2(0.f, 0.f);
+            for (int e = 0; e < 8; ++e) v[e] = in ? spectrum(line * N + ln.t + e * T) : make_float2(0.f, 0.f);
             p2_fft<N, WARP, 0>(v, ln);
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
@@ -1477,7 +1490,7 @@ __global__ void __launch_bounds__(SEP_THREADS, 2) sep_desc_kernel(const __grid_c
         const float inv_n = 1.0f / (float)n;
         for (int e = threadIdx.x; e < rows * n; e += blockDim.x) {
             const int l = fdiv(e, inv_n), i = e - l * n;
-            s.a[l * pitch + spad(i)] = skipped(l) ? make_float2(0.f, 0.f) : swapf(V[e]);
+            s.a[l * pitch + spad(i)] = skipped(l) ? make_float2(0.f, 0.f) : spectrum(e);
         }
         float2* r = transform(lv.ax[2], s.a, s.b, s.tw, rows, pitch);
         if (!lv.fuse) {
@@ -1620,6 +1633,7 @@ sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__
     const SepLevel& lv = bk.lv;
     float2* sm = sep_smem;
     const SepTier& t = tb.tier[bk.tier];
+    if (bk.part * (last_ax(lv).fast ? SEP_BLOCK_PTS / (lv.colsL * last_ax(lv).n) : 1) >= t.npair) return;
     int x0, y;
     const ColGroup g = last_axis(lv, bk.block, x0, y);
     const SepAxis& ax = last_ax(lv);
@@ -1647,7 +1661,7 @@ sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__
                     else gr[e * SEP_THREADS] = norm * v[e].x;
                 }
             }
-            for (int p0 = 0; p0 < t.npair; p0 += c.slots) {
+            for (int p0 = bk.part * c.slots; p0 < t.npair; p0 += bk.parts * c.slots) {
                 const int p = p0 + c.slot;
                 const bool on = p < t.npair;
                 float2 v[8];
@@ -1710,7 +1724,7 @@ sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__
         const float2* r = transform(ax, s.a, s.b, s.tw, g.L, pitch);
         own([&](int, int e, int at) { gs[b * total + e] = make_float2(norm * r[at].x, MULTI ? -norm * r[at].y : 0.f); });
     }
-    for (int p = 0; p < t.npair; ++p) {
+    for (int p = bk.part; p < t.npair; p += bk.parts) {
         float2 acc[SEP_OWN];
 #pragma unroll
         for (int q = 0; q < SEP_OWN; ++q) acc[q] = make_float2(0.f, 0.f);
