@@ -6,6 +6,8 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "loss.cuh"
 
@@ -437,32 +439,57 @@ void launch_final(const FinalSeg* segs, int nseg, int64_t blocks, int sub, cudaS
 // memory: stream ordered, no host synchronisation, and valid inside a graph capture.  Different
 // lanes read different parameter words, which the constant path serves one address at a time:
 // 16 bytes a thread and a warp per block keep that serial chain short (15 KB: 6.0 -> 2.3 us).
+// The parameters are copied whole at every launch, so they come in sizes: the host spends 25 us on
+// the descriptor of a 32^2 field (2 KB), 28 with 30 KB.
 constexpr int BLOB_BYTES = 30720;
+template <int BYTES>
 struct Blob {
     unsigned int quads;
-    uint4 data[BLOB_BYTES / 16];
+    uint4 data[BYTES / 16];
 };
 
-__global__ void __launch_bounds__(32) blob_kernel(const __grid_constant__ Blob b, uint4* __restrict__ dst) {
+template <int BYTES>
+__global__ void __launch_bounds__(32) blob_kernel(const __grid_constant__ Blob<BYTES> b, uint4* __restrict__ dst) {
     dep_wait();
     dep_trigger();
     const unsigned int i = blockIdx.x * 32 + threadIdx.x;
     if (i < b.quads) dst[i] = b.data[i];
 }
 
+namespace {
+template <int BYTES>
+void blob_part(const unsigned char* src, size_t n, unsigned char* dst, cudaStream_t s) {
+    static thread_local Blob<BYTES> b;
+    const size_t quads = (n + 15) / 16;
+    if (n % 16) memset(&b.data[quads - 1], 0, 16);
+    memcpy(b.data, src, n);
+    b.quads = (unsigned int)quads;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)((quads + 31) / 32));
+    cfg.blockDim = dim3(32);
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    // by pointer: the parameters are copied once, by the launch
+    uint4* out = reinterpret_cast<uint4*>(dst);
+    void* args[] = {&b, &out};
+    cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(blob_kernel<BYTES>), args);
+}
+}  // namespace
+
 void launch_blob(const void* host, size_t bytes, void* dst, cudaStream_t s) {
     const unsigned char* src = static_cast<const unsigned char*>(host);
     unsigned char* out = static_cast<unsigned char*>(dst);
-    size_t off = 0;
-    static thread_local Blob b;
-    while (off < bytes) {
-        const size_t n = bytes - off < (size_t)BLOB_BYTES ? bytes - off : (size_t)BLOB_BYTES;
-        const size_t quads = (n + 15) / 16;
-        if (n % 16) memset(&b.data[quads - 1], 0, 16);
-        memcpy(b.data, src + off, n);
-        b.quads = (unsigned int)quads;
-        launch_dep(blob_kernel, (unsigned)((quads + 31) / 32), 32, 0, s, b, reinterpret_cast<uint4*>(out + off));
-        off += quads * 16;
+    for (size_t off = 0; off < bytes;) {
+        const size_t n = std::min<size_t>(bytes - off, BLOB_BYTES);
+        if (n <= 2048) blob_part<2048>(src + off, n, out + off, s);
+        else if (n <= 4096) blob_part<4096>(src + off, n, out + off, s);
+        else if (n <= 10240) blob_part<10240>(src + off, n, out + off, s);
+        else blob_part<BLOB_BYTES>(src + off, n, out + off, s);
+        off += (n + 15) / 16 * 16;
     }
 }
 
