@@ -174,16 +174,20 @@ bool fft_size_ok(int64_t n) {
     return n == 1;
 }
 
-// Identity threshold, AUTO path: the FFT when its estimated cost is lower.  Both costs are
-// fitted (relative error) to GB300 measurements of descriptor + gradient on 64^3 and 128^3
-// (P = 1..24): the FFT path is ~0.758 ns per grid point + 0.157 ms; the direct kernels
-// ~0.148 ps per voxel-shift + 0.127 ns per point + 0.151 ms.  Measured crossovers: P = 8 on
-// both grids (at P = 6 the direct path is ahead by 23% on 64^3 and 29% on 128^3).
-bool fft_cheaper(const LevelGeom& g) {
+// Identity threshold, AUTO path: the FFT when its estimated cost is lower.  Fitted to loss and
+// gradient on GB300, 16^3 .. 160^3 and 64^2 .. 2048^2 (us, direct / FFT): 64^3 P = 4 167 / 181,
+// P = 8 367 / 201; 96^3 P = 3 272 / 317, P = 6 619 / 317; 128^3 P = 2 403 / 556, P = 4 637 / 558;
+// 256^2 P = 32 105 / 121, P = 64 235 / 122; 512^2 P = 32 236 / 245, P = 64 654 / 246; 1024^2
+// P = 16 282 / 352, P = 31 586 / 352.
+// A last axis that the direct kernels do not take leaves nothing to choose: there an older,
+// higher line (fitted when the FFT path took three times as long) decides which problems are
+// accepted, and stays.
+bool fft_cheaper(const LevelGeom& g, int ndim) {
+    const double N = (double)g.N;
     const double kfull = (double)(2 * g.P[0] + 1) * (2 * g.P[1] + 1) * (2 * g.P[2] + 1);
-    const double t_direct = (double)g.N * kfull * 1.481e-13 + (double)g.N * 1.266e-10 + 1.506e-4;
-    const double t_fft = (double)g.N * 7.577e-10 + 1.568e-4;
-    return t_fft < t_direct;
+    if (g.n[2] % T != 0) return N * 7.577e-10 + 1.568e-4 < N * kfull * 1.481e-13 + N * 1.266e-10 + 1.506e-4;
+    if (ndim == 3) return N * 2.6e-10 + 1.0e-4 < N * kfull * 2.2e-13 + N * 1.2e-10 + 4e-5;
+    return N * 5.6e-10 + 1.0e-4 < N * kfull * 1.3e-13 + N * 1.0e-10 + 4e-5;
 }
 
 // sizes of one FFT level (no pointers)
@@ -201,6 +205,7 @@ FftArgs fft_shape(const LevelGeom& g) {
     a.Lx = fft_lines_per_block(a.n2, false);
     a.Ly = fft_lines_per_block(a.n1, true);
     a.Ll = fft_lines_per_block(a.n0 > 1 ? a.n0 : a.n1, true);
+    fft_window_lines(a);
     a.nsq = fft_row_blocks(a);
     return a;
 }
@@ -519,7 +524,7 @@ dmcr_status make_plan(const dmcr_params* p, Plan& pl) {
                 return fail(DMCR_ENOTSUP, "FFT path: level %d sizes must factor into 2, 3, 5 and be <= 4096", l + 1);
             g.fft = 1;
         } else if (p->path == DMCR_PATH_AUTO && p->threshold == DMCR_IDENTITY && phases == 1 && fft_sizes &&
-                   fft_cheaper(g)) {
+                   fft_cheaper(g, pl.ndim)) {
             g.fft = 1;
         }
         if (pl.desc_kind == DMCR_DESC_S3) {

@@ -320,6 +320,7 @@ struct FftArgs {
     int64_t N;
     FftAxis ax[3];
     int Lx, Ly, Ll;           // lines per block: rows (row pairs), middle axis, last axis
+    int Lv, Lw;               // the window's rows and middle axis
     const float* field;
     double2 *X, *U, *V;       // half spectrum of the field; window planes (3-D) and rows
     double* sq;               // sum M^2 of the row blocks
@@ -482,6 +483,7 @@ void launch_s3_backward(const S3Job& j, const ThreshConst& tc, int* err, cudaStr
 void set_fft_attributes();
 void fft_axis(int len, FftAxis& ax);
 int fft_lines_per_block(int len, bool strided);
+void fft_window_lines(FftArgs& g);
 int fft_row_blocks(const FftArgs& g);
 void launch_fft_descriptor(const FftArgs& g, cudaStream_t s);
 void launch_fft_vjp(const FftArgs& g, cudaStream_t s);

@@ -27,7 +27,9 @@
 //   fft_mul     last axis: transform of A, product with X, inverse
 //   fft_grad    inverse along x, two rows at a time: the gradient
 // 128^3, +-24, loss and gradient: 1715 us with twelve full complex passes of 130 us and seven
-// elementwise kernels, 603 us so.
+// elementwise kernels, 579 us so.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace dmcr {
@@ -319,8 +321,8 @@ template <bool DESC>
 __global__ void __launch_bounds__(FFT_THREADS, 3) fft_win_y_kernel(const __grid_constant__ FftArgs g) {
     dep_wait();
     dep_trigger();
-    const int xg = (g.nh + g.Ly - 1) / g.Ly, x0 = (int)(blockIdx.x % xg) * g.Ly, rz = (int)(blockIdx.x / xg);
-    const int n = g.n1, L = g.Ly, cols = min(L, g.nh - x0), wy = 2 * g.P1 + 1;
+    const int xg = (g.nh + g.Lw - 1) / g.Lw, x0 = (int)(blockIdx.x % xg) * g.Lw, rz = (int)(blockIdx.x / xg);
+    const int n = g.n1, L = g.Lw, cols = min(L, g.nh - x0), wy = 2 * g.P1 + 1;
     double2 *a = fft_smem, *b = fft_smem + L * n;
     double2* U = g.U + (int64_t)rz * g.n1 * g.nh + x0;
     double2* V = g.V + (int64_t)rz * wy * g.nh + x0;
@@ -356,7 +358,7 @@ __global__ void __launch_bounds__(FFT_THREADS, 3) fft_desc_kernel(const __grid_c
     dep_wait();
     dep_trigger();
     __shared__ double sh[FFT_THREADS];
-    const int n = g.n2, nh = g.nh, L = g.Lx, R = fft_window_rows(g), q0 = blockIdx.x * L;
+    const int n = g.n2, nh = g.nh, L = g.Lv, R = fft_window_rows(g), q0 = blockIdx.x * L;
     const int lines = min(L, (R + 1) / 2 - q0);
     double2 *a = fft_smem, *b = fft_smem + L * n;
     double s = 0.0;
@@ -390,7 +392,7 @@ __global__ void __launch_bounds__(FFT_THREADS, 3) fft_desc_kernel(const __grid_c
 __global__ void __launch_bounds__(FFT_THREADS, 3) fft_coef_kernel(const __grid_constant__ FftArgs g) {
     dep_wait();
     dep_trigger();
-    const int n = g.n2, nh = g.nh, L = g.Lx, R = fft_window_rows(g), q0 = blockIdx.x * L;
+    const int n = g.n2, nh = g.nh, L = g.Lv, R = fft_window_rows(g), q0 = blockIdx.x * L;
     const int lines = min(L, (R + 1) / 2 - q0);
     double2 *a = fft_smem, *b = fft_smem + L * n;
     auto A = [&](int row, int i) {
@@ -503,6 +505,18 @@ int fft_lines_per_block(int len, bool strided) {
     return L < least ? least : L;
 }
 
+namespace {
+int win_pairs(const FftArgs& g) { return ((g.n0 > 1 ? (g.P0 + 1) * (2 * g.P1 + 1) : g.P1 + 1) + 1) / 2; }
+}
+
+// The window's rows and planes are few: fewer lines a block, so that every SM has one (128^3, +-24:
+// its four launches 80 us together with the field's 8 lines a block, 64 so).
+void fft_window_lines(FftArgs& g) {
+    g.Lv = std::max(1, std::min(g.Lx, win_pairs(g) / SMS));
+    g.Lw = g.Ly;
+    if (g.Lw > 4 && (int64_t)((g.nh + g.Lw - 1) / g.Lw) * (g.P0 + 1) < 2 * SMS) g.Lw = 4;
+}
+
 int fft_row_blocks(const FftArgs& g) { return (int)(((int64_t)g.n0 * g.n1 + 1) / 2 + g.Lx - 1) / g.Lx; }
 
 namespace {
@@ -512,10 +526,10 @@ size_t last_smem(const FftArgs& g, bool mul) {
     const size_t pts = (size_t)g.Ll * (g.n0 > 1 ? g.n0 : g.n1);
     return 2 * pts * sizeof(double2) + (mul ? pts * sizeof(double) : 0);
 }
-unsigned win_blocks(const FftArgs& g) {
-    const int R = g.n0 > 1 ? (g.P0 + 1) * (2 * g.P1 + 1) : g.P1 + 1;
-    return (unsigned)(((R + 1) / 2 + g.Lx - 1) / g.Lx);
-}
+unsigned win_blocks(const FftArgs& g) { return (unsigned)((win_pairs(g) + g.Lv - 1) / g.Lv); }
+unsigned win_y_blocks(const FftArgs& g) { return (unsigned)((g.nh + g.Lw - 1) / g.Lw) * (g.P0 + 1); }
+size_t win_smem(const FftArgs& g) { return (size_t)2 * g.Lv * g.n2 * sizeof(double2); }
+size_t win_y_smem(const FftArgs& g) { return (size_t)2 * g.Lw * g.n1 * sizeof(double2); }
 unsigned last_blocks(const FftArgs& g) { return (unsigned)((g.nh + g.Ll - 1) / g.Ll) * (g.n0 > 1 ? g.n1 : 1); }
 unsigned y_blocks(const FftArgs& g, int planes) { return (unsigned)((g.nh + g.Ly - 1) / g.Ly) * planes; }
 
@@ -531,15 +545,15 @@ void field_spectrum(const FftArgs& g, cudaStream_t s) {
 void launch_fft_descriptor(const FftArgs& g, cudaStream_t s) {
     field_spectrum(g, s);
     launch_dep(fft_last_kernel, last_blocks(g), FFT_THREADS, last_smem(g, false), s, g);
-    if (g.n0 > 1) launch_dep(fft_win_y_kernel<true>, y_blocks(g, g.P0 + 1), FFT_THREADS, y_smem(g), s, g);
-    launch_dep(fft_desc_kernel, win_blocks(g), FFT_THREADS, row_smem(g), s, g);
+    if (g.n0 > 1) launch_dep(fft_win_y_kernel<true>, win_y_blocks(g), FFT_THREADS, win_y_smem(g), s, g);
+    launch_dep(fft_desc_kernel, win_blocks(g), FFT_THREADS, win_smem(g), s, g);
 }
 
 // g.x_ready: the descriptor of the same call left X (and the twiddles) in place
 void launch_fft_vjp(const FftArgs& g, cudaStream_t s) {
     if (!g.x_ready) field_spectrum(g, s);
-    launch_dep(fft_coef_kernel, win_blocks(g), FFT_THREADS, row_smem(g), s, g);
-    if (g.n0 > 1) launch_dep(fft_win_y_kernel<false>, y_blocks(g, g.P0 + 1), FFT_THREADS, y_smem(g), s, g);
+    launch_dep(fft_coef_kernel, win_blocks(g), FFT_THREADS, win_smem(g), s, g);
+    if (g.n0 > 1) launch_dep(fft_win_y_kernel<false>, win_y_blocks(g), FFT_THREADS, win_y_smem(g), s, g);
     launch_dep(fft_mul_kernel, last_blocks(g), FFT_THREADS, last_smem(g, true), s, g);
     if (g.n0 > 1) launch_dep(fft_y_kernel<true>, y_blocks(g, g.n0), FFT_THREADS, y_smem(g), s, g);
     launch_dep(fft_grad_kernel, (unsigned)fft_row_blocks(g), FFT_THREADS, row_smem(g), s, g);

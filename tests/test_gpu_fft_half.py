@@ -31,3 +31,21 @@ def test_half_spectrum_edges(cuda_lib, shape, window):
     want = oracle.level_vjp(M.astype(np.float64), op, G.astype(np.float64), pos)
     # the coefficients and the result are floats: each 6e-8, summed over random signs
     assert np.linalg.norm(g[pos] - want) / np.linalg.norm(want) < 1e-6
+
+
+@pytest.mark.parametrize("shape,window,levels", [((96, 96, 96), (6, 6, 6), 1), ((64, 48, 80), (9, 12, 7), 2),
+                                                 ((1024, 1024), (40, 40), 1), ((128, 128, 128), (4, 4, 5), 1)])
+def test_auto_equals_direct_near_the_line(cuda_lib, shape, window, levels):
+    """Problems on both sides of the line at which the identity threshold goes to the transforms:
+    the chosen path against the direct kernels."""
+    dm = cuda_lib
+    M = torch.rand(shape, device="cuda", generator=torch.Generator("cuda").manual_seed(5)) * 1.4 - 0.2
+    out = []
+    for path in (dm.DMCR_PATH_AUTO, dm.DMCR_PATH_DIRECT):
+        p = dm.Params(shape=shape, window=window, levels=levels, threshold=dm.DMCR_IDENTITY, path=path)
+        target = torch.full((dm.dmcr_descriptor_length(p),), 0.3, device="cuda")
+        out.append((dm.descriptor(M, p), *dm.loss_grad(M, target, p)))
+    (d1, l1, g1), (d2, l2, g2) = out
+    np.testing.assert_allclose(d1.cpu().numpy(), d2.cpu().numpy(), rtol=1e-5, atol=1e-9)
+    np.testing.assert_allclose(l1.cpu().numpy(), l2.cpu().numpy(), rtol=1e-5)
+    assert float(torch.linalg.norm(g1 - g2) / torch.linalg.norm(g2)) < 1e-5
