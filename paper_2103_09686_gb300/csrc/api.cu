@@ -635,7 +635,7 @@ dmcr_status make_plan(const dmcr_params* p, Plan& pl) {
         if (nr > INT32_MAX || ns > INT32_MAX) return fail(DMCR_EINVAL, "window too large: the descriptor has too many blocks");
         pl.nred = (int)nr;
         pl.nsep = (int)ns;
-        pl.nexc = (int)std::min<int64_t>(NPEN_BLOCKS, ceil_div(Nall, 2048));
+        pl.nexc = (int)std::min<int64_t>(1024, ceil_div(Nall, 2048));
         pl.o_excess = o; o = align_up(o + (size_t)std::max(pl.nexc, PREP_BLOCKS) * sizeof(float4));
         pl.o_sums = o; o = align_up(o + (size_t)std::max(nr, ns) * sizeof(float4));
     }

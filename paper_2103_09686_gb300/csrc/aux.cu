@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(256, 5) stats_kernel(const PenSeg* __restrict_
     const PenSeg& sg = segs[blockIdx.y];
     if (sg.done != nullptr && *sg.done) return;
     if ((int)blockIdx.x >= sg.nblk) return;
-    __shared__ DF sh[32];
+    __shared__ DF sh[3 * 8];
     const int64_t stride = (int64_t)sg.nblk * blockDim.x;
     const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     // per-thread compensated (Kahan) FP32 sums in a fixed order -- FP64 arithmetic is slow on
@@ -258,12 +258,11 @@ __global__ void __launch_bounds__(256, 5) stats_kernel(const PenSeg* __restrict_
         }
     }
     // Kahan's (sum, comp) stands for sum - comp
-    const DF R2 = block_sum_df(df_two_sum(r2, -r2c), sh);
-    const DF T2 = block_sum_df(df_two_sum(t2, -t2c), sh);
-    const DF E2 = block_sum_df(df_two_sum(e2, -e2c), sh);
+    DF v[3] = {df_two_sum(r2, -r2c), df_two_sum(t2, -t2c), df_two_sum(e2, -e2c)};
+    block_sums_df(v, sh);
     if (threadIdx.x == 0) {
-        sg.sums[blockIdx.x] = make_float4(R2.hi, R2.lo, T2.hi, T2.lo);
-        sg.excess[blockIdx.x] = make_float4(E2.hi, E2.lo, 0.f, 0.f);
+        sg.sums[blockIdx.x] = make_float4(v[0].hi, v[0].lo, v[1].hi, v[1].lo);
+        sg.excess[blockIdx.x] = make_float4(v[2].hi, v[2].lo, 0.f, 0.f);
     }
     loss_arrive(*sg.loss, sg.nblk, sh);
 }

@@ -20,7 +20,7 @@ constexpr int S3_SHIFTS = 32;      // three-point gradient gather: shifts per pa
 
 // offset of C_m inside a coefficient block: (C_m, C_m, C_m+1, C_m+1) after the 8 (A, A, B, B)
 __host__ __device__ inline int gblock_c(int m) { return 4 * T + 2 * m; }
-constexpr int NPEN_BLOCKS = 1024;  // most blocks of the loss statistics of one instance
+constexpr int NPEN_BLOCKS = 512;   // most blocks of the loss statistics of one instance
 
 // Double-float sums: an FP32 pair hi + lo carries about 48 significant bits.  FP64
 // arithmetic is slow on this part, and the reductions below sit on the critical path of
@@ -43,23 +43,36 @@ __device__ __forceinline__ DF df_add(DF a, DF b) {
     return {hi, lo - (hi - s.hi)};
 }
 
-// fixed-order sum over the block (blockDim.x a multiple of 32, <= 1024): xor butterflies in
-// each warp, then over the warp results in warp 0; the result is valid in thread 0.  sh holds
-// 32 entries.
-__device__ __forceinline__ DF block_sum_df(DF v, DF* sh) {
-    for (int o = 16; o > 0; o >>= 1)
-        v = df_add(v, DF{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)});
+// fixed-order sums over the block (blockDim.x a multiple of 32): xor butterflies in each warp, then
+// over the warp results in warp 0, all NV values side by side; the results are valid in warp 0.
+// sh holds NV entries for every warp.
+template <int NV>
+__device__ __forceinline__ void block_sums_df(DF (&v)[NV], DF* sh) {
+    auto warp_sums = [&]() {
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int i = 0; i < NV; ++i)
+                v[i] = df_add(v[i], DF{__shfl_xor_sync(0xffffffffu, v[i].hi, o), __shfl_xor_sync(0xffffffffu, v[i].lo, o)});
+    };
+    warp_sums();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     __syncthreads();   // sh may still be read by a previous call
-    if (lane == 0) sh[warp] = v;
+    if (lane == 0)
+#pragma unroll
+        for (int i = 0; i < NV; ++i) sh[warp * NV + i] = v[i];
     __syncthreads();
     if (warp == 0) {
-        v = lane < nw ? sh[lane] : DF{0.f, 0.f};
-        for (int o = 16; o > 0; o >>= 1)
-            v = df_add(v, DF{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)});
+#pragma unroll
+        for (int i = 0; i < NV; ++i) v[i] = lane < nw ? sh[lane * NV + i] : DF{0.f, 0.f};
+        warp_sums();
     }
-    return v;
 }
+__device__ __forceinline__ DF block_sum_df(DF v, DF* sh) {
+    DF a[1] = {v};
+    block_sums_df(a, sh);
+    return a[0];
+}
+
 // Programmatic dependent launch.  A kernel launched with launch_dep may start while its
 // predecessor in the stream still runs; dep_wait() returns once every earlier kernel has
 // completed and its writes are visible, and dep_trigger() lets the successor start.  Every

@@ -20,38 +20,52 @@ __device__ __forceinline__ float box_excess(float M) {
     return M > 1.f ? M - 1.f : (M < 0.f ? -M : 0.f);
 }
 
-// One thread: E, E^2, E_bc, lambda, L, rel_err and the gradient scalars from
+// Warp 0: E, E^2, E_bc, lambda, L, rel_err and the gradient scalars from
 // sum (D - D_des)^2, sum D_des^2 and the sum of the squared box excess; in a reconstruction
 // also the stopping test and the Adam step bookkeeping.
+// In FP64: the double-float sums keep about 48 bits, and the square roots and quotients below
+// keep them, so E, rel_err and L reach the output rounded once to FP32.  An FP64 root or quotient
+// is a chain of several hundred cycles and every other block waits for this one, so a lane each
+// takes the three roots, then the four quotients that depend on nothing else, at once.
 __device__ __forceinline__ void loss_scalars(const LossSeg& sg, DF e2s, DF t2s, DF x2s) {
-    const LossParams lp = sg.lp;
+    const LossParams& lp = sg.lp;
     Scalars* sc = sg.sc;
-    float* loss_out = sg.loss_out;
-    float* history = sg.history;
-    // the scalars in FP64 on this one thread (a few dozen FP64 operations once per
-    // evaluation): the double-float sums keep about 48 bits, and the square roots and
-    // quotients below keep them, so E, rel_err and L reach the output rounded once to FP32
+    const int lane = threadIdx.x & 31;
     const double E2 = (double)e2s.hi + (double)e2s.lo;
     const double T2 = (double)t2s.hi + (double)t2s.lo;
     const double ex2 = (double)x2s.hi + (double)x2s.lo;
     const double N = (double)lp.N;
     const double lam0 = lp.bc_on ? (double)lp.lambda0 : 0.0;
-    const double E = sqrt(E2);
-    const double Ebc = ex2 / (N * N);
+    // beta^t products stay FP64: they are multiplied once per step over many steps
+    const double b1t = sc->b1t * (double)lp.beta1;
+    const double b2t = sc->b2t * (double)lp.beta2;
+    const double root = sqrt(lane == 0 ? E2 : (lane == 1 ? T2 : 1.0 - b2t));
+    const double E = __shfl_sync(0xffffffffu, root, 0);
+    const double rootT = __shfl_sync(0xffffffffu, root, 1), rootB = __shfl_sync(0xffffffffu, root, 2);
     const double phi = lp.mode == 0 ? E : E2;
     const double lam = lam0 * phi;
+    // E / |D_des|, E_bc, the penalty's gradient factor, Adam's step
+    const double num = lane == 0 ? E : (lane == 1 ? ex2 : (lane == 2 ? 2.0 * lam0 * phi : (double)lp.lr * rootB));
+    const double den = lane == 0 ? rootT : (lane <= 2 ? N * N : 1.0 - b1t);
+    const double quot = num / den;
+    const double Ebc = __shfl_sync(0xffffffffu, quot, 1);
+    const float pen_coef = (float)__shfl_sync(0xffffffffu, quot, 2);
+    const float lr_t = (float)__shfl_sync(0xffffffffu, quot, 3);
+    if (lane != 0) return;
     const double L = phi + lam * Ebc;
-    const double rel = T2 > 0.0 ? E / sqrt(T2) : (double)INFINITY;
-    const float out[6] = {(float)E, (float)E2, (float)Ebc, (float)lam, (float)L, (float)rel};
-    for (int i = 0; i < 6; ++i) sc->loss[i] = out[i];
-    if (loss_out != nullptr)
-        for (int i = 0; i < 6; ++i) loss_out[i] = out[i];
+    const double rel = T2 > 0.0 ? quot : (double)INFINITY;
     // dL/dD = phi'(E) (1 + lam0 E_bc) dE/dD ;  dL/dM (penalty) = lam0 phi dE_bc/dM
     double gs;
     if (lp.mode == 0) gs = E > 0.0 ? (1.0 + lam0 * Ebc) / E : 0.0;
     else gs = 2.0 * (1.0 + lam0 * Ebc);
     sc->gscale = (float)gs;
-    sc->pen_coef = (float)(2.0 * lam0 * phi / (N * N));
+    sc->pen_coef = pen_coef;
+    float* loss_out = sg.loss_out;
+    float* history = sg.history;
+    const float out[6] = {(float)E, (float)E2, (float)Ebc, (float)lam, (float)L, (float)rel};
+    for (int i = 0; i < 6; ++i) sc->loss[i] = out[i];
+    if (loss_out != nullptr)
+        for (int i = 0; i < 6; ++i) loss_out[i] = out[i];
     if (!lp.recon) return;
     const int it = sc->iter;
     if (history != nullptr && it < lp.max_iters) {
@@ -64,30 +78,26 @@ __device__ __forceinline__ void loss_scalars(const LossSeg& sg, DF e2s, DF t2s, 
     if (lp.tol_rel > 0.f && (it % lp.check_every) == 0 && out[5] < lp.tol_rel) { sc->done = 1; return; }
     if (it + 1 > lp.max_iters) { sc->done = 3; return; }
     sc->adam_step = sc->adam_step + 1;
-    // beta^t products stay FP64: they are multiplied once per step over many steps
-    const double b1t = sc->b1t * (double)lp.beta1;
-    const double b2t = sc->b2t * (double)lp.beta2;
     sc->b1t = b1t;
     sc->b2t = b2t;
-    sc->lr_t = (float)((double)lp.lr * sqrt(1.0 - b2t) / (1.0 - b1t));
+    sc->lr_t = lr_t;
 }
 
-// Whole block: sums the instance's block sums in a fixed order and finishes the loss.
+// Whole block: sums the instance's block sums in a fixed order and finishes the loss.  `sh`: three
+// entries for every warp.
 __device__ __forceinline__ void loss_finish(const LossSeg& sg, DF* sh) {
-    DF r2{0.f, 0.f}, t2{0.f, 0.f}, x2{0.f, 0.f};
+    DF v[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
     for (int i = threadIdx.x; i < sg.nsum; i += blockDim.x) {
-        const float4 v = __ldcg(sg.sums + i);
-        r2 = df_add(r2, DF{v.x, v.y});
-        t2 = df_add(t2, DF{v.z, v.w});
+        const float4 s = __ldcg(sg.sums + i);
+        v[0] = df_add(v[0], DF{s.x, s.y});
+        v[1] = df_add(v[1], DF{s.z, s.w});
     }
     for (int i = threadIdx.x; i < sg.nexc; i += blockDim.x) {
-        const float4 v = __ldcg(sg.excess + i);
-        x2 = df_add(x2, DF{v.x, v.y});
+        const float4 s = __ldcg(sg.excess + i);
+        v[2] = df_add(v[2], DF{s.x, s.y});
     }
-    const DF e2s = block_sum_df(r2, sh);
-    const DF t2s = block_sum_df(t2, sh);
-    const DF x2s = block_sum_df(x2, sh);
-    if (threadIdx.x == 0) loss_scalars(sg, e2s, t2s, x2s);
+    block_sums_df(v, sh);
+    if (threadIdx.x < 32) loss_scalars(sg, v[0], v[1], v[2]);
 }
 
 // Called by every block (all threads) of the launch that leaves an instance's `count` block

@@ -1395,7 +1395,7 @@ __device__ __forceinline__ int half_index(const SepLevel& lv, int rz, int ry, in
 __global__ void __launch_bounds__(SEP_THREADS, 2) sep_desc_kernel(const __grid_constant__ SepTables tb,
                                                                   const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
-    __shared__ DF dsh[32];
+    __shared__ DF dsh[3 * SEP_THREADS / 32];
     if (!enter<true>(tb, items, nitem, bk, sep_smem, axis_x)) return;
     const SepLevel& lv = bk.lv;
     float2* sm = sep_smem;
@@ -1517,10 +1517,10 @@ __global__ void __launch_bounds__(SEP_THREADS, 2) sep_desc_kernel(const __grid_c
     }
     if (lv.loss == nullptr) return;
     // Kahan's (sum, comp) stands for sum - comp
-    const DF R2 = block_sum_df(df_two_sum(r2, -r2c), dsh);
-    const DF T2 = block_sum_df(df_two_sum(t2, -t2c), dsh);
+    DF sums[2] = {df_two_sum(r2, -r2c), df_two_sum(t2, -t2c)};
+    block_sums_df(sums, dsh);
     const int blocks = (R + lv.rowsW - 1) / lv.rowsW;
-    if (threadIdx.x == 0) lv.sums[lv.sumStart + pair * blocks + bk.block] = make_float4(R2.hi, R2.lo, T2.hi, T2.lo);
+    if (threadIdx.x == 0) lv.sums[lv.sumStart + pair * blocks + bk.block] = make_float4(sums[0].hi, sums[0].lo, sums[1].hi, sums[1].lo);
     loss_arrive(*lv.loss, lv.arrive, dsh);
 }
 
