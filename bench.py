@@ -52,11 +52,7 @@ MIX_KEY = {"corr_fwd": "forward_pairs", "corr_adj": "adjoint_pairs"}
 # DRAM bytes (read + write) per launch of each correlation kernel, from one ncu capture of the
 # bench's own command per workload (dram__bytes_read.sum + dram__bytes_write.sum); None
 # whenever a kernel changed since its last capture.
-NCU_TRAFFIC_BYTES = {("grf512", "corr_adj"): 2780160 + 256, ("grf512", "corr_fwd"): 1457152 + 1024,
-                     ("mp3_512", "corr_adj"): 16121344 + 45945088, ("mp3_512", "corr_fwd"): 4216832 + 45588480,
-                     ("grf128_3d", "corr_adj"): 17604096 + 51608320, ("grf128_3d", "corr_fwd"): 39135744 + 242014464,
-                     ("grf64", "corr_adj"): 114688 + 0, ("grf64", "corr_fwd"): 93440 + 0,
-                     ("batch256", "corr_adj"): 135313408 + 1368981248, ("batch256", "corr_fwd"): 86752256 + 615229184}
+NCU_TRAFFIC_BYTES = {}
 
 WORKLOADS = {
     "grf512": dict(shape=(512, 512), window=(64, 64), levels=3,
@@ -984,6 +980,10 @@ def main():
         pairs_adj += nsum * kfull
         pairs_fwd += nsum * ((kfull + 1) // 2)
     pairs = pairs_adj if name.startswith("corr_adj") else (pairs_fwd if name.startswith("corr_fwd") else None)
+    # separable instances evaluate no pairs (their gated correlation launches find nothing to do)
+    separable = any(k.startswith("sep_") for k in prof)
+    if separable:
+        pairs = None
     sm_count = torch.cuda.get_device_properties(dev).multi_processor_count
     max_mhz = clocks.get("sm_max_mhz") or 2070.0
     avg_ms = kms / max(kcnt, 1)
@@ -1019,8 +1019,20 @@ def main():
                     "binding_frac": max(achieved / peak, mufu / mufu_peak),
                     "pairs_per_launch": pairs, "pairs_per_s": pairs / t,
                     "avg_launch_ms": avg_ms, "launches": kcnt}
-    # kernels of this library per step (the profiled pass launches the same kernels as a graph
-    # replay: the replay's scalar set-up kernel stands in for the direct path's), times steps
+    elif separable:
+        # the step against what no method avoids: a transform there and back for the correlation
+        # of each ordered phase pair and its gradient the same again, 5 N log2 N operations each
+        flops = sum(nph * nph * 4 * 5.0 * n * np.log2(n) for sh, _, lev, _ in insts for n in level_sizes(sh, lev))
+        peak = sm_count * pipes["ffma2_lanes"] * 2 * max_mhz * 1e6 / 1e12
+        achieved = flops / (total_s / args.steps) / 1e12
+        roofline = {"bound": "alu", "kernel": name, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+                    "frac": achieved / peak, "traffic": None,
+                    "peak_basis": "measured FP32 pipe (FFMA2 probe) at the max SM clock; achieved = transform "
+                                  "operations of the exact correlation and its gradient / step time (the separable "
+                                  "path runs about a dozen such transforms, one per pair of features)",
+                    "avg_launch_ms": avg_ms, "launches": kcnt}
+    # kernels of this library per step (the profiled pass launches the kernels of a graph replay
+    # directly), times steps
     launches = int(round(sum(c for _, c in prof.values()) / max(prof_steps, 1) * args.steps))
 
     cpu = None

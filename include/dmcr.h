@@ -61,8 +61,13 @@ enum { DMCR_SOFT = 0, DMCR_IDENTITY = 1 };           /* threshold (Sec. 3.2.4; f
  * autocorrelation by hand-written FP64 FFTs -- exact (up to rounding) for the identity
  * threshold, and for the soft threshold of BINARY fields through the App. A mapping
  * (descriptor only; use it to characterise binary targets).  Every level size must factor
- * into 2, 3 and 5 and be <= 4096 per axis.  AUTO: DIRECT for the soft threshold; for the
- * identity threshold the cheaper of the two per level (measured crossover). */
+ * into 2, 3 and 5 and be <= 4096 per axis.  AUTO: for the identity threshold the cheaper of
+ * the two per level (measured crossover); for the soft threshold DIRECT, or, where it is
+ * estimated to be faster, the separable path: f((u + v) / 2)^2 as a short sum of products
+ * over a range of values, evaluated by FP32 transforms with FP32-level accuracy.  The range
+ * is taken from the field on the device; NaN and fields beyond [-2.25, 2.5] (alpha = 10) are
+ * left to the DIRECT kernels of the same call.  The first separable call of an alpha on a
+ * device copies its table of coefficients there on a private stream. */
 enum { DMCR_PATH_AUTO = 0, DMCR_PATH_DIRECT = 1, DMCR_PATH_FFT = 2 };
 enum { DMCR_LOSS_NORM = 0, DMCR_LOSS_SQUARED = 1 };  /* L = E(1 + lambda0 E_bc)  |  E^2 (1 + lambda0 E_bc) */
 enum { DMCR_PROLONG_ADJOINT_ACCUMULATE = 0, DMCR_PROLONG_INJECT = 1 };
@@ -249,8 +254,8 @@ dmcr_status dmcr_reconstruct(const dmcr_params* p, const dmcr_recon_opts* opts,
  *   The first call with a given set of arguments (params, the options above, every pointer,
  *   ws_bytes, the current device) captures the iteration into a CUDA graph that the library
  *   keeps (the 16 most recently used sets); a later call with the same arguments launches
- *   one small kernel with this call's step count and replays the graph, with the same
- *   results bit for bit.  While `stream` is being captured by the caller, or while the
+ *   one small kernel with this call's scalars and tables and replays the graph, with the
+ *   same results bit for bit.  While `stream` is being captured by the caller, or while the
  *   dmcr_profile timers are on, the kernels are launched directly instead.
  */
 dmcr_status dmcr_adam_step(const dmcr_params* p, const dmcr_recon_opts* opts, const float* target_desc,

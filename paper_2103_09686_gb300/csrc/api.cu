@@ -764,7 +764,7 @@ dmcr_status check_ws(const Plan& pl, void* ws, size_t ws_bytes) {
 //   upload (scalars, tables) -> prep (pyramid, value range) -> corr_fwd -> fwd_reduce (and the
 //   loss, finished by its last block) -> corr_adj -> final (gradient assembly, optional Adam
 //   step); separable instances run the sep_* kernels instead (sep.cu), FFT and three-point
-//   ones theirs, with the statistics and the loss in two further launches.
+//   ones theirs, with the statistics and the loss in one further launch.
 enum : unsigned {
     F_FWD = 2u,      // pyramid + descriptor
     F_LOSS = 4u,     // penalty + loss
