@@ -14,7 +14,7 @@
 // are packed in pairs, z = p_1 + i p_2: Re IDFT(|Z|^2) = autocorr(p_1) + autocorr(p_2), and a
 // real even G acts on both parts at once, so no mirrored frequency is ever read.
 //
-//   sep_range   the tier (basis) that covers the field's values; none: the direct kernels run
+//   prep_kernel (aux.cu) the tier (basis) that covers the field's values; none: the direct kernels run
 //   sep_feat    features of whole rows + transform along x             -> Z
 //   sep_fft_y   3-D: transform along y, in place
 //   sep_power   last axis: transform, sum_k s_k conj(Z^a_k) Z^b_k, inverse along the same
@@ -874,7 +874,10 @@ __device__ __forceinline__ Line<N> row_line(float2* sm, int line, int t, int lin
 
 // item: (level, phase a); blocks: groups of rows.  Features of whole rows and their transform
 // along x.  Every block combines the range blocks' tiers; the first block of the finest
-// level leaves the result for the later kernels.
+// level leaves the result for the later kernels.  Bound by latency (coefficient gathers from L1,
+// exchanges): it issues 35 % of the time.  Seven pairs: 512^2, three levels 24 us; 1024^2, five
+// levels 79 us; 128^3, two levels 89 us (one series over the whole range instead of local
+// polynomials: twice the instructions).
 __global__ void __launch_bounds__(SEP_ROW_THREADS, 4) sep_feat_kernel(const __grid_constant__ SepTables tb,
                                                                       const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
@@ -1038,7 +1041,8 @@ __device__ __forceinline__ void load_cols(const float2* __restrict__ src, const 
 
 // Middle axis of 3-D, in place on Z (forward) or on the product spectra (INVERSE).  item:
 // (level, phase a); blocks: groups of planes' columns (x fastest, then z).  A block walks the
-// feature pairs, loading the next pair's columns while it transforms the current ones.
+// feature pairs, loading the next pair's columns while it transforms the current ones (128^3, two
+// levels, seven pairs: 53 us; a block for every pair: 99).
 template <bool INVERSE>
 __global__ void __launch_bounds__(SEP_THREADS, 2) sep_fft_y_kernel(const __grid_constant__ SepTables tb,
                                                                    const SepItem* __restrict__ items, int nitem) {
@@ -1113,7 +1117,9 @@ __device__ __forceinline__ float2 split(double v) {
 
 // item: (level, phases a, b).  Sums s_k conj(Z^a_k) Z^b_k over the feature pairs and writes the
 // inverse along the last axis, cropped to r = 0 .. P (-r belongs to the pair (b, a)).  CROSS:
-// a and b may differ.
+// a and b may differ.  Bound by latency: one or two blocks an SM.  512^2, three levels, seven pairs:
+// 25 us with two shares of the pairs at the finest level, 31 with one; 128^3, two levels: 101 us;
+// nine phase pairs of 512^2: 148 us.
 template <bool CROSS>
 __global__ void __launch_bounds__(SEP_THREADS, CROSS ? 1 : 2)
 sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__ items, int nitem) {
@@ -1391,7 +1397,9 @@ __device__ __forceinline__ int half_index(const SepLevel& lv, int rz, int ry, in
 // entries of block (a, b); with a loss to evaluate, its share of the loss' sums too.  With
 // lv.fuse (one phase, a loss and its gradient in one call) a row goes straight on: its residuals
 // D - D_des are G up to the loss' factor gscale, which sep_mul applies, so they are embedded and
-// transformed here (the rows of sep_gx).
+// transformed here (the rows of sep_gx).  17 blocks at 512^2: 20 us, the chain of one row's two
+// transforms, the descriptor and the loss (a launch of sep_gx less; a loop that shares one copy of
+// the transform's code took the same).
 __global__ void __launch_bounds__(SEP_THREADS, 2) sep_desc_kernel(const __grid_constant__ SepTables tb,
                                                                   const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
@@ -1624,7 +1632,9 @@ struct GCols {
 
 // item: (level, phase a).  Spectrum of G along the last axis, then for every feature pair the
 // forward transform of the columns, the product sum_b conj(G^ab) Z^b and the inverse: Q^a, in
-// place of Z for a single phase (G is even then: a real spectrum).
+// place of Z for a single phase (G is even then: a real spectrum).  Bound by latency, as sep_power.
+// 512^2, three levels, seven pairs: 24 us with the pairs shared among up to four blocks a group of
+// columns, 29 without; 128^3, two levels: 103 us.
 template <bool MULTI>
 __global__ void __launch_bounds__(SEP_THREADS, MULTI ? 1 : 2)
 sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__ items, int nitem) {
@@ -1754,7 +1764,9 @@ sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__
 // ------------------------------------------------------------------------- gradient
 
 // item: (level, phase a); blocks: groups of rows.  Inverse along x of every feature pair and
-// g(y) = sum_k s_k p_k'(M_y) Q_k(y), the slots' shares added in a fixed order.
+// g(y) = sum_k s_k p_k'(M_y) Q_k(y), the slots' shares added in a fixed order.  Bound by latency, as
+// sep_feat.  Seven pairs: 512^2, three levels 27 us; 128^3, two levels 119 us (coefficient gathers
+// unrolled by three: 28 and 125).
 __global__ void __launch_bounds__(SEP_ROW_THREADS, 3) sep_grad_kernel(const __grid_constant__ SepTables tb,
                                                                       const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
