@@ -12,7 +12,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(PKG, "libdmcr.so")
 BUILD_DIR = os.path.join(PKG, "_build")
-SOURCES = ["corr.cu", "sep.cu", "aux.cu", "fft.cu", "gram.cu", "api.cu"]
+SOURCES = ["corr.cu", "sep.cu", "sep_basis.cpp", "aux.cu", "fft.cu", "gram.cu", "api.cu"]
 # the benchmark's pipe-rate microbenchmark: a library of its own, not part of the C ABI
 PIPES_SRC = "pipes.cu"
 PIPES_LIB = os.path.join(PKG, "libdmcr_pipes.so")
@@ -55,7 +55,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     cmd = [nvcc, *ARCH, *NVCC_FLAGS, "-c", os.path.join(CSRC, PIPES_SRC), "-o", pipes_obj]
     procs.append((cmd, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)))
     for src in SOURCES:
-        obj = os.path.join(BUILD_DIR, src.replace(".cu", ".o"))
+        obj = os.path.join(BUILD_DIR, os.path.splitext(src)[0] + ".o")
         objs.append(obj)
         cmd = [nvcc, *ARCH, *NVCC_FLAGS, "-c", os.path.join(CSRC, src), "-o", obj]
         if verbose:

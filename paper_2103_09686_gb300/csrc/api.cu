@@ -156,7 +156,8 @@ struct Plan {
     std::shared_ptr<const SepBasis> basis;
     int sep_tiers = 0, sep_pairs = 0;   // tiers worth running, feature pairs of the widest of them
     size_t o_tier = 0, o_tiers = 0, o_z[MAX_LEVELS] = {}, o_q[MAX_LEVELS] = {}, o_u[MAX_LEVELS] = {},
-           o_v[MAX_LEVELS] = {}, o_sdc[MAX_LEVELS] = {}, o_spart[MAX_LEVELS] = {};
+           o_v[MAX_LEVELS] = {}, o_sdc[MAX_LEVELS] = {}, o_spart[MAX_LEVELS] = {}, o_phi[MAX_LEVELS] = {},
+           o_gsum[MAX_LEVELS] = {}, o_msum = 0, o_center = 0;
     // block sums of the loss, left by the descriptor kernels (two-point descriptor without FFT levels)
     bool sums = false;
     size_t o_excess = 0, o_sums = 0;
@@ -218,7 +219,7 @@ int64_t fft_v_len(const FftArgs& a) {
 size_t table_bound(const Plan& pl) {
     const int levels = pl.levels, phases = pl.phases;
     const size_t pp = (size_t)phases * phases;
-    const size_t sep = !pl.sep ? 0 : 16 + pl.basis->coef.size() * sizeof(float2) +
+    const size_t sep = !pl.sep ? 0 : 16 + pl.basis->coef.size() * sizeof(SepCoef) +
                                          (size_t)levels * (sizeof(SepLevel) + (size_t)SEP_KERNELS * pp * sizeof(SepItem));
     return sep + (size_t)levels *
                (pp * (sizeof(FwdSeg) + sizeof(RedSeg) + sizeof(GSeg) + sizeof(AdjSeg)) +
@@ -339,6 +340,13 @@ void plan_level(LevelGeom& g, const int tune[4], int phases, int level) {
 int64_t sep_u_len(const LevelGeom& g) { return g.n[0] > 1 ? (int64_t)(g.P[0] + 1) * g.n[1] * g.n[2] : 0; }
 int64_t sep_v_rows(const LevelGeom& g) {
     return g.n[0] > 1 ? (int64_t)(g.P[0] + 1) * (2 * g.P[1] + 1) : g.P[1] + 1;
+}
+
+// blocks of sep_feat and sep_grad, one phase
+int64_t sep_feature_blocks(const LevelGeom& g) {
+    SepAxis ax;
+    sep_axis(g.n[2], ax);
+    return ceil_div(g.n[0] * g.n[1], sep_feature_rows(ax, g.n[0] * g.n[1]));
 }
 
 // shape of one level for sep.cu (no pointers)
@@ -608,6 +616,8 @@ dmcr_status make_plan(const dmcr_params* p, Plan& pl) {
     if (pl.sep) {
         pl.o_tier = o; o = align_up(o + sizeof(int));
         pl.o_tiers = o; o = align_up(o + PREP_BLOCKS * sizeof(int));
+        pl.o_msum = o; o = align_up(o + (size_t)PREP_BLOCKS * pl.phases * sizeof(float));
+        pl.o_center = o; o = align_up(o + (size_t)pl.phases * sizeof(float));
         std::vector<PairShare> power;
         for (int l = 0; l < pl.levels; ++l) {
             SepLevel lv;
@@ -661,11 +671,13 @@ dmcr_status make_plan(const dmcr_params* p, Plan& pl) {
             pl.o_gl[l] = o; o = align_up(o + Kp * Kp * sizeof(uint16_t));
             pl.o_amax[l] = o; o = align_up(o + 2 * sizeof(float));
         } else if (pl.sep) {
-            // gradient of the level and window means, then the buffers of the path that runs:
+            // gradient of the level, window means and sums, then the buffers of the path that runs:
             // spectra (separable) or partials (direct, for fields outside the separable ranges) -- a call uses one of the two
             const size_t pp = ph * ph;
             pl.o_spart[l] = o; o = align_up(o + ph * g.N * sizeof(float));
             pl.o_sdc[l] = o; o = align_up(o + pp * pl.sep_parts[l] * sizeof(float2));
+            pl.o_phi[l] = o; o = align_up(o + pp * sep_feature_blocks(g) * (SEP_ROW_THREADS / 32) * sizeof(float));
+            pl.o_gsum[l] = o; o = align_up(o + pp * sizeof(float));
             const size_t start = o;
             pl.o_z[l] = o; o = align_up(o + ph * pl.sep_pairs * g.N * sizeof(float2));
             pl.o_q[l] = pl.o_z[l];
@@ -941,6 +953,13 @@ void prepare_sep(const std::vector<Inst>& in, unsigned flags, const std::vector<
             lv.U = reinterpret_cast<float2*>(x.ws + pl.o_u[l]);
             lv.V = reinterpret_cast<float2*>(x.ws + pl.o_v[l]);
             lv.dc = reinterpret_cast<float2*>(x.ws + pl.o_sdc[l]);
+            if (flags & F_FWD) lv.phi = reinterpret_cast<float*>(x.ws + pl.o_phi[l]);
+            const int64_t fgroups = sep_feature_blocks(g);
+            lv.nphi = (int)fgroups * (SEP_ROW_THREADS / 32);
+            lv.gsum = reinterpret_cast<float*>(x.ws + pl.o_gsum[l]);
+            lv.msum = reinterpret_cast<const float*>(x.ws + pl.o_msum);
+            lv.center = reinterpret_cast<float*>(x.ws + pl.o_center);
+            lv.invN1 = (float)(1.0 / (double)pl.N1);
             lv.tier = reinterpret_cast<int*>(x.ws + pl.o_tier);
             lv.tiers = reinterpret_cast<int*>(x.ws + pl.o_tiers);
             lv.ntiers = prep_blocks(pl);
@@ -968,8 +987,6 @@ void prepare_sep(const std::vector<Inst>& in, unsigned flags, const std::vector<
             lv.done = lv_done = x.use_done ? &x.sc->done : nullptr;
             lv_tier = lv.tier;
             const bool d3 = lv.n0 > 1;
-            const int64_t rows = (int64_t)lv.n0 * lv.n1;
-            const int64_t fgroups = ceil_div(rows, lv.rowsF);
             const int64_t xl = ceil_div(lv.n2, lv.colsL), xy = ceil_div(lv.n2, lv.colsY);
             const int64_t last = d3 ? xl * lv.n1 : xl;
             // planes of the middle axis side by side in one block
@@ -1013,6 +1030,9 @@ void prepare_sep(const std::vector<Inst>& in, unsigned flags, const std::vector<
     const float2* coef = sep_device_coef(*basis);
     if (coef == nullptr) P.o_sep_coef = push(P.tb, basis->coef);
     for (int t = 0; t < SEP_TIERS; ++t) P.sept.tier[t] = basis->tier[t];
+    P.sept.alpha = P.tc.alpha;
+    P.sept.c1 = P.tc.c1;
+    P.sept.c3 = P.tc.c3;
     P.sept.level = P.at<SepLevel>(P.o_sep_level);
     P.sept.coef = coef != nullptr ? coef : P.at<float2>(P.o_sep_coef);
     for (int k = 0; k < SEP_KERNELS; ++k) {
@@ -1106,6 +1126,7 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
             for (int l = 0; l < p.coarse; ++l) p.lv[l] = const_cast<float*>(x.lv[l + 1]);
             if (pl.sep) {
                 p.tiers = reinterpret_cast<int*>(x.ws + pl.o_tiers);
+                p.sums = reinterpret_cast<float*>(x.ws + pl.o_msum);
                 p.ntier = pl.sep_tiers;
                 for (int t = 0; t < pl.sep_tiers; ++t) p.lo[t] = pl.basis->tier[t].lo, p.hi[t] = pl.basis->tier[t].hi;
                 if ((flags & F_LOSS) && pl.sums && x.lp.bc_on) p.excess = reinterpret_cast<float4*>(x.ws + pl.o_excess);

@@ -48,19 +48,30 @@ __global__ void restrict_kernel(const RestrictSeg* __restrict__ segs, int nseg) 
 
 // All coarser levels of a tile in one pass over the finest field (each the mean of its 2^d
 // children, summed as restrict_one does), with the tier of the values' range and the box
-// excess, which need the same pass.  A thread reads a 2^d block; the coarser means go through
+// excess, which need the same pass (and the phases that are bright enough for the transforms).  A thread reads a 2^d block; the coarser means go through
 // shared memory.  One launch of a microsecond or two instead of one per level.
 template <int ND>
 __device__ __forceinline__ void prep_tiles(const PrepSeg& sg, int blk, float* sh, float& lo, float& hi, int& bad,
-                                           float& e2, float& e2c) {
+                                           int& bright, float* msh, float& e2, float& e2c) {
     constexpr int TILE = ND == 2 ? PREP_TILE2 : PREP_TILE3, H = TILE / 2;
     constexpr int CELLS = ND == 2 ? H * H : H * H * H;        // level-2 cells of a tile
     const int n0 = sg.n[0], n1 = sg.n[1], n2 = sg.n[2];
     const int64_t N = (int64_t)n0 * n1 * n2;
     const int t0 = ND == 2 ? 1 : (n0 + TILE - 1) / TILE, t1 = (n1 + TILE - 1) / TILE, t2 = (n2 + TILE - 1) / TILE;
     const int64_t tiles = (int64_t)t0 * t1 * t2 * sg.phases;
-    auto see = [&](float v) {
+    // sum of the values of one phase: each warp its own share, msh[phase][warp]
+    float sum = 0.f;
+    int summed = 0;
+    auto flush = [&]() {
+        if (sg.tiers == nullptr) return;
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if ((threadIdx.x & 31) == 0) msh[summed * (ELEM_TH / 32) + (threadIdx.x >> 5)] += sum;
+        sum = 0.f;
+    };
+    auto see = [&](float v, int ph) {
+        sum += v;
         bad |= !(v == v);
+        bright |= (int)(v >= SEP_WEAK) << ph;
         lo = fminf(lo, v);
         hi = fmaxf(hi, v);
         const float ex = box_excess(v);
@@ -70,6 +81,10 @@ __device__ __forceinline__ void prep_tiles(const PrepSeg& sg, int blk, float* sh
         const int x0 = (int)(tile % t2) * TILE, y0 = (int)(tile / t2 % t1) * TILE;
         const int z0 = ND == 2 ? 0 : (int)(tile / ((int64_t)t2 * t1) % t0) * TILE;
         const int ph = (int)(tile / ((int64_t)t2 * t1 * t0));
+        if (ph != summed) {
+            flush();
+            summed = ph;
+        }
         const float* f = sg.field + ph * N;
         for (int c = threadIdx.x; c < CELLS; c += ELEM_TH) {
             const int cx = c % H, cy = c / H % H, cz = ND == 2 ? 0 : c / (H * H);
@@ -81,7 +96,7 @@ __device__ __forceinline__ void prep_tiles(const PrepSeg& sg, int blk, float* sh
                 v[k] = xx < n2 && yy < n1 && zz < n0 ? f[((int64_t)zz * n1 + yy) * n2 + xx] : 0.f;
             }
 #pragma unroll
-            for (int k = 0; k < (ND == 2 ? 4 : 8); ++k) see(v[k]);
+            for (int k = 0; k < (ND == 2 ? 4 : 8); ++k) see(v[k], ph);
             if (sg.coarse == 0) continue;
             float s;
             if constexpr (ND == 2) s = ((v[0] + v[1]) + (v[2] + v[3])) * 0.25f;
@@ -115,6 +130,7 @@ __device__ __forceinline__ void prep_tiles(const PrepSeg& sg, int blk, float* sh
         }
         __syncthreads();
     }
+    flush();
 }
 
 __global__ void __launch_bounds__(ELEM_TH) prep_kernel(const PrepSeg* __restrict__ segs, int nseg) {
@@ -125,12 +141,15 @@ __global__ void __launch_bounds__(ELEM_TH) prep_kernel(const PrepSeg* __restrict
     if (sg.done != nullptr && *sg.done) return;
     __shared__ float sh[640];        // 2-D: 256 + 64 + 16 + 4 + 1; 3-D: 512 + 64 + 8 + 1
     __shared__ DF dsh[32];
-    __shared__ int tsh[ELEM_TH / 32];
+    __shared__ int tsh[ELEM_TH / 32], bsh[ELEM_TH / 32];
     const int blk = (int)((int64_t)blockIdx.x - sg.blockStart);
     float lo = 0.f, hi = 0.f, e2 = 0.f, e2c = 0.f;
-    int bad = 0;
-    if (sg.ndim == 2) prep_tiles<2>(sg, blk, sh, lo, hi, bad, e2, e2c);
-    else prep_tiles<3>(sg, blk, sh, lo, hi, bad, e2, e2c);
+    int bad = 0, bright = 0;
+    __shared__ float msh[MAX_PHASES * (ELEM_TH / 32)];
+    if ((threadIdx.x & 31) == 0)
+        for (int ph = 0; ph < MAX_PHASES; ++ph) msh[ph * (ELEM_TH / 32) + (threadIdx.x >> 5)] = 0.f;
+    if (sg.ndim == 2) prep_tiles<2>(sg, blk, sh, lo, hi, bad, bright, msh, e2, e2c);
+    else prep_tiles<3>(sg, blk, sh, lo, hi, bad, bright, msh, e2, e2c);
     if (sg.excess != nullptr) {
         const DF E = block_sum_df(df_two_sum(e2, -e2c), dsh);
         if (threadIdx.x == 0) sg.excess[blk] = make_float4(E.hi, E.lo, 0.f, 0.f);
@@ -141,11 +160,17 @@ __global__ void __launch_bounds__(ELEM_TH) prep_kernel(const PrepSeg* __restrict
     while (t < sg.ntier && !(lo >= sg.lo[t] && hi <= sg.hi[t])) ++t;
     if (bad || t >= sg.ntier) t = SEP_TIERS;
     t = __reduce_max_sync(0xffffffffu, t);
-    if ((threadIdx.x & 31) == 0) tsh[threadIdx.x >> 5] = t;
+    bright = __reduce_or_sync(0xffffffffu, bright);
+    if ((threadIdx.x & 31) == 0) tsh[threadIdx.x >> 5] = t, bsh[threadIdx.x >> 5] = bright;
     __syncthreads();
+    if (threadIdx.x < sg.phases) {
+        float m = 0.f;
+        for (int w = 0; w < ELEM_TH / 32; ++w) m += msh[threadIdx.x * (ELEM_TH / 32) + w];
+        sg.sums[blk * sg.phases + threadIdx.x] = m;
+    }
     if (threadIdx.x == 0) {
-        for (int w = 1; w < ELEM_TH / 32; ++w) t = max(t, tsh[w]);
-        sg.tiers[blk] = t;
+        for (int w = 1; w < ELEM_TH / 32; ++w) t = max(t, tsh[w]), bright |= bsh[w];
+        sg.tiers[blk] = t | bright << 8;
     }
 }
 

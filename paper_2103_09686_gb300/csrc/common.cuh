@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "scalars.h"
+#include "sep_basis.h"
 
 namespace dmcr {
 
@@ -274,7 +275,9 @@ struct PrepSeg {
     int n[3];                    // finest sizes (3-D embedded)
     const float* field;
     float* lv[PREP_LEVELS2];     // level 2, 3, ... (phases stacked)
-    int* tiers;                  // separable path: one tier per block, null otherwise
+    int* tiers;                  // separable path: one word per block, null otherwise: its tier, and from bit 8
+                                 // on one bit per phase that shows a value of at least SEP_WEAK
+    float* sums;                 // separable path: sum of the block's values, [block][phase]
     int ntier;
     float lo[8], hi[8];          // its ranges
     float4* excess;              // box excess: sum of squares per block (hi, lo), null: not wanted
@@ -349,15 +352,11 @@ struct FftArgs {
 };
 
 // ---------------------------------------------------------------- separable path (sep.cu)
-constexpr int SEP_TIERS = 6;        // value ranges with a basis of their own; tier SEP_TIERS: direct kernels
-constexpr int SEP_MAX_PAIRS = 28;   // packed pairs of features of one basis at most
 constexpr int SEP_THREADS = 512;    // threads of the transform kernels
 constexpr int SEP_BLOCK_PTS = 8 * SEP_THREADS;   // points a block holds in registers (power-of-two axes)
 constexpr int SEP_ROW_THREADS = 256;   // threads of the feature and gradient kernels
 constexpr int SEP_SLOTS = 8;        // feature pairs a row block holds side by side at most
 constexpr int SEP_FAST_PHASES = 3;  // phases whose spectra fit behind the line buffers of sep_mul
-constexpr int SEP_SEG = 8;          // segments of the value range per unit
-constexpr int SEP_MAX_NC = 14;      // coefficients of a feature in one segment at most
 constexpr int SEP_MAX_N = 2048;     // longest axis
 constexpr int64_t SEP_MAX_POINTS = 1 << 28;   // points of one grid (32-bit offsets)
 constexpr int SEP_MAX_RAD = 12;
@@ -378,20 +377,6 @@ __host__ __device__ inline int sep_pitch(int n, int L) {
     return p + ((want - p) % 16 + 16) % 16;
 }
 
-struct SepTier {
-    float lo, hi;
-    int seg0, nseg, nc;       // first segment, segments, coefficients per segment
-    int npair, npos;          // packed pairs of features, the first npos of them with s = +1
-    int coef;                 // offset of this tier's coefficients
-};
-
-struct SepBasis {
-    float alpha = 0.f;
-    int ntier = 0;
-    SepTier tier[SEP_TIERS] = {};
-    std::vector<float2> coef;
-};
-
 // one (instance, level)
 struct SepLevel {
     int n0, n1, n2;
@@ -405,7 +390,13 @@ struct SepLevel {
     float2 *U, *V;            // window spectra (3-D: [r0][y][x]; [row][x]), one per ordered phase pair
     int64_t strideU, strideV;
     float2* dc;               // scaleD sum_k s_k conj(Z^a_k(0)) Z^b_k(0) per phase pair (hi, lo)
-    int* tiers;               // tiers of the range blocks
+    const float* msum;        // PrepSeg.sums: [range block][phase]
+    float invN1;              // 1 / points of the finest level
+    float* center;            // per phase, the value that the features vanish at (sep_feat)
+    float* phi;               // sums of F(M^a, center_b) by the warps of sep_feat, nphi per phase pair; null: not wanted
+    int nphi;
+    float* gsum;              // sum of G over the window, one per phase pair
+    int* tiers;               // tiers of the range blocks (PrepSeg.tiers)
     int ntiers;
     int* tier;                // the instance's tier
     int first;                // finest level: writes *tier
@@ -439,6 +430,7 @@ struct SepTables {
     const SepLevel* level;
     const float2* coef;
     SepTier tier[SEP_TIERS];
+    float alpha, c1, c3;      // of the threshold (ThreshConst)
 };
 
 enum SepKernel {
@@ -446,7 +438,6 @@ enum SepKernel {
     SEP_GRAD, SEP_KERNELS
 };
 
-std::shared_ptr<const SepBasis> sep_basis(float alpha);
 const float2* sep_device_coef(const SepBasis& b);
 bool sep_axis(int64_t n, SepAxis& ax);
 double sep_axis_cost(const SepAxis& ax);

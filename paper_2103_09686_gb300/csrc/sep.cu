@@ -2,32 +2,35 @@
 // (sm_103a).  Paper: arXiv 2103.09686, Sec. 3.2.2-3.2.4 and the gradient of Sec. 3.1/3.3.
 //
 // The pair function F(u, v) = f((u + v) / 2)^2 is smooth on the bounded range of a relaxed
-// field, so its integral operator has rapidly decaying eigenvalues:
-//     F(u, v) = sum_k s_k p_k(u) p_k(v),  s_k = +-1,  p_k polynomials,
-// with 16 terms to 1e-10 on [-1/16, 17/16] at alpha = 10 (SepBasis, built on the host in
-// FP64).  The descriptor is then a sum of autocorrelations of R feature fields p_k(M), and the
-// gradient a sum of convolutions of the same features with the window coefficients G:
-//     S(r) = (1/N) sum_k s_k sum_x p_k(M_x) p_k(M_{x+r}),
-//     g(y) = sum_k s_k p_k'(M_y) sum_r G(r) p_k(M_{y+r}).
+// field, so around a value c it is, to FP32 accuracy, a short sum over features that vanish at c:
+//     F(u, v) = F(u, c) + F(c, v) - F(c, c) + sum_k s_k q_k(u) q_k(v),  s_k = +-1,
+//     q_k(u) = p_k(u) - p_k(c), p_k piecewise polynomials (sep_basis.cpp, built on the host in FP64),
+// 14 terms on [-1/16, 17/16] at alpha = 10.  c is the mean of the field, or 0 for a field whose
+// mean lies near 0: what most pairs of a field consist of is then evaluated directly, not as a
+// difference of features rounded to FP32.  The descriptor is a mean and a sum of autocorrelations of
+// R feature fields, and the gradient a sum of convolutions of the same features with the window
+// coefficients G:
+//     S(r) = (2/N) sum_x F(M_x, c) - F(c, c) + (1/N) sum_k s_k sum_x q_k(M_x) q_k(M_{x+r}),
+//     g(y) = F_u(M_y, c) sum_r G(r) + sum_k s_k p_k'(M_y) sum_r G(r) q_k(M_{y+r}).
+// (Several phases: a value each, F(M^a, c_b) and F(c_a, M^b).)
 // Both are diagonal in Fourier space: the work per position falls from the window's K pair
 // evaluations (8321 at +-64) to R transforms (5 R log2 N operations).  Features of equal sign
 // are packed in pairs, z = p_1 + i p_2: Re IDFT(|Z|^2) = autocorr(p_1) + autocorr(p_2), and a
 // real even G acts on both parts at once, so no mirrored frequency is ever read.
 //
 //   prep_kernel (aux.cu) the tier (basis) that covers the field's values; none: the direct kernels run
-//   sep_feat    features of whole rows + transform along x             -> Z
+//   sep_feat    features of whole rows + transform along x             -> Z; sums of F(M, c)
 //   sep_fft_y   3-D: transform along y, in place
 //   sep_power   last axis: transform, sum_k s_k conj(Z^a_k) Z^b_k, inverse along the same
-//               axis, cropped to the window
+//               axis, cropped to the window; the mean of F(M, c) joins the frequency 0
 //   sep_inv_y   3-D: inverse along y, cropped to the window
 //   sep_desc    inverse along x, cropped to the window: the descriptor
 //   sep_gx/gy   the window's coefficients G embedded and transformed along x (and y)
-//   sep_mul     last axis: transform of G, then per feature pair transform, product, inverse
-//   sep_grad    inverse along x and sum_k s_k p_k'(M_y) Q_k(y): the gradient of the level
+//   sep_mul     last axis: transform of G, then per feature pair transform, product, inverse; sum of G
+//   sep_grad    inverse along x, sum_k s_k p_k'(M_y) Q_k(y) and the term of F_u(M, c): the gradient
 //
-// The frequency 0 carries the means, which are orders of magnitude above the fluctuations:
-// its power is summed in FP64 and added after the inverse transform, so the FP32 transforms
-// only carry fluctuations.  Fixed grids and orders: results are bitwise reproducible.
+// The power of the frequency 0, the features' means, is summed in FP64 with the mean of F(M, c) and
+// added after the inverse transform, so the FP32 transforms only carry fluctuations.  Fixed grids and orders: results are bitwise reproducible.
 #include <math.h>
 
 #include <algorithm>
@@ -40,289 +43,14 @@
 
 namespace dmcr {
 
-// ------------------------------------------------------------------------- basis (host)
-
-namespace {
-
-struct PairFn {
-    double a, c1, c3;
-    explicit PairFn(double alpha) : a(alpha) {
-        const double s0 = 1.0 / (1.0 + exp(0.75 * a)), s1 = 1.0 / (1.0 + exp(-0.25 * a));
-        c1 = 1.0 / (s1 - s0);
-        c3 = -c1 * s0;
-    }
-    double f(double t) const { return c1 / (1.0 + exp(-a * (0.5 * t - 0.75))) + c3; }
-    double F(double t) const { const double v = f(t); return v * v; }          // t = u + v
-    double Fu(double t) const {
-        const double s = 1.0 / (1.0 + exp(-a * (0.5 * t - 0.75)));
-        return (c1 * s + c3) * c1 * a * s * (1.0 - s);
-    }
-};
-
-// Symmetric eigenproblem by cyclic Jacobi rotations (Golub & Van Loan, Matrix Computations,
-// Sec. 8.5): A (n x n) becomes diagonal, V holds the eigenvectors in its columns.
-void jacobi_eigen(std::vector<double>& A, std::vector<double>& V, int n) {
-    V.assign((size_t)n * n, 0.0);
-    for (int i = 0; i < n; ++i) V[(size_t)i * n + i] = 1.0;
-    for (int sweep = 0; sweep < 30; ++sweep) {
-        double off = 0.0, dia = 0.0;
-        for (int i = 0; i < n; ++i)
-            for (int j = 0; j < n; ++j) (i == j ? dia : off) += A[(size_t)i * n + j] * A[(size_t)i * n + j];
-        if (off <= 1e-30 * dia) break;
-        for (int p = 0; p < n; ++p)
-            for (int q = p + 1; q < n; ++q) {
-                const double apq = A[(size_t)p * n + q];
-                if (apq == 0.0) continue;
-                const double th = (A[(size_t)q * n + q] - A[(size_t)p * n + p]) / (2.0 * apq);
-                const double t = (th >= 0 ? 1.0 : -1.0) / (fabs(th) + sqrt(th * th + 1.0));
-                const double c = 1.0 / sqrt(t * t + 1.0), s = t * c;
-                for (int k = 0; k < n; ++k) {
-                    const double x = A[(size_t)k * n + p], y = A[(size_t)k * n + q];
-                    A[(size_t)k * n + p] = c * x - s * y;
-                    A[(size_t)k * n + q] = s * x + c * y;
-                }
-                for (int k = 0; k < n; ++k) {
-                    const double x = A[(size_t)p * n + k], y = A[(size_t)q * n + k];
-                    A[(size_t)p * n + k] = c * x - s * y;
-                    A[(size_t)q * n + k] = s * x + c * y;
-                }
-                for (int k = 0; k < n; ++k) {
-                    const double x = V[(size_t)k * n + p], y = V[(size_t)k * n + q];
-                    V[(size_t)k * n + p] = c * x - s * y;
-                    V[(size_t)k * n + q] = s * x + c * y;
-                }
-            }
-    }
-}
-
-// One tier: eigenfunctions of F on the range of the segments k0 .. k1 (segment k holds the
-// values within half a segment of k / SEP_SEG), discretised at Chebyshev nodes, as one short
-// polynomial per segment.  False when SEP_MAX_PAIRS packed pairs, or polynomials of SEP_MAX_NC
-// coefficients, do not reach the tolerances (largest error of F and of dF/du over the range).
-bool build_tier(const PairFn& fn, int k0, int k1, double tolF, double tolFu, SepTier& t,
-                std::vector<float2>& coef) {
-    const double lo = (k0 - 0.5) / SEP_SEG, hi = (k1 + 0.5) / SEP_SEG;
-    const double mid = 0.5 * (lo + hi), half = 0.5 * (hi - lo);
-    // nodes: the degree grows with the range measured in widths of the sigmoid
-    const int n = (int)std::min(160.0, std::max(48.0, 24.0 + 2.6 * (hi - lo) * fn.a));
-    std::vector<double> ct(4 * n);                       // cos(pi m / (2 n))
-    for (int m = 0; m < 4 * n; ++m) ct[m] = cos(M_PI * m / (2 * n));
-    auto node = [&](int i) { return ct[2 * i + 1]; };
-    std::vector<double> A((size_t)n * n);
-    for (int i = 0; i < n; ++i)
-        for (int j = 0; j < n; ++j) A[(size_t)i * n + j] = fn.F(2.0 * mid + half * (node(i) + node(j))) / n;
-    // numerical range of A: Gram-Schmidt on its columns, largest residual first, each
-    // direction orthogonalised twice
-    const int rmax = std::min(n, 2 * SEP_MAX_PAIRS + 8);
-    std::vector<double> W(A), Q;                          // W: residual columns; Q: r rows of length n
-    int r = 0;
-    double first = 0.0;
-    for (; r < rmax; ++r) {
-        int best = 0;
-        double bestn = -1.0;
-        for (int j = 0; j < n; ++j) {
-            double s = 0.0;
-            for (int i = 0; i < n; ++i) s += W[(size_t)i * n + j] * W[(size_t)i * n + j];
-            if (s > bestn) bestn = s, best = j;
-        }
-        if (r == 0) first = bestn;
-        if (!(bestn > 1e-28 * first)) break;
-        std::vector<double> q(n);
-        for (int i = 0; i < n; ++i) q[i] = W[(size_t)i * n + best];
-        for (int k = 0; k < r; ++k) {
-            double d = 0.0;
-            for (int i = 0; i < n; ++i) d += q[i] * Q[(size_t)k * n + i];
-            for (int i = 0; i < n; ++i) q[i] -= d * Q[(size_t)k * n + i];
-        }
-        double nn = 0.0;
-        for (double v : q) nn += v * v;
-        nn = 1.0 / sqrt(nn);
-        for (double& v : q) v *= nn;
-        for (int j = 0; j < n; ++j) {
-            double d = 0.0;
-            for (int i = 0; i < n; ++i) d += q[i] * W[(size_t)i * n + j];
-            for (int i = 0; i < n; ++i) W[(size_t)i * n + j] -= d * q[i];
-        }
-        Q.insert(Q.end(), q.begin(), q.end());
-    }
-    // A restricted to it, and its eigenvectors
-    std::vector<double> AQ((size_t)r * n), B((size_t)r * r), V;
-    for (int k = 0; k < r; ++k)
-        for (int i = 0; i < n; ++i) {
-            double s = 0.0;
-            for (int j = 0; j < n; ++j) s += A[(size_t)i * n + j] * Q[(size_t)k * n + j];
-            AQ[(size_t)k * n + i] = s;
-        }
-    for (int k = 0; k < r; ++k)
-        for (int m = 0; m < r; ++m) {
-            double s = 0.0;
-            for (int i = 0; i < n; ++i) s += Q[(size_t)m * n + i] * AQ[(size_t)k * n + i];
-            B[(size_t)k * r + m] = s;
-        }
-    for (int k = 0; k < r; ++k)
-        for (int m = 0; m < k; ++m)
-            B[(size_t)k * r + m] = B[(size_t)m * r + k] = 0.5 * (B[(size_t)k * r + m] + B[(size_t)m * r + k]);
-    jacobi_eigen(B, V, r);
-    std::vector<int> ord(r);
-    for (int i = 0; i < r; ++i) ord[i] = i;
-    std::stable_sort(ord.begin(), ord.end(),
-                     [&](int a, int b) { return fabs(B[(size_t)a * r + a]) > fabs(B[(size_t)b * r + b]); });
-    // Chebyshev coefficients of sqrt(|lambda_k| n) v_k
-    auto series = [&](int k) {
-        std::vector<double> v(n, 0.0), c(n);
-        for (int m = 0; m < r; ++m)
-            for (int i = 0; i < n; ++i) v[i] += V[(size_t)m * r + ord[k]] * Q[(size_t)m * n + i];
-        const double sc = sqrt(fabs(B[(size_t)ord[k] * r + ord[k]]) * n);
-        for (int j = 0; j < n; ++j) {
-            double s = 0.0;
-            for (int i = 0; i < n; ++i) s += v[i] * ct[(int)((int64_t)j * (2 * i + 1) % (4 * n))];
-            c[j] = s * sc * (j == 0 ? 1.0 : 2.0) / n;
-        }
-        return c;
-    };
-    constexpr int GRID = 97;
-    std::vector<double> E((size_t)GRID * GRID), D((size_t)GRID * GRID);
-    auto gx = [&](int i) { return -1.0 + 2.0 * i / (GRID - 1); };
-    for (int i = 0; i < GRID; ++i)
-        for (int j = 0; j < GRID; ++j) {
-            const double tt = 2.0 * mid + half * (gx(i) + gx(j));
-            E[(size_t)i * GRID + j] = fn.F(tt);
-            D[(size_t)i * GRID + j] = fn.Fu(tt);
-        }
-    std::vector<std::vector<double>> pos, neg;
-    bool ok = false;
-    for (int k = 0; k < r; ++k) {
-        const bool plus = B[(size_t)ord[k] * r + ord[k]] > 0.0;
-        std::vector<std::vector<double>>& side = plus ? pos : neg;
-        // once accurate, further terms are taken only while they fill a half-empty pair
-        if (ok && side.size() % 2 == 0) break;
-        if ((int)((pos.size() + 1) / 2 + (neg.size() + 1) / 2) + (side.size() % 2 == 0) > SEP_MAX_PAIRS) break;
-        const std::vector<double> c = series(k);
-        side.push_back(c);
-        std::vector<double> p(GRID), dp(GRID);
-        for (int i = 0; i < GRID; ++i) {
-            const double xx = gx(i);
-            double T0 = 1.0, T1 = xx, U0 = 1.0, U1 = 2.0 * xx, s = c[0] + c[1] * xx, d = c[1];
-            for (int j = 2; j < n; ++j) {
-                const double T2 = 2.0 * xx * T1 - T0;
-                s += c[j] * T2;
-                d += c[j] * j * U1;          // T_j' = j U_{j-1}
-                T0 = T1, T1 = T2;
-                const double U2 = 2.0 * xx * U1 - U0;
-                U0 = U1, U1 = U2;
-            }
-            p[i] = s;
-            dp[i] = d / half;
-        }
-        double eF = 0.0, eD = 0.0;
-        for (int i = 0; i < GRID; ++i)
-            for (int j = 0; j < GRID; ++j) {
-                E[(size_t)i * GRID + j] -= (plus ? 1.0 : -1.0) * p[i] * p[j];
-                D[(size_t)i * GRID + j] -= (plus ? 1.0 : -1.0) * dp[i] * p[j];
-                eF = std::max(eF, fabs(E[(size_t)i * GRID + j]));
-                eD = std::max(eD, fabs(D[(size_t)i * GRID + j]));
-            }
-        if (eF < tolF && eD < tolFu) ok = true;
-    }
-    if (!ok) return false;
-    // local polynomials in u = SEP_SEG M - k, |u| <= 1/2: interpolation at SEP_MAX_NC + 4
-    // Chebyshev points, cut where the rest is below the rounding of the largest terms
-    constexpr int m = SEP_MAX_NC + 4;
-    const int nseg = k1 - k0 + 1, npos = (int)(pos.size() + 1) / 2, npair = npos + (int)(neg.size() + 1) / 2;
-    std::vector<double> local((size_t)2 * npair * nseg * m, 0.0);       // [feature][segment][power]
-    int nc = 4;
-    for (int side = 0; side < 2; ++side)
-        for (size_t k = 0; k < (side ? neg : pos).size(); ++k) {
-            const std::vector<double>& c = (side ? neg : pos)[k];
-            const size_t feature = (side ? 2 * npos : 0) + k;
-            for (int sg = 0; sg < nseg; ++sg) {
-                double y[m], ch[m];
-                for (int i = 0; i < m; ++i) {
-                    const double M = (k0 + sg + 0.5 * cos((i + 0.5) * M_PI / m)) / SEP_SEG, xx = (M - mid) / half;
-                    double b1 = 0.0, b2 = 0.0;                          // Clenshaw
-                    for (int q = n - 1; q >= 1; --q) {
-                        const double b0 = c[q] + 2.0 * xx * b1 - b2;
-                        b2 = b1, b1 = b0;
-                    }
-                    y[i] = c[0] + xx * b1 - b2;
-                }
-                for (int q = 0; q < m; ++q) {
-                    double v = 0.0;
-                    for (int i = 0; i < m; ++i) v += y[i] * cos(q * (i + 0.5) * M_PI / m);
-                    ch[q] = v * (q == 0 ? 1.0 : 2.0) / m;
-                    if (q < SEP_MAX_NC + 1 && fabs(ch[q]) > 3e-9) nc = std::max(nc, q + 1);
-                }
-                if (nc > SEP_MAX_NC) return false;
-                // Chebyshev in 2 u to powers of u, terms up to nc of this and later features alike
-                std::vector<double> t0(m, 0.0), t1(m, 0.0), pw(m, 0.0);
-                t0[0] = 1.0;
-                t1[1] = 2.0;
-                for (int q = 0; q < SEP_MAX_NC; ++q) {
-                    if (fabs(ch[q]) > 1e-13)
-                        for (int e = 0; e <= q; ++e) pw[e] += ch[q] * t0[e];
-                    std::vector<double> t2(m, 0.0);
-                    for (int e = 0; e + 1 < m; ++e) t2[e + 1] += 4.0 * t1[e];
-                    for (int e = 0; e < m; ++e) t2[e] -= t0[e];
-                    t0 = t1, t1 = t2;
-                }
-                for (int e = 0; e < m; ++e) local[(feature * nseg + sg) * m + e] = pw[e];
-            }
-        }
-    t.lo = (float)lo;
-    t.hi = (float)hi;
-    t.seg0 = k0;
-    t.nseg = nseg;
-    t.nc = nc;
-    t.npos = npos;
-    t.npair = npair;
-    t.coef = (int)coef.size();
-    // coefficients [power][pair][segment] of the features (2p, 2p + 1)
-    for (int e = 0; e < nc; ++e)
-        for (int p = 0; p < npair; ++p)
-            for (int sg = 0; sg < nseg; ++sg)
-                coef.push_back(make_float2((float)local[((size_t)(2 * p) * nseg + sg) * m + e],
-                                           (float)local[((size_t)(2 * p + 1) * nseg + sg) * m + e]));
-    return true;
-}
-
-}  // namespace
-
-// The basis of one alpha.  The first range, [-1/16, 17/16], is a field between the phases with
-// the overshoot of an optimiser step or two; the penalty weakens as the loss falls, so fields of
-// long runs spread over the wider ones, up to [-2.3, 2.6] (measured over 3000 Adam steps:
-// [-1.7, 1.9]).  A wider range needs more features: 7 .. 25 packed pairs at alpha = 10.
-std::shared_ptr<const SepBasis> sep_basis(float alpha) {
-    static std::mutex mu;
-    static std::vector<std::shared_ptr<const SepBasis>>* cache = new std::vector<std::shared_ptr<const SepBasis>>();
-    constexpr size_t KEEP = 16;
-    std::lock_guard<std::mutex> lk(mu);
-    for (size_t i = 0; i < cache->size(); ++i)
-        if ((*cache)[i]->alpha == alpha) {
-            std::rotate(cache->begin(), cache->begin() + i, cache->begin() + i + 1);   // most recent first
-            return cache->front();
-        }
-    auto b = std::make_shared<SepBasis>();
-    b->alpha = alpha;
-    const PairFn fn((double)alpha);
-    const int ranges[SEP_TIERS][2] = {{0, 8}, {-2, 10}, {-4, 12}, {-8, 13}, {-12, 16}, {-18, 20}};   // segments
-    for (int t = 0; t < SEP_TIERS; ++t) {
-        // below the FP32 rounding of a pair's value and derivative
-        if (!build_tier(fn, ranges[t][0], ranges[t][1], t == 0 ? 1.5e-9 : 1e-8, 3e-7, b->tier[t],
-                        b->coef))
-            break;
-        b->ntier = t + 1;
-    }
-    cache->insert(cache->begin(), b);
-    if (cache->size() > KEEP) cache->pop_back();
-    return b;
-}
+// ------------------------------------------------------------------------- coefficients (host)
 
 // Coefficients in device memory: the first SEP_SLOTS_DEV alphas a process uses get a slot of a
 // static array, filled once per device by a synchronous copy on a stream of its own (also while
 // another stream is being captured); slots are never rewritten, so kernels and graphs may keep
 // reading them.  Null when there is no slot: the call uploads the coefficients with its tables.
 namespace {
-constexpr int SEP_SLOTS_DEV = 8, SEP_SLOT_LEN = 24576;
+constexpr int SEP_SLOTS_DEV = 8, SEP_SLOT_LEN = 32768;
 __device__ float2 g_sep_coef[SEP_SLOTS_DEV][SEP_SLOT_LEN];
 }  // namespace
 
@@ -355,7 +83,7 @@ const float2* sep_device_coef(const SepBasis& b) {
     bool ok = cudaGetSymbolAddress(&base, g_sep_coef) == cudaSuccess &&
               cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess;
     float2* dst = static_cast<float2*>(base) + (size_t)used * SEP_SLOT_LEN;
-    ok = ok && cudaMemcpyAsync(dst, b.coef.data(), b.coef.size() * sizeof(float2), cudaMemcpyHostToDevice, s) == cudaSuccess;
+    ok = ok && cudaMemcpyAsync(dst, b.coef.data(), b.coef.size() * sizeof(SepCoef), cudaMemcpyHostToDevice, s) == cudaSuccess;
     if (s) ok = cudaStreamSynchronize(s) == cudaSuccess && ok;
     if (s) cudaStreamDestroy(s);
     cudaThreadExchangeStreamCaptureMode(&mode);
@@ -850,6 +578,24 @@ __device__ __forceinline__ void eval_features(const float2* __restrict__ cf, int
     }
 }
 
+// F(M, c) and its derivative by M.  z = exp((alpha / 2)(1.5 - c - M)) is
+// wanted to 1e-7 of itself: c is a multiple of 2^-10, so 1.5 - c is exact, and the exponent keeps its
+// rounding errors.  (Beyond exp(80) f is its limit.)
+__device__ __forceinline__ float pair_with(const SepTables& tb, float M, float c, float& slope) {
+    const float h = 0.5f * tb.alpha;
+    const DF d = df_two_sum(1.5f - c, -M);
+    const float e = fminf(h * d.hi, 80.f), low = e < 80.f ? fmaf(h, d.lo, fmaf(h, d.hi, -e)) : 0.f;
+    float z = expf(e);
+    z = fmaf(z, low, z);
+    const float s = __fdividef(1.f, 1.f + z), f = fmaf(tb.c1, s, tb.c3);       // 1 + z < 2^126
+    slope = f * (tb.c1 * tb.alpha * s) * (z * s);
+    return f * f;
+}
+__device__ __forceinline__ float pair_with(const SepTables& tb, float M, float c) {
+    float slope;
+    return pair_with(tb, M, c, slope);
+}
+
 // rows of a block of the feature and gradient kernels: SLOTS feature pairs side by side
 template <int N>
 struct RowShape {
@@ -873,28 +619,53 @@ __device__ __forceinline__ Line<N> row_line(float2* sm, int line, int t, int lin
 }  // namespace
 
 // item: (level, phase a); blocks: groups of rows.  Features of whole rows and their transform
-// along x.  Every block combines the range blocks' tiers; the first block of the finest
-// level leaves the result for the later kernels.  Bound by latency (coefficient gathers from L1,
-// exchanges): it issues 35 % of the time.  Seven pairs: 512^2, three levels 24 us; 1024^2, five
-// levels 79 us; 128^3, two levels 89 us (one series over the whole range instead of local
-// polynomials: twice the instructions).
+// along x, and the warps' sums of F(M, c).  Every block combines the range blocks' tiers and sums;
+// the first block of the finest level leaves the tier and c for the later kernels.  Bound by
+// latency (coefficient gathers from L1, exchanges): it issues 35 % of the time.  Seven pairs:
+// 512^2, three levels 27 us; 1024^2, five levels 86 us; 128^3, two levels 97 us, 8 % of it for the
+// features' offsets and F(M, c) (one series over the whole range instead of local polynomials:
+// twice the instructions).
 __global__ void __launch_bounds__(SEP_ROW_THREADS, 4) sep_feat_kernel(const __grid_constant__ SepTables tb,
                                                                       const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
-    __shared__ int tsh[SEP_ROW_THREADS / 32];
+    constexpr int NW = SEP_ROW_THREADS / 32;
+    __shared__ int tsh[NW], bsh[NW];
+    __shared__ float csh[MAX_PHASES][NW];
+    __shared__ float2 offset[SEP_MAX_PAIRS];      // p_k(c)
     if (!enter<false>(tb, items, nitem, bk, sep_smem, axis_x)) return;
     const SepLevel& lv = bk.lv;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     {
-        int t = 0;
-        for (int i = threadIdx.x; i < lv.ntiers; i += blockDim.x) t = max(t, lv.tiers[i]);
+        int t = 0, bright = 0;
+        for (int i = threadIdx.x; i < lv.ntiers; i += blockDim.x) {
+            t = max(t, lv.tiers[i] & 0xff);
+            bright |= lv.tiers[i] >> 8;
+        }
+        for (int ph = 0; ph < lv.phases; ++ph) {
+            float m = 0.f;
+            for (int i = threadIdx.x; i < lv.ntiers; i += blockDim.x) m += lv.msum[i * lv.phases + ph];
+            for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+            if (lane == 0) csh[ph][warp] = m;
+        }
         t = __reduce_max_sync(0xffffffffu, t);
-        if ((threadIdx.x & 31) == 0) tsh[threadIdx.x >> 5] = t;
+        bright = __reduce_or_sync(0xffffffffu, bright);
+        if (lane == 0) tsh[warp] = t, bsh[warp] = bright;
     }
     float2* sm = sep_smem;
     const int rowsN = lv.n0 * lv.n1, n = lv.n2;
     __syncthreads();
-    int tier = tsh[0];
-    for (int i = 1; i < SEP_ROW_THREADS / 32; ++i) tier = max(tier, tsh[i]);
+    int tier = tsh[0], bright = bsh[0];
+    for (int i = 1; i < NW; ++i) tier = max(tier, tsh[i]), bright |= bsh[i];
+    if (bright != (1 << lv.phases) - 1) tier = SEP_TIERS;      // a phase without a value of SEP_WEAK
+    // the values c: the means on a grid of 2^-10, 0 for those in the segment around 0 (where the
+    // features of the background are exactly 0 already)
+    auto center = [&](int ph) {
+        float m = 0.f;
+        for (int i = 0; i < NW; ++i) m += csh[ph][i];
+        m *= lv.invN1;
+        return m > 0.5f / SEP_SEG ? rintf(1024.f * m) * (1.f / 1024.f) : 0.f;
+    };
+    if (lv.first && bk.a == 0 && bk.block == 0 && threadIdx.x < lv.phases) lv.center[threadIdx.x] = center(threadIdx.x);
     if (lv.first && bk.a == 0 && bk.block == 0 && threadIdx.x == 0) *lv.tier = tier;
     if (tier >= SEP_TIERS) return;
     const SepTier& t = tb.tier[tier];
@@ -903,6 +674,25 @@ __global__ void __launch_bounds__(SEP_ROW_THREADS, 4) sep_feat_kernel(const __gr
     const int row0 = bk.block * lv.rowsF, rows = min(lv.rowsF, rowsN - row0);
     const float* __restrict__ field = lv.field + (int64_t)bk.a * lv.N + (int64_t)row0 * n;
     float2* __restrict__ Z = lv.Z + (int64_t)bk.a * lv.maxPairs * lv.N + (int64_t)row0 * n;
+    const float own = center(bk.a);
+    if (threadIdx.x < t.npair) {
+        const float x[1] = {own};
+        float u[1];
+        int seg[1];
+        float2 f[1];
+        locate<1>(t, x, seg, u);
+        eval_features<false, 1>(cf + threadIdx.x * t.nseg, step, t.nc, seg, u, f);
+        offset[threadIdx.x] = f[0];
+    }
+    if (lv.phi != nullptr)
+        for (int b = 0; b < lv.phases; ++b) {
+            const float c = center(b);
+            float s = 0.f;
+            for (int e = threadIdx.x; e < rows * n; e += blockDim.x) s += pair_with(tb, field[e], c);
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) lv.phi[(int64_t)(bk.a * lv.phases + b) * lv.nphi + bk.block * NW + warp] = s;
+        }
+    __syncthreads();
     if (lv.ax[2].fast) {
         for_pow2(lv.ax[2].fast, [&](auto c) {
             constexpr int N = decltype(c)::value;
@@ -919,7 +709,12 @@ __global__ void __launch_bounds__(SEP_ROW_THREADS, 4) sep_feat_kernel(const __gr
                 for (int p0 = 0; p0 < t.npair; p0 += S::SLOTS) {
                     const bool live = in && p0 + p < t.npair;
                     float2 v[8];
-                    if (live) eval_features<false, 8>(cf + (p0 + p) * t.nseg, step, t.nc, seg, u, v);
+                    if (live) {
+                        eval_features<false, 8>(cf + (p0 + p) * t.nseg, step, t.nc, seg, u, v);
+                        const float2 c = offset[p0 + p];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) v[e] = csubf(v[e], c);
+                    }
                     p2_fft<N, S::WARP, 0>(v, opaque(ln));
                     if (live) {
                         float2* out = Z + (int64_t)(p0 + p) * lv.N + row * N + ln.t;
@@ -948,7 +743,7 @@ __global__ void __launch_bounds__(SEP_ROW_THREADS, 4) sep_feat_kernel(const __gr
             locate<1>(t, x, seg, u);
             float2 f[1];
             eval_features<false, 1>(cf + (p0 + c) * t.nseg, step, t.nc, seg, u, f);
-            s.a[q * pitch + spad(i)] = f[0];
+            s.a[q * pitch + spad(i)] = csubf(f[0], offset[p0 + c]);
         }
         const float2* r = transform(lv.ax[2], s.a, s.b, s.tw, rows * nc, pitch);
         for (int e = threadIdx.x; e < rows * nc * n; e += blockDim.x) {
@@ -1116,15 +911,16 @@ __device__ __forceinline__ float2 split(double v) {
 }  // namespace
 
 // item: (level, phases a, b).  Sums s_k conj(Z^a_k) Z^b_k over the feature pairs and writes the
-// inverse along the last axis, cropped to r = 0 .. P (-r belongs to the pair (b, a)).  CROSS:
-// a and b may differ.  Bound by latency: one or two blocks an SM.  512^2, three levels, seven pairs:
-// 25 us with two shares of the pairs at the finest level, 31 with one; 128^3, two levels: 101 us;
-// nine phase pairs of 512^2: 148 us.
+// inverse along the last axis, cropped to r = 0 .. P (-r belongs to the pair (b, a)).  The block that
+// holds the frequency 0 adds the means of F(M, c) there.  CROSS: a and b may differ.  Bound by latency: one or two blocks an SM.  512^2, three levels, seven pairs:
+// 27 us with two shares of the pairs at the finest level (33 with one); 128^3, two levels: 101 us;
+// nine phase pairs of 512^2: 153 us.
 template <bool CROSS>
 __global__ void __launch_bounds__(SEP_THREADS, CROSS ? 1 : 2)
 sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
     __shared__ double dcs[SEP_THREADS / 2];
+    __shared__ DF psh[SEP_THREADS / 32];  // sum F(M^a, c_b) + sum F(c_a, M^b), one share a warp
     if (!enter<true>(tb, items, nitem, bk, sep_smem, axis_last)) return;
     const SepLevel& lv = bk.lv;
     float2* sm = sep_smem;
@@ -1141,6 +937,22 @@ sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict
     // 3-D: U[r][y][x]; 2-D: V[r][x]
     float2* out = (lv.n0 > 1 ? lv.U : lv.V) + (int64_t)(pair + bk.part) * (lv.n0 > 1 ? lv.strideU : lv.strideV) + g.base;
     const bool cross = CROSS && bk.a != bk.b;
+    if (dc_block && bk.part == 0) {
+        DF v{0.f, 0.f};
+        const float* pa = lv.phi + (int64_t)(bk.a * lv.phases + bk.b) * lv.nphi;
+        const float* pb = lv.phi + (int64_t)(bk.b * lv.phases + bk.a) * lv.nphi;
+        for (int i = threadIdx.x; i < lv.nphi; i += blockDim.x) v = df_add(v, df_two_sum(pa[i], pb[i]));
+        for (int o = 16; o > 0; o >>= 1)
+            v = df_add(v, DF{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)});
+        if ((threadIdx.x & 31) == 0) psh[threadIdx.x >> 5] = v;
+    }
+    // by the thread that holds the frequency 0, a barrier or more later
+    auto means = [&]() {
+        DF v = psh[0];
+        for (int w = 1; w < SEP_THREADS / 32; ++w) v = df_add(v, psh[w]);
+        const double twice = (double)pair_with(tb, lv.center[bk.a], lv.center[bk.b]);
+        return (double)lv.N * (((double)v.hi + (double)v.lo) - (double)lv.N * twice);
+    };
     if (ax.fast) {
         for_pow2(ax.fast, [&](auto cc) {
             constexpr int N = decltype(cc)::value, T = N / 8;
@@ -1218,6 +1030,7 @@ sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict
             if (has_dc && c.slot == 0) {
                 double s = dcs[0];
                 for (int k = 1; k < c.slots; ++k) s += dcs[k];
+                if (bk.part == 0) s += means();
                 lv.dc[pair + bk.part] = split(s * lv.scaleD);
             }
             if (has_dc) acc[0] = make_float2(0.f, 0.f);
@@ -1271,6 +1084,7 @@ sep_power_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict
         });
     }
     if (has_dc) {
+        if (bk.part == 0) dc += means();
         lv.dc[pair + bk.part] = split(dc * lv.scaleD);
         acc[0] = make_float2(0.f, 0.f);
     }
@@ -1632,9 +1446,10 @@ struct GCols {
 
 // item: (level, phase a).  Spectrum of G along the last axis, then for every feature pair the
 // forward transform of the columns, the product sum_b conj(G^ab) Z^b and the inverse: Q^a, in
-// place of Z for a single phase (G is even then: a real spectrum).  Bound by latency, as sep_power.
-// 512^2, three levels, seven pairs: 24 us with the pairs shared among up to four blocks a group of
-// columns, 29 without; 128^3, two levels: 103 us.
+// place of Z for a single phase (G is even then: a real spectrum).  Its frequency 0, the sum of G over
+// the window, is left for the term of F_u(M, c).  Bound by latency, as sep_power.
+// 512^2, three levels, seven pairs: 23 us with the pairs shared among up to four blocks a group of
+// columns, 29 without; 128^3, two levels: 100 us.
 template <bool MULTI>
 __global__ void __launch_bounds__(SEP_THREADS, MULTI ? 1 : 2)
 sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__ items, int nitem) {
@@ -1648,7 +1463,8 @@ sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__
     const ColGroup g = last_axis(lv, bk.block, x0, y);
     const SepAxis& ax = last_ax(lv);
     // of the unnormalised inverse; sep_desc's rows still lack the loss' factor
-    const float norm = (lv.fuse && lv.sc != nullptr ? lv.sc->gscale : 1.f) / (float)lv.N;
+    const float gscale = lv.fuse && lv.sc != nullptr ? lv.sc->gscale : 1.f, norm = gscale / (float)lv.N;
+    const bool has_sum = x0 == 0 && y == 0 && bk.part == 0 && threadIdx.x == 0;   // its first point is frequency 0
     if (ax.fast && (!MULTI || lv.phases <= SEP_FAST_PHASES)) {
         for_pow2(ax.fast, [&](auto cc) {
             constexpr int N = decltype(cc)::value, T = N / 8;
@@ -1665,6 +1481,7 @@ sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__
                     v[e] = c.l < g.cols ? gc.at(c.ln.t + e * T, c.l) : make_float2(0.f, 0.f);
                 p2_fft<N, false, 0>(v, opaque(c.ln));
                 if (PAR1) __syncthreads();
+                if (has_sum) lv.gsum[bk.a * lv.phases + b] = gscale * v[0].x;
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     if (MULTI) gs[(b * 8 + e) * SEP_THREADS] = make_float2(norm * v[e].x, -norm * v[e].y);
@@ -1733,6 +1550,7 @@ sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__
         }
         const float2* r = transform(ax, s.a, s.b, s.tw, g.L, pitch);
         own([&](int, int e, int at) { gs[b * total + e] = make_float2(norm * r[at].x, MULTI ? -norm * r[at].y : 0.f); });
+        if (has_sum) lv.gsum[bk.a * lv.phases + b] = gscale * r[0].x;
     }
     for (int p = bk.part; p < t.npair; p += bk.parts) {
         float2 acc[SEP_OWN];
@@ -1764,9 +1582,9 @@ sep_mul_kernel(const __grid_constant__ SepTables tb, const SepItem* __restrict__
 // ------------------------------------------------------------------------- gradient
 
 // item: (level, phase a); blocks: groups of rows.  Inverse along x of every feature pair and
-// g(y) = sum_k s_k p_k'(M_y) Q_k(y), the slots' shares added in a fixed order.  Bound by latency, as
-// sep_feat.  Seven pairs: 512^2, three levels 27 us; 128^3, two levels 119 us (coefficient gathers
-// unrolled by three: 28 and 125).
+// g(y) = F_u(M_y, c) sum G + sum_k s_k p_k'(M_y) Q_k(y), the slots' shares added in a fixed order.
+// Bound by latency, as sep_feat.  Seven pairs: 512^2, three levels 28 us; 128^3, two levels 124 us,
+// 5 of them for F_u(M, c) (coefficient gathers unrolled by three: 1 and 6 us more).
 __global__ void __launch_bounds__(SEP_ROW_THREADS, 3) sep_grad_kernel(const __grid_constant__ SepTables tb,
                                                                       const SepItem* __restrict__ items, int nitem) {
     __shared__ SepBlock bk;
@@ -1781,6 +1599,20 @@ __global__ void __launch_bounds__(SEP_ROW_THREADS, 3) sep_grad_kernel(const __gr
     const float* __restrict__ field = lv.field + (int64_t)bk.a * lv.N + (int64_t)row0 * n;
     const float2* __restrict__ Q = lv.Q + (int64_t)bk.a * lv.maxPairs * lv.N + (int64_t)row0 * n;
     float* __restrict__ part = lv.part + (int64_t)bk.a * lv.N + (int64_t)row0 * n;
+    __shared__ float2 csh[MAX_PHASES];           // (c_b, sum_r G^ab(r))
+    if (threadIdx.x < lv.phases) csh[threadIdx.x] = make_float2(lv.center[threadIdx.x], lv.gsum[bk.a * lv.phases + threadIdx.x]);
+    // sum_b F_u(M, c_b) sum_r G^ab(r) at element o of the block's rows
+    auto background = [&](int o) {
+        const float M = field[o];
+        float s = 0.f;
+        for (int b = 0; b < lv.phases; ++b) {
+            const float2 c = csh[b];
+            float slope;
+            pair_with(tb, M, c.x, slope);
+            s = fmaf(slope, c.y, s);
+        }
+        return s;
+    };
     __syncthreads();
     if (lv.ax[2].fast) {
         for_pow2(lv.ax[2].fast, [&](auto cc) {
@@ -1826,19 +1658,34 @@ __global__ void __launch_bounds__(SEP_ROW_THREADS, 3) sep_grad_kernel(const __gr
                     if (in) {
 #pragma unroll
                         for (int e = 0; e < 8; ++e) part[row * N + ln.t + e * S::T] = g[e];
+                        // (one at a time: eight side by side spill)
+#pragma unroll 1
+                        for (int e = 0; e < 8; ++e)
+                            part[row * N + ln.t + e * S::T] += background(row * N + ln.t + e * S::T);
                     }
                     continue;
+                }
+                // the positions this thread finishes: their background terms before the barrier
+                constexpr int FIN = (S::ROWS * N + SEP_ROW_THREADS - 1) / SEP_ROW_THREADS;
+                const int here = min(S::ROWS, rows - rb) * N;
+                float bg[FIN];
+#pragma unroll
+                for (int j = 0; j < FIN; ++j) {
+                    const int o = threadIdx.x + j * SEP_ROW_THREADS;
+                    bg[j] = o < here ? background(rb * N + o) : 0.f;
                 }
                 __syncthreads();
 #pragma unroll
                 for (int e = 0; e < 8; ++e) red[(p * S::ROWS + r0) * N + ln.t + e * S::T] = g[e];
                 __syncthreads();
-                const int here = min(S::ROWS, rows - rb) * N;
-                for (int o = threadIdx.x; o < here; o += SEP_ROW_THREADS) {
+#pragma unroll
+                for (int j = 0; j < FIN; ++j) {
+                    const int o = threadIdx.x + j * SEP_ROW_THREADS;
+                    if (o >= here) break;
                     float s = red[o];
 #pragma unroll
                     for (int k = 1; k < S::SLOTS; ++k) s += red[k * S::ROWS * N + o];
-                    part[rb * N + o] = s;
+                    part[rb * N + o] = s + bg[j];
                 }
                 __syncthreads();
             }
@@ -1881,7 +1728,7 @@ __global__ void __launch_bounds__(SEP_ROW_THREADS, 3) sep_grad_kernel(const __gr
 #pragma unroll
     for (int q = 0; q < SEP_OWN; ++q) {
         const int e = threadIdx.x + q * SEP_ROW_THREADS;
-        if (e < rows * n) part[e] = g[q];
+        if (e < rows * n) part[e] = g[q] + background(e);
     }
 }
 
