@@ -157,7 +157,7 @@ struct Plan {
     int sep_tiers = 0, sep_pairs = 0;   // tiers worth running, feature pairs of the widest of them
     size_t o_tier = 0, o_tiers = 0, o_z[MAX_LEVELS] = {}, o_q[MAX_LEVELS] = {}, o_u[MAX_LEVELS] = {},
            o_v[MAX_LEVELS] = {}, o_sdc[MAX_LEVELS] = {}, o_spart[MAX_LEVELS] = {}, o_phi[MAX_LEVELS] = {},
-           o_gsum[MAX_LEVELS] = {}, o_msum = 0, o_center = 0;
+           o_gsum[MAX_LEVELS] = {}, o_msum = 0, o_center = 0, o_next = 0;
     // block sums of the loss, left by the descriptor kernels (two-point descriptor without FFT levels)
     bool sums = false;
     size_t o_excess = 0, o_sums = 0;
@@ -341,6 +341,9 @@ int64_t sep_u_len(const LevelGeom& g) { return g.n[0] > 1 ? (int64_t)(g.P[0] + 1
 int64_t sep_v_rows(const LevelGeom& g) {
     return g.n[0] > 1 ? (int64_t)(g.P[0] + 1) * (2 * g.P[1] + 1) : g.P[1] + 1;
 }
+
+// counters of the gated launches of one instance: forward, reduction and adjoint of every level and phase pair
+size_t gated_segments(const Plan& pl) { return (size_t)3 * pl.levels * pl.phases * pl.phases; }
 
 // blocks of sep_feat and sep_grad, one phase
 int64_t sep_feature_blocks(const LevelGeom& g) {
@@ -618,6 +621,7 @@ dmcr_status make_plan(const dmcr_params* p, Plan& pl) {
         pl.o_tiers = o; o = align_up(o + PREP_BLOCKS * sizeof(int));
         pl.o_msum = o; o = align_up(o + (size_t)PREP_BLOCKS * pl.phases * sizeof(float));
         pl.o_center = o; o = align_up(o + (size_t)pl.phases * sizeof(float));
+        pl.o_next = o; o = align_up(o + gated_segments(pl) * sizeof(unsigned));
         std::vector<PairShare> power;
         for (int l = 0; l < pl.levels; ++l) {
             SepLevel lv;
@@ -1127,6 +1131,8 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
             if (pl.sep) {
                 p.tiers = reinterpret_cast<int*>(x.ws + pl.o_tiers);
                 p.sums = reinterpret_cast<float*>(x.ws + pl.o_msum);
+                p.next = reinterpret_cast<unsigned*>(x.ws + pl.o_next);
+                p.nnext = (int)gated_segments(pl);
                 p.ntier = pl.sep_tiers;
                 for (int t = 0; t < pl.sep_tiers; ++t) p.lo[t] = pl.basis->tier[t].lo, p.hi[t] = pl.basis->tier[t].hi;
                 if ((flags & F_LOSS) && pl.sums && x.lp.bc_on) p.excess = reinterpret_cast<float4*>(x.ws + pl.o_excess);
@@ -1199,6 +1205,8 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
                         it.f.partial = reinterpret_cast<float*>(x.ws + x.pl->o_fwd[l]) + blk * g.fwdTiles * g.Khalf;
                         it.f.done = x.use_done ? &x.sc->done : nullptr;
                         it.f.gate = gate;
+                        unsigned* next = reinterpret_cast<unsigned*>(x.ws + x.pl->o_next) + 3 * (l * (int64_t)nph * nph + blk);
+                        if (gate) it.f.next = next;
                         it.work = (int64_t)g.TY * g.PPB;
                         it.blocks = g.fwdTiles * g.fwdGroupBlocks;
                         items.push_back(it);
@@ -1208,6 +1216,7 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
                         r.desc = x.desc + x.pl->off[l] + blk * g.Khalf;
                         r.done = it.f.done;
                         r.gate = gate;
+                        if (gate) r.next = next + 1;
                         r.scale = (float)((double)x.pl->w[l] / (double)g.N);
                         const int64_t own = ceil_div(g.Khalf, RED_K);
                         if (loss != nullptr) {
@@ -1379,6 +1388,7 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
                         it.a.part = pblk;
                         it.a.done = done;
                         it.a.gate = gate;
+                        if (gate) it.a.next = reinterpret_cast<unsigned*>(x.ws + x.pl->o_next) + 3 * (l * (int64_t)nph * nph + blk) + 2;
                         it.work = (int64_t)g.RZ * g.RY * g.NBc;
                         it.blocks = g.adjTiles * g.nChunks;
                         items.push_back(it);

@@ -155,6 +155,8 @@ __global__ void __launch_bounds__(ELEM_TH) prep_kernel(const PrepSeg* __restrict
         if (threadIdx.x == 0) sg.excess[blk] = make_float4(E.hi, E.lo, 0.f, 0.f);
     }
     if (sg.tiers == nullptr) return;
+    if (blk == 0)
+        for (int i = threadIdx.x; i < sg.nnext; i += ELEM_TH) sg.next[i] = 0;
     // the narrowest range that holds the block's values; NaN and wider fields: the direct kernels
     int t = 0;
     while (t < sg.ntier && !(lo >= sg.lo[t] && hi <= sg.hi[t])) ++t;

@@ -190,6 +190,7 @@ struct FwdSeg {
     const float* tip;       // tips of the pairs (x + r): the same field, or another phase's
     float* partial;
     const int* gate;        // gated launches only: run when *gate >= SEP_TIERS
+    unsigned* next;         // gated launches only: the first block that nobody has taken (prep_kernel sets it to 0)
     const int* done;
     int64_t blockStart;
 };
@@ -198,6 +199,7 @@ struct RedSeg {
     const float* partial;
     float* desc;
     const int* gate;        // gated launches only: run when *gate >= SEP_TIERS
+    unsigned* next;         // gated launches only: the first block that nobody has taken (prep_kernel sets it to 0)
     const int* done;
     float scale;             // w_l / N_l
     // loss: this segment's target, its block sums (one per block), the instance's loss and the
@@ -232,6 +234,7 @@ struct AdjSeg {
     CoefSrc c;
     float* part;
     const int* gate;        // gated launches only: run when *gate >= SEP_TIERS
+    unsigned* next;         // gated launches only: the first block that nobody has taken (prep_kernel sets it to 0)
     const int* done;
     int64_t blockStart;
 };
@@ -278,6 +281,8 @@ struct PrepSeg {
     int* tiers;                  // separable path: one word per block, null otherwise: its tier, and from bit 8
                                  // on one bit per phase that shows a value of at least SEP_WEAK
     float* sums;                 // separable path: sum of the block's values, [block][phase]
+    unsigned* next;              // separable path: the gated segments' counters, set to 0 (nnext of them)
+    int nnext;
     int ntier;
     float lo[8], hi[8];          // its ranges
     float4* excess;              // box excess: sum of squares per block (hi, lo), null: not wanted

@@ -528,10 +528,13 @@ corr_fwd_kernel(const FwdSeg* __restrict__ segs, int nseg, ThreshConst tc) {
     corr_fwd_block<IDENT>(sg, (int64_t)blockIdx.x - sg.blockStart, tc);
 }
 
-// Gated launches: the segments belong to instances on the separable path, and run here only
-// when their field left every range that path has a basis for.  A small grid that all but
-// always finds nothing to do: one parallel look at the gates, then a block-strided walk over
-// the blocks of the segments whose gate is open.
+// Gated launches: the segments belong to instances on the separable path, and run here only when
+// their field left every range that path has a basis for.  A grid of the resident blocks, which
+// all but always finds nothing to do after one parallel look at the gates; otherwise its blocks
+// take the segments' blocks one by one, as the hardware hands them out in an ungated launch
+// (8192 blocks with a fixed share of them each, blockIdx + k gridDim: 25.2 and 60.4 ms, forward
+// and adjoint, instead of 22.7 and 55.3 for 128^3, +-24, two levels; and 10 and 4 us longer when
+// there is nothing to do).
 template <typename S>
 __device__ __forceinline__ bool gate_open(const S& sg) {
     return !(sg.done != nullptr && *sg.done) && *sg.gate >= SEP_TIERS;
@@ -539,16 +542,26 @@ __device__ __forceinline__ bool gate_open(const S& sg) {
 
 template <typename S, typename F>
 __device__ __forceinline__ void run_gated(const S* __restrict__ segs, int nseg, int64_t total, F block) {
+    __shared__ unsigned taken;
     int any = 0;
     for (int i = threadIdx.x; i < nseg; i += blockDim.x) any |= gate_open(segs[i]);
     if (!__syncthreads_or(any)) return;
     for (int i = 0; i < nseg; ++i) {
-        if (!gate_open(segs[i])) continue;
         const int64_t count = (i + 1 < nseg ? segs[i + 1].blockStart : total) - segs[i].blockStart;
-        for (int64_t local = blockIdx.x; local < count; local += gridDim.x) {
-            block(segs[i], local);
+        // thread 0 decides for the block: an instance may stop while later blocks look at its gate
+        unsigned mine = 0;
+        if (threadIdx.x == 0) taken = gate_open(segs[i]) ? atomicAdd(segs[i].next, 1u) : 0xffffffffu;
+        for (;;) {
             __syncthreads();
+            const unsigned local = taken;
+            if ((int64_t)local >= count) break;
+            // the next one is asked for while this one runs
+            if (threadIdx.x == 0) mine = atomicAdd(segs[i].next, 1u);
+            block(segs[i], (int64_t)local);
+            __syncthreads();
+            if (threadIdx.x == 0) taken = mine;
         }
+        __syncthreads();
     }
 }
 
@@ -911,9 +924,8 @@ void launch_corr_adj(const AdjSeg* segs, int nseg, int64_t blocks, size_t smem, 
     else launch_dep(corr_adj_kernel<false>, (unsigned)blocks, ADJ_THREADS, smem, s, segs, nseg, tc);
 }
 
-// blocks of a gated launch at most: enough for the hardware to balance them when the gate is
-// open, few enough to be dismissed in a few microseconds when it is not
-constexpr int64_t GATED_BLOCKS = 8192, GATED_SMALL = 8192;
+// blocks of a gated launch at most: what is resident at once (launch bounds)
+constexpr int64_t GATED_BLOCKS = 4 * SMS, GATED_REDUCE_BLOCKS = 8 * SMS;
 
 void launch_corr_fwd_gated(const FwdSeg* segs, int nseg, int64_t blocks, size_t smem, const ThreshConst& tc,
                            cudaStream_t s) {
@@ -923,7 +935,7 @@ void launch_corr_fwd_gated(const FwdSeg* segs, int nseg, int64_t blocks, size_t 
 
 void launch_fwd_reduce_gated(const RedSeg* segs, int nseg, int64_t blocks, cudaStream_t s) {
     if (blocks <= 0) return;
-    launch_dep(fwd_reduce_gated_kernel, (unsigned)std::min(blocks, GATED_SMALL), 256, 0, s, segs, nseg, blocks);
+    launch_dep(fwd_reduce_gated_kernel, (unsigned)std::min(blocks, GATED_REDUCE_BLOCKS), 256, 0, s, segs, nseg, blocks);
 }
 
 void launch_corr_adj_gated(const AdjSeg* segs, int nseg, int64_t blocks, size_t smem, const ThreshConst& tc,
