@@ -97,7 +97,10 @@ typedef struct {
     int tune[4];             /* launch shape (0 = built-in choice): forward tile rows {2,4,8,16,32},
                                 adjoint ry rows per shift chunk (1..16), adjoint chunk target
                                 limit (1..64), adjoint rx blocks of 8 shifts per chunk at most
-                                (1..32).  Results agree to rounding across shapes. */
+                                (1..32).  Results agree to rounding across shapes.  It shapes the
+                                DIRECT kernels: a problem that AUTO gives to the separable or the
+                                FFT path runs as it would without it (path = DMCR_PATH_DIRECT
+                                runs the direct kernels in this shape) */
     int descriptor;          /* DMCR_DESC_S2 (default), DMCR_DESC_S3 or DMCR_DESC_S2_TILDE */
     int phases;              /* phase fields (1..8; 0 means 1).  See "Several phases" below. */
 } dmcr_params;

@@ -8,7 +8,8 @@ kernel), then the adjoint's rx blocks per chunk (they set how many ry rows fit i
 memory), its ry rows, and its chunk limit -- and returns the params with the fastest shape
 in ``tune``.  Results are cached in a JSON file keyed by the problem class and the GPU, so a
 shape is measured once per machine.  Shapes change only the blocking and summation order:
-results agree to rounding.
+results agree to rounding.  A problem that AUTO gives to the separable or the FFT path does not
+run these kernels and is not tuned; tune it with ``path=DMCR_PATH_DIRECT`` where those are wanted.
 """
 from __future__ import annotations
 
@@ -95,10 +96,28 @@ def search(p: _lib.Params, seed: int = 0, device="cuda", timer=None) -> tuple[tu
     return best, best_ms, trials
 
 
+def runs_direct_kernels(p: _lib.Params) -> bool:
+    """Whether p, or one of its levels, is planned onto the kernels that ``tune`` shapes: not the
+    three-point descriptor, and not the separable path or the FFT path at every level (their scratch
+    is another than the direct kernels')."""
+    if p.descriptor == _lib.DMCR_DESC_S3 or p.path == _lib.DMCR_PATH_FFT:
+        return False
+    if p.path == _lib.DMCR_PATH_DIRECT:
+        return True
+    size = _lib.dmcr_workspace_size(p)
+    if p.threshold == _lib.DMCR_SOFT:        # separable: all levels or none
+        return size == _lib.dmcr_workspace_size(dataclasses.replace(p, path=_lib.DMCR_PATH_DIRECT))
+    try:
+        return size != _lib.dmcr_workspace_size(dataclasses.replace(p, path=_lib.DMCR_PATH_FFT))
+    except _lib.DmcrError:                   # lengths that the transforms do not take
+        return True
+
+
 def tuned(p: _lib.Params, cache: str | None = None) -> _lib.Params:
-    """params with the cached (or freshly measured) fastest launch shape.  The three-point
-    descriptor does not run the tuned kernels: its params come back unchanged."""
-    if p.descriptor == _lib.DMCR_DESC_S3:
+    """params with the cached (or freshly measured) fastest launch shape.  Problems that do not run
+    the tuned kernels (``runs_direct_kernels``) come back unchanged: their time does not depend
+    on the shape."""
+    if not runs_direct_kernels(p):
         return p
     path = _cache_path(cache)
     key = _key(p)
