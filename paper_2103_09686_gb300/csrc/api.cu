@@ -1458,9 +1458,9 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
     }
     if (need_pyr) prepare_sep(in, flags, loss_sep, P);
     if (P.tb.h.size() > cap) return fail(DMCR_ENOMEM, "segment tables (%zu bytes) exceed their region", P.tb.h.size());
-    // every fused launch indexes its blocks with a 1-D grid
+    // every fused launch indexes its blocks with a 1-D grid (a gated one with a 32-bit counter)
     int64_t most = std::max({P.fwd.blocks, P.red.blocks, P.gco.blocks, P.adj.blocks, P.fin.blocks, P.fin_small.blocks,
-                             P.tmap.blocks});
+                             P.tmap.blocks, P.gfwd.blocks, P.gred.blocks, P.gadj.blocks});
     for (const Prepared::R& r : P.sep) most = std::max(most, r.blocks);
     for (const Prepared::R& r : P.restricts) most = std::max(most, r.blocks);
     if (most > (int64_t)INT32_MAX)
