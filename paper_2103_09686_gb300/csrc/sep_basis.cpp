@@ -351,6 +351,8 @@ void build(SepBasis& b) {
     const double deltas[] = {0.2, 0.05, 0.02, 0.014, 0.01, 0.007, 0.005};
     constexpr int ND = sizeof deltas / sizeof deltas[0];
     int d = 0;
+    b.ntier = 0;
+    b.coef.clear();
     for (int t = 0; t < SEP_TIERS; ++t) {
         TierResult res = TIER_ROUNDED;
         for (d = t == 0 ? 0 : std::max(2, d - 1); d < ND; ++d) {
@@ -367,21 +369,30 @@ void build(SepBasis& b) {
 }  // namespace
 
 std::shared_ptr<const SepBasis> sep_basis(float alpha) {
+    // one build takes about 0.1 s: outside the lock, so that only callers of the same new alpha wait
+    struct Entry {
+        SepBasis basis;
+        std::once_flag built;
+    };
     static std::mutex mu;
-    static std::vector<std::shared_ptr<const SepBasis>>* cache = new std::vector<std::shared_ptr<const SepBasis>>();
+    static std::vector<std::shared_ptr<Entry>>* cache = new std::vector<std::shared_ptr<Entry>>();
     constexpr size_t KEEP = 16;
-    std::lock_guard<std::mutex> lk(mu);
-    for (size_t i = 0; i < cache->size(); ++i)
-        if ((*cache)[i]->alpha == alpha) {
-            std::rotate(cache->begin(), cache->begin() + i, cache->begin() + i + 1);   // most recent first
-            return cache->front();
+    std::shared_ptr<Entry> e;
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        size_t i = 0;
+        while (i < cache->size() && (*cache)[i]->basis.alpha != alpha) ++i;
+        if (i == cache->size()) {
+            auto fresh = std::make_shared<Entry>();
+            fresh->basis.alpha = alpha;
+            cache->push_back(fresh);
         }
-    auto b = std::make_shared<SepBasis>();
-    b->alpha = alpha;
-    build(*b);
-    cache->insert(cache->begin(), b);
-    if (cache->size() > KEEP) cache->pop_back();
-    return b;
+        std::rotate(cache->begin(), cache->begin() + i, cache->begin() + i + 1);   // most recent first
+        if (cache->size() > KEEP) cache->pop_back();
+        e = cache->front();
+    }
+    std::call_once(e->built, [&] { build(e->basis); });
+    return std::shared_ptr<const SepBasis>(e, &e->basis);
 }
 
 }  // namespace dmcr

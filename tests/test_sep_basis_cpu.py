@@ -10,16 +10,18 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_2103_09686_gb300", "csrc")
 
 
-@pytest.fixture(scope="module")
-def probe(tmp_path_factory):
+def _compile(source, exe):
     cxx = shutil.which("g++") or shutil.which("c++")
     if cxx is None:
         pytest.skip("no C++ compiler")
-    exe = str(tmp_path_factory.mktemp("sep") / "probe")
     subprocess.check_call([cxx, "-O2", "-std=c++17", "-Wall", "-Werror", "-pthread", "-I", CSRC,
-                           os.path.join(ROOT, "tests", "sep_basis_probe.cpp"), os.path.join(CSRC, "sep_basis.cpp"),
-                           "-o", exe])
+                           os.path.join(ROOT, "tests", source), os.path.join(CSRC, "sep_basis.cpp"), "-o", exe])
     return exe
+
+
+@pytest.fixture(scope="module")
+def probe(tmp_path_factory):
+    return _compile("sep_basis_probe.cpp", str(tmp_path_factory.mktemp("sep") / "probe"))
 
 
 @pytest.mark.parametrize("alpha,least", [(0.5, 6), (2.0, 6), (5.0, 6), (8.0, 6), (10.0, 6), (12.0, 4), (15.0, 2), (20.0, 1),
@@ -33,3 +35,8 @@ def test_pairs_of_every_range(probe, alpha, least):
         # the bound of an entry (tests/test_gpu_parity.py) for every single pair of values; accepted
         # at other values than these, whose rounding differs
         assert rel < 1.3 and upper < 1.3
+
+
+def test_a_new_slope_holds_up_nobody(tmp_path):
+    out = subprocess.run([_compile("sep_basis_threads_probe.cpp", str(tmp_path / "probe"))], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout + out.stderr
