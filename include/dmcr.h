@@ -312,7 +312,9 @@ dmcr_status dmcr_profile_reset(void);
 dmcr_status dmcr_profile_read(int index, char* name, int name_len, double* total_ms, int64_t* launches);
 
 /*
- * dmcr_descriptor_noalloc -- the same descriptor as dmcr_descriptor, for callers that
+ * dmcr_descriptor_noalloc -- the descriptor that dmcr_descriptor computes, always by the
+ *   DIRECT evaluation: bit for bit that of path = DMCR_PATH_DIRECT; a problem that AUTO gives
+ *   to the separable path agrees to rounding (1e-5 of an entry).  For callers that
  *   cannot allocate device memory (no cudaMalloc, no caching allocator) at the point of
  *   the call: code running under a runtime that forbids allocation during execution, or
  *   deployments that reserve all device memory up front.  The paper has no counterpart;

@@ -6,6 +6,7 @@ Bounds: descriptor entries within 1e-5 relative plus 1e-9 absolute of FP64, grad
 normwise, as in test_gpu_parity.py.  Against the direct kernels, whose own error is below 1e-6
 relative, 1.1e-5.
 """
+import ctypes
 import dataclasses
 
 import numpy as np
@@ -200,3 +201,21 @@ def test_the_path_of_other_slopes(cuda_lib, alpha, separable):
     a = dm.descriptor(f, p).cpu().numpy().astype(np.float64)
     b = dm.descriptor(f, dataclasses.replace(p, path=dm.DMCR_PATH_DIRECT)).cpu().numpy().astype(np.float64)
     _check_descriptor(dm, p, M, a, b)
+
+
+@pytest.mark.parametrize("vf,pixel", [(0.01, 2.0), (0.35, 1.0)])
+def test_noalloc_is_the_direct_evaluation(cuda_lib, vf, pixel):
+    """dmcr_descriptor_noalloc on a problem that dmcr_descriptor runs by transforms."""
+    dm = cuda_lib
+    from paper_2103_09686_gb300 import _lib
+    M = synthetic.target_2d_grf(SHAPE[0], 6.0, vf, seed=3)
+    M[5, 7] = pixel
+    p, f = dm.Params(shape=SHAPE, window=WINDOW, levels=LEVELS), _dev(M)
+    assert _separable(dm, p, f)
+    got = torch.empty(dm.dmcr_descriptor_length(p), device="cuda")
+    lib = _lib.load()
+    st = lib.dmcr_descriptor_noalloc(ctypes.byref(p.c()), f.data_ptr(), got.data_ptr(),
+                                     torch.cuda.current_stream().cuda_stream)
+    assert st == 0, lib.dmcr_last_error().decode()
+    assert torch.equal(got, dm.descriptor(f, dataclasses.replace(p, path=dm.DMCR_PATH_DIRECT)))
+    np.testing.assert_allclose(got.cpu().numpy(), dm.descriptor(f, p).cpu().numpy(), rtol=1.1 * RTOL, atol=ATOL)
