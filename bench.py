@@ -1025,12 +1025,14 @@ def main():
         flops = sum(nph * nph * 4 * 5.0 * n * np.log2(n) for sh, _, lev, _ in insts for n in level_sizes(sh, lev))
         peak = sm_count * pipes["ffma2_lanes"] * 2 * max_mhz * 1e6 / 1e12
         achieved = flops / (total_s / args.steps) / 1e12
-        roofline = {"bound": "alu", "kernel": name, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+        step_ms = total_s / args.steps * 1e3
+        roofline = {"bound": "alu", "kernel": "whole step", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                     "frac": achieved / peak, "traffic": None,
                     "peak_basis": "measured FP32 pipe (FFMA2 probe) at the max SM clock; achieved = transform "
                                   "operations of the exact correlation and its gradient / step time (the separable "
                                   "path runs about a dozen such transforms, one per pair of features)",
-                    "avg_launch_ms": avg_ms, "launches": kcnt}
+                    "avg_launch_ms": step_ms, "launches": args.steps,
+                    "slowest_kernel": {"kernel": name, "avg_launch_ms": avg_ms, "launches": kcnt}}
     # kernels of this library per step (the profiled pass launches the kernels of a graph replay
     # directly), times steps
     launches = int(round(sum(c for _, c in prof.values()) / max(prof_steps, 1) * args.steps))
