@@ -949,7 +949,6 @@ void prepare_sep(const std::vector<Inst>& in, unsigned flags, const std::vector<
             const LevelGeom& g = pl.g[l];
             SepLevel lv;
             sep_shape(g, pl.phases, pl.sep_pairs, lv);
-            lv.ntier = pl.sep_tiers;
             lv.parts = pl.sep_parts[l];
             lv.field = x.lv[l];
             lv.Z = reinterpret_cast<float2*>(x.ws + pl.o_z[l]);

@@ -387,7 +387,6 @@ struct SepLevel {
     int n0, n1, n2;
     int P0, P1, P2;
     int phases, maxPairs;
-    int ntier;                // tiers this problem uses (wider fields: the direct kernels)
     int64_t N, Khalf;
     SepAxis ax[3];
     const float* field;       // this level's field(s)
