@@ -52,7 +52,7 @@ MIX_KEY = {"corr_fwd": "forward_pairs", "corr_adj": "adjoint_pairs"}
 # DRAM bytes (read + write) per launch of each correlation kernel, from one ncu capture of the
 # bench's own command per workload (dram__bytes_read.sum + dram__bytes_write.sum); None
 # whenever a kernel changed since its last capture.
-NCU_TRAFFIC_BYTES = {}
+NCU_TRAFFIC_BYTES = {("grf64", "corr_adj"): 90112 + 0, ("grf64", "corr_fwd"): 93696 + 0}
 
 WORKLOADS = {
     "grf512": dict(shape=(512, 512), window=(64, 64), levels=3,
