@@ -155,6 +155,7 @@ struct Plan {
     bool sep = false;
     std::shared_ptr<const SepBasis> basis;
     int sep_tiers = 0, sep_pairs = 0;   // tiers worth running, feature pairs of the widest of them
+    int sep_vjp = 0;                    // of these, the ones worth running for a gradient alone
     size_t o_tier = 0, o_tiers = 0, o_z[MAX_LEVELS] = {}, o_q[MAX_LEVELS] = {}, o_u[MAX_LEVELS] = {},
            o_v[MAX_LEVELS] = {}, o_sdc[MAX_LEVELS] = {}, o_spart[MAX_LEVELS] = {}, o_phi[MAX_LEVELS] = {},
            o_gsum[MAX_LEVELS] = {}, o_msum = 0, o_center = 0, o_next = 0;
@@ -410,8 +411,8 @@ int usual_pairs(const SepBasis& b) { return std::max(b.tier[0].npair, b.tier[1].
 // The separable path for the soft threshold's two-point descriptor: when a basis of this
 // alpha exists, every axis of every level can be transformed, its buffers stay moderate and
 // the direct kernels are estimated to be slower in each of the three kinds of call.  All levels
-// of an instance or none, and one path for every kind of call (the loss of a field that equals
-// its target is exactly 0).  Seconds, fitted to GB300 measurements of both paths (2-D 16^2 ..
+// of an instance or none, and one path for every call that evaluates a descriptor (the loss of a
+// field that equals its target is exactly 0).  Seconds, fitted to GB300 measurements of both paths (2-D 16^2 ..
 // 2048^2, 3-D 16^3 .. 160^3, windows 2 .. 64; captured calls, GPU time), the direct kernels with
 // the padding of their 64 x 32 (adjoint) and 32-wide (forward) tiles.  Loss and gradient, direct
 // and separable: 64^2, +-16: 41 and 49 us; 128^2, +-32, 2 levels: 112 and 57 us; 512^2, +-8: 118
@@ -419,10 +420,17 @@ int usual_pairs(const SepBasis& b) { return std::max(b.tier[0].npair, b.tier[1].
 // (its VJP 187 and 407 us); 600^2 (8 * 3 * 5^2), +-16: 207 and 326 us, +-48: 1032 and 328 us.  The
 // separable cost of a tier grows with its feature pairs (7 in the narrowest), so wide ranges
 // are left to the direct kernels where the window is small.
+// Blocks of the column kernels that hold little cost the same: a strided axis that is short and no
+// power of two from 16 up (2 x 512^2, +-(1, 20, 20): 0.83 ms direct, 3.2 ms separable).  Several phases
+// whose spectra do not fit beside the lines go through the staged kernels, every ordered pair by itself:
+// 100 x 120, +-20, five phases: descriptor 105 us direct, 150 us separable.  There a gradient alone
+// (its upstream coefficients given, so no value depends on the path) may be better off on the direct
+// kernels though the loss is not: 256^2, +-8, five phases: loss and gradient 575 us direct, 511 us
+// separable, VJP 190 and 409 us.
 bool choose_sep(const dmcr_params* p, Plan& pl) {
     if (p->path != DMCR_PATH_AUTO || p->threshold != DMCR_SOFT || pl.desc_kind == DMCR_DESC_S3) return false;
     const double ph = pl.phases;
-    double fwd = 0.0, adj = 0.0, bytes = 0.0, points = 0.0, N = 0.0;
+    double fwd = 0.0, adj = 0.0, bytes = 0.0, points = 0.0, thin = 0.0, N = 0.0;
     bool fast = true;
     for (int l = 0; l < pl.levels; ++l) {
         const LevelGeom& g = pl.g[l];
@@ -433,10 +441,17 @@ bool choose_sep(const dmcr_params* p, Plan& pl) {
         fwd += pairs * padx;
         adj += pairs * padx * (double)(g.adjTilesY * ADJ_ROWS) / (double)g.n[1];
         bytes += 8.0 * (double)g.N * ph * (pl.phases > 1 ? 2 : 1);
-        double per = 0.0;
-        for (int a = 0; a < 3; ++a)
-            if (g.n[a] > 1) per += sep_axis_cost(lv.ax[a]), fast = fast && lv.ax[a].fast;
+        double per = 0.0, few = 0.0;
+        const int last = g.n[0] > 1 ? 0 : 1;
+        for (int a = 0; a < 3; ++a) {
+            if (g.n[a] == 1) continue;
+            per += sep_axis_cost(lv.ax[a]);
+            fast = fast && lv.ax[a].fast;
+            const int held = lv.ax[a].n * (a == last ? lv.colsL : lv.colsY);       // points of a block
+            if (a < 2 && !lv.ax[a].fast && held < 512) few += (a == last ? 1.9e-7 : 0.6e-7) / held;
+        }
         points += ph * (double)g.N * per;
+        thin += ph * (double)g.N * few;
         N += ph * ph * (double)g.N;
     }
     const bool d3 = pl.g[0].n[0] > 1;
@@ -445,15 +460,24 @@ bool choose_sep(const dmcr_params* p, Plan& pl) {
     const double direct_v = 2.2e-5 + 4.15e-13 * adj + 0.6e-10 * N;
     // start-up of the chain of kernels; lengths that are no power of two run more, slower stages
     const double start = fast ? 1.0 : 2.2;
+    const bool staged = pl.phases > 1 && (pl.phases > SEP_FAST_PHASES || !fast);
+    const double staged_d = staged && !fast ? 2.3e-10 * N : 0.0;
+    const double staged_v = staged ? (fast ? 1.7e-10 : 2.1e-10) * N : 0.0, start_v = staged ? 5e-5 : 0.0;
     auto worth = [&](int npair) {
-        const double w = points * npair / 7.0;
-        return bytes * npair <= 16e9 && direct_lg > 1.03 * (4.9e-5 * start + w) && direct_d > 2.5e-5 * start + 0.5 * w &&
+        const double k = npair / 7.0, w = points * k, lg = 1.03 * (4.9e-5 * start + w + thin * k);
+        return bytes * npair <= 16e9 && direct_lg > lg && direct_d > 2.5e-5 * start + 0.5 * w &&
+               direct_d * std::min(4.0, direct_lg / lg) > 2.5e-5 * start + 0.5 * w + staged_d * k &&
                direct_v > 3.3e-5 * start + 0.8 * w;
+    };
+    auto worth_vjp = [&](int npair) {
+        const double k = npair / 7.0;
+        return direct_v > 3.3e-5 * start + start_v + (0.8 * (points + thin) + staged_v) * k;
     };
     if (!worth(1)) return false;
     pl.basis = sep_basis(p->alpha);
     while (pl.sep_tiers < pl.basis->ntier && worth(pl.basis->tier[pl.sep_tiers].npair)) {
         pl.sep_pairs = std::max(pl.sep_pairs, pl.basis->tier[pl.sep_tiers].npair);
+        if (pl.sep_vjp == pl.sep_tiers && worth_vjp(pl.basis->tier[pl.sep_tiers].npair)) ++pl.sep_vjp;
         ++pl.sep_tiers;
     }
     return pl.sep_tiers > 0;
@@ -2122,6 +2146,13 @@ dmcr_status dmcr_loss_grad(const dmcr_params* p, const dmcr_loss_opts* opts, con
                        "dmcr_loss_grad launch");
 }
 
+// The plan of a call for the gradient alone (the workspace holds both paths' buffers).
+static void plan_vjp(Plan& pl) {
+    if (!pl.sep) return;
+    pl.sep = pl.sep_vjp > 0;
+    pl.sep_tiers = pl.sep_vjp;
+}
+
 dmcr_status dmcr_descriptor_vjp(const dmcr_params* p, const float* field, const float* grad_desc, float* grad_field,
                                 void* ws, size_t ws_bytes, void* stream) {
     Plan pl;
@@ -2130,6 +2161,7 @@ dmcr_status dmcr_descriptor_vjp(const dmcr_params* p, const float* field, const 
         return fail(DMCR_EINVAL, "field/grad_desc/grad_field is NULL");
     DMCR_TRY(check_ws(pl, ws, ws_bytes));
     DMCR_TRY(prepare_device());
+    plan_vjp(pl);
     Inst x = single(pl, ws);
     x.field = field;
     x.target = grad_desc;
@@ -2286,6 +2318,7 @@ dmcr_status dmcr_descriptor_vjp_batched(int count, const dmcr_params* params, co
         return fail(DMCR_EINVAL, "NULL pointer array");
     DMCR_TRY(batch_ws(B, ws, ws_bytes));
     DMCR_TRY(prepare_device());
+    for (Plan& pl : B.plans) plan_vjp(pl);
     std::vector<Inst> in = batch_insts(B, ws);
     for (int i = 0; i < count; ++i) {
         if (fields[i] == nullptr || grad_descs[i] == nullptr || grad_fields[i] == nullptr)
