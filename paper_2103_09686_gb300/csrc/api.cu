@@ -927,13 +927,17 @@ S3Job s3_job(const Inst& x, int l, bool loss) {
     return j;
 }
 
-// blocks of one instance in the pyramid launch
+// the pyramid launch: the coarser levels of fields that are not large, and what the separable path
+// wants to know of the values
+bool one_pass(const Plan& pl) { return pl.sep || (pl.levels > 1 && pl.N1 <= PREP_BELOW); }
+
+// its blocks for one instance: few on the separable path, whose kernels read what each of them leaves
 int prep_blocks(const Plan& pl) {
     const LevelGeom& g = pl.g[0];
     const int64_t tiles = (pl.ndim == 2 ? 1 : ceil_div(g.n[0], PREP_TILE3)) *
                           ceil_div(g.n[1], pl.ndim == 2 ? PREP_TILE2 : PREP_TILE3) *
                           ceil_div(g.n[2], pl.ndim == 2 ? PREP_TILE2 : PREP_TILE3) * pl.phases;
-    return (int)std::min<int64_t>(PREP_BLOCKS, tiles);
+    return (int)std::min<int64_t>(pl.sep ? PREP_BLOCKS : 16 * PREP_BLOCKS, tiles);
 }
 
 // sep_desc goes straight on to the rows of G
@@ -1142,7 +1146,7 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
         int64_t pb = 0;
         for (const Inst& x : in) {
             const Plan& pl = *x.pl;
-            if (pl.levels == 1 && !pl.sep) continue;
+            if (!one_pass(pl)) continue;
             PrepSeg p{};
             p.ndim = pl.ndim;
             p.coarse = std::min(pl.levels - 1, pl.ndim == 2 ? PREP_LEVELS2 : PREP_LEVELS3);
@@ -1170,7 +1174,7 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
             std::vector<RestrictSeg> v;
             int64_t b = 0;
             for (const Inst& x : in) {
-                if (x.pl->levels <= l || l <= (x.pl->ndim == 2 ? PREP_LEVELS2 : PREP_LEVELS3)) continue;
+                if (x.pl->levels <= l || (one_pass(*x.pl) && l <= (x.pl->ndim == 2 ? PREP_LEVELS2 : PREP_LEVELS3))) continue;
                 const LevelGeom& g = x.pl->g[l];
                 for (int ph = 0; ph < x.pl->phases; ++ph) {
                     RestrictSeg r{};
@@ -1456,7 +1460,7 @@ dmcr_status prepare(std::vector<Inst>& in, unsigned flags, char* tab, size_t cap
                     fvs.push_back(f);
                 } else {
                     f.blockStart = fb;
-                    fb += ceil_div(N1, ELEM_TH);
+                    fb += ceil_div(N1, (int64_t)ELEM_TH * fin_rounds(N1));
                     fv.push_back(f);
                 }
             }

@@ -59,6 +59,7 @@ __device__ __forceinline__ void prep_tiles(const PrepSeg& sg, int blk, float* sh
     const int64_t N = (int64_t)n0 * n1 * n2;
     const int t0 = ND == 2 ? 1 : (n0 + TILE - 1) / TILE, t1 = (n1 + TILE - 1) / TILE, t2 = (n2 + TILE - 1) / TILE;
     const int64_t tiles = (int64_t)t0 * t1 * t2 * sg.phases;
+    const bool look = sg.tiers != nullptr || sg.excess != nullptr;
     // sum of the values of one phase: each warp its own share, msh[phase][warp]
     float sum = 0.f;
     int summed = 0;
@@ -95,8 +96,10 @@ __device__ __forceinline__ void prep_tiles(const PrepSeg& sg, int blk, float* sh
                 const int xx = x + (k & 1), yy = y + (k >> 1 & 1), zz = z + (k >> 2);
                 v[k] = xx < n2 && yy < n1 && zz < n0 ? f[((int64_t)zz * n1 + yy) * n2 + xx] : 0.f;
             }
+            if (look) {
 #pragma unroll
-            for (int k = 0; k < (ND == 2 ? 4 : 8); ++k) see(v[k], ph);
+                for (int k = 0; k < (ND == 2 ? 4 : 8); ++k) see(v[k], ph);
+            }
             if (sg.coarse == 0) continue;
             float s;
             if constexpr (ND == 2) s = ((v[0] + v[1]) + (v[2] + v[3])) * 0.25f;
@@ -413,10 +416,11 @@ __global__ void __launch_bounds__(ELEM_TH) final_kernel(const FinalSeg* __restri
     const FinalArgs& a = sg.a;
     const int64_t N1 = a.n1[0] * a.n1[1] * a.n1[2];
     const int q = threadIdx.x / NPOS, pl = threadIdx.x % NPOS;
-    const int64_t i = ((int64_t)blockIdx.x - sg.blockStart) * NPOS + pl;
-    const bool valid = i < N1;
+    const int rounds = SUB == 1 ? fin_rounds(N1) : 1;
+    int64_t i = ((int64_t)blockIdx.x - sg.blockStart) * NPOS * rounds + pl;
     float M = 0.f, m0 = 0.f, v0 = 0.f;
-    if (valid && q == 0) {
+    auto load = [&]() {
+        if (i >= N1 || q != 0) return;
         if (a.M != nullptr) {
             M = a.M[i];
             m0 = a.m[i];
@@ -424,32 +428,38 @@ __global__ void __launch_bounds__(ELEM_TH) final_kernel(const FinalSeg* __restri
         } else if (a.sc != nullptr && a.field != nullptr) {
             M = a.field[i];
         }
-    }
+    };
+    load();
     dep_wait();
     dep_trigger();
     if (sg.done != nullptr && *sg.done) return;
-    float g = valid ? chunk_sums<SUB>(a, i, q) : 0.f;
-    if constexpr (SUB > 1) {
-        __shared__ float part[SUB][NPOS];
-        part[q][pl] = g;
-        __syncthreads();
-        if (q != 0) return;
-        for (int u = 1; u < SUB; ++u) g += part[u][pl];
-    }
-    if (!valid) return;
-    if (a.sc != nullptr && a.field != nullptr) {
-        const float f = a.M != nullptr && a.M != a.field ? a.field[i] : M;
-        const float ex = box_excess(f);
-        const float dex = f > 1.f ? 1.f : (f < 0.f ? -1.f : 0.f);
-        g = fmaf(a.sc->pen_coef * ex, dex, g);
-    }
-    if (a.grad_out != nullptr) a.grad_out[i] = g;
-    if (a.M != nullptr) {
-        const float m = fmaf(a.beta1, m0, (1.f - a.beta1) * g);
-        const float v = fmaf(a.beta2, v0, (1.f - a.beta2) * g * g);
-        a.m[i] = m;
-        a.v[i] = v;
-        a.M[i] = M - a.sc->lr_t * m / (sqrtf(v) + a.eps);
+    for (int r = 0;;) {
+        float g = i < N1 ? chunk_sums<SUB>(a, i, q) : 0.f;
+        if constexpr (SUB > 1) {
+            __shared__ float part[SUB][NPOS];
+            part[q][pl] = g;
+            __syncthreads();
+            if (q != 0) return;
+            for (int u = 1; u < SUB; ++u) g += part[u][pl];
+        }
+        if (i >= N1) return;
+        if (a.sc != nullptr && a.field != nullptr) {
+            const float f = a.M != nullptr && a.M != a.field ? a.field[i] : M;
+            const float ex = box_excess(f);
+            const float dex = f > 1.f ? 1.f : (f < 0.f ? -1.f : 0.f);
+            g = fmaf(a.sc->pen_coef * ex, dex, g);
+        }
+        if (a.grad_out != nullptr) a.grad_out[i] = g;
+        if (a.M != nullptr) {
+            const float m = fmaf(a.beta1, m0, (1.f - a.beta1) * g);
+            const float v = fmaf(a.beta2, v0, (1.f - a.beta2) * g * g);
+            a.m[i] = m;
+            a.v[i] = v;
+            a.M[i] = M - a.sc->lr_t * m / (sqrtf(v) + a.eps);
+        }
+        if (++r >= rounds) return;
+        i += NPOS;
+        load();
     }
 }
 

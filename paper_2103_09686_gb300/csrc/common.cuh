@@ -505,6 +505,13 @@ constexpr int ELEM_TH = 256;   // pixels per restrict block; threads per final b
 constexpr int FIN_SUB = 8;     // gradient assembly of a small field: threads per position (each sums
                                // every 8th chunk)
 constexpr int64_t FIN_SUB_BELOW = 1 << 16;   // fields of fewer positions use FIN_SUB threads each
+// Positions of one thread of the gradient assembly: several in a large field, whose blocks each read
+// their arguments and wait once (8192^2, three levels: 884 us with one, 765 with four, 742 with eight; 1024^2:
+// 23 with one, 29 with four).
+__host__ __device__ inline int fin_rounds(int64_t N1) { return N1 >= 1 << 23 ? 8 : (N1 >= 1 << 21 ? 4 : 1); }
+// Fields from here on build their levels one launch each where only levels are wanted: the tiles of the
+// one-pass pyramid pay for short launches (2048^2 21 us and 23, 4096^2, two levels 47 and 28).
+constexpr int64_t PREP_BELOW = (int64_t)1 << 22;
 
 // Segment of linear block b: the last segment whose blockStart <= b.
 template <typename S>
