@@ -66,9 +66,11 @@ enum { DMCR_SOFT = 0, DMCR_IDENTITY = 1 };           /* threshold (Sec. 3.2.4; f
  * estimated to be faster, the separable path: f((u + v) / 2)^2 as a short sum of products
  * over a range of values, evaluated by FP32 transforms with FP32-level accuracy.  The range
  * is taken from the field on the device; NaN, fields beyond [-2.25, 2.5] (alpha = 10) and dark
- * fields (a phase without a value of 1/2) are left to the DIRECT kernels of the same call.  The first plan of an alpha in a
- * process builds its tables on the host (about 0.1 s), its first separable call on a device copies
- * them there on a private stream. */
+ * fields (a phase without a value of 1/2) are left to the DIRECT kernels of the same call.  A
+ * problem has one path for all calls that evaluate its descriptor; dmcr_descriptor_vjp may take the
+ * DIRECT kernels where they are faster for it.  The first plan of an alpha in a process builds
+ * its tables on the host (about 0.1 s), its first separable call on a device copies them there on
+ * a private stream. */
 enum { DMCR_PATH_AUTO = 0, DMCR_PATH_DIRECT = 1, DMCR_PATH_FFT = 2 };
 enum { DMCR_LOSS_NORM = 0, DMCR_LOSS_SQUARED = 1 };  /* L = E(1 + lambda0 E_bc)  |  E^2 (1 + lambda0 E_bc) */
 enum { DMCR_PROLONG_ADJOINT_ACCUMULATE = 0, DMCR_PROLONG_INJECT = 1 };

@@ -48,8 +48,9 @@ __global__ void restrict_kernel(const RestrictSeg* __restrict__ segs, int nseg) 
 
 // All coarser levels of a tile in one pass over the finest field (each the mean of its 2^d
 // children, summed as restrict_one does), with the tier of the values' range and the box
-// excess, which need the same pass (and the phases that are bright enough for the transforms).  A thread reads a 2^d block; the coarser means go through
-// shared memory.  One launch of a microsecond or two instead of one per level.
+// excess, which need the same pass (and the phases that are bright enough for the transforms).  A
+// thread reads a 2^d block; the coarser means go through shared memory.  One launch of a microsecond
+// or two instead of one per level.
 template <int ND>
 __device__ __forceinline__ void prep_tiles(const PrepSeg& sg, int blk, float* sh, float& lo, float& hi, int& bad,
                                            int& bright, float* msh, float& e2, float& e2c) {
